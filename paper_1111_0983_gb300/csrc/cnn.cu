@@ -11,14 +11,21 @@
 // by di*d*Wp + dj*d -- is a shift of the operand's start address by a whole
 // number of 16-byte rows: the implicit GEMM needs no im2col copy.
 //
-// Convolution (forward, and backward to the input): a CTA owns 128
-// consecutive pixels (M = 128), N = output channels, K = input channels in
-// slices of 16, summed over the 9 taps; the three input row segments it
-// needs (di = -1, 0, 1, each 128 + 2d pixels) are staged in shared memory
-// once, the weights too, and one thread issues the 9 * C_in / 16 MMAs into
-// a TMEM accumulator.  The epilogue (bias, ReLU, BF16) runs from TMEM.
-// Weight gradients: D_t[c_out][c_in] = sum_q dz[q][c_out] x[q + s_t][c_in]
-// with the pixels as K, both operands MN-major, one accumulator per tap.
+// Tiles and chains.  A tile is 128 consecutive pixels of one image row (M =
+// 128 of the MMAs).  With dilation d the tiles of rows i, i + d, i + 2d, ... in
+// one column of tiles share their input rows: row i is tap row +1, 0 and -1 of
+// three successive tiles.  A CTA therefore walks down such a chain with a ring
+// of four row segments of 128 + 2d pixels in shared memory: each tile brings in
+// one new segment (18.6 KB at d = 81) instead of three.
+//
+// Convolution (forward, and backward to the input): N = output channels, K =
+// input channels in slices of 16, summed over the 9 taps.  Warp roles: a
+// producer (bulk copies), an MMA issuer, four epilogue warps; four TMEM
+// accumulators, so that loads, MMAs and epilogues of different tiles overlap.
+// Weight gradients: D[slot, ci][tap column, co] = sum_q x[q][ci] dz[q - s][co]
+// with the pixels as K, both operands MN-major; the 16 channel groups of the
+// whole ring (4 slots x 4 groups) are the M = 128 rows of one MMA and three
+// shifted copies of dz its N = 96 columns, so one MMA serves all nine taps.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
@@ -39,8 +46,11 @@ constexpr int kCin[kLayers] = {4, 32, 32, 32, 32, 32};
 constexpr int kCout[kLayers] = {32, 32, 32, 32, 32, 2};
 constexpr int kTile = 128;            // pixels per CTA (M)
 constexpr int kMaxDil = 96;
-constexpr int kSeg = kTile + 2 * kMaxDil;   // staged pixels per row segment
-constexpr long kWaitLimit = 1L << 24; // bounded mbarrier polls
+constexpr int kRing = 4;              // row segments in shared memory
+constexpr int kAcc = 4;               // TMEM accumulators of the convolution
+constexpr int kDzStages = 4;          // staged gradient tiles of the weight gradients
+constexpr int kConvThreads = 192;     // producer, MMA issuer, four epilogue warps
+constexpr long kWaitLimit = 1L << 22; // bounded mbarrier polls
 
 // ------------------------------------------------------------- PTX helpers
 __device__ __forceinline__ uint32_t smem_u32(const void *p) {
@@ -75,9 +85,12 @@ __device__ __forceinline__ void mma_commit(uint32_t mbar) {
                  : "memory");
 }
 
-__device__ __forceinline__ void mbar_init(uint32_t mbar) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(mbar) : "memory");
+__device__ __forceinline__ void mbar_init(uint32_t mbar, uint32_t count) {
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(mbar), "r"(count) : "memory");
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+}
+__device__ __forceinline__ void mbar_arrive(uint32_t mbar) {
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(mbar) : "memory");
 }
 
 // polls the barrier's phase with a bound; false if it never completed
@@ -133,36 +146,31 @@ __device__ __forceinline__ float bf16_hi(uint32_t w) { return __uint_as_float(w 
 struct Geo {
     int npix, Hp, Wp, H, W, P;
     int gs;        // rows between channel groups (npix plus zero guard rows on both sides)
-    __device__ __forceinline__ bool interior(int q, int *b, int *i, int *j) const {
-        const int plane = Hp * Wp;
-        *b = q / plane;
-        const int rem = q - *b * plane;
-        *i = rem / Wp;
-        *j = rem - *i * Wp;
-        return *i >= P && *i < P + H && *j >= P && *j < P + W;
+};
+
+// ------------------------------------------------------------ convolution
+// Chains: item = ((image * cols + column) * res + residue) * parts + part; its
+// tiles are rows residue + (part * len + k) * dil, k < cnt.
+struct Chains {
+    int H, dil, cols, res, parts, len, items;
+    // false: the part lies past the chain's end
+    __device__ __forceinline__ bool item(int t, int *b, int *c, int *row0, int *cnt) const {
+        const int part = t % parts;
+        t /= parts;
+        const int r = t % res;
+        t /= res;
+        *c = t % cols;
+        *b = t / cols;
+        const int n = (H - r + dil - 1) / dil, j0 = part * len;
+        *row0 = r + j0 * dil;
+        *cnt = min(len, n - j0);
+        return *cnt > 0;
     }
 };
 
-// stages the three row segments (di = -1, 0, 1) of G channel groups around
-// pixels [q0, q0 + 128): smem[g][s][r] = x[g][q0 + (s-1) d Wp - d + r]
-template <int G>
-__device__ __forceinline__ void stage_halo(uint4 *sm, const uint4 *__restrict__ x, int npix, int gs, int q0, int Wp,
-                                           int dil) {
-    const int len = kTile + 2 * dil;
-    for (int e = threadIdx.x; e < G * 3 * len; e += blockDim.x) {
-        const int g = e / (3 * len);
-        const int rem = e - g * 3 * len;
-        const int s = rem / len, r = rem - s * len;
-        const int q = q0 + (s - 1) * dil * Wp - dil + r;
-        uint4 v = make_uint4(0, 0, 0, 0);
-        if (q >= 0 && q < npix) v = x[(size_t)g * gs + q];
-        sm[(g * 3 + s) * kSeg + r] = v;
-    }
-}
-
-// ------------------------------------------------------------ convolution
 // MODE 0: y = bf16(relu(acc + bias)); 1: out[b][c][i][j] = acc + bias (c < 2);
-// 2: y = bf16(acc * (gate > 0)) (backward to the input of the layer below)
+// 2: y = bf16(acc * (gate > 0)) (backward to the input of the layer below) and
+// db[c] += the sum of the stored values over the pixels
 struct ConvArgs {
     const uint4 *x;       // [GIN][npix] pixel rows
     const uint4 *w;       // [9][GIN][NOUT] rows of 8 input channels
@@ -170,7 +178,9 @@ struct ConvArgs {
     uint4 *y;             // [NOUT / 8][npix]
     float *out;           // MODE 1: [B][2][H][W]
     const uint4 *gate;    // MODE 2: [NOUT / 8][npix]
+    float *db;            // MODE 2: NOUT
     Geo geo;
+    Chains ch;
     int dil;
     int *err;
 };
@@ -187,266 +197,450 @@ __device__ __forceinline__ void mbar_expect(uint32_t mbar, uint32_t bytes) {
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(mbar), "r"(bytes) : "memory");
 }
 
-// Persistent convolution: a CTA keeps the layer's weights in shared memory
-// and walks the tiles blockIdx.x, blockIdx.x + gridDim.x, ...  The three
-// input row segments of the next tile are brought in by bulk copies into the
-// other half of a double buffer while the current tile's MMAs and epilogue
-// run.  The activation buffers carry zero guard rows before and after each
-// channel group, so every segment lies inside the allocation.
+// Positions number the segments a CTA loads, over all of its items; position p
+// lies in ring slot p % kRing.  Tile k of an item whose first segment has
+// position p0 reads positions p0 + k, + 1, + 2 (tap rows -1, 0, +1).
+// Every wait is bounded; after one that ran out (ok = false) a role waits no
+// more, and the kernel reports it through a.err.
+// Four CTAs an SM at small dilations, two at 81 (TMEM columns, shared memory):
+// with one segment in flight a CTA, several CTAs hide the copies' latency.
+// Measured, 8 images of 513^2, 32 -> 32 channels, forward: 366 us a layer with
+// three segments a tile, one accumulator and the border's tiles computed too;
+// 81-96 us so (2.9-3.4 TB/s of activations read and written once).  Backward to
+// the input 721 -> 124-149 us (reads the gate too).
 template <int GIN, int NOUT, int MODE>
-__global__ void __launch_bounds__(128) k_conv(ConvArgs a, int ntiles) {
+__global__ void __launch_bounds__(kConvThreads) k_conv(ConvArgs a) {
     extern __shared__ __align__(128) unsigned char smem[];
-    constexpr int HALO = GIN * 3 * kSeg;                          // rows per buffer
-    uint4 *sx = reinterpret_cast<uint4 *>(smem);                  // 2 buffers
-    uint4 *sw = sx + 2 * HALO;                                    // 9 * GIN * NOUT rows
-    uint64_t *mbar = reinterpret_cast<uint64_t *>(sw + 9 * GIN * NOUT);   // full[2], mma
-    uint32_t *tslot = reinterpret_cast<uint32_t *>(mbar + 3);
+    const int seg = kTile + 2 * a.dil;                            // pixels of a segment
+    uint4 *sx = reinterpret_cast<uint4 *>(smem);                  // [kRing][GIN][seg]
+    uint4 *sw = sx + kRing * GIN * seg;                           // 9 * GIN * NOUT rows
+    uint64_t *bars = reinterpret_cast<uint64_t *>(sw + 9 * GIN * NOUT);
+    uint32_t *tslot = reinterpret_cast<uint32_t *>(bars + 2 * kRing + 2 * kAcc + 1);
+    const uint32_t full = smem_u32(bars), empty = full + 8 * kRing, afull = empty + 8 * kRing,
+                   afree = afull + 8 * kAcc, wbar = afree + 8 * kAcc;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int len = kTile + 2 * a.dil;
-    const uint32_t seg_bytes = (uint32_t)len * 16;
-    const uint32_t full0 = smem_u32(&mbar[0]), full1 = smem_u32(&mbar[1]), mma_bar = smem_u32(&mbar[2]);
 
-    if (warp == 0) tmem_alloc<32>(smem_u32(tslot));
+    if (warp == 1) tmem_alloc<kAcc * NOUT>(smem_u32(tslot));
     if (threadIdx.x == 0) {
-        mbar_init(full0);
-        mbar_init(full1);
-        mbar_init(mma_bar);
+        for (int i = 0; i < kRing; i++) {
+            mbar_init(full + 8 * i, 1);
+            mbar_init(empty + 8 * i, 1);
+        }
+        for (int i = 0; i < kAcc; i++) {
+            mbar_init(afull + 8 * i, 1);
+            mbar_init(afree + 8 * i, 4);   // one arrival an epilogue warp
+        }
+        mbar_init(wbar, 1);
     }
-    for (int e = threadIdx.x; e < 9 * GIN * NOUT; e += blockDim.x) sw[e] = a.w[e];
-    fence_async_smem();
     tc_before();
     __syncthreads();
     tc_after();
     const uint32_t tmem = *tslot;
-
-    // the producer: the segments of tile t into buffer b
-    auto load_tile = [&](int t, int b) {
-        const uint32_t fb = b ? full1 : full0;
-        mbar_expect(fb, (uint32_t)(GIN * 3) * seg_bytes);
-        const int q0 = t * kTile;
-        for (int g = 0; g < GIN; g++)
-            for (int sgm = 0; sgm < 3; sgm++) {
-                const int q = q0 + (sgm - 1) * a.dil * a.geo.Wp - a.dil;
-                bulk_g2s(smem_u32(sx + b * HALO + (g * 3 + sgm) * kSeg), a.x + (size_t)g * a.geo.gs + q, seg_bytes,
-                         fb);
-            }
-    };
-    if (threadIdx.x == 0 && (int)blockIdx.x < ntiles) load_tile(blockIdx.x, 0);
-
-    uint32_t ph_full[2] = {0, 0}, ph_mma = 0;
     bool ok = true;
-    int k = 0;
-#pragma unroll 1
-    for (int t = blockIdx.x; t < ntiles; t += gridDim.x, k++) {
-        const int b = k & 1;
-        const bool w1 = mbar_wait(b ? full1 : full0, ph_full[b]);
-        ph_full[b] ^= 1;
-        ok = ok && w1;
-        if (threadIdx.x == 0) {
-            constexpr uint32_t idesc = idesc_bf16(kTile, NOUT, 0, 0);
-            const uint32_t xa = smem_u32(sx + b * HALO), wa = smem_u32(sw);
-            uint32_t acc = 0;
-#pragma unroll 1
-            for (int tap = 0; tap < 9; tap++) {
-                const int sgm = tap / 3, dj = tap % 3 - 1;
-                const int r0 = a.dil + dj * a.dil;
-#pragma unroll
-                for (int gp = 0; gp < GIN / 2; gp++) {
-                    const uint64_t ad = sdesc(xa + ((2 * gp * 3 + sgm) * kSeg + r0) * 16, 3 * kSeg * 16, 128);
-                    const uint64_t bd = sdesc(wa + ((tap * GIN + 2 * gp) * NOUT) * 16, NOUT * 16, 128);
-                    mma_bf16(tmem, ad, bd, idesc, acc);
-                    acc = 1;
+    auto wait = [&](uint32_t bar, uint32_t parity) {
+        if (ok) ok = mbar_wait(bar, parity & 1u);
+    };
+    int b, c, row0, cnt;
+
+    if (warp == 0) {
+        if (lane == 0) {   // producer
+            mbar_expect(wbar, 9 * GIN * NOUT * 16);
+            bulk_g2s(smem_u32(sw), a.w, 9 * GIN * NOUT * 16, wbar);
+            int pos = 0;
+            for (int t = blockIdx.x; t < a.ch.items; t += gridDim.x) {
+                if (!a.ch.item(t, &b, &c, &row0, &cnt)) continue;
+                // pixel of the first segment: row row0 - dil, columns from dil before the tile
+                long q = ((long)b * a.geo.Hp + a.geo.P + row0 - a.dil) * a.geo.Wp + a.geo.P + c * kTile - a.dil;
+                for (int p = 0; p < cnt + 2; p++, pos++, q += (long)a.dil * a.geo.Wp) {
+                    const int s = pos % kRing;
+                    wait(empty + 8 * s, (uint32_t)(pos / kRing) + 1u);
+                    if (!ok) break;
+                    mbar_expect(full + 8 * s, (uint32_t)(GIN * seg * 16));
+                    for (int g = 0; g < GIN; g++)
+                        bulk_g2s(smem_u32(sx + (s * GIN + g) * seg), a.x + (long)g * a.geo.gs + q, (uint32_t)(seg * 16),
+                                 full + 8 * s);
                 }
+                if (!ok) break;
             }
-            mma_commit(mma_bar);
-            // the other buffer held the previous tile, whose MMAs completed
-            // before its epilogue (below, in the previous iteration)
-            if (t + (int)gridDim.x < ntiles) load_tile(t + gridDim.x, b ^ 1);
+            // every copy has landed before the CTA ends (in a complete run the
+            // MMAs have waited for them already)
+            for (int p = max(0, pos - kRing); p < pos; p++) mbar_wait(full + 8 * (p % kRing), (uint32_t)(p / kRing) & 1u);
+            mbar_wait(wbar, 0);
         }
         __syncwarp();
-        const bool w2 = mbar_wait(mma_bar, ph_mma);
-        ph_mma ^= 1;
-        ok = ok && w2;
-        tc_after();
-
-        float v[NOUT];
-        const uint32_t lane_addr = tmem + ((uint32_t)(warp * 32) << 16);
-        tmem_ld16(lane_addr, v);
-        if (NOUT == 32) tmem_ld16(lane_addr + 16, v + 16);
-
-        const int q = t * kTile + warp * 32 + lane;
-        int bb, i, j;
-        if (q < a.geo.npix) {
-            const bool in = a.geo.interior(q, &bb, &i, &j) && ok;
-            if (MODE == 1) {
-                if (in) {
-                    const int H = a.geo.H, W = a.geo.W, P = a.geo.P;
-                    for (int c = 0; c < 2; c++)
-                        a.out[(((size_t)bb * 2 + c) * H + (i - P)) * W + (j - P)] = v[c] + a.bias[c];
-                }
-            } else {
+    } else if (warp == 1) {
+        if (lane == 0) {   // MMA issuer
+            constexpr uint32_t idesc = idesc_bf16(kTile, NOUT, 0, 0);
+            const uint32_t xa = smem_u32(sx), wa = smem_u32(sw);
+            int pos = 0, tile = 0;
+            wait(wbar, 0);
+            for (int t = blockIdx.x; t < a.ch.items && ok; t += gridDim.x) {
+                if (!a.ch.item(t, &b, &c, &row0, &cnt)) continue;
+                for (int k = 0; k < cnt; k++, tile++) {
+                    for (int p = k ? pos + k + 2 : pos; p <= pos + k + 2; p++)
+                        wait(full + 8 * (p % kRing), (uint32_t)(p / kRing));
+                    const int ac = tile % kAcc;
+                    wait(afree + 8 * ac, (uint32_t)(tile / kAcc) + 1u);
+                    if (!ok) break;
+                    tc_after();
+                    const uint32_t d = tmem + (uint32_t)(ac * NOUT);
+                    uint32_t acc = 0;
+#pragma unroll 1
+                    for (int tr = 0; tr < 3; tr++) {
+                        const uint32_t xs = xa + (uint32_t)(((pos + k + tr) % kRing) * GIN * seg) * 16;
 #pragma unroll
-                for (int g = 0; g < NOUT / 8; g++) {
-                    float o[8];
-                    if (MODE == 0) {
+                        for (int tc = 0; tc < 3; tc++)
 #pragma unroll
-                        for (int e = 0; e < 8; e++) o[e] = in ? fmaxf(v[8 * g + e] + a.bias[8 * g + e], 0.0f) : 0.0f;
-                    } else {
-                        const uint4 gt = a.gate[(size_t)g * a.geo.gs + q];
-                        const uint32_t gw[4] = {gt.x, gt.y, gt.z, gt.w};
-#pragma unroll
-                        for (int e = 0; e < 4; e++) {
-                            o[2 * e] = (in && bf16_lo(gw[e]) > 0.0f) ? v[8 * g + 2 * e] : 0.0f;
-                            o[2 * e + 1] = (in && bf16_hi(gw[e]) > 0.0f) ? v[8 * g + 2 * e + 1] : 0.0f;
-                        }
+                            for (int gp = 0; gp < GIN / 2; gp++) {
+                                const uint64_t ad = sdesc(xs + (uint32_t)(2 * gp * seg + tc * a.dil) * 16, seg * 16, 128);
+                                const uint64_t bd =
+                                    sdesc(wa + (((tr * 3 + tc) * GIN + 2 * gp) * NOUT) * 16, NOUT * 16, 128);
+                                mma_bf16(d, ad, bd, idesc, acc);
+                                acc = 1;
+                            }
                     }
-                    a.y[(size_t)g * a.geo.gs + q] = make_uint4(pack_bf16(o[0], o[1]), pack_bf16(o[2], o[3]),
-                                                               pack_bf16(o[4], o[5]), pack_bf16(o[6], o[7]));
+                    mma_commit(afull + 8 * ac);
+                    mma_commit(empty + 8 * ((pos + k) % kRing));
+                    if (k + 1 == cnt) {   // the item's last two segments serve no other tile
+                        mma_commit(empty + 8 * ((pos + k + 1) % kRing));
+                        mma_commit(empty + 8 * ((pos + k + 2) % kRing));
+                    }
+                }
+                pos += cnt + 2;
+            }
+        }
+        __syncwarp();
+    } else {   // epilogue: warp w reads the TMEM lanes 32 (w % 4)
+        const int ew = warp & 3;
+        const uint32_t lane_addr = tmem + ((uint32_t)(ew * 32) << 16);
+        float dbs[MODE == 2 ? NOUT : 1];
+#pragma unroll
+        for (int e = 0; e < (MODE == 2 ? NOUT : 1); e++) dbs[e] = 0.0f;
+        float bias[MODE == 0 ? NOUT : 1];
+        if (MODE == 0) {
+#pragma unroll
+            for (int e = 0; e < NOUT; e++) bias[MODE == 0 ? e : 0] = a.bias[e];
+        }
+        int tile = 0;
+        for (int t = blockIdx.x; t < a.ch.items && ok; t += gridDim.x) {
+            if (!a.ch.item(t, &b, &c, &row0, &cnt)) continue;
+            const int j = c * kTile + ew * 32 + lane;
+            const bool in = j < a.geo.W;
+            for (int k = 0; k < cnt && ok; k++, tile++) {
+                const int i = row0 + k * a.dil;
+                const long q = ((long)b * a.geo.Hp + a.geo.P + i) * a.geo.Wp + a.geo.P + j;
+                uint4 gt[MODE == 2 ? NOUT / 8 : 1];
+                if (MODE == 2 && in) {
+#pragma unroll
+                    for (int g = 0; g < NOUT / 8; g++) gt[g] = a.gate[(long)g * a.geo.gs + q];
+                }
+                const int ac = tile % kAcc;
+                wait(afull + 8 * ac, (uint32_t)(tile / kAcc));
+                ok = __all_sync(0xffffffffu, ok);
+                if (!ok) break;
+                tc_after();
+                float v[NOUT];
+                tmem_ld16(lane_addr + (uint32_t)(ac * NOUT), v);
+                if (NOUT == 32) tmem_ld16(lane_addr + (uint32_t)(ac * NOUT) + 16, v + 16);
+                tc_before();   // the accumulator is read: the issuer may overwrite it
+                __syncwarp();
+                if (lane == 0) mbar_arrive(afree + 8 * ac);
+                if (!in) continue;
+                if (MODE == 1) {
+                    for (int ch = 0; ch < 2; ch++)
+                        a.out[(((size_t)b * 2 + ch) * a.geo.H + i) * a.geo.W + j] = v[ch] + a.bias[ch];
+                } else {
+#pragma unroll
+                    for (int g = 0; g < NOUT / 8; g++) {
+                        float o[8];
+                        if (MODE == 0) {
+#pragma unroll
+                            for (int e = 0; e < 8; e++) o[e] = fmaxf(v[8 * g + e] + bias[MODE == 0 ? 8 * g + e : 0], 0.0f);
+                        } else {
+                            const uint32_t gw[4] = {gt[g].x, gt[g].y, gt[g].z, gt[g].w};
+#pragma unroll
+                            for (int e = 0; e < 4; e++) {
+                                o[2 * e] = bf16_lo(gw[e]) > 0.0f ? v[8 * g + 2 * e] : 0.0f;
+                                o[2 * e + 1] = bf16_hi(gw[e]) > 0.0f ? v[8 * g + 2 * e + 1] : 0.0f;
+                            }
+                        }
+                        const uint32_t w[4] = {pack_bf16(o[0], o[1]), pack_bf16(o[2], o[3]), pack_bf16(o[4], o[5]),
+                                               pack_bf16(o[6], o[7])};
+                        if (MODE == 2) {
+#pragma unroll
+                            for (int e = 0; e < 4; e++) {
+                                dbs[8 * g + 2 * e] += bf16_lo(w[e]);
+                                dbs[8 * g + 2 * e + 1] += bf16_hi(w[e]);
+                            }
+                        }
+                        a.y[(long)g * a.geo.gs + q] = make_uint4(w[0], w[1], w[2], w[3]);
+                    }
                 }
             }
         }
-        // the accumulator is read before the next tile's MMAs overwrite it
-        tc_before();
-        __syncthreads();
-        tc_after();
+        if (MODE == 2) {
+#pragma unroll
+            for (int e = 0; e < NOUT; e++) {
+                float s = dbs[e];
+                for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+                if (lane == 0) atomicAdd(&a.db[e], s);
+            }
+        }
     }
-    if (!ok && threadIdx.x == 0) atomicExch(a.err, 1);
+    if (!ok) atomicExch(a.err, 1);
+    tc_before();
     __syncthreads();
-    if (warp == 0) {
+    if (warp == 1) {
         tc_after();
-        tmem_free<32>(tmem);
+        tmem_free<kAcc * NOUT>(tmem);
     }
 }
 
 // --------------------------------------------------------- weight gradient
-// D_t[co][ci] += sum over the CTA's pixel tiles of dz[q][co] x[q + s_t][ci];
-// rows co >= 8 GA of the M = 128 operand read unrelated shared memory and
-// are never stored.
+// dw[co][ci][t] += sum over the CTA's tiles of x[q][ci] dz[q - s_t][co], with
+// the chains of k_conv.  A ring slot holds one row's 128 pixels of x; a
+// gradient tile is staged three times, shifted by the tap columns, so that one
+// MMA multiplies all 4 slots x GB groups (M rows) of x by the 3 x 8 GA columns
+// of the gradient (K = 16 pixels): the MMA's time is that of reading its A
+// operand, whatever N.  A slot holds tap row (slot - first position) mod 4 of
+// the tile, so the accumulators are kept per class = first position mod 4; the
+// class's fourth slot (being loaded, or of the next item) yields rows nobody
+// reads.  Pixels past the image's last column are staged as zeros.  Bound by
+// the latency of the one x segment in flight (the ring's fourth slot).
+// Measured, 8 images of 513^2: 2469 us a layer with a tap and 16 pixels an MMA
+// and nothing staged ahead, 253 us with the ring and one MMA a tap column, 195
+// us with one MMA for the three.
 struct DwArgs {
     const uint4 *dz;      // [GA][npix]
     const uint4 *x;       // [GB][npix]
     float *dw;            // [co][ci][9] of this layer (FP32, accumulated)
     int cout, cin;        // real channel counts
     Geo geo;
+    Chains ch;
     int dil;
-    int ntiles;
     int *err;
 };
-
-constexpr int kDwARows = 16 * kTile;   // 16 m-groups of a 128-pixel tile
 
 template <int GA, int GB>
 __global__ void __launch_bounds__(128, 1) k_conv_dw(DwArgs a) {
     extern __shared__ __align__(128) unsigned char smem[];
-    uint4 *sa = reinterpret_cast<uint4 *>(smem);                  // [16][kTile] rows (first GA filled)
-    uint4 *sx = sa + kDwARows;                                    // [GB][3][kSeg]
-    uint64_t *mbar = reinterpret_cast<uint64_t *>(sx + GB * 3 * kSeg);
-    uint32_t *tslot = reinterpret_cast<uint32_t *>(mbar + 1);
-    constexpr int N = 8 * GB;
+    constexpr int N = 3 * 8 * GA;                                 // (tap column, output channel)
+    uint4 *sx = reinterpret_cast<uint4 *>(smem);                  // [kRing][GB][kTile], 16 groups readable
+    uint4 *sz = sx + 16 * kTile;                                  // [kDzStages][3][GA][kTile]
+    float *red = reinterpret_cast<float *>(sz + kDzStages * 3 * GA * kTile);   // [9][32 ci][32 co]
+    uint64_t *bars = reinterpret_cast<uint64_t *>(red + 9 * 32 * 32);
+    uint32_t *tslot = reinterpret_cast<uint32_t *>(bars + 2 * kRing + 2 * kDzStages + 1);
+    const uint32_t full = smem_u32(bars), empty = full + 8 * kRing, zfull = empty + 8 * kRing,
+                   zempty = zfull + 8 * kDzStages, done = zempty + 8 * kDzStages;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
-    if (warp == 0) tmem_alloc<512>(smem_u32(tslot));
-    if (threadIdx.x == 0) mbar_init(smem_u32(mbar));
-    for (int e = threadIdx.x + GA * kTile; e < kDwARows; e += blockDim.x) sa[e] = make_uint4(0, 0, 0, 0);
+    if (warp == 1) tmem_alloc<512>(smem_u32(tslot));
+    if (threadIdx.x == 0) {
+        for (int i = 0; i < kRing; i++) {
+            mbar_init(full + 8 * i, 1);
+            mbar_init(empty + 8 * i, 1);
+        }
+        for (int i = 0; i < kDzStages; i++) {
+            mbar_init(zfull + 8 * i, 1);
+            mbar_init(zempty + 8 * i, 1);
+        }
+        mbar_init(done, 1);
+    }
+    for (int e = threadIdx.x; e < 9 * 32 * 32; e += blockDim.x) red[e] = 0.0f;
     tc_before();
     __syncthreads();
     tc_after();
     const uint32_t tmem = *tslot;
-    constexpr uint32_t idesc = idesc_bf16(kTile, N, 1, 1);
-    uint32_t phase = 0;
     bool ok = true;
-    int iter = 0;
-#pragma unroll 1
-    for (int tile = blockIdx.x; tile < a.ntiles; tile += gridDim.x, iter++) {
-        const int q0 = tile * kTile;
-        if (iter > 0) {   // the previous tile's MMAs have read shared memory
-            const bool w = mbar_wait(smem_u32(mbar), phase);
-            ok = ok && w;
-            phase ^= 1;
-            tc_after();
+    auto wait = [&](uint32_t bar, uint32_t parity) {
+        if (ok) ok = mbar_wait(bar, parity & 1u);
+    };
+    int b, c, row0, cnt;
+    unsigned used = 0;   // classes with an accumulator (the same in every thread)
+    {
+        int pos = 0;
+        for (int t = blockIdx.x; t < a.ch.items; t += gridDim.x) {
+            if (!a.ch.item(t, &b, &c, &row0, &cnt)) continue;
+            for (int k = 0; k < min(cnt, kRing); k++) used |= 1u << ((pos + k) % kRing);
+            pos += cnt + 2;
         }
-        for (int e = threadIdx.x; e < GA * kTile; e += blockDim.x) {
-            const int g = e / kTile, r = e - g * kTile;
-            const int q = q0 + r;
-            sa[e] = q < a.geo.npix ? a.dz[(size_t)g * a.geo.gs + q] : make_uint4(0, 0, 0, 0);
-        }
-        stage_halo<GB>(sx, a.x, a.geo.npix, a.geo.gs, q0, a.geo.Wp, a.dil);
-        fence_async_smem();
-        tc_before();
-        __syncthreads();
-        tc_after();
-        if (threadIdx.x == 0) {
-            const uint32_t aa = smem_u32(sa), xa = smem_u32(sx);
-#pragma unroll 1
-            for (int kk = 0; kk < kTile / 16; kk++) {
-                const uint64_t ad = sdesc(aa + kk * 16 * 16, 128, kTile * 16);
-#pragma unroll 1
-                for (int t = 0; t < 9; t++) {
-                    const int s = t / 3, dj = t % 3 - 1;
-                    const int r0 = a.dil + dj * a.dil + 16 * kk;
-                    const uint64_t bd = sdesc(xa + (s * kSeg + r0) * 16, 128, 3 * kSeg * 16);
-                    mma_bf16(tmem + (uint32_t)(t * N), ad, bd, idesc, (iter > 0 || kk > 0) ? 1u : 0u);
+    }
+
+    if (warp == 0) {   // producer (the whole warp: it zeroes the tail of a gradient tile)
+        int pos = 0, tile = 0;
+        for (int t = blockIdx.x; t < a.ch.items && ok; t += gridDim.x) {
+            if (!a.ch.item(t, &b, &c, &row0, &cnt)) continue;
+            const long q0 = ((long)b * a.geo.Hp + a.geo.P + row0) * a.geo.Wp + a.geo.P + c * kTile;
+            const int width = min(kTile, a.geo.W - c * kTile), padded = (width + 15) & ~15;
+            for (int p = 0; p < cnt + 2 && ok; p++, pos++) {
+                const long q = q0 + (long)(p - 1) * a.dil * a.geo.Wp;
+                const int s = pos % kRing;
+                wait(empty + 8 * s, (uint32_t)(pos / kRing) + 1u);
+                ok = __all_sync(0xffffffffu, ok);
+                if (!ok) break;
+                if (lane == 0) {
+                    mbar_expect(full + 8 * s, (uint32_t)(GB * kTile * 16));
+                    for (int g = 0; g < GB; g++)
+                        bulk_g2s(smem_u32(sx + (s * GB + g) * kTile), a.x + (long)g * a.geo.gs + q, kTile * 16,
+                                 full + 8 * s);
                 }
+                if (p < 1 || p > cnt) continue;   // the gradient tile of this row
+                const int z = tile % kDzStages;
+                wait(zempty + 8 * z, (uint32_t)(tile / kDzStages) + 1u);
+                ok = __all_sync(0xffffffffu, ok);
+                if (!ok) {
+                    pos++;   // this position's segment is on its way
+                    break;
+                }
+                for (int e = lane; e < 3 * GA * (padded - width); e += 32) {
+                    const int g = e / (padded - width), r = width + e % (padded - width);
+                    sz[(z * 3 * GA + g) * kTile + r] = make_uint4(0, 0, 0, 0);
+                }
+                fence_async_smem();
+                __syncwarp();
+                if (lane == 0) {
+                    mbar_expect(zfull + 8 * z, (uint32_t)(3 * GA * width * 16));
+                    for (int tc = 0; tc < 3; tc++)
+                        for (int g = 0; g < GA; g++)
+                            bulk_g2s(smem_u32(sz + ((z * 3 + tc) * GA + g) * kTile),
+                                     a.dz + (long)g * a.geo.gs + q + (1 - tc) * a.dil, (uint32_t)(width * 16),
+                                     zfull + 8 * z);
+                }
+                tile++;
             }
-            mma_commit(smem_u32(mbar));
+        }
+        if (lane == 0) {   // every copy has landed before the CTA ends
+            for (int p = max(0, pos - kRing); p < pos; p++) mbar_wait(full + 8 * (p % kRing), (uint32_t)(p / kRing) & 1u);
+            for (int p = max(0, tile - kDzStages); p < tile; p++)
+                mbar_wait(zfull + 8 * (p % kDzStages), (uint32_t)(p / kDzStages) & 1u);
+        }
+        __syncwarp();
+    } else if (warp == 1) {
+        if (lane == 0) {   // MMA issuer
+            constexpr uint32_t idesc = idesc_bf16(kTile, N, 1, 1);
+            const uint32_t xa = smem_u32(sx), za = smem_u32(sz);
+            int pos = 0, tile = 0;
+            unsigned begun = 0;
+            for (int t = blockIdx.x; t < a.ch.items && ok; t += gridDim.x) {
+                if (!a.ch.item(t, &b, &c, &row0, &cnt)) continue;
+                const int steps = (min(kTile, a.geo.W - c * kTile) + 15) / 16;
+                for (int k = 0; k < cnt; k++, tile++) {
+                    for (int p = k ? pos + k + 2 : pos; p <= pos + k + 2; p++)
+                        wait(full + 8 * (p % kRing), (uint32_t)(p / kRing));
+                    const int z = tile % kDzStages, cls = (pos + k) % kRing;
+                    wait(zfull + 8 * z, (uint32_t)(tile / kDzStages));
+                    if (!ok) break;
+                    tc_after();
+#pragma unroll 1
+                    for (int ks = 0; ks < steps; ks++) {
+                        const uint64_t ad = sdesc(xa + (uint32_t)(16 * ks) * 16, 128, kTile * 16);
+                        const uint64_t bd = sdesc(za + (uint32_t)(z * 3 * GA * kTile + 16 * ks) * 16, 128, kTile * 16);
+                        mma_bf16(tmem + (uint32_t)(cls * N), ad, bd, idesc, (begun >> cls & 1u) | (ks > 0 ? 1u : 0u));
+                    }
+                    begun |= 1u << cls;
+                    mma_commit(zempty + 8 * z);
+                    mma_commit(empty + 8 * cls);
+                    if (k + 1 == cnt) {
+                        mma_commit(empty + 8 * ((pos + k + 1) % kRing));
+                        mma_commit(empty + 8 * ((pos + k + 2) % kRing));
+                    }
+                }
+                pos += cnt + 2;
+            }
+            mma_commit(done);
+            if (!mbar_wait(done, 0)) ok = false;
         }
         __syncwarp();
     }
-    if (iter > 0) {
-        const bool w = mbar_wait(smem_u32(mbar), phase);
-        ok = ok && w;
-        tc_after();
-    }
-    if (!ok && threadIdx.x == 0) atomicExch(a.err, 2);
-    if (iter > 0 && ok && warp == 0) {
-        for (int t = 0; t < 9; t++) {
-            for (int c0 = 0; c0 < N; c0 += 16) {
-                float v[16];
-                tmem_ld16(tmem + (uint32_t)(t * N + c0), v);
-                const int co = lane;
-                if (co < a.cout)
-                    for (int k = 0; k < 16; k++)
-                        if (c0 + k < a.cin) atomicAdd(&a.dw[((size_t)co * a.cin + c0 + k) * 9 + t], v[k]);
+    if (!ok) atomicExch(a.err, 2);
+    tc_before();
+    const bool good = __syncthreads_and(ok);
+    tc_after();
+    if (good) {
+        // M row 32 warp + lane is (slot, ci); in step s warp w adds tap row
+        // (w + s) mod 4 of its slot (GB = 4): no two warps touch the same sums
+        const int row = 32 * warp + lane, slot = row / (8 * GB), ci = row % (8 * GB);
+        for (int s = 0; s < kRing; s++) {
+            const int di = (warp + s) & 3;
+            // GB = 2: a warp holds two slots, whose lanes take the same tap row one after the other
+            for (int h = 0; h < 4 / GB; h++) {
+                const int sl = GB == 4 ? warp : 2 * warp + h;   // warp uniform
+                const int cls = (sl - di) & 3;
+                if (sl < kRing && di < 3 && (used >> cls & 1u)) {
+                    for (int tc = 0; tc < 3; tc++)
+#pragma unroll
+                        for (int c0 = 0; c0 < 8 * GA; c0 += 16) {
+                            float v[16];
+                            tmem_ld16(tmem + ((uint32_t)(32 * warp) << 16) + (uint32_t)(cls * N + tc * 8 * GA + c0), v);
+                            if (slot == sl)
+#pragma unroll
+                                for (int k = 0; k < 16; k++) red[((di * 3 + tc) * 32 + ci) * 32 + ((c0 + k + ci) & 31)] += v[k];
+                        }
+                }
+                __syncwarp();
             }
+            __syncthreads();
+        }
+        for (int e = threadIdx.x; e < a.cout * a.cin * 9; e += blockDim.x) {
+            const int t = e % 9, ci = (e / 9) % a.cin, co = e / (9 * a.cin);
+            atomicAdd(&a.dw[e], red[(t * 32 + ci) * 32 + ((co + ci) & 31)]);
         }
     }
     tc_before();
     __syncthreads();
-    if (warp == 0) {
+    if (warp == 1) {
         tc_after();
         tmem_free<512>(tmem);
     }
 }
 
 // ---------------------------------------------------------- small kernels
-// input [B][4][H][W] FP32 -> [2][npix] rows (channels 4..15 zero, border zero)
-__global__ void k_pack_input(const float *__restrict__ in, uint4 *__restrict__ x, Geo geo) {
-    const int q = blockIdx.x * blockDim.x + threadIdx.x;
-    if (q >= geo.npix) return;
-    int b, i, j;
-    float c[4] = {0, 0, 0, 0};
-    if (geo.interior(q, &b, &i, &j)) {
-        const size_t plane = (size_t)geo.H * geo.W;
-        const size_t off = (size_t)(i - geo.P) * geo.W + (j - geo.P);
-        for (int k = 0; k < 4; k++) c[k] = in[((size_t)b * 4 + k) * plane + off];
+// input [B][4][H][W] FP32 -> [2][npix] rows at the image pixels (channels
+// 4..15 zero; the border and the second group are zero from the start)
+__global__ void k_pack_input(const float *__restrict__ in, uint4 *__restrict__ x, Geo geo, int B) {
+    const int plane = geo.H * geo.W, e = blockIdx.x * blockDim.x + threadIdx.x;
+    if (e >= plane) return;
+    const int i = e / geo.W, j = e - i * geo.W;
+    for (int b = blockIdx.y; b < B; b += gridDim.y) {
+        float c[4];
+#pragma unroll
+        for (int k = 0; k < 4; k++) c[k] = in[((size_t)b * 4 + k) * plane + e];
+        x[((size_t)b * geo.Hp + geo.P + i) * geo.Wp + geo.P + j] =
+            make_uint4(pack_bf16(c[0], c[1]), pack_bf16(c[2], c[3]), 0, 0);
     }
-    x[q] = make_uint4(pack_bf16(c[0], c[1]), pack_bf16(c[2], c[3]), 0, 0);
-    x[(size_t)geo.gs + q] = make_uint4(0, 0, 0, 0);
 }
 
-// dL/dout [B][2][H][W] FP32 -> [2][npix] rows (channels 2..15 zero)
-__global__ void k_pack_dout(const float *__restrict__ d, uint4 *__restrict__ x, Geo geo) {
-    const int q = blockIdx.x * blockDim.x + threadIdx.x;
-    if (q >= geo.npix) return;
-    int b, i, j;
-    float c[2] = {0, 0};
-    if (geo.interior(q, &b, &i, &j)) {
-        const size_t plane = (size_t)geo.H * geo.W;
-        const size_t off = (size_t)(i - geo.P) * geo.W + (j - geo.P);
-        for (int k = 0; k < 2; k++) c[k] = d[((size_t)b * 2 + k) * plane + off];
+// dL/dout [B][2][H][W] FP32 -> [2][npix] rows at the image pixels (channels
+// 2..15 zero), and the bias gradient of the last layer: db[c] += sum of the
+// rounded values
+__global__ void __launch_bounds__(256) k_pack_dout(const float *__restrict__ d, uint4 *__restrict__ x, Geo geo, int B, float *db) {
+    const int plane = geo.H * geo.W;
+    float s0 = 0.0f, s1 = 0.0f;
+    for (int b = blockIdx.y; b < B; b += gridDim.y)
+        for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < plane; e += gridDim.x * blockDim.x) {
+            const int i = e / geo.W, j = e - i * geo.W;
+            const uint32_t w = pack_bf16(d[(size_t)b * 2 * plane + e], d[((size_t)b * 2 + 1) * plane + e]);
+            const size_t q = ((size_t)b * geo.Hp + geo.P + i) * geo.Wp + geo.P + j;
+            x[q] = make_uint4(w, 0, 0, 0);
+            x[(size_t)geo.gs + q] = make_uint4(0, 0, 0, 0);
+            s0 += bf16_lo(w);
+            s1 += bf16_hi(w);
+        }
+    for (int o = 16; o > 0; o >>= 1) {
+        s0 += __shfl_xor_sync(0xffffffffu, s0, o);
+        s1 += __shfl_xor_sync(0xffffffffu, s1, o);
     }
-    x[q] = make_uint4(pack_bf16(c[0], c[1]), 0, 0, 0);
-    x[(size_t)geo.gs + q] = make_uint4(0, 0, 0, 0);
+    __shared__ float part[2][8];
+    if ((threadIdx.x & 31) == 0) {
+        part[0][threadIdx.x >> 5] = s0;
+        part[1][threadIdx.x >> 5] = s1;
+    }
+    __syncthreads();
+    if (threadIdx.x < 2) {
+        float t = 0.0f;
+        for (int w = 0; w < 8; w++) t += part[threadIdx.x][w];
+        atomicAdd(&db[threadIdx.x], t);
+    }
 }
 
 // masked squared error of channel 0 ([B][2][plane] arrays): dout_0 = 2 (out_0 -
@@ -519,25 +713,6 @@ __global__ void k_lap_grad(const float *__restrict__ s, const float *__restrict_
     }
 }
 
-// db[c] += sum over pixels of the G-group gradient rows (BF16 values)
-__global__ void k_bias_grad(const uint4 *__restrict__ dz, int G, int cout, int npix, int gs, float *db) {
-    float acc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-    const int g = blockIdx.y;
-    for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < npix; q += gridDim.x * blockDim.x) {
-        const uint4 v = dz[(size_t)g * gs + q];
-        const uint32_t w[4] = {v.x, v.y, v.z, v.w};
-        for (int k = 0; k < 4; k++) {
-            acc[2 * k] += bf16_lo(w[k]);
-            acc[2 * k + 1] += bf16_hi(w[k]);
-        }
-    }
-    for (int k = 0; k < 8; k++) {
-        float s = acc[k];
-        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-        if ((threadIdx.x & 31) == 0 && 8 * g + k < cout) atomicAdd(&db[8 * g + k], s);
-    }
-}
-
 // BF16 operand copies of one layer's FP32 weights w[co][ci][9]:
 // forward rows  wf[t][g][co][8] = w[co][8g + k][t]            (GIN groups, NOUT rows)
 // backward rows wb[t][g][ci][8] = w[8g + k][ci][8 - t]         (GOUT groups, 32 rows)
@@ -594,7 +769,7 @@ struct gcmg_cnn {
     int adam_t = 0;
     int sms = 148;
     size_t guard = 0;            // zero rows before and after each channel group
-    size_t smem_conv4 = 0, smem_conv2 = 0, smem_dw = 0;
+    size_t smem_sm = 0;          // shared memory of an SM
     std::string err;
     std::vector<void *> allocs;
 };
@@ -627,9 +802,36 @@ T *alloc(gcmg_cnn *c, size_t n) {
 int groups_in(int l) { return l == 0 ? 2 : 4; }
 int nout_of(int l) { return l == kLayers - 1 ? 16 : 32; }
 
-size_t conv_smem(int gin, int nout, size_t slack) {
-    const size_t need = (size_t)(2 * gin * 3 * kSeg + 9 * gin * nout) * 16 + 32;
-    return std::max(need, slack);
+// shared memory of the convolution: the ring, the weights, the barriers
+size_t conv_smem(int gin, int nout, int dil) {
+    return (size_t)(kRing * gin * (kTile + 2 * dil) + 9 * gin * nout) * 16 + 16 * 16;
+}
+// of the weight gradients: 16 channel groups of x (the MMA's M rows), the
+// staged gradients, the reduction buffer, the barriers; the kernel holds 512
+// TMEM columns, so it asks for enough to sit alone on an SM
+size_t dw_smem(int ga) {
+    const size_t need = (size_t)(16 * kTile + kDzStages * 3 * ga * kTile) * 16 + 9 * 32 * 32 * 4 + 24 * 16;
+    return std::max(need, (size_t)120 * 1024);
+}
+
+// work items of a chain kernel: chains cut into parts of at most `len` tiles,
+// short enough that every resident CTA (`slots`) gets about three
+Chains make_chains(const gcmg_cnn *c, int dil, int slots) {
+    Chains h;
+    h.H = c->H;
+    h.dil = dil;
+    h.cols = (c->W + kTile - 1) / kTile;
+    h.res = std::min(dil, c->H);
+    const int nmax = (c->H + dil - 1) / dil;   // tiles of the longest chain
+    const int64_t chains = (int64_t)c->batch * h.cols * h.res;
+    // a part of n tiles loads n + 2 segments: parts below 8 tiles only where a
+    // chain is that short or the CTAs would idle
+    const int64_t want = std::max<int64_t>(1, (int64_t)3 * slots / chains);
+    int len = std::max<int>(4, (int)((nmax + want - 1) / want));
+    h.parts = (nmax + len - 1) / len;
+    h.len = (nmax + h.parts - 1) / h.parts;
+    h.items = (int)(chains * h.parts);
+    return h;
 }
 
 #define CNN_GUARD(c, ...)                                             \
@@ -657,18 +859,28 @@ void prep_weights(gcmg_cnn *c) {
 }
 
 template <int GIN, int NOUT, int MODE>
-void launch_conv(gcmg_cnn *c, const ConvArgs &a, size_t smem) {
-    const int ntiles = (c->geo.npix + kTile - 1) / kTile;
-    int per_sm = 1;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_conv<GIN, NOUT, MODE>, 128, smem);
-    const unsigned grid = (unsigned)std::min(ntiles, std::max(per_sm, 1) * c->sms);
-    k_conv<GIN, NOUT, MODE><<<grid, 128, smem, c->stream>>>(a, ntiles);
+void launch_conv(gcmg_cnn *c, ConvArgs a) {
+    const size_t smem = conv_smem(GIN, NOUT, a.dil);
+    // resident CTAs an SM: shared memory (1 KB each is the system's), TMEM columns
+    const int per_sm = std::max(1, std::min({(int)(c->smem_sm / (smem + 1024)), 512 / (kAcc * NOUT), 4}));
+    a.ch = make_chains(c, a.dil, per_sm * c->sms);
+    const unsigned grid = (unsigned)std::min(a.ch.items, per_sm * c->sms);
+    k_conv<GIN, NOUT, MODE><<<grid, kConvThreads, smem, c->stream>>>(a);
     ck(cudaGetLastError(), "conv launch");
+}
+
+template <int GA, int GB>
+void launch_dw(gcmg_cnn *c, DwArgs d) {
+    d.ch = make_chains(c, d.dil, c->sms);
+    const unsigned grid = (unsigned)std::min(d.ch.items, c->sms);
+    k_conv_dw<GA, GB><<<grid, 128, dw_smem(GA), c->stream>>>(d);
+    ck(cudaGetLastError(), "dw launch");
 }
 
 void forward(gcmg_cnn *c, const float *in, float *out) {
     const Geo g = c->geo;
-    k_pack_input<<<(g.npix + 255) / 256, 256, 0, c->stream>>>(in, c->act[0], g);
+    const unsigned images = (unsigned)std::min(c->batch, 65535);
+    k_pack_input<<<dim3((unsigned)((c->H * c->W + 255) / 256), images), 256, 0, c->stream>>>(in, c->act[0], g, c->batch);
     for (int l = 0; l < kLayers; l++) {
         ConvArgs a{};
         a.x = c->act[l];
@@ -679,13 +891,13 @@ void forward(gcmg_cnn *c, const float *in, float *out) {
         a.err = c->d_err;
         if (l == 0) {
             a.y = c->act[1];
-            launch_conv<2, 32, 0>(c, a, c->smem_conv2);
+            launch_conv<2, 32, 0>(c, a);
         } else if (l < kLayers - 1) {
             a.y = c->act[l + 1];
-            launch_conv<4, 32, 0>(c, a, c->smem_conv4);
+            launch_conv<4, 32, 0>(c, a);
         } else {
             a.out = out;
-            launch_conv<4, 16, 1>(c, a, c->smem_conv4);
+            launch_conv<4, 16, 1>(c, a);
         }
     }
 }
@@ -694,10 +906,11 @@ void forward(gcmg_cnn *c, const float *in, float *out) {
 void backward(gcmg_cnn *c, const float *dout) {
     const Geo g = c->geo;
     ck(cudaMemsetAsync(c->grad, 0, c->nparams * sizeof(float), c->stream), "memset");
-    k_pack_dout<<<(g.npix + 255) / 256, 256, 0, c->stream>>>(dout, c->dz[0], g);
+    const int plane = c->H * c->W;
+    k_pack_dout<<<dim3((unsigned)std::min((plane + 255) / 256, std::max(1, 8 * c->sms / c->batch)),
+                       (unsigned)std::min(c->batch, 65535)),
+                  256, 0, c->stream>>>(dout, c->dz[0], g, c->batch, c->grad + c->boff[kLayers - 1]);
     int cur = 0;
-    const int ntiles = (g.npix + kTile - 1) / kTile;
-    const int sms = c->sms;
     for (int l = kLayers - 1; l >= 0; l--) {
         const int ga = l == kLayers - 1 ? 2 : 4;
         DwArgs d{};
@@ -708,26 +921,22 @@ void backward(gcmg_cnn *c, const float *dout) {
         d.cin = kCin[l];
         d.geo = g;
         d.dil = c->dil[l];
-        d.ntiles = ntiles;
         d.err = c->d_err;
-        const unsigned grid = (unsigned)std::min(ntiles, sms);
-        if (ga == 2) k_conv_dw<2, 4><<<grid, 128, c->smem_dw, c->stream>>>(d);
-        else if (l == 0) k_conv_dw<4, 2><<<grid, 128, c->smem_dw, c->stream>>>(d);
-        else k_conv_dw<4, 4><<<grid, 128, c->smem_dw, c->stream>>>(d);
-        ck(cudaGetLastError(), "dw launch");
-        k_bias_grad<<<dim3(64, ga), 256, 0, c->stream>>>(c->dz[cur], ga, kCout[l], g.npix, g.gs,
-                                                         c->grad + c->boff[l]);
+        if (ga == 2) launch_dw<2, 4>(c, d);
+        else if (l == 0) launch_dw<4, 2>(c, d);
+        else launch_dw<4, 4>(c, d);
         if (l == 0) break;
         ConvArgs a{};
         a.x = c->dz[cur];
         a.w = reinterpret_cast<const uint4 *>(c->wb[l]);
         a.y = c->dz[cur ^ 1];
         a.gate = c->act[l];
+        a.db = c->grad + c->boff[l - 1];
         a.geo = g;
         a.dil = c->dil[l];
         a.err = c->d_err;
-        if (ga == 2) launch_conv<2, 32, 2>(c, a, c->smem_conv2);
-        else launch_conv<4, 32, 2>(c, a, c->smem_conv4);
+        if (ga == 2) launch_conv<2, 32, 2>(c, a);
+        else launch_conv<4, 32, 2>(c, a);
         cur ^= 1;
     }
 }
@@ -806,19 +1015,21 @@ gcmg_status gcmg_cnn_create(int batch, int H, int W, const int *dilations, void 
         c->d_loss = alloc<double>(c, 1);
         c->d_err = alloc<int>(c, 1);
         ck(cudaMemset(c->d_err, 0, sizeof(int)), "memset");
-        // shared memory: the weight-gradient kernel holds 512 TMEM columns, so
-        // it asks for enough shared memory to sit alone on an SM
-        c->smem_conv4 = conv_smem(4, 32, 0);
-        c->smem_conv2 = conv_smem(2, 32, 0);
-        c->smem_dw = std::max((size_t)(kDwARows + 4 * 3 * kSeg) * 16 + 16, (size_t)140 * 1024);
-        ck(cudaFuncSetAttribute(k_conv<2, 32, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)c->smem_conv2), "attr");
-        ck(cudaFuncSetAttribute(k_conv<4, 32, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)c->smem_conv4), "attr");
-        ck(cudaFuncSetAttribute(k_conv<4, 16, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)c->smem_conv4), "attr");
-        ck(cudaFuncSetAttribute(k_conv<2, 32, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)c->smem_conv2), "attr");
-        ck(cudaFuncSetAttribute(k_conv<4, 32, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)c->smem_conv4), "attr");
-        ck(cudaFuncSetAttribute(k_conv_dw<2, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)c->smem_dw), "attr");
-        ck(cudaFuncSetAttribute(k_conv_dw<4, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)c->smem_dw), "attr");
-        ck(cudaFuncSetAttribute(k_conv_dw<4, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)c->smem_dw), "attr");
+        int most = 0, per_sm = 0;
+        ck(cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, c->device), "attr");
+        ck(cudaDeviceGetAttribute(&per_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, c->device), "attr");
+        c->smem_sm = (size_t)per_sm;
+        const auto allow = [&](auto *kernel) {
+            ck(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, most), "attr");
+        };
+        allow(k_conv<2, 32, 0>);
+        allow(k_conv<4, 32, 0>);
+        allow(k_conv<4, 16, 1>);
+        allow(k_conv<2, 32, 2>);
+        allow(k_conv<4, 32, 2>);
+        allow(k_conv_dw<2, 4>);
+        allow(k_conv_dw<4, 4>);
+        allow(k_conv_dw<4, 2>);
         // zero every activation once: borders and guards stay zero from then on
         for (int l = 0; l < kLayers; l++) ck(cudaMemset(c->act[l] - c->guard, 0, (l ? 4 : 2) * gs * 16), "memset");
         ck(cudaMemset(c->dz[0] - c->guard, 0, 4 * gs * 16), "memset");
