@@ -330,14 +330,16 @@ gcmg_status gcmg_kernel_timing_ex(gcmg_ctx *ctx, int64_t *launches, double *tota
 
 /* How the 3D boundary relaxation (the ghost sweep, the lambda band sweeps
  * of Sec. 3.2 and the junction sweeps) is launched; every mode gives the same
- * results bitwise.  mode 0 (default): one launch per phase, the store of
- * each Jacobi ghost sweep merged into the launch of the next red band or
- * junction-zone sweep; 1: on levels whose ghost, band and junction lists
+ * results bitwise.  mode 0 (default): on small levels all phases, on the
+ * others the junction sweeps, as one thread-block cluster whose CTAs hold the
+ * values in shared memory and send each other what they read; the remaining
+ * phases one launch each, the store of each Jacobi ghost sweep merged into the
+ * launch of the next red band or junction-zone sweep; 1: on levels whose ghost, band and junction lists
  * hold at most 65,536 entries all phases as one thread-block cluster of 16
- * CTAs with hardware barriers between them, mode 0 on the other levels; 2:
- * all phases as one grid with software barriers.  Modes 1 and 2 measured
- * slower on GB300 (the per-phase launches overlap inside the solve's graph
- * and spread each phase's gathers over every SM).  Not in the paper. */
+ * CTAs with hardware barriers between them and the values in global memory,
+ * one launch a phase on the other levels; 2: all phases as one grid with
+ * software barriers.  Modes 1 and 2 measured slower on GB300 (a phase costs a
+ * round trip to L2 besides the barrier).  Not in the paper. */
 gcmg_status gcmg_set_boundary3d(gcmg_ctx *ctx, int mode);
 
 /* Mode 2 of gcmg_set_boundary3d with test controls: every software barrier
@@ -386,10 +388,12 @@ gcmg_status gcmg_set_junction_blocks(gcmg_ctx *ctx, int enable);
  * bitwise.  GCMG_E_ARG for a negative count.  Not in the paper. */
 gcmg_status gcmg_set_split2d(gcmg_ctx *ctx, int min_strips);
 
-/* How level l's junction sweeps run in the context's cycle precision (3D
- * mixed form: the FP32 programs, which need less shared memory): 0 on global
+/* The form of level l's junction program in the context's cycle precision (3D
+ * mixed form: the FP32 programs, which need less shared memory): 0 global
  * lists (or no junction zone), 1 whole components in shared memory, 2 blocks
- * in shared memory; -1 for a bad context or level.  Not in the paper. */
+ * in shared memory; -1 for a bad context or level.  Launch mode 0 of
+ * gcmg_set_boundary3d runs the zone as a cluster instead where that fits and
+ * gcmg_set_junction_blocks is off.  Not in the paper. */
 int gcmg_junction_mode(const gcmg_ctx *ctx, int l);
 
 /* Sweep 2's work on level l: number of items (0: the level uses sweep 1)

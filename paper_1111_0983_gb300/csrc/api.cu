@@ -47,6 +47,15 @@ int kslots(int dim) { return dim == 2 ? 9 : 27; }
 // threads: four entries a thread a phase)
 constexpr int64_t kClusterWork = 65536;
 
+// 3D levels with at most this many ghosts (FP32 / FP64 cycles) run all boundary
+// phases of a relaxation as one cluster over distributed shared memory, larger
+// ones the junction zone alone.  Beyond, the 16 SMs' work a phase (and their
+// shared memory: 29 values a ghost) costs more than a launch saves.  A cycle of
+// the torus, launch a phase -> cluster: 33^3 173 -> 142 us, 65^3 376 -> 275,
+// 97^3 (two levels) 469 -> 316, FP64 65^3 746 -> 513; the zone alone on 129^3
+// and 257^3: 46 -> 21 and 52 -> 25 us a relaxation
+constexpr int64_t kC3Ghosts32 = 12000, kC3Ghosts64 = 6000;
+
 // Rows of the Kaczmarz comparison smoother on level l (2D): the ghosts and the
 // inside nodes of the band, grouped by the colour (i mod 5) + 5 (j mod 5) of
 // their node, increasing node index within a colour
@@ -428,9 +437,22 @@ T *relax(gcmg_ctx *c, LevelView<T> v, T *out, T *wb, int l, bool extra) {
         // thread-block cluster with hardware barriers between the phases;
         // 2: all phases as one grid with software barriers
         bool done = false, zdone = false;
+        // mode 0: the cluster program of the level, if it has one
+        const Cluster3Dev *C3 = nullptr;
+        if (dim == 3 && extra && c->p.smoother == 0 && !c->coop3d && !c->cluster3d && !c->junction_blocks &&
+            c->c3[l].records && (sizeof(T) == 4 ? c->c3[l].fits32 : c->c3[l].fits64))
+            C3 = &c->c3[l];
+        const int mu = !c->p.junction_solve && g.jz.ncomp > 0 ? c->p.junction_sweeps : 0;
+        if (C3 && C3->band) {
+            timer_mark(c, GCMG_KERNEL_BOUNDARY, l);
+            launch_cluster3<T>(v, *C3, true, c->p.lambda, mu, c->stream);
+            timer_mark(c, GCMG_KERNEL_BOUNDARY, l);
+            done = true;
+            zdone = !c->p.junction_solve;
+        }
         BoundaryProgram3 P;
         const bool jz_smem = dim == 3 && sizeof(T) == 4 ? g.jz.in_smem32 : g.jz.in_smem;
-        if (dim == 3 && c->p.smoother == 0 && g.ng > 0) {
+        if (!done && dim == 3 && c->p.smoother == 0 && g.ng > 0) {
             P.red = g.red;
             P.nred = g.nred;
             P.black = g.black;
@@ -471,7 +493,8 @@ T *relax(gcmg_ctx *c, LevelView<T> v, T *out, T *wb, int l, bool extra) {
         const bool merged = !done && dim == 3 && extra && c->p.smoother == 0 && g.ng > 0 && g.red_src &&
                             !c->coop3d;
         if (merged) {
-            const bool zmerge = !c->p.junction_solve && c->p.junction_sweeps > 0 && g.jz.ncomp > 0 &&
+            const bool zcluster = C3 && mu > 0;
+            const bool zmerge = !zcluster && !c->p.junction_solve && c->p.junction_sweeps > 0 && g.jz.ncomp > 0 &&
                                 !jz_smem && g.jz.zred_src;
             launch_ghost_new<T>(v, nullptr, g.ng, c->stream);
             for (int k = 0; k < c->p.lambda; k++) {
@@ -491,6 +514,10 @@ T *relax(gcmg_ctx *c, LevelView<T> v, T *out, T *wb, int l, bool extra) {
                 return v.u;
             }
             launch_ghost_store<T>(v, nullptr, g.ng, c->stream);
+            if (zcluster) {
+                launch_cluster3<T>(v, *C3, false, 0, mu, c->stream);
+                return v.u;
+            }
         } else if (!done) {
             launch_ghost_relax<T>(v, dim, c->stream);
             if (extra)
@@ -545,6 +572,32 @@ void check_program_fits(gcmg_ctx *c, LocalDev &z) {
     // the attribute is per kernel: allow the device maximum once for all levels
     local_prepare<double>(c->p.dim, (size_t)dev_max);
     local_prepare<float>(c->p.dim, (size_t)dev_max);
+}
+
+// (re)builds level l's cluster program (3D) for its current junction zone: the
+// band and zone phases together where the level is small, else the zone alone
+void update_cluster3(gcmg_ctx *c, int l) {
+    if (c->p.dim != 3) return;
+    if (c->c3.empty()) c->c3.resize(c->H.size());
+    Cluster3Dev &d = c->c3[l];
+    free_tracked(c, d.records);
+    d = Cluster3Dev{};
+    const HostLevel &L = c->H[l];
+    if (L.ng() == 0) return;
+    const bool f32 = c->p.precision == 1;
+    for (int band = L.ng() <= (f32 ? kC3Ghosts32 : kC3Ghosts64) ? 1 : 0; band >= 0; band--) {
+        const Cluster3Program P = build_cluster3(L, band != 0);
+        if (P.records.empty()) continue;
+        const bool ok32 = cluster3_fits<float>(P.lay, c->device), ok64 = cluster3_fits<double>(P.lay, c->device);
+        if (!(f32 ? ok32 : ok64)) continue;
+        d.lay = P.lay;
+        d.band = P.band;
+        d.fits32 = ok32;
+        d.fits64 = ok64;
+        d.records = upload<uint8_t>(c, P.records.data(), P.records.size());
+        ck(cudaStreamSynchronize(c->stream), "sync");   // the host records die at return
+        return;
+    }
 }
 
 // TGCS (Sec. 2.4) applied recursively: V (gamma = 1) or W (gamma = 2) cycle
@@ -641,7 +694,7 @@ double fine_defect_norm(gcmg_ctx *c) {
     return read_norm(c);
 }
 
-// whether a bounded barrier wait of k_boundary3d ran out since the last
+// whether a bounded wait of k_boundary3d ran out since the last
 // check (synchronises the stream); if so the flag and the barrier words are
 // cleared for the next launch
 bool barrier_timed_out(gcmg_ctx *c) {
@@ -890,6 +943,7 @@ gcmg_status create_from_levels(const gcmg_params &q, std::vector<HostLevel> &&H,
             c->D32.resize(nl);
             for (int l = 0; l < nl; l++) alloc_data<float>(c, l, c->D32[l], true);
         }
+        for (int l = 0; l < nl; l++) update_cluster3(c, l);
         c->d_norm = dalloc<unsigned long long>(c, 2);
         c->d_rel = dalloc<double>(c, 257);
         c->d_r0 = dalloc<double>(c, 2);   // r0, the last relative residual
@@ -1172,6 +1226,7 @@ gcmg_status gcmg_set_bc_types(gcmg_ctx *c, int l, const uint8_t *types) {
             upload_program(c, L.junction, c->G[l].jz);
             check_program_fits(c, c->G[l].jz);
         }
+        update_cluster3(c, l);
         upload_ghost_data<double>(c, l, c->D64[l], false);
         if (!c->D32.empty()) upload_ghost_data<float>(c, l, c->D32[l], false);
         return GCMG_OK;

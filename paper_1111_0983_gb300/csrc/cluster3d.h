@@ -1,0 +1,75 @@
+// 3D boundary phases as one thread-block cluster over distributed shared
+// memory: the host-built program (cluster3d.cpp) and its kernel (cluster3d.cu).
+#pragma once
+
+#include <cuda_runtime.h>
+#include <stdint.h>
+
+#include <vector>
+
+#include "gcmg_internal.h"
+
+namespace gcmg {
+
+constexpr int C3_RANKS = 16;      // CTAs of the cluster
+constexpr int C3_THREADS = 512;
+
+// Header of a rank's record: counts and list bounds (ints).  Inside entries
+// are ordered by colour, within a colour band only | band and zone | zone
+// only, so that a band sweep and a zone sweep each take one range.
+enum {
+    C3_NIN,                   // inside slots (own updated nodes first)
+    C3_NGS,                   // ghost slots (own updated ghosts first)
+    C3_OWN_IN, C3_OWN_G,      // updated nodes of this rank, written back
+    C3_RB0, C3_RB1,           // red entries of a band sweep
+    C3_RZ0, C3_RZ1,           // red entries of a zone sweep
+    C3_BB0, C3_BB1, C3_BZ0, C3_BZ1,   // black
+    C3_GZ,                    // first zone ghost among the own ghosts
+    C3_HDR = 16
+};
+
+// The partition of the updated nodes over the cluster's ranks.  Every rank
+// has a record of `stride` bytes with the same section offsets:
+//   ints    header
+//   lnode   int32 per slot: global node (inside slots, then ghost slots)
+//   ent     8 x uint16 per inside entry: own slot, 6 sources in the order of
+//           the sweeps' sum, first copy (0xffff: none)
+//   gq      int32 per own ghost: ghost number
+//   gst     4 x max_g x 8 uint16: the 27 stencil sources, first copy
+//   copies  uint32: rank << 16 | slot, bit 31 = last; where the entry's value
+//           is also kept (the ranks that read it)
+// A source is an inside slot, or 0x8000 | (max_in + ghost slot).
+struct Cluster3Layout {
+    int stride = 0, lnode = 0, ent = 0, gq = 0, gst = 0, copies = 0;   // bytes
+    int max_in = 0, max_gs = 0, max_e = 0, max_g = 0;                  // most per rank
+};
+
+struct Cluster3Program {
+    bool band = false;               // holds the band sweeps too (else the zone sweeps alone)
+    Cluster3Layout lay;
+    std::vector<uint8_t> records;    // C3_RANKS * stride; empty: no program
+};
+
+// Program of level L's junction zone (L.junction's lists) and, with `band`,
+// of its ghost and band sweeps.  Empty if there is nothing to do or a rank's
+// slots do not fit 15 bits.
+Cluster3Program build_cluster3(const HostLevel &L, bool band);
+
+// Device copy of a program.
+struct Cluster3Dev {
+    Cluster3Layout lay;
+    uint8_t *records = nullptr;
+    bool band = false;
+    bool fits32 = false, fits64 = false;   // per precision: shared memory, and the cluster can be resident
+};
+
+template <typename T>
+size_t cluster3_smem(const Cluster3Layout &l);
+// whether a cluster of this program's size can be resident on the device
+template <typename T>
+bool cluster3_fits(const Cluster3Layout &l, int device);
+// lead: the relaxation's ghost sweep first; then lambda band sweeps, mu zone sweeps
+template <typename T>
+void launch_cluster3(const LevelView<T> &v, const Cluster3Dev &P, bool lead, int lambda, int mu, cudaStream_t s);
+
+}  // namespace gcmg

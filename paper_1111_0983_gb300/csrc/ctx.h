@@ -6,6 +6,7 @@
 #include <string>
 #include <vector>
 
+#include "cluster3d.h"
 #include "gcmg_internal.h"
 
 using gcmg::DevData;
@@ -23,6 +24,7 @@ struct gcmg_ctx {
     std::vector<DevGeom> G;
     std::vector<DevData<double>> D64;
     std::vector<DevData<float>> D32;
+    std::vector<gcmg::Cluster3Dev> c3;      // 3D: the levels' boundary phases as one cluster launch
     bool rhs_set = false;
     bool js64 = false;                      // FP64 junction-solve inverses kept (single relaxations)
     // the fused coarse cycle (coarse.cu): its first level (-1: per-level
