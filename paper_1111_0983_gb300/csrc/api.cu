@@ -237,14 +237,12 @@ void free_tracked(gcmg_ctx *c, void *p) {
 void upload_program(gcmg_ctx *c, const LocalProgram &J, LocalDev &z) {
     int32_t **arrs[] = {&z.node_off, &z.wb_cnt, &z.lnode, &z.int_off, &z.red_cnt, &z.int_glob,
                         &z.int_me, &z.int_nb, &z.gh_off, &z.gh_me, &z.gh_q, &z.gh_stn,
-                        &z.zred, &z.zblack, &z.zghost, &z.wb_list, &z.node_base,
-                        &z.pre_off, &z.pre_red_cnt, &z.pre_me, &z.pre_nb, &z.pre_glob, &z.zred_src};
+                        &z.zred, &z.zblack, &z.zghost, &z.wb_list, &z.node_base, &z.zred_src};
     for (int32_t **a : arrs) { free_tracked(c, *a); *a = nullptr; }
     z.ncomp = J.ncomp();
     z.max_nodes = J.max_nodes;
     z.max_int = J.max_int;
     z.max_gh = J.max_gh;
-    z.max_pre = J.max_pre;
     z.max_colour = 0;
     for (int k = 0; k < J.ncomp(); k++)
         z.max_colour = std::max({z.max_colour, J.red_cnt[k], J.int_off[k + 1] - J.int_off[k] - J.red_cnt[k]});
@@ -254,12 +252,6 @@ void upload_program(gcmg_ctx *c, const LocalProgram &J, LocalDev &z) {
     z.wb_cnt = upload<int32_t>(c, J.wb_cnt.data(), J.wb_cnt.size());
     z.lnode = upload<int32_t>(c, J.lnode.data(), J.lnode.size());
     z.node_base = upload<int32_t>(c, J.node_base.data(), J.node_base.size());
-    z.has_pre = !J.pre_me.empty();
-    z.pre_off = upload<int32_t>(c, J.pre_off.data(), J.pre_off.size());
-    z.pre_red_cnt = upload<int32_t>(c, J.pre_red_cnt.data(), J.pre_red_cnt.size());
-    z.pre_me = upload<int32_t>(c, J.pre_me.data(), J.pre_me.size());
-    z.pre_nb = upload<int32_t>(c, J.pre_nb.data(), J.pre_nb.size());
-    z.pre_glob = upload<int32_t>(c, J.pre_glob.data(), J.pre_glob.size());
     z.int_off = upload<int32_t>(c, J.int_off.data(), J.int_off.size());
     z.red_cnt = upload<int32_t>(c, J.red_cnt.data(), J.red_cnt.size());
     z.int_glob = upload<int32_t>(c, J.int_glob.data(), J.int_glob.size());
@@ -283,6 +275,26 @@ void upload_program(gcmg_ctx *c, const LocalProgram &J, LocalDev &z) {
     z.nwb = (int)wb.size();
     z.wb_list = upload<int32_t>(c, wb.data(), wb.size());
     ck(cudaStreamSynchronize(c->stream), "sync");
+}
+
+// uploads the boundary blocks of level l as per-thread records
+void upload_blocks2(gcmg_ctx *c, int l) {
+    const Block2Host B = build_blocks2(c->H[l]);
+    Block2Dev &d = c->G[l].b2;
+    d = B.d;
+    if (d.m == 0) return;
+    auto put = [&](const std::vector<uint32_t> &v) {
+        return reinterpret_cast<uint4 *>(upload<uint32_t>(c, v.data(), v.size()));
+    };
+    d.node = upload<int32_t>(c, B.node.data(), B.node.size());
+    d.w = reinterpret_cast<int2 *>(upload<int32_t>(c, B.w.data(), B.w.size()));
+    d.e_red = put(B.e_red);
+    d.e_black = put(B.e_black);
+    d.p_red = put(B.p_red);
+    d.p_black = put(B.p_black);
+    d.g0 = put(B.g0);
+    d.g1 = put(B.g1);
+    ck(cudaStreamSynchronize(c->stream), "sync");   // the host records die at return
 }
 
 // sets NODE_WB in the device type grid of level l at the boundary blocks'
@@ -347,48 +359,49 @@ template <typename T>
 T *relax(gcmg_ctx *c, LevelView<T> v, T *out, T *wb, int l, bool extra) {
     const int dim = c->p.dim;
     const DevGeom &g = c->G[l];
-    if constexpr (std::is_same<T, float>::value) {
-        // FP32 2D: the interior sweep, the ghost sweep and the band sweeps in one
-        // launch (strips and boundary blocks both read v.u, write out); the
-        // blocks store straight into out, so no write-back is pending
-        if (dim == 2 && extra && g.nstrips > 0 && g.bz.ncomp > 0 && g.bz.in_smem && g.bz.pre_in_smem) {
-            // algorithmic bytes: the interior sweep's (u, f read and u written
-            // once per inside node) and the boundary blocks' distinct values
-            const double bytes = c->timing_kind >= 0
-                                     ? ((double)c->bz_units[l] + 3.0 * (double)c->H[l].n_in) * sizeof(T)
-                                     : 0.0;
-            timer_mark(c, GCMG_KERNEL_SMOOTH, l, bytes);
-            timer_mark(c, GCMG_KERNEL_BOUNDARY, l, bytes);
+    // 2D: the interior sweep, the ghost sweep and the band sweeps in one launch
+    // (strips and boundary blocks both read v.u, write out); the blocks store
+    // straight into out, so no write-back is pending
+    if (dim == 2 && extra && c->p.smoother == 0 && g.nstrips > 0 && g.strip_rows == 8 && g.b2.m > 0) {
+        // algorithmic bytes: the interior sweep's (u, f read and u written
+        // once per inside node) and the boundary blocks' distinct values
+        const double bytes = c->timing_kind >= 0
+                                 ? ((double)c->bz_units[l] + 3.0 * (double)c->H[l].n_in) * sizeof(T)
+                                 : 0.0;
+        timer_mark(c, GCMG_KERNEL_SMOOTH, l, bytes);
+        timer_mark(c, GCMG_KERNEL_BOUNDARY, l, bytes);
+        bool split = false;
+        if constexpr (std::is_same<T, float>::value) {
             if (c->split2d_strips > 0 && g.nstrips >= c->split2d_strips) {
                 if (!c->sstream) {
                     ck(cudaStreamCreateWithFlags(&c->sstream, cudaStreamNonBlocking), "cudaStreamCreate");
                     ck(cudaEventCreateWithFlags(&c->ev_fork, cudaEventDisableTiming), "cudaEventCreate");
                     ck(cudaEventCreateWithFlags(&c->ev_join, cudaEventDisableTiming), "cudaEventCreate");
                 }
-                launch_relax2d_split(v, out, g, lview<T>(g.bz, v), c->p.lambda, c->stream, c->sstream, c->ev_fork,
+                launch_relax2d_split(v, out, g, b2view<T>(g.b2, v), c->p.lambda, c->stream, c->sstream, c->ev_fork,
                                      c->ev_join);
-            } else {
-                launch_relax2d(v, out, g, lview<T>(g.bz, v), c->p.lambda, c->stream);
+                split = true;
             }
-            timer_mark(c, GCMG_KERNEL_BOUNDARY, l);
-            timer_mark(c, GCMG_KERNEL_SMOOTH, l);
-            v.u = out;
-            if (c->p.junction_solve) {
-                const DevData<T> &D = data<T>(c)[l];
-                launch_junction_solve<T>(v, g, D.js_inv, D.js_r, c->stream, nullptr);
-            } else if (c->p.junction_sweeps > 0 && g.jz.ncomp > 0) {
-                if (g.jz.in_smem) {
-                    launch_local<T>(lview<T>(g.jz, v), dim, 0, c->p.junction_sweeps, c->stream);
-                } else {
-                    for (int k = 0; k < c->p.junction_sweeps; k++) {
-                        launch_rb_list<T>(v, dim, g.jz.zred, g.jz.nzred, c->stream);
-                        launch_rb_list<T>(v, dim, g.jz.zblack, g.jz.nzblack, c->stream);
-                        launch_ghost_relax_list<T>(v, dim, g.jz.zghost, g.jz.nzghost, c->stream);
-                    }
+        }
+        if (!split) launch_relax2d<T>(v, out, g, b2view<T>(g.b2, v), c->p.lambda, c->stream);
+        timer_mark(c, GCMG_KERNEL_BOUNDARY, l);
+        timer_mark(c, GCMG_KERNEL_SMOOTH, l);
+        v.u = out;
+        if (c->p.junction_solve) {
+            const DevData<T> &D = data<T>(c)[l];
+            launch_junction_solve<T>(v, g, D.js_inv, D.js_r, c->stream, nullptr);
+        } else if (c->p.junction_sweeps > 0 && g.jz.ncomp > 0) {
+            if (g.jz.in_smem) {
+                launch_local<T>(lview<T>(g.jz, v), dim, 0, c->p.junction_sweeps, c->stream);
+            } else {
+                for (int k = 0; k < c->p.junction_sweeps; k++) {
+                    launch_rb_list<T>(v, dim, g.jz.zred, g.jz.nzred, c->stream);
+                    launch_rb_list<T>(v, dim, g.jz.zblack, g.jz.nzblack, c->stream);
+                    launch_ghost_relax_list<T>(v, dim, g.jz.zghost, g.jz.nzghost, c->stream);
                 }
             }
-            return v.u;
         }
+        return v.u;
     }
     if (dim == 2) {
         timer_mark(c, GCMG_KERNEL_SMOOTH, l);
@@ -567,8 +580,6 @@ void check_program_fits(gcmg_ctx *c, LocalDev &z) {
     z.in_smem32 = local_smem_bytes<float>(lview<float>(z, dummy32), c->p.dim) <= (size_t)dev_max &&
                   local_fits_registers(z.max_int);
     if (!z.in_smem && !z.in_smem32) return;    // relaxed from global memory instead
-    z.pre_in_smem = z.in_smem && z.has_pre &&
-                    local_smem_bytes<float>(lview<float>(z, dummy32), c->p.dim, true) <= (size_t)dev_max;
     // the attribute is per kernel: allow the device maximum once for all levels
     local_prepare<double>(c->p.dim, (size_t)dev_max);
     local_prepare<float>(c->p.dim, (size_t)dev_max);
@@ -935,6 +946,7 @@ gcmg_status create_from_levels(const gcmg_params &q, std::vector<HostLevel> &&H,
             for (int l = 0; l < nl; l++) {
                 upload_program(c, c->H[l].boundary, c->G[l].bz);
                 check_program_fits(c, c->G[l].bz);
+                upload_blocks2(c, l);
                 mark_writeback(c, l);
             }
         c->D64.resize(nl);

@@ -142,17 +142,27 @@ LocalView<T> lview(const LocalDev &z, const LevelView<T> &v, T *wb = nullptr) {
     J.max_nodes = z.max_nodes;
     J.max_int = z.max_int;
     J.max_gh = z.max_gh;
-    J.max_pre = z.max_pre;
     J.max_colour = z.max_colour;
     J.ng = v.ng;
     J.node_off = z.node_off; J.wb_cnt = z.wb_cnt; J.lnode = z.lnode; J.node_base = z.node_base;
-    J.pre_off = z.pre_off; J.pre_red_cnt = z.pre_red_cnt; J.pre_me = z.pre_me; J.pre_nb = z.pre_nb;
-    J.pre_glob = z.pre_glob;
     J.int_off = z.int_off; J.red_cnt = z.red_cnt; J.int_glob = z.int_glob; J.int_me = z.int_me; J.int_nb = z.int_nb;
     J.gh_off = z.gh_off; J.gh_me = z.gh_me; J.gh_q = z.gh_q; J.gh_stn = z.gh_stn;
     J.wb_list = z.wb_list;
     J.nwb = z.nwb;
     J.u = v.u; J.f = v.f; J.gg = v.gg; J.gc = v.gc; J.gw = v.gw;
+    J.h2 = v.h2;
+    return J;
+}
+
+template <typename T>
+Block2View<T> b2view(const Block2Dev &b, const LevelView<T> &v) {
+    Block2View<T> J;
+    J.p = b;
+    J.f = v.f;
+    J.gg = v.gg;
+    J.gc = v.gc;
+    J.gw = v.gw;
+    J.ng = v.ng;
     J.h2 = v.h2;
     return J;
 }

@@ -66,7 +66,7 @@ struct LocalProgram {
     // components are overlapping blocks (3D junction zone): each writes back
     // through a separate grid, copied into u after the launch
     bool blocked = false;
-    int max_nodes = 0, max_int = 0, max_gh = 0, max_pre = 0;
+    int max_nodes = 0, max_int = 0, max_gh = 0;
     int ncomp() const { return (int)wb_cnt.size(); }
 };
 
@@ -209,12 +209,9 @@ void build_boundary_blocks(HostLevel &L, int lambda, int block);
 // --------------------------------------------------------------- device side
 // A LocalProgram on the device.
 struct LocalDev {
-    int ncomp = 0, max_nodes = 0, max_int = 0, max_gh = 0, max_pre = 0;
+    int ncomp = 0, max_nodes = 0, max_int = 0, max_gh = 0;
     int max_colour = 0;   // most inside entries of one colour in a component
     int32_t *node_off = nullptr, *wb_cnt = nullptr, *lnode = nullptr, *node_base = nullptr;
-    int32_t *pre_off = nullptr, *pre_red_cnt = nullptr, *pre_me = nullptr, *pre_nb = nullptr, *pre_glob = nullptr;
-    bool has_pre = false;
-    bool pre_in_smem = false;  // the FP32 program with its pre-sweep lists fits in shared memory
     int32_t *int_off = nullptr, *red_cnt = nullptr, *int_glob = nullptr, *int_me = nullptr, *int_nb = nullptr;
     int32_t *gh_off = nullptr, *gh_me = nullptr, *gh_q = nullptr, *gh_stn = nullptr;
     int nzred = 0, nzblack = 0, nzghost = 0;
@@ -227,6 +224,30 @@ struct LocalDev {
     bool in_smem32 = true;     // the same for the FP32 program (smaller: 3D FP32 cycles use it)
 };
 
+// The 2D boundary blocks of a relaxation as per-thread records (k_relax2d):
+// component c's records start at c times the section's length, thread t takes
+// records t, t + nt, ...; a record past the component's count has node
+// or ghost -1.  Sources are 16 bits: a staged node's slot, or 0x8000 | (nodes +
+// j) for the component's updated ghost j (which has two values, see block2).
+struct Block2Dev {
+    int ncomp = 0;
+    int m = 0, nt = 0;       // records per thread and colour (1 or 2; 0: does not fit), threads (256 or 512)
+    int nodes = 0, gh = 0, red = 0, black = 0, pred = 0, pblack = 0, wb = 0;   // section lengths
+    int32_t *node = nullptr; // staged nodes
+    uint4 *e_red = nullptr, *e_black = nullptr;     // own slot, 4 sources; .w = node
+    uint4 *p_red = nullptr, *p_black = nullptr;     // pre-sweep: the same form, slots only
+    uint4 *g0 = nullptr, *g1 = nullptr;             // 9 sources; g1.z = node, g1.w = ghost number
+    int2 *w = nullptr;       // write-back: node, source
+};
+
+// A boundary-block program (with pre-sweep) as the sections of a Block2Dev, on
+// the host; m = 0 if a component exceeds what two records a thread hold.
+struct Block2Host {
+    Block2Dev d;   // counts only
+    std::vector<int32_t> node, w;
+    std::vector<uint32_t> e_red, e_black, p_red, p_black, g0, g1;   // 4 words a record
+};
+Block2Host build_blocks2(const HostLevel &L);
 // Integer geometry of a level on the device (shared by both precisions).
 struct DevGeom {
     int dim = 2, n = 0;
@@ -266,6 +287,7 @@ struct DevGeom {
     int32_t *unk_node = nullptr, *unk_ghost = nullptr;
     std::vector<int> wave;       // host copy of the wavefront offsets
     LocalDev jz, bz;             // junction zone / boundary blocks
+    Block2Dev b2;                // the boundary blocks as per-thread records (2D)
     // exact junction solve: js_n rows in js_ncomp components.  On the device
     // each component's inverse has rows padded to a multiple of 4 entries
     // (zeros) and starts at js_aoff[c], a multiple of 4; its defects sit at
@@ -345,12 +367,20 @@ struct BoundaryProgram3 {
     unsigned spin = 0;         // polls before a wait gives up
 };
 
+// Kernel view of a Block2Dev program in precision T.
+template <typename T>
+struct Block2View {
+    Block2Dev p;
+    const T *f, *gg, *gc, *gw;
+    int ng;
+    T h2;
+};
+
 // Kernel view of a LocalDev program in precision T.
 template <typename T>
 struct LocalView {
-    int ncomp, max_nodes, max_int, max_gh, max_pre, max_colour, ng;
+    int ncomp, max_nodes, max_int, max_gh, max_colour, ng;
     const int32_t *node_off, *wb_cnt, *lnode, *node_base;
-    const int32_t *pre_off, *pre_red_cnt, *pre_me, *pre_nb, *pre_glob;
     const int32_t *int_off, *red_cnt, *int_glob, *int_me, *int_nb;
     const int32_t *gh_off, *gh_me, *gh_q, *gh_stn;
     T *u;

@@ -1333,49 +1333,47 @@ void launch_rb(const LevelView<T> &v, int dim, int color, cudaStream_t s) {
 // v.u and the stored node sets are disjoint, so nothing is written twice and
 // no CTA reads a value another one writes.
 // EPT: inside entries per thread and colour the boundary blocks need
-template <int SR, int EPT>
-__global__ void __launch_bounds__(LOCAL_THREADS, 2)
-    k_relax2d(LevelView<float> v, float *__restrict__ out, const int32_t *__restrict__ strips, int ns, int nsc,
-              LocalView<float> J, int lambda) {
-    pdl_trigger();
+// One 2D relaxation up to the band sweeps: the first nsc CTAs take the strips
+// (one a warp), the others a boundary block each.  Both read the grid before
+// the relaxation and store disjoint nodes of `out`, so nothing is written twice
+// and no CTA reads what another writes.
+template <typename T, int SR, int NT, int M>
+__global__ void __launch_bounds__(NT, M == 1 ? 2 : 1)
+    k_relax2d(LevelView<T> v, T *__restrict__ out, const int32_t *__restrict__ strips, int ns, int nsc,
+              Block2View<T> J, int lambda) {
+    if (sizeof(T) == 4) pdl_trigger();
     if ((int)blockIdx.x < nsc) {
-        const int s = blockIdx.x * (LOCAL_THREADS / 32) + (threadIdx.x >> 5);
+        const int s = blockIdx.x * (NT / 32) + (threadIdx.x >> 5);
         const int32_t st = s < ns ? strips[s] : 0;   // static: read before the wait
         pdl_wait();
-        if (s < ns) rb_strip<float, SR, true>(v, out, st);   // uniform over the warp
+        if (s < ns) rb_strip<T, SR, true>(v, out, st);   // uniform over the warp
         return;
     }
-    // the block copies its index lists before waiting for the previous launch
-    local_body<float, 2, EPT>(J, v.u, out, (int)blockIdx.x - nsc, 1, lambda, true, true);
+    block2<T, NT, M>(J, v.u, out, (int)blockIdx.x - nsc, lambda, true);
 }
 
-template <int SR, int EPT>
-void launch_relax2d_as(dim3 grid, size_t smem, cudaStream_t s, const LevelView<float> &v, float *out,
-                       const DevGeom &g, int nsc, const LocalView<float> &J, int lambda) {
-    static size_t opted = 0;   // dynamic shared memory opted in for this instance
-    if (smem > opted) {
-        cudaFuncSetAttribute(k_relax2d<SR, EPT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        opted = smem;
-    }
-    pdl_launch(k_relax2d<SR, EPT>, grid, dim3(LOCAL_THREADS), smem, s, v, out, g.strips, g.nstrips, nsc, J, lambda);
+// the blocks, after the CTAs of the first ns strips (0: the blocks alone)
+template <typename T, int SR, int NT, int M>
+void launch_relax2d_as(cudaStream_t s, const LevelView<T> &v, T *out, const DevGeom &g, int ns, const Block2View<T> &J,
+                       int lambda) {
+    const int nsc = (ns + NT / 32 - 1) / (NT / 32);
+    pdl_launch(k_relax2d<T, SR, NT, M>, dim3((unsigned)(nsc + J.p.ncomp)), dim3(NT), block2_smem<T>(J.p), s, v, out,
+               g.strips, ns, nsc, J, lambda);
 }
 
-void launch_relax2d(const LevelView<float> &v, float *out, const DevGeom &g, const LocalView<float> &J, int lambda,
+template <typename T>
+void launch_relax2d_strips(cudaStream_t s, const LevelView<T> &v, T *out, const DevGeom &g, int ns,
+                           const Block2View<T> &J, int lambda) {
+    if (J.p.nt == 512) launch_relax2d_as<T, 8, 512, 2>(s, v, out, g, ns, J, lambda);
+    else if (J.p.m == 2) launch_relax2d_as<T, 8, 256, 2>(s, v, out, g, ns, J, lambda);
+    else launch_relax2d_as<T, 8, 256, 1>(s, v, out, g, ns, J, lambda);
+}
+
+template <typename T>
+void launch_relax2d(const LevelView<T> &v, T *out, const DevGeom &g, const Block2View<T> &J, int lambda,
                     cudaStream_t s) {
     g_launches++;
-    const int per = LOCAL_THREADS / 32;
-    const int nsc = (g.nstrips + per - 1) / per;
-    const size_t smem = local_smem_bytes(J, 2, true);
-    const dim3 grid((unsigned)(nsc + J.ncomp));
-    if (J.max_colour <= LOCAL_THREADS) {
-        if (g.strip_rows == 32) launch_relax2d_as<32, 1>(grid, smem, s, v, out, g, nsc, J, lambda);
-        else if (g.strip_rows == 16) launch_relax2d_as<16, 1>(grid, smem, s, v, out, g, nsc, J, lambda);
-        else launch_relax2d_as<8, 1>(grid, smem, s, v, out, g, nsc, J, lambda);
-    } else {
-        if (g.strip_rows == 32) launch_relax2d_as<32, LOCAL_EPT>(grid, smem, s, v, out, g, nsc, J, lambda);
-        else if (g.strip_rows == 16) launch_relax2d_as<16, LOCAL_EPT>(grid, smem, s, v, out, g, nsc, J, lambda);
-        else launch_relax2d_as<8, LOCAL_EPT>(grid, smem, s, v, out, g, nsc, J, lambda);
-    }
+    launch_relax2d_strips<T>(s, v, out, g, g.nstrips, J, lambda);
 }
 
 // both colours in one pass over the active 2D strips: 4 warps a CTA, one strip a warp
@@ -1394,7 +1392,7 @@ static void launch_strips_interior(const LevelView<float> &v, float *out, const 
                g.nstrips);
 }
 
-void launch_relax2d_split(const LevelView<float> &v, float *out, const DevGeom &g, const LocalView<float> &J,
+void launch_relax2d_split(const LevelView<float> &v, float *out, const DevGeom &g, const Block2View<float> &J,
                           int lambda, cudaStream_t s, cudaStream_t side, cudaEvent_t fork, cudaEvent_t join) {
     // the boundary blocks (k_relax2d without strips) on the side stream, the
     // strips (interior nodes off the band) on the main one: both read v.u and
@@ -1402,20 +1400,8 @@ void launch_relax2d_split(const LevelView<float> &v, float *out, const DevGeom &
     g_launches += 2;
     cudaEventRecord(fork, s);
     cudaStreamWaitEvent(side, fork, 0);
-    const size_t smem = local_smem_bytes(J, 2, true);
-    const dim3 grid((unsigned)J.ncomp);
-    if (J.max_colour <= LOCAL_THREADS) {
-        if (g.strip_rows == 32) launch_relax2d_as<32, 1>(grid, smem, side, v, out, g, 0, J, lambda);
-        else if (g.strip_rows == 16) launch_relax2d_as<16, 1>(grid, smem, side, v, out, g, 0, J, lambda);
-        else launch_relax2d_as<8, 1>(grid, smem, side, v, out, g, 0, J, lambda);
-    } else {
-        if (g.strip_rows == 32) launch_relax2d_as<32, LOCAL_EPT>(grid, smem, side, v, out, g, 0, J, lambda);
-        else if (g.strip_rows == 16) launch_relax2d_as<16, LOCAL_EPT>(grid, smem, side, v, out, g, 0, J, lambda);
-        else launch_relax2d_as<8, LOCAL_EPT>(grid, smem, side, v, out, g, 0, J, lambda);
-    }
-    if (g.strip_rows == 32) launch_strips_interior<32>(v, out, g, s);
-    else if (g.strip_rows == 16) launch_strips_interior<16>(v, out, g, s);
-    else launch_strips_interior<8>(v, out, g, s);
+    launch_relax2d_strips<float>(side, v, out, g, 0, J, lambda);
+    launch_strips_interior<8>(v, out, g, s);
     cudaEventRecord(join, side);
     cudaStreamWaitEvent(s, join, 0);
 }
@@ -1879,12 +1865,10 @@ void launch_junction_solve(const LevelView<T> &v, const DevGeom &g, const T *inv
 }
 
 template <typename T>
-size_t local_smem_bytes(const LocalView<T> &J, int dim, bool pre) {
+size_t local_smem_bytes(const LocalView<T> &J, int dim) {
     const int K = dim == 2 ? 9 : 27;
-    size_t b = sizeof(T) * ((size_t)J.max_nodes + (size_t)(K + 3) * J.max_gh + J.max_int) +
+    return sizeof(T) * ((size_t)J.max_nodes + (size_t)(K + 3) * J.max_gh + J.max_int) +
                sizeof(int) * ((size_t)(K + 2) * J.max_gh + J.max_nodes + J.max_int);
-    if (pre) b = (b + sizeof(T) - 1) / sizeof(T) * sizeof(T) + (sizeof(T) + sizeof(int) * (2 + 2 * dim)) * (size_t)J.max_pre;
-    return b;
 }
 
 bool local_fits_registers(int max_int_per_colour) { return max_int_per_colour <= LOCAL_THREADS * LOCAL_EPT; }
@@ -1998,9 +1982,11 @@ void launch_add_correction(const DevGeom &g, double *u64, const float *e32, cuda
     template void launch_rb_zmarch<T>(const LevelView<T> &, T *, const DevGeom &, cudaStream_t);    \
     template void launch_rb_stream3d<T>(const LevelView<T> &, T *, const DevGeom &, cudaStream_t);  \
     template bool launch_rb_rows<T>(const LevelView<T> &, const DevGeom &, cudaStream_t);           \
+    template void launch_relax2d<T>(const LevelView<T> &, T *, const DevGeom &, const Block2View<T> &, int,  \
+                                    cudaStream_t);                                                       \
     template bool launch_boundary3d<T>(const LevelView<T> &, BoundaryProgram3, int, cudaStream_t);  \
     template bool launch_boundary3d_cluster<T>(const LevelView<T> &, const BoundaryProgram3 &, cudaStream_t); \
-    template size_t local_smem_bytes<T>(const LocalView<T> &, int, bool);                                 \
+    template size_t local_smem_bytes<T>(const LocalView<T> &, int);                                       \
     template void launch_local<T>(const LocalView<T> &, int, int, int, cudaStream_t);               \
     template void launch_local_copyback<T>(const LocalView<T> &, cudaStream_t);                      \
     template void local_prepare<T>(int, size_t);

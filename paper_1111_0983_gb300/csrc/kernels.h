@@ -18,14 +18,18 @@ void launch_kaczmarz(const LevelView<double> &v, const int32_t *rows, const std:
 
 template <typename T>
 void launch_rb(const LevelView<T> &v, int dim, int color, cudaStream_t s);
-// one FP32 2D relaxation (interior sweep, ghost sweep, band sweeps) in one
-// launch: strips and boundary blocks both read v.u and write out
+// one 2D relaxation (interior sweep, ghost sweep, band sweeps) in one launch:
+// strips (of 8 rows) and boundary blocks both read v.u and write out
+template <typename T>
+void launch_relax2d(const LevelView<T> &v, T *out, const DevGeom &g, const Block2View<T> &J, int lambda,
+                    cudaStream_t s);
 // the same as two launches side by side: the boundary blocks on `side`, the
 // strips' interior nodes on `s` (fork and join through the two events)
-void launch_relax2d_split(const LevelView<float> &v, float *out, const DevGeom &g, const LocalView<float> &J,
+void launch_relax2d_split(const LevelView<float> &v, float *out, const DevGeom &g, const Block2View<float> &J,
                           int lambda, cudaStream_t s, cudaStream_t side, cudaEvent_t fork, cudaEvent_t join);
-void launch_relax2d(const LevelView<float> &v, float *out, const DevGeom &g, const LocalView<float> &J, int lambda,
-                    cudaStream_t s);
+// dynamic shared memory of the boundary blocks
+template <typename T>
+size_t block2_smem(const Block2Dev &p) { return sizeof(T) * ((size_t)p.nodes + 2 * (size_t)p.gh); }
 // both colours of a 2D sweep over the active strips (one warp a strip, rows
 // in registers): reads v.u, writes out
 template <typename T>
@@ -109,7 +113,7 @@ bool launch_rb_rows(const LevelView<T> &v, const DevGeom &g, cudaStream_t s);
 bool launch_rb_span3d(const LevelView<float> &v, float *out, const DevGeom &g, cudaStream_t s);
 
 template <typename T>
-size_t local_smem_bytes(const LocalView<T> &J, int dim, bool pre = false);
+size_t local_smem_bytes(const LocalView<T> &J, int dim);
 // shared-memory programs; a program with a write-back grid (J.wb) leaves its
 // write-back to launch_local_copyback or to launch_junction_solve
 template <typename T>

@@ -35,13 +35,6 @@ __device__ __forceinline__ void cp_async(W *smem, const W *gmem) {
 // waits until this thread's asynchronous copies have landed (and are visible to it)
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
-// start of the pre-sweep lists in a local program's shared memory: the end
-// of the other lists rounded up to a word of T
-template <typename T>
-__device__ __forceinline__ void *local_pre_base(int *end) {
-    return (void *)(((uintptr_t)end + sizeof(T) - 1) & ~(uintptr_t)(sizeof(T) - 1));
-}
-
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 // lets the launch that depends on this grid start its CTAs now: they run
 // whatever precedes their pdl_wait (reads of data no launch writes) while
@@ -246,6 +239,16 @@ constexpr int STRIP_PD = 3;    // rows loaded ahead
 __device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
 __device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
 
+// s / 4.  FP64: two off the exponent (exact, like the product) keeps it off
+// GB300's FP64 pipe, which takes 64 cycles a warp instruction; the product only
+// where that is not the quotient (0, subnormal, Inf, NaN)
+__device__ __forceinline__ float quarter(float s) { return s * 0.25f; }
+__device__ __forceinline__ double quarter(double s) {
+    const int hi = __double2hiint(s);
+    if ((((unsigned)hi >> 20) & 0x7ffu) - 3u < 0x7fcu) return __hiloint2double(hi - (2 << 20), __double2loint(s));
+    return s * 0.25;
+}
+
 // INTERIOR_ONLY: store only the inside nodes outside the boundary band (the
 // boundary blocks of the same launch store the band nodes and the ghosts)
 template <typename T, int SR, bool INTERIOR_ONLY = false>
@@ -302,15 +305,15 @@ __device__ __forceinline__ void rb_strip(const LevelView<T> &v, T *__restrict__ 
         const T uL = __shfl_up_sync(FULL, ub1, 1), uR = __shfl_down_sync(FULL, ub0, 1);
         const bool red0 = ((x + c0) & 1) == 0;   // c1 has the other colour
         T r0 = ub0, r1 = ub1;
-        if ((kc0 & NODE_KIND) == NODE_IN && red0) r0 = (mul_rn(h2, fc0) + ua0 + uc0 + uL + ub1) * (T)0.25;
-        if ((kc1 & NODE_KIND) == NODE_IN && !red0) r1 = (mul_rn(h2, fc1) + ua1 + uc1 + ub0 + uR) * (T)0.25;
+        if ((kc0 & NODE_KIND) == NODE_IN && red0) r0 = quarter(mul_rn(h2, fc0) + ua0 + uc0 + uL + ub1);
+        if ((kc1 & NODE_KIND) == NODE_IN && !red0) r1 = quarter(mul_rn(h2, fc1) + ua1 + uc1 + ub0 + uR);
         if (x > i0) {   // row o = x - 1 of the strip is complete (warp-uniform)
             const int o = x - 1;
             const T RL = __shfl_up_sync(FULL, rb1, 1), RR = __shfl_down_sync(FULL, rb0, 1);
             // a column's colour flips from row to row: c0 is black in row o when it is red in row x
             T o0 = rb0, o1 = rb1;
-            if ((kp0 & NODE_KIND) == NODE_IN && red0) o0 = (mul_rn(h2, fp0) + ra0 + r0 + RL + rb1) * (T)0.25;
-            if ((kp1 & NODE_KIND) == NODE_IN && !red0) o1 = (mul_rn(h2, fp1) + ra1 + r1 + rb0 + RR) * (T)0.25;
+            if ((kp0 & NODE_KIND) == NODE_IN && red0) o0 = quarter(mul_rn(h2, fp0) + ra0 + r0 + RL + rb1);
+            if ((kp1 & NODE_KIND) == NODE_IN && !red0) o1 = quarter(mul_rn(h2, fp1) + ra1 + r1 + rb0 + RR);
             if (own && o < n) {
                 const int b = o * pitch;
                 auto stored = [](uint8_t k) {
@@ -385,18 +388,12 @@ __device__ __forceinline__ void rb_fused2d_body(const LevelView<T> &v, T *__rest
 // the gathers through them (each thread gathers through the entries it copied
 // itself), so a component costs two memory round trips to stage whatever its
 // size.
-// wait_lists: the caller has not waited for the launches it depends on yet;
-// the index lists (static) are copied first, then it waits.
-// pre: also stage the pre-sweep's nodes and run its red then black interior
-// update first (the relaxation's interior sweep over what the component
-// reads, from `src` holding the grid before that sweep; the same sums as the
-// sweep kernels: h^2 f rounded on its own, neighbours in axis order)
 template <typename T, int D, int EPT = LOCAL_EPT>
 __device__ __forceinline__ void local_body(const LocalView<T> &J, const T *src, T *dst, int c, int lead_ghost,
-                                           int reps, bool pre = false, bool wait_lists = false) {
+                                           int reps) {
     constexpr int K = D == 2 ? 9 : 27;
     extern __shared__ __align__(16) unsigned char smem_dyn[];
-    const int n0 = J.node_off[c], nl = pre ? J.node_off[c + 1] - n0 : J.node_base[c];
+    const int n0 = J.node_off[c], nl = J.node_base[c];
     const int i0 = J.int_off[c], ni = J.int_off[c + 1] - i0, nred = J.red_cnt[c];
     const int g0 = J.gh_off[c], ngh = J.gh_off[c + 1] - g0;
     T *val = reinterpret_cast<T *>(smem_dyn);
@@ -410,11 +407,6 @@ __device__ __forceinline__ void local_body(const LocalView<T> &J, const T *src, 
     int *sln = gme + J.max_gh;                            // staged global nodes
     int *sgq = sln + J.max_nodes;                         // ghost numbers
     int *sig = sgq + J.max_gh;                            // inside entries' global nodes
-    T *pf = reinterpret_cast<T *>(local_pre_base<T>(sig + J.max_int));   // pre-sweep: f, slot, node, neighbours
-    int *pme = reinterpret_cast<int *>(pf + J.max_pre);
-    int *pgl = pme + J.max_pre;
-    int *pnb = pgl + J.max_pre;
-    const int p0 = pre ? J.pre_off[c] : 0, np = pre ? J.pre_off[c + 1] - p0 : 0;
     const int tid = threadIdx.x, nt = blockDim.x;
     for (int i = tid; i < nl; i += nt) cp_async(&sln[i], &J.lnode[n0 + i]);
     for (int e = tid; e < ngh; e += nt) {
@@ -423,11 +415,6 @@ __device__ __forceinline__ void local_body(const LocalView<T> &J, const T *src, 
     }
     for (int i = tid; i < ngh * K; i += nt) cp_async(&gst[i], &J.gh_stn[(size_t)g0 * K + i]);
     for (int i = tid; i < ni; i += nt) cp_async(&sig[i], &J.int_glob[i0 + i]);
-    for (int i = tid; i < np; i += nt) {
-        cp_async(&pme[i], &J.pre_me[p0 + i]);
-        cp_async(&pgl[i], &J.pre_glob[p0 + i]);
-    }
-    for (int i = tid; i < np * 2 * D; i += nt) cp_async(&pnb[i], &J.pre_nb[(size_t)p0 * 2 * D + i]);
     int rme[EPT], rnb[EPT][2 * D], bme[EPT], bnb[EPT][2 * D];
     T rf[EPT], bf[EPT];
 #pragma unroll
@@ -447,7 +434,6 @@ __device__ __forceinline__ void local_body(const LocalView<T> &J, const T *src, 
         }
     }
     cp_async_wait_all();
-    if (wait_lists) pdl_wait();   // the gathers read what earlier launches wrote
     for (int i = tid; i < nl; i += nt) cp_async(&val[i], &src[sln[i]]);
     for (int e = tid; e < ngh; e += nt) {
         const int q = sgq[e];
@@ -456,7 +442,6 @@ __device__ __forceinline__ void local_body(const LocalView<T> &J, const T *src, 
         for (int k = 0; k < K; k++) cp_async(&gw[e * K + k], &J.gw[(int64_t)k * J.ng + q]);
     }
     for (int i = tid; i < ni; i += nt) cp_async(&sf[i], &J.f[sig[i]]);
-    for (int i = tid; i < np; i += nt) cp_async(&pf[i], &J.f[pgl[i]]);
     cp_async_wait_all();
     __syncthreads();
 #pragma unroll
@@ -480,19 +465,6 @@ __device__ __forceinline__ void local_body(const LocalView<T> &J, const T *src, 
         return s;
     };
     const T inv = (T)(1.0 / (2 * D));
-    if (pre) {
-        const int npr = J.pre_red_cnt[c];
-        auto update = [&](int e) {
-            T s = mul_rn(J.h2, pf[e]);
-#pragma unroll
-            for (int a = 0; a < 2 * D; a++) s += val[pnb[e * 2 * D + a]];
-            val[pme[e]] = s * inv;
-        };
-        for (int e = threadIdx.x; e < npr; e += blockDim.x) update(e);
-        __syncthreads();
-        for (int e = npr + threadIdx.x; e < np; e += blockDim.x) update(e);
-        __syncthreads();
-    }
     auto ghost_sweep = [&]() {
         for (int e = threadIdx.x; e < ngh; e += blockDim.x) {
             T s = 0;
@@ -518,6 +490,154 @@ __device__ __forceinline__ void local_body(const LocalView<T> &J, const T *src, 
     }
     const int nw = J.wb_cnt[c];
     for (int i = tid; i < nw; i += nt) dst[sln[i]] = val[i];
+}
+
+// One boundary block of a 2D relaxation by one CTA of NT threads, from
+// the grid before the relaxation: the interior red and black update over every
+// inside node the block reads (the sums of the strips), the ghost sweep, then
+// reps x (red band, black band, Jacobi ghosts) on the band nodes and ghosts
+// within the reach of those phases (the block's halo); the block's own band
+// nodes and ghosts are stored into dst.  A phase is one record a thread (M at
+// most), held in registers with its weights and h^2 f, so that it costs its
+// shared-memory reads, its sum and one barrier: the records are loaded at once
+// by the threads that use them (one round trip, before the wait for the
+// previous launch where `early`), then the values through them (another).
+// Updated ghosts have two values, the ghost sweep reads one and writes the
+// other, so it takes one barrier instead of two.
+// Measured, the flower at 1025^2, a block's lists staged in shared memory by 512
+// threads (720 cycles a red / black / ghost sweep, two barriers a ghost sweep) ->
+// this form (430): a relaxation with its junction solve 8.6 -> 7.2 us; FP64 30
+// -> 20 us, where the interior sweep and the blocks had been two launches.
+template <typename T, int NT, int M>
+__device__ __forceinline__ void block2(const Block2View<T> &J, const T *__restrict__ src, T *__restrict__ dst, int c,
+                                       int reps, bool early) {
+    constexpr int RP = M + 1, RN = 4 * M, RW = 2 * M;
+    extern __shared__ __align__(16) unsigned char smem_dyn[];
+    T *val = reinterpret_cast<T *>(smem_dyn);   // nodes, then two values a ghost
+    const Block2Dev &p = J.p;
+    const int tid = threadIdx.x;
+    const uint4 none = make_uint4(0, 0, 0, 0xffffffffu);
+    auto rec = [&](const uint4 *a, int per, int k) { return tid + k * NT < per ? a[(size_t)c * per + tid + k * NT] : none; };
+    int nd[RN];
+    uint4 er[M], eb[M], pr[RP], pb[RP], ga[M], gb[M];
+    int2 wb[RW];
+#pragma unroll
+    for (int k = 0; k < RN; k++) nd[k] = tid + k * NT < p.nodes ? p.node[(size_t)c * p.nodes + tid + k * NT] : -1;
+#pragma unroll
+    for (int k = 0; k < RP; k++) {
+        pr[k] = rec(p.p_red, p.pred, k);
+        pb[k] = rec(p.p_black, p.pblack, k);
+    }
+#pragma unroll
+    for (int k = 0; k < M; k++) {
+        gb[k] = rec(p.g1, p.gh, k);
+        ga[k] = rec(p.g0, p.gh, k);
+        er[k] = rec(p.e_red, p.red, k);
+        eb[k] = rec(p.e_black, p.black, k);
+    }
+#pragma unroll
+    for (int k = 0; k < RW; k++)
+        wb[k] = tid + k * NT < p.wb ? p.w[(size_t)c * p.wb + tid + k * NT] : make_int2(-1, 0);
+    T w[M][9], gc[M];
+#pragma unroll
+    for (int k = 0; k < M; k++)
+        if ((int)gb[k].w >= 0) {
+            gc[k] = J.gc[gb[k].w];
+#pragma unroll
+            for (int i = 0; i < 9; i++) w[k][i] = J.gw[(int64_t)i * J.ng + gb[k].w];
+        }
+    if (early) pdl_wait();
+    T v[RN], fr[M], fb[M], fpr[RP], fpb[RP], gg[M], g0[M];
+#pragma unroll
+    for (int k = 0; k < RN; k++)
+        if (nd[k] >= 0) v[k] = src[nd[k]];
+#pragma unroll
+    for (int k = 0; k < RP; k++) {
+        if ((int)pr[k].w >= 0) fpr[k] = J.f[pr[k].w];
+        if ((int)pb[k].w >= 0) fpb[k] = J.f[pb[k].w];
+    }
+#pragma unroll
+    for (int k = 0; k < M; k++) {
+        if ((int)gb[k].w >= 0) {
+            g0[k] = src[gb[k].z];
+            gg[k] = J.gg[gb[k].w];
+        }
+        if ((int)er[k].w >= 0) fr[k] = J.f[er[k].w];
+        if ((int)eb[k].w >= 0) fb[k] = J.f[eb[k].w];
+    }
+#pragma unroll
+    for (int k = 0; k < RN; k++)
+        if (nd[k] >= 0) val[tid + k * NT] = v[k];
+#pragma unroll
+    for (int k = 0; k < M; k++)
+        if ((int)gb[k].w >= 0) val[p.nodes + tid + k * NT] = g0[k];
+    __syncthreads();
+    auto presweep = [&](const uint4 &r, T f) {
+        if ((int)r.w < 0) return;
+        T s = mul_rn(J.h2, f);   // h^2 f rounded on its own, neighbours in axis order
+        s += val[r.x >> 16];
+        s += val[r.y & 0xffffu];
+        s += val[r.y >> 16];
+        s += val[r.z];
+        val[r.x & 0xffffu] = quarter(s);
+    };
+#pragma unroll
+    for (int k = 0; k < RP; k++) presweep(pr[k], fpr[k]);
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < RP; k++) presweep(pb[k], fpb[k]);
+    __syncthreads();
+    int pn = 0;   // offset of the ghosts' current values
+    auto at = [&](unsigned s) -> T { return val[(s & 0x7fffu) + ((s >> 15) ? pn : 0)]; };
+    auto inside = [&](const uint4 &r, T h2f) {
+        if ((int)r.w < 0) return;
+        T s = h2f;
+        s += at(r.x >> 16);
+        s += at(r.y & 0xffffu);
+        s += at(r.y >> 16);
+        s += at(r.z);
+        val[r.x & 0xffffu] = quarter(s);
+    };
+    auto ghosts = [&]() {
+        const int po = p.gh - pn;
+#pragma unroll
+        for (int k = 0; k < M; k++)
+            if ((int)gb[k].w >= 0) {
+                T s = 0;
+                s += w[k][0] * at(ga[k].x & 0xffffu);
+                s += w[k][1] * at(ga[k].x >> 16);
+                s += w[k][2] * at(ga[k].y & 0xffffu);
+                s += w[k][3] * at(ga[k].y >> 16);
+                s += w[k][4] * at(ga[k].z & 0xffffu);
+                s += w[k][5] * at(ga[k].z >> 16);
+                s += w[k][6] * at(ga[k].w & 0xffffu);
+                s += w[k][7] * at(ga[k].w >> 16);
+                s += w[k][8] * at(gb[k].x);
+                const int j = p.nodes + tid + k * NT;
+                val[j + po] = val[j + pn] + gc[k] * (gg[k] - s);
+            }
+        pn = po;
+    };
+#pragma unroll
+    for (int k = 0; k < M; k++) {
+        fr[k] = mul_rn(J.h2, fr[k]);
+        fb[k] = mul_rn(J.h2, fb[k]);
+    }
+    ghosts();
+    __syncthreads();
+    for (int it = 0; it < reps; it++) {
+#pragma unroll
+        for (int k = 0; k < M; k++) inside(er[k], fr[k]);
+        __syncthreads();
+#pragma unroll
+        for (int k = 0; k < M; k++) inside(eb[k], fb[k]);
+        __syncthreads();
+        ghosts();
+        __syncthreads();
+    }
+#pragma unroll
+    for (int k = 0; k < RW; k++)
+        if (wb[k].x >= 0) dst[wb[k].x] = at((unsigned)wb[k].y);
 }
 
 // write-back node i of the flat list: u = wb

@@ -558,7 +558,6 @@ struct ProgramBuilder {
         P.max_nodes = std::max(P.max_nodes, (int)nodes.size());
         P.max_int = std::max(P.max_int, nint);
         P.max_gh = std::max(P.max_gh, ngh);
-        P.max_pre = std::max(P.max_pre, P.pre_off.back() - P.pre_off[P.pre_off.size() - 2]);
         for (int64_t p : nodes) local[p] = -1;
     }
     // union lists of the updated nodes of all components (global fallback)
@@ -747,6 +746,91 @@ void build_boundary_blocks(HostLevel &L, int lambda, int block) {
     std::sort(all.begin(), all.end());
     PB.finish(all);
     L.boundary = std::move(prog);
+}
+
+Block2Host build_blocks2(const HostLevel &L) {
+    Block2Host out;
+    const LocalProgram &P = L.boundary;
+    Block2Dev &d = out.d;
+    d.ncomp = P.ncomp();
+    if (L.dim != 2 || d.ncomp == 0 || P.pre_me.empty()) return out;
+    // section lengths: the largest component's counts
+    for (int c = 0; c < d.ncomp; c++) {
+        const int ni = P.int_off[c + 1] - P.int_off[c], np = P.pre_off[c + 1] - P.pre_off[c];
+        d.nodes = std::max(d.nodes, P.node_off[c + 1] - P.node_off[c]);
+        d.gh = std::max(d.gh, P.gh_off[c + 1] - P.gh_off[c]);
+        d.red = std::max(d.red, P.red_cnt[c]);
+        d.black = std::max(d.black, ni - P.red_cnt[c]);
+        d.pred = std::max(d.pred, P.pre_red_cnt[c]);
+        d.pblack = std::max(d.pblack, np - P.pre_red_cnt[c]);
+        d.wb = std::max(d.wb, P.wb_cnt[c]);
+    }
+    // 256 threads hold the blocks of a band of 3 h; a wide band takes 512
+    for (int v = 0; v < 3 && d.m == 0; v++) {
+        const int m = v == 0 ? 1 : 2, T = v == 2 ? 512 : 256;
+        if (std::max({d.gh, d.red, d.black}) <= m * T && std::max(d.pred, d.pblack) <= (m + 1) * T &&
+            d.nodes <= 4 * m * T && d.wb <= 2 * m * T) {
+            d.m = m;
+            d.nt = T;
+        }
+    }
+    if (d.m == 0 || d.nodes + d.gh >= 0x8000) {
+        d.m = 0;
+        return out;
+    }
+    const uint32_t none = 0xffffffffu;
+    out.node.assign((size_t)d.ncomp * d.nodes, -1);
+    out.w.assign((size_t)d.ncomp * d.wb * 2, -1);
+    auto records = [&](std::vector<uint32_t> &v, int per) {
+        v.assign((size_t)d.ncomp * per * 4, 0);
+        for (size_t i = 3; i < v.size(); i += 4) v[i] = none;
+    };
+    records(out.e_red, d.red);
+    records(out.e_black, d.black);
+    records(out.p_red, d.pred);
+    records(out.p_black, d.pblack);
+    records(out.g0, d.gh);
+    records(out.g1, d.gh);
+    std::vector<uint16_t> src;   // slot -> source
+    for (int c = 0; c < d.ncomp; c++) {
+        const int n0 = P.node_off[c], nl = P.node_off[c + 1] - n0, g0 = P.gh_off[c], ngh = P.gh_off[c + 1] - g0;
+        src.resize(nl);
+        for (int i = 0; i < nl; i++) {
+            src[i] = (uint16_t)i;
+            out.node[(size_t)c * d.nodes + i] = P.lnode[n0 + i];
+        }
+        for (int j = 0; j < ngh; j++) src[P.gh_me[g0 + j]] = (uint16_t)(0x8000 | (d.nodes + j));
+        auto entry = [](uint32_t *r, int me, const int32_t *nb, const std::vector<uint16_t> *map, int32_t node) {
+            auto s = [&](int k) { return map ? (uint32_t)(*map)[nb[k]] : (uint32_t)nb[k]; };
+            r[0] = (uint32_t)me | s(0) << 16;
+            r[1] = s(1) | s(2) << 16;
+            r[2] = s(3);
+            r[3] = (uint32_t)node;
+        };
+        for (int e = P.int_off[c]; e < P.int_off[c + 1]; e++) {
+            const int k = e - P.int_off[c], nr = P.red_cnt[c];
+            uint32_t *r = k < nr ? &out.e_red[((size_t)c * d.red + k) * 4] : &out.e_black[((size_t)c * d.black + k - nr) * 4];
+            entry(r, P.int_me[e], &P.int_nb[(size_t)e * 4], &src, P.int_glob[e]);
+        }
+        for (int e = P.pre_off[c]; e < P.pre_off[c + 1]; e++) {
+            const int k = e - P.pre_off[c], nr = P.pre_red_cnt[c];
+            uint32_t *r = k < nr ? &out.p_red[((size_t)c * d.pred + k) * 4] : &out.p_black[((size_t)c * d.pblack + k - nr) * 4];
+            entry(r, P.pre_me[e], &P.pre_nb[(size_t)e * 4], nullptr, P.pre_glob[e]);
+        }
+        for (int j = 0; j < ngh; j++) {
+            uint32_t *a = &out.g0[((size_t)c * d.gh + j) * 4], *b = &out.g1[((size_t)c * d.gh + j) * 4];
+            const int32_t *st = &P.gh_stn[(size_t)(g0 + j) * 9];
+            for (int k = 0; k < 4; k++) a[k] = (uint32_t)src[st[2 * k]] | (uint32_t)src[st[2 * k + 1]] << 16;
+            b[0] = src[st[8]];
+            b[2] = (uint32_t)P.lnode[n0 + P.gh_me[g0 + j]];
+            b[3] = (uint32_t)P.gh_q[g0 + j];
+        }
+        for (int i = 0; i < P.wb_cnt[c]; i++) {
+            out.w[((size_t)c * d.wb + i) * 2] = P.lnode[n0 + i];
+            out.w[((size_t)c * d.wb + i) * 2 + 1] = src[i];
+        }
+    }
+    return out;
 }
 
 bool partial_transfer_weights(const HostLevel &F, int64_t p, bool interior, double *wt) {
