@@ -650,26 +650,28 @@ T *cycle(gcmg_ctx *c, int l, T *u) {
     return u;
 }
 
-// ||(f, g)||_inf: f over the inside nodes (those of the active chunks where
-// the level has them), g over the ghosts
+// calls visit(p) at every inside node of a level, a warp a row segment
+template <typename F>
+__device__ __forceinline__ void for_inside(const LevelView<double> &lv, F &&visit) {
+    const int lane = threadIdx.x & 31, nw = (int)((gridDim.x * blockDim.x) >> 5);
+    for (int q = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5); q < lv.nsegs; q += nw) {
+        const int2 sg = lv.segs[q];
+        const int k0 = sg.y & 0xffff, k1 = (int)((unsigned)sg.y >> 16);
+        for (int k = k0 + lane; k <= k1; k += 32) visit((int64_t)sg.x * lv.n + k);
+    }
+}
+// CTAs of such a launch (256 threads), at most `most`
+unsigned inside_blocks(const LevelView<double> &lv, int64_t more, unsigned most) {
+    return (unsigned)std::max<int64_t>(1, std::min<int64_t>((std::max<int64_t>(32 * (int64_t)lv.nsegs, more) + 255) / 256, most));
+}
+
+// ||(f, g)||_inf: f over the inside nodes, g over the ghosts
 __global__ void k_rhs_norm(LevelView<double> lv, const double *g, int ng, unsigned long long *bits) {
     __shared__ double wmax[32];
-    const uint8_t *type = lv.type;
     const double *f = lv.f;
-    const int64_t nt = lv.chunks ? lv.nchunks * CHUNK : lv.nn;
     double v = 0.0;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < nt || i < ng;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        int64_t p = i;
-        bool ok = i < nt;
-        if (ok && lv.chunks) {   // thread i: node i % CHUNK of chunk i / CHUNK
-            ok = (int)(i % CHUNK) < (lv.clen[i / CHUNK] & 63);
-            p = (int64_t)lv.chunks[i / CHUNK] + i % CHUNK;
-        }
-        if (ok && (type[p] & NODE_KIND) == NODE_IN) v = fmax(v, fabs(f[p]));
-        if (i < ng) v = fmax(v, fabs(g[i]));
-        if (v != v) v = __longlong_as_double(0x7ff0000000000000ll);
-    }
+    for_inside(lv, [&](int64_t p) { v = fmax(v, fabs(f[p])); });
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < ng; i += gridDim.x * blockDim.x) v = fmax(v, fabs(g[i]));
     for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, o));
     if ((threadIdx.x & 31) == 0) wmax[threadIdx.x >> 5] = v;
     __syncthreads();
@@ -761,9 +763,7 @@ void solve_prologue(gcmg_ctx *c, cudaGraphConditionalHandle h) {
     const HostLevel &L0 = c->H[0];
     ck(cudaMemsetAsync(c->d_norm + 1, 0, sizeof(unsigned long long), c->stream), "memset");
     const LevelView<double> lv = view<double>(c, 0, c->D64[0]);
-    const int64_t cnt = std::max<int64_t>(lv.chunks ? lv.nchunks * CHUNK : L0.nn, L0.ng());
-    const unsigned nb = (unsigned)std::min<int64_t>((cnt + 255) / 256, 4096);
-    k_rhs_norm<<<nb, 256, 0, c->stream>>>(lv, c->D64[0].gg, g0.ng, c->d_norm + 1);
+    k_rhs_norm<<<inside_blocks(lv, L0.ng(), 4096), 256, 0, c->stream>>>(lv, c->D64[0].gg, g0.ng, c->d_norm + 1);
     g_launches++;
     fine_defect(c);
     k_loop_start<<<1, 1, 0, c->stream>>>(h, c->d_norm, c->d_r0, c->d_rel, c->d_m, c->p.rtol);
@@ -1414,9 +1414,7 @@ gcmg_status gcmg_residual(gcmg_ctx *c, const double *u_dev, double *r_dev, doubl
         LevelView<double> v = view<double>(c, 0, c->D64[0]);
         // ||(f, g)|| into slot 1, the defect's norm into slot 0
         ck(cudaMemsetAsync(c->d_norm, 0, 2 * sizeof(unsigned long long), c->stream), "memset");
-        const int64_t cnt = std::max<int64_t>(v.chunks ? v.nchunks * CHUNK : L0.nn, L0.ng());
-        const unsigned nb = (unsigned)std::min<int64_t>((cnt + 255) / 256, 4096);
-        k_rhs_norm<<<nb, 256, 0, c->stream>>>(v, c->D64[0].gg, g0.ng, c->d_norm + 1);
+        k_rhs_norm<<<inside_blocks(v, L0.ng(), 4096), 256, 0, c->stream>>>(v, c->D64[0].gg, g0.ng, c->d_norm + 1);
         g_launches++;
         v.u = const_cast<double *>(u_dev);
         v.r = r_dev;
@@ -1536,9 +1534,7 @@ gcmg_status gcmg_solve(gcmg_ctx *c, double *u_dev, gcmg_stats *stats) {
             ck(cudaMemsetAsync(c->d_norm, 0, sizeof(unsigned long long), c->stream), "memset");
             {
                 const LevelView<double> lv = view<double>(c, 0, c->D64[0]);
-                const int64_t cnt = std::max<int64_t>(lv.chunks ? lv.nchunks * CHUNK : L0.nn, L0.ng());
-                const unsigned nb = (unsigned)std::min<int64_t>((cnt + 255) / 256, 4096);
-                k_rhs_norm<<<nb, 256, 0, c->stream>>>(lv, c->D64[0].gg, g0.ng, c->d_norm);
+                k_rhs_norm<<<inside_blocks(lv, L0.ng(), 4096), 256, 0, c->stream>>>(lv, c->D64[0].gg, g0.ng, c->d_norm);
                 g_launches++;
             }
             check_launch();
@@ -1583,18 +1579,8 @@ gcmg_status gcmg_solve(gcmg_ctx *c, double *u_dev, gcmg_stats *stats) {
 // f at the inside nodes of the finest level, read by the device straight from
 // a host buffer it can address (page-locked memory): the solver reads f only
 // on Omega_h, so the other n^d - |Omega_h| values need not cross the link.
-// Nodes visited as in k_rhs_norm (the active chunks in 3D, else every node).
 __global__ void k_gather_inside(LevelView<double> lv, const double *__restrict__ src, double *__restrict__ dst) {
-    const uint8_t *type = lv.type;
-    const int64_t nt = lv.chunks ? lv.nchunks * CHUNK : lv.nn;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < nt; i += (int64_t)gridDim.x * blockDim.x) {
-        int64_t p = i;
-        if (lv.chunks) {
-            if ((int)(i % CHUNK) >= (lv.clen[i / CHUNK] & 63)) continue;
-            p = (int64_t)lv.chunks[i / CHUNK] + i % CHUNK;
-        }
-        if ((type[p] & NODE_KIND) == NODE_IN) dst[p] = src[p];
-    }
+    for_inside(lv, [&](int64_t p) { dst[p] = src[p]; });
 }
 
 // u (all nn values) stored by the device straight into a host buffer it can
@@ -1632,9 +1618,7 @@ gcmg_status gcmg_solve_host(gcmg_ctx *c, const double *f_host, const double *g_h
         const void *f_mapped = mapped_host(f_host);
         if (f_mapped) {
             const LevelView<double> lv = view<double>(c, 0, c->D64[0]);
-            const int64_t cnt = lv.chunks ? lv.nchunks * CHUNK : L.nn;
-            const unsigned nb = (unsigned)std::min<int64_t>((cnt + 255) / 256, 8192);
-            k_gather_inside<<<nb, 256, 0, c->stream>>>(lv, static_cast<const double *>(f_mapped), c->D64[0].f);
+            k_gather_inside<<<inside_blocks(lv, 0, 8192), 256, 0, c->stream>>>(lv, static_cast<const double *>(f_mapped), c->D64[0].f);
             g_launches++;
             check_launch();
         } else {

@@ -120,9 +120,9 @@ struct HostLevel {
     // interval (the sweep then falls back to the tiles).
     std::vector<int32_t> sp_rows, sp;
     int sp_cols = 0;
-    // segments of up to 64 consecutive inside nodes of a row, as pairs
-    // (i * n + j, first | last << 16), in increasing node order: the work of
-    // the one-colour row sweep (any domain)
+    // segments of up to 64 consecutive inside nodes of a row, as pairs (row,
+    // first | last << 16), in increasing node order, the row i (2D) or i * n +
+    // j (3D): the work of the passes over the inside nodes (any domain)
     std::vector<int32_t> sp_list;
     // defect extension of this level (before restricting to the next coarser one)
     std::vector<int32_t> ext_node;      // ordered by upwind wavefront
@@ -342,7 +342,7 @@ struct LevelView {
     const int32_t *chunks = nullptr;
     const uint8_t *clen = nullptr;
     int64_t nchunks = 0;
-    // 3D: segments of up to 64 consecutive inside nodes of a row (DevGeom::sp_list)
+    // segments of up to 64 consecutive inside nodes of a row (DevGeom::sp_list)
     const int2 *segs = nullptr;
     int nsegs = 0;
     // 3D: ghost stencils as boxes (DevGeom::gcode, gbase; null: gstn only)

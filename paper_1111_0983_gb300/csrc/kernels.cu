@@ -619,13 +619,12 @@ __global__ void __launch_bounds__(256) k_rb_rows(LevelView<T> v, const int2 *__r
     }
 }
 
-// The defect f + Lap_h u (TGCS step 3) at every inside node of a 3D level
-// into r, over the row segments: a warp takes G segments at once, lane l the
+// The defect f + Lap_h u (TGCS step 3) at every inside node of a level into r, over the row segments: a warp takes G segments at once, lane l the
 // nodes k0 + l and k0 + l + 32 of each, all loads issued before the first
 // store; with norm, its max-norm.  MIXED (the FP64 finest level of the mixed
 // form): also f32 = the defect rounded to FP32 and e32 = 0 at those nodes.
 // The expression of defect_node.
-template <typename T, int G, bool MIXED>
+template <typename T, int D, int G, bool MIXED>
 __global__ void __launch_bounds__(256) k_defect_rows(LevelView<T> v, unsigned long long *norm, float *__restrict__ f32,
                                                     float *__restrict__ e32) {
     if (MIXED) pdl_trigger();
@@ -650,7 +649,7 @@ __global__ void __launch_bounds__(256) k_defect_rows(LevelView<T> v, unsigned lo
                 const int k = k0 + lane + 32 * h;
                 on[2 * g + h] = k <= k1;
                 p[2 * g + h] = (int64_t)sg.x * n + k;
-                if (on[2 * g + h]) d[2 * g + h] = inside_defect<T, 3>(v, p[2 * g + h]);
+                if (on[2 * g + h]) d[2 * g + h] = inside_defect<T, D>(v, p[2 * g + h]);
             }
         }
 #pragma unroll
@@ -668,68 +667,87 @@ __global__ void __launch_bounds__(256) k_defect_rows(LevelView<T> v, unsigned lo
     reduce_norm(norm, __longlong_as_double((long long)mb));
 }
 
-// The interpolation of the coarse correction added at every unknown of a 3D
-// level (Sec. 2.6; the sums of prolong_node_early): the inside nodes over
-// the row segments, G at once, lane l the nodes k0 + l and k0 + l + 32 of
-// each, every parent's type and value loaded before the first sum; past
-// them the ghosts, a thread each.
-template <typename T, int G>
+// The interpolation of the coarse correction added at every unknown of a
+// level (Sec. 2.6; the sums of prolong_node): the inside nodes over the row
+// segments, G at once, lane l the nodes k0 + l and k0 + l + 32 of each; past
+// them the ghosts, 32 a warp at once.  The segments and the parents' types are
+// fixed: those of a warp's first group are read before the wait for the
+// previous launch; every parent's value is loaded before the first sum.
+template <typename T, int D, int G>
 __global__ void __launch_bounds__(256) k_prolong_rows(LevelView<T> F, LevelView<T> C, const T *__restrict__ e,
                                                       T *__restrict__ out) {
+    constexpr int NP = 1 << D;   // parents, in the order of prolong_node's loops
     if (sizeof(T) == 4) pdl_trigger();
     const int lane = threadIdx.x & 31;
     const int nw = (int)((gridDim.x * blockDim.x) >> 5);
     const int n = F.n, nseg = F.nsegs;
-    pdl_wait();
-    for (int q = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5) * G; q < nseg; q += nw * G) {
-        T ev[2 * G][8], old[2 * G];
-        bool use[2 * G][8], on[2 * G];
-        int64_t pp[2 * G];
-        int cnt[2 * G];
+    int64_t pp[2 * G], X0[2 * G];
+    unsigned use[2 * G];   // bit s: parent s lies in Omega_2h u Gamma_2h
+    int cnt[2 * G];        // parents by parity; 0: no node
+    auto parent = [&](int s) -> int64_t {
+        return D == 3 ? (s >> 2) * C.s0 + ((s >> 1) & 1) * C.s1 + (s & 1) : (s >> 1) * C.s0 + (s & 1);
+    };
+    // node x of the group: node k of row `row`, if any
+    auto node = [&](int x, int row, int k, bool on) {
+        const int i = D == 3 ? row / n : row, j = D == 3 ? row - i * n : 0;
+        pp[x] = (int64_t)row * n + k;
+        X0[x] = (int64_t)(i / 2) * C.s0 + (D == 3 ? (int64_t)(j / 2) * C.s1 : 0) + k / 2;
+        // the parents whose offset the node's parity allows, per axis
+        const unsigned odd = D == 3 ? (i & 1) << 2 | (j & 1) << 1 | (k & 1) : (i & 1) << 1 | (k & 1);
+        cnt[x] = on ? 1 << __popc(odd) : 0;
+        use[x] = 0;
+#pragma unroll
+        for (int s = 0; s < NP; s++)
+            if (on && (s & ~odd) == 0) {
+                const uint8_t kc = C.type[X0[x] + parent(s)] & NODE_KIND;
+                use[x] |= (unsigned)(kc == NODE_IN || kc == NODE_GHOST) << s;
+            }
+    };
+    const int last = nseg + (F.ng + 31) / 32;   // ghost groups follow the segments
+    auto fixed = [&](int q) {
 #pragma unroll
         for (int g = 0; g < G; g++) {
-            const int2 sg = q + g < nseg ? F.segs[q + g] : make_int2(0, 0x0000ffff);
-            const int i = sg.x / n, j = sg.x - (sg.x / n) * n;
-            const int k0 = sg.y & 0xffff, k1 = (int)((unsigned)sg.y >> 16);
-#pragma unroll
-            for (int h = 0; h < 2; h++) {
-                const int e_ = 2 * g + h, k = k0 + lane + 32 * h;
-                on[e_] = k <= k1;
-                pp[e_] = (int64_t)sg.x * n + k;
-                const int n1 = (i & 1) ? 2 : 1, n2 = (j & 1) ? 2 : 1, n3 = (k & 1) ? 2 : 1;
-                cnt[e_] = n1 * n2 * n3;
-                const int64_t X0 = (int64_t)(i / 2) * C.s0 + (int64_t)(j / 2) * C.s1 + k / 2;
-#pragma unroll
-                for (int s8 = 0; s8 < 8; s8++) {
-                    const int a = s8 >> 2, b = (s8 >> 1) & 1, c = s8 & 1;
-                    const int64_t X = X0 + a * C.s0 + b * C.s1 + c;
-                    use[e_][s8] = false;
-                    if (on[e_] && a < n1 && b < n2 && c < n3) {
-                        const uint8_t kc = C.type[X] & NODE_KIND;
-                        use[e_][s8] = kc == NODE_IN || kc == NODE_GHOST;   // parents in Omega_2h u Gamma_2h
-                    }
-                    ev[e_][s8] = use[e_][s8] ? e[X] : (T)0;
-                }
-                old[e_] = on[e_] ? out[pp[e_]] : (T)0;
+            if (q + g < nseg) {
+                const int2 sg = F.segs[q + g];
+                const int k0 = sg.y & 0xffff, k1 = (int)((unsigned)sg.y >> 16);
+                node(2 * g, sg.x, k0 + lane, k0 + lane <= k1);
+                node(2 * g + 1, sg.x, k0 + lane + 32, k0 + lane + 32 <= k1);
+            } else {
+                const int e_ = (q + g - nseg) * 32 + lane;
+                const int p = q + g < last && e_ < F.ng ? F.gnode[e_] : -1;
+                node(2 * g, p < 0 ? 0 : p / n, p < 0 ? 0 : p % n, p >= 0);
+                cnt[2 * g + 1] = 0;
+                use[2 * g + 1] = 0;
             }
         }
+    };
+    int q = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5) * G;
+    if (q < last) fixed(q);
+    pdl_wait();
+    for (; q < last; q += nw * G) {
+        T ev[2 * G][NP], old[2 * G];
 #pragma unroll
-        for (int e_ = 0; e_ < 2 * G; e_++) {
-            if (!on[e_]) continue;
+        for (int x = 0; x < 2 * G; x++) {
+#pragma unroll
+            for (int s = 0; s < NP; s++) ev[x][s] = (use[x] >> s & 1u) ? e[X0[x] + parent(s)] : (T)0;
+            old[x] = cnt[x] ? out[pp[x]] : (T)0;
+        }
+#pragma unroll
+        for (int x = 0; x < 2 * G; x++) {
+            if (!cnt[x]) continue;
             T num = 0, den = 0;
-            const T w = (T)1 / (T)cnt[e_];   // a power of two: exact
+            const T w = (T)1 / (T)cnt[x];   // a power of two: exact
 #pragma unroll
-            for (int s8 = 0; s8 < 8; s8++)
-                if (use[e_][s8]) {
-                    num += w * ev[e_][s8];
+            for (int s = 0; s < NP; s++)
+                if (use[x] >> s & 1u) {
+                    num += w * ev[x][s];
                     den += w;
                 }
             const T val = den > (T)0 ? num / den : (T)0;
-            out[pp[e_]] = old[e_] + val;
+            out[pp[x]] = old[x] + val;
         }
+        if (q + nw * G < last) fixed(q + nw * G);
     }
-    for (int qg = (int)(blockIdx.x * blockDim.x + threadIdx.x); qg < F.ng; qg += (int)(gridDim.x * blockDim.x))
-        prolong_node<T, 3>(F, C, e, out, true, F.gnode[qg]);
 }
 
 // u64 += e32 at the inside nodes over the row segments (G at once) and, past
@@ -771,6 +789,18 @@ __global__ void __launch_bounds__(256) k_add_rows(LevelView<double> v, double *_
         const int64_t g = v.gnode[q];
         u64[g] += (double)e32[g];
     }
+}
+
+// SMs of the current device (queried once)
+static int num_sms() {
+    static int count = 0;
+    if (count <= 0) {
+        int d = 0, m = 0;
+        if (cudaGetDevice(&d) == cudaSuccess && cudaDeviceGetAttribute(&m, cudaDevAttrMultiProcessorCount, d) ==
+                                                     cudaSuccess)
+            count = m;
+    }
+    return count > 0 ? count : 1;
 }
 
 template <typename K>
@@ -1141,18 +1171,24 @@ __global__ void k_descend(LevelView<T> F, LevelView<T> C, T *__restrict__ fc, T 
         if (has) descend_node<T, D, FROM_R>(F, C, fc, uc, i, split);
         return;
     }
-    if (sizeof(T) == 8) {
-        // the thread-per-index form: in FP64 the terms are plain reads of r
-        pdl_wait();
-        descend_item<T, D, FROM_R>(F, C, fc, gc, uc, ptr, col, val, blockIdx.x * (int64_t)blockDim.x + threadIdx.x);
+    // 2D: the first 32 C.ng threads take the coarse ghost rows, a warp each; the
+    // next ones the segments of coarse inside nodes, a thread a node.  Both read
+    // their static data before waiting for the previous launch.  Every other
+    // node of fc and uc is 0 from the start.
+    const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, nw = 32 * (int64_t)C.ng;
+    if (t < nw) {   // uniform over the warp
+        const int q = (int)(t >> 5);
+        descend_ghost_row_warp_early<T, D, FROM_R>(F, gc, ptr, col, val, q);
+        if ((t & 31) == 0) uc[C.gnode[q]] = 0;
         return;
     }
-    // 2D: the first 32 C.ng threads take the coarse ghost rows, a warp each;
-    // the rest the coarse nodes, a thread each; both read their static data
-    // before waiting for the previous launch
-    const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, nw = 32 * (int64_t)C.ng;
-    if (t < nw) descend_ghost_row_warp_early<T, D, FROM_R>(F, gc, ptr, col, val, (int)(t >> 5));   // uniform over the warp
-    else if (t - nw < C.nn) descend_node_early<T, D, FROM_R>(F, C, fc, uc, t - nw);
+    const int64_t sgi = (t - nw) >> 6;   // 64 threads a segment
+    const int2 sg = sgi < C.nsegs ? C.segs[sgi] : make_int2(0, 0x0000ffff);
+    const int k = (sg.y & 0xffff) + (int)((t - nw) & 63);
+    if (k <= (int)((unsigned)sg.y >> 16))
+        descend_inside_early<T, D, FROM_R>(F, fc, uc, (int64_t)sg.x * C.n + k, 2 * ((int64_t)sg.x * F.s0 + k));
+    else
+        pdl_wait();
 }
 
 // 3D descent at the coarse inside nodes whose fine neighbourhood is partly
@@ -1233,15 +1269,12 @@ __global__ void k_ghost_transfer(const T *__restrict__ rf, const int32_t *__rest
 }
 
 // ------------------------------------------------------------ interpolation
+// on every node of the box (0 off Omega_h u Gamma_h), for a caller's grid and full multigrid
 template <typename T, int D>
-__global__ void k_prolong(LevelView<T> F, LevelView<T> C, const T *__restrict__ e, T *__restrict__ out, bool add) {
-    if (sizeof(T) == 4) pdl_trigger();
-    if (!add) F.chunks = nullptr;   // every node of out is written: the whole box
-    int64_t p;
-    if (level_node(F, blockIdx.x * (int64_t)blockDim.x + threadIdx.x, p))
-        prolong_node_early<T, D>(F, C, e, out, add, p);   // waits after reading the types
-    else
-        pdl_wait();
+__global__ void k_prolong(LevelView<T> F, LevelView<T> C, const T *__restrict__ e, T *__restrict__ out) {
+    pdl_wait();
+    const int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (p < F.nn) prolong_node<T, D>(F, C, e, out, false, p);
 }
 
 // --------------------------------------------------------------- coarsest
@@ -1254,29 +1287,9 @@ __global__ void k_coarse_solve(LevelView<T> v, const int32_t *__restrict__ unk_n
 }
 
 // ------------------------------------------------------- mixed precision
-// FP64 defect of the finest level (r, its norm) that also sets up the next
-// FP32 correction problem: right-hand side = the defect rounded to FP32 at
-// inside nodes, 0 elsewhere; initial correction e32 = 0 everywhere
-template <int D>
-__global__ void k_defect_interior_mixed(LevelView<double> v, unsigned long long *norm, float *__restrict__ f32,
-                                        float *__restrict__ e32) {
-    pdl_trigger();
-    pdl_wait();
-    const int64_t nt = v.chunks ? v.nchunks * CHUNK : v.nn;
-    double m = 0.0;
-    for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < nt; t += (int64_t)gridDim.x * blockDim.x) {
-        int64_t p;
-        if (!level_node(v, t, p)) continue;   // nodes off the chunks stay 0
-        const double val = defect_node<double, D>(v, p, false);   // 0 off Omega_h
-        f32[p] = (float)val;
-        e32[p] = 0.0f;
-        m = fmax(m, abs_keep_nan(val));
-    }
-    reduce_norm(norm, m);
-}
-
-// ... and its ghost rows: the ghost defects rounded to FP32
-// (e32: when not null, also e32 = 0 at the ghosts)
+// Ghost rows of the FP64 defect of the finest level that sets up the next FP32
+// correction problem (the inside nodes: k_defect_rows): r, the defects rounded
+// to FP32 into g32, e32 = 0 at the ghosts
 template <int K>
 __global__ void k_defect_ghost_mixed(LevelView<double> v, unsigned long long *norm, float *__restrict__ g32,
                                      float *__restrict__ e32) {
@@ -1287,20 +1300,9 @@ __global__ void k_defect_ghost_mixed(LevelView<double> v, unsigned long long *no
     if (q < v.ng) {
         val = defect_ghost_item<double, K>(v, q);
         g32[q] = (float)val;
-        if (e32) e32[v.gnode[q]] = 0.0f;
+        e32[v.gnode[q]] = 0.0f;
     }
     reduce_norm(norm, val);
-}
-
-// u64 += e32 on Omega_h u Gamma_h
-__global__ void k_add_correction(LevelView<double> v, double *__restrict__ u64, const float *__restrict__ e32) {
-    pdl_trigger();
-    pdl_wait();
-    const uint8_t *__restrict__ type = v.type;
-    int64_t p;
-    if (!level_node(v, blockIdx.x * (int64_t)blockDim.x + threadIdx.x, p)) return;
-    const uint8_t k = type[p] & NODE_KIND;
-    if (k == NODE_IN || k == NODE_GHOST) u64[p] += (double)e32[p];
 }
 
 // keep u = 0 off Omega_h u Gamma_h
@@ -1626,15 +1628,29 @@ void launch_ghost_relax_list(const LevelView<T> &v, int dim, const int32_t *list
     pdl_launch(k_ghost_store_list<T>, dim3(blocks_for(cnt)), dim3(kThreads), 0, s, v, list, cnt);
 }
 
+// k_defect_rows with G segments a warp, or one where G would leave SMs idle: G
+// at once pay the memory's latency once for G, but a warp's arithmetic (the
+// FP64 form's exact sum above all) is a chain
+template <typename T, int D, int G, bool MIXED>
+static void launch_defect_rows(const LevelView<T> &v, unsigned long long *norm, float *f32, float *e32, cudaStream_t s) {
+    static unsigned resident = 0, resident1 = 0;
+    if (v.nsegs >= 32 * G * num_sms())
+        pdl_launch(k_defect_rows<T, D, G, MIXED>,
+                   dim3(segment_blocks(k_defect_rows<T, D, G, MIXED>, v.nsegs, G, resident)), dim3(256), 0, s, v, norm,
+                   f32, e32);
+    else
+        pdl_launch(k_defect_rows<T, D, 1, MIXED>,
+                   dim3(segment_blocks(k_defect_rows<T, D, 1, MIXED>, v.nsegs, 1, resident1)), dim3(256), 0, s, v, norm,
+                   f32, e32);
+}
+
 template <typename T>
 void launch_defect(const LevelView<T> &v, int dim, bool zero_rest, unsigned long long *norm, cudaStream_t s) {
     g_launches += v.ng > 0 ? 2 : 1;
     const unsigned nb = std::min(blocks_for(level_threads(v, !zero_rest)), kNormBlocks);
-    if (dim == 3 && !zero_rest && v.nsegs > 0) {   // inside nodes over the row segments
-        constexpr int G = 4;
-        static unsigned resident = 0;
-        pdl_launch(k_defect_rows<T, G, false>, dim3(segment_blocks(k_defect_rows<T, G, false>, v.nsegs, G, resident)),
-                   dim3(256), 0, s, v, norm, (float *)nullptr, (float *)nullptr);
+    if (!zero_rest) {   // inside nodes over the row segments
+        if (dim == 2) launch_defect_rows<T, 2, 4, false>(v, norm, nullptr, nullptr, s);
+        else launch_defect_rows<T, 3, 4, false>(v, norm, nullptr, nullptr, s);
     } else if (dim == 2) pdl_launch(k_defect_interior<T, 2>, dim3(nb), dim3(kThreads), 0, s, v, zero_rest, norm);
     else pdl_launch(k_defect_interior<T, 3>, dim3(nb), dim3(kThreads), 0, s, v, zero_rest, norm);
     if (v.ng > 0) {
@@ -1674,20 +1690,15 @@ void launch_restrict(const LevelView<T> &F, const LevelView<T> &C, int dim, T *f
 template <typename T>
 void launch_descend(const LevelView<T> &F, const LevelView<T> &C, const DevGeom &gf, const T *gt_val, T *fc, T *gc,
                     T *uc, cudaStream_t s, const T *pt_w) {
-    const bool warp_rows = sizeof(T) == 4 && gf.dim == 2;   // 2D FP32: a warp per coarse ghost row
-    const int64_t n = gf.dim == 3 ? level_threads(C, true) : warp_rows ? C.nn + 32 * (int64_t)C.ng
-                                                                      : std::max<int64_t>(C.nn, C.ng);
+    // 3D: a thread a node of the coarse chunks; 2D: a warp per coarse ghost row, two per coarse segment
+    const int64_t n = gf.dim == 3 ? level_threads(C, true) : 64 * (int64_t)C.nsegs + 32 * (int64_t)C.ng;
     if (gf.dim == 3 && F.nsegs > 0) {
         // 3D with row segments: one defect pass first (inside nodes over the
         // segments, then the ghosts), so that each fine defect is computed
         // once rather than once per coarse node whose 27-node neighbourhood
         // holds it (27/8 times on average); the same values as on the spot
-        constexpr int G = 4;
-        static unsigned resident = 0;
-        const unsigned blocks = segment_blocks(k_defect_rows<T, G, false>, F.nsegs, G, resident);
         g_launches++;
-        pdl_launch(k_defect_rows<T, G, false>, dim3(blocks), dim3(256), 0, s, F, (unsigned long long *)nullptr,
-                   (float *)nullptr, (float *)nullptr);
+        launch_defect_rows<T, 3, 4, false>(F, nullptr, nullptr, nullptr, s);
         if (F.ng > 0) {
             g_launches++;
             pdl_launch(k_defect_ghost<T, 27>, dim3(blocks_for(F.ng)), dim3(kThreads), 0, s, F,
@@ -1744,16 +1755,19 @@ template <typename T>
 void launch_prolong(const LevelView<T> &F, const LevelView<T> &C, int dim, const T *e, T *out, bool add,
                     cudaStream_t s) {
     g_launches++;
-    if (dim == 3 && add && F.nsegs > 0) {   // inside nodes over the row segments, then the ghosts
-        constexpr int G = 1;
-        static unsigned resident = 0;
-        pdl_launch(k_prolong_rows<T, G>, dim3(segment_blocks(k_prolong_rows<T, G>, F.nsegs, G, resident)), dim3(256),
-                   0, s, F, C, e, out);
+    if (add) {   // inside nodes over the row segments, then the ghosts
+        static unsigned resident2 = 0, resident3 = 0;
+        const int groups = F.nsegs + (F.ng + 31) / 32;
+        if (dim == 2)
+            pdl_launch(k_prolong_rows<T, 2, 1>, dim3(segment_blocks(k_prolong_rows<T, 2, 1>, groups, 1, resident2)),
+                       dim3(256), 0, s, F, C, e, out);
+        else
+            pdl_launch(k_prolong_rows<T, 3, 1>, dim3(segment_blocks(k_prolong_rows<T, 3, 1>, groups, 1, resident3)),
+                       dim3(256), 0, s, F, C, e, out);
         return;
     }
-    const int64_t nt = level_threads(F, add);
-    if (dim == 2) pdl_launch(k_prolong<T, 2>, dim3(blocks_for(nt)), dim3(kThreads), 0, s, F, C, e, out, add);
-    else pdl_launch(k_prolong<T, 3>, dim3(blocks_for(nt)), dim3(kThreads), 0, s, F, C, e, out, add);
+    if (dim == 2) pdl_launch(k_prolong<T, 2>, dim3(blocks_for(F.nn)), dim3(kThreads), 0, s, F, C, e, out);
+    else pdl_launch(k_prolong<T, 3>, dim3(blocks_for(F.nn)), dim3(kThreads), 0, s, F, C, e, out);
 }
 
 template <typename T>
@@ -1824,18 +1838,6 @@ __global__ void __launch_bounds__(256)
     }
     pdl_wait();
     dev::js_apply_span<T, R>(u, node, comp, off, aoff, roff, inv, r, k0, min(k0 + R, n), threadIdx.x & 31);
-}
-
-// SMs of the current device (queried once)
-int num_sms() {
-    static int count = 0;
-    if (count <= 0) {
-        int d = 0, m = 0;
-        if (cudaGetDevice(&d) == cudaSuccess && cudaDeviceGetAttribute(&m, cudaDevAttrMultiProcessorCount, d) ==
-                                                     cudaSuccess)
-            count = m;
-    }
-    return count > 0 ? count : 1;
 }
 
 template <typename T>
@@ -1911,23 +1913,13 @@ void launch_mask_unknowns(const uint8_t *type, T *u, int64_t nn, cudaStream_t s)
 void launch_defect_mixed(const LevelView<double> &v, int dim, unsigned long long *norm, float *f32, float *g32,
                          float *e32, cudaStream_t s) {
     g_launches += v.ng > 0 ? 2 : 1;
-    const unsigned nb = std::min(blocks_for(level_threads(v, true)), kNormBlocks);
-    // 3D with row segments: the inside nodes over the segments, e32 = 0 at
-    // the ghosts by the ghost launch; the other nodes of f32 and e32 are 0
-    // from the start and nothing writes them
-    const bool rows = dim == 3 && v.nsegs > 0;
-    if (rows) {
-        constexpr int G = 2;
-        static unsigned resident = 0;
-        pdl_launch(k_defect_rows<double, G, true>,
-                   dim3(segment_blocks(k_defect_rows<double, G, true>, v.nsegs, G, resident)), dim3(256), 0, s, v,
-                   norm, f32, e32);
-    } else if (dim == 2) pdl_launch(k_defect_interior_mixed<2>, dim3(nb), dim3(kThreads), 0, s, v, norm, f32, e32);
-    else pdl_launch(k_defect_interior_mixed<3>, dim3(nb), dim3(kThreads), 0, s, v, norm, f32, e32);
-    float *ge = rows ? e32 : nullptr;
+    // the inside nodes over the segments, e32 = 0 at the ghosts by the ghost
+    // launch; the other nodes of f32 and e32 are 0 from the start
+    if (dim == 2) launch_defect_rows<double, 2, 2, true>(v, norm, f32, e32, s);
+    else launch_defect_rows<double, 3, 2, true>(v, norm, f32, e32, s);
     if (v.ng > 0) {
-        if (dim == 2) pdl_launch(k_defect_ghost_mixed<9>, dim3(blocks_for(v.ng)), dim3(kThreads), 0, s, v, norm, g32, ge);
-        else pdl_launch(k_defect_ghost_mixed<27>, dim3(blocks_for(v.ng)), dim3(kThreads), 0, s, v, norm, g32, ge);
+        if (dim == 2) pdl_launch(k_defect_ghost_mixed<9>, dim3(blocks_for(v.ng)), dim3(kThreads), 0, s, v, norm, g32, e32);
+        else pdl_launch(k_defect_ghost_mixed<27>, dim3(blocks_for(v.ng)), dim3(kThreads), 0, s, v, norm, g32, e32);
     }
 }
 
@@ -1936,22 +1928,14 @@ void launch_add_correction(const DevGeom &g, double *u64, const float *e32, cuda
     LevelView<double> v{};
     v.n = g.n;
     v.nn = g.nn;
-    v.type = g.type;
-    v.chunks = g.chunks;
-    v.clen = g.chunk_len;
-    v.nchunks = g.nchunks;
-    if (g.dim == 3 && g.nspl > 0) {   // inside nodes over the row segments, then the ghosts
-        constexpr int G = 4;
-        static unsigned resident = 0;
-        v.segs = reinterpret_cast<const int2 *>(g.sp_list);
-        v.nsegs = g.nspl;
-        v.ng = g.ng;
-        v.gnode = g.gnode;
-        pdl_launch(k_add_rows<G>, dim3(segment_blocks(k_add_rows<G>, v.nsegs, G, resident)), dim3(256), 0, s, v, u64,
-                   e32);
-        return;
-    }
-    pdl_launch(k_add_correction, dim3(blocks_for(level_threads(v, true))), dim3(kThreads), 0, s, v, u64, e32);
+    // inside nodes over the row segments, then the ghosts
+    constexpr int G = 4;
+    static unsigned resident = 0;
+    v.segs = reinterpret_cast<const int2 *>(g.sp_list);
+    v.nsegs = g.nspl;
+    v.ng = g.ng;
+    v.gnode = g.gnode;
+    pdl_launch(k_add_rows<G>, dim3(segment_blocks(k_add_rows<G>, v.nsegs, G, resident)), dim3(256), 0, s, v, u64, e32);
 }
 
 #define GCMG_INSTANTIATE(T)                                                                              \

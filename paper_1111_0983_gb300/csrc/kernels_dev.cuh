@@ -923,17 +923,14 @@ __device__ __forceinline__ T transfer_term(const LevelView<T> &F, int col) {
     return FROM_R ? F.r[F.gnode[col]] : ghost_defect<T, D == 2 ? 9 : 27>(F, col);
 }
 
-// descend_node in a launch that starts before its predecessor ends: the
-// node types are read first, then pdl_wait, then the defects
+// descend_node at coarse inside node i (fine image p) in a launch that starts
+// before its predecessor ends: the node types are read first, then pdl_wait
+// (again harmless when the warp has waited before), then the defects
 template <typename T, int D, bool FROM_R>
-__device__ __forceinline__ void descend_node_early(const LevelView<T> &F, const LevelView<T> &C,
-                                                   T *__restrict__ fc, T *__restrict__ uc, int64_t i) {
-    T v = 0;
-    if ((C.type[i] & NODE_KIND) == NODE_IN)
-        v = partial_transfer_of<T, D>(F, fine_image<D>(i, C.s0, C.s1, F.s0, F.s1), true,
-                                      [&](int64_t q) { return FROM_R ? F.r[q] : inside_defect<T, D>(F, q); }, true);
-    else
-        pdl_wait();
+__device__ __forceinline__ void descend_inside_early(const LevelView<T> &F, T *__restrict__ fc, T *__restrict__ uc,
+                                                     int64_t i, int64_t p) {
+    const T v = partial_transfer_of<T, D>(F, p, true,
+                                          [&](int64_t q) { return FROM_R ? F.r[q] : inside_defect<T, D>(F, q); }, true);
     uc[i] = 0;
     fc[i] = v;
 }
@@ -1087,62 +1084,6 @@ __device__ __forceinline__ void prolong_node(const LevelView<T> &F, const LevelV
                 num += w * e[X];
                 den += w;
             }
-    const T val = den > (T)0 ? num / den : (T)0;
-    if (add) out[p] += val;
-    else out[p] = val;
-}
-
-// prolong_node in a launch that starts before its predecessor ends: the
-// node's and its parents' types are read first, then pdl_wait, then e and
-// out.  The same sums as prolong_node.
-template <typename T, int D>
-__device__ __forceinline__ void prolong_node_early(const LevelView<T> &F, const LevelView<T> &C,
-                                                   const T *__restrict__ e, T *__restrict__ out, bool add, int64_t p) {
-    const uint8_t k = F.type[p] & NODE_KIND;
-    const bool on = k == NODE_IN || k == NODE_GHOST;
-    int j[3] = {0, 0, 0};
-    int64_t rem = p;
-    j[0] = (int)idx_div(rem, F.s0);
-    rem -= (int64_t)j[0] * F.s0;
-    if (D == 2) {
-        j[1] = (int)rem;
-    } else {
-        j[1] = (int)idx_div(rem, F.s1);
-        j[2] = (int)(rem - (int64_t)j[1] * F.s1);
-    }
-    const int n1 = (j[0] & 1) ? 2 : 1, n2 = (j[1] & 1) ? 2 : 1, n3 = (D == 3 && (j[2] & 1)) ? 2 : 1;
-    // up to 2^D parents in fixed slots (a, b, c), every load of a phase issued
-    // before the first use
-    constexpr int NS = D == 3 ? 8 : 4;
-    int64_t X[NS];
-    bool use[NS];
-#pragma unroll
-    for (int s = 0; s < NS; s++) {
-        const int a = D == 3 ? s >> 2 : s >> 1, b = D == 3 ? (s >> 1) & 1 : s & 1, c = D == 3 ? s & 1 : 0;
-        X[s] = (int64_t)(j[0] / 2 + a) * C.s0 +
-               (D == 2 ? (int64_t)(j[1] / 2 + b) : (int64_t)(j[1] / 2 + b) * C.s1 + (j[2] / 2 + c));
-        use[s] = false;
-        if (on && a < n1 && b < n2 && c < n3) {
-            const uint8_t kc = C.type[X[s]] & NODE_KIND;
-            use[s] = kc == NODE_IN || kc == NODE_GHOST;   // parents in Omega_2h u Gamma_2h
-        }
-    }
-    pdl_wait();
-    if (!on) {
-        if (!add) out[p] = 0;
-        return;
-    }
-    T ev[NS];
-#pragma unroll
-    for (int s = 0; s < NS; s++) ev[s] = use[s] ? e[X[s]] : (T)0;
-    T num = 0, den = 0;
-    const T w = (T)1 / (T)(n1 * n2 * n3);   // a power of two: exact
-#pragma unroll
-    for (int s = 0; s < NS; s++)   // (a, b, c) order, as prolong_node
-        if (use[s]) {
-            num += w * ev[s];
-            den += w;
-        }
     const T val = den > (T)0 ? num / den : (T)0;
     if (add) out[p] += val;
     else out[p] = val;

@@ -1094,13 +1094,12 @@ static void span_items_for(const HostLevel &L, int C, int seg, std::vector<int32
     }
 }
 
-// Work of the one-colour row sweep: every run of consecutive inside nodes of
-// a row (i, j), cut into segments of at most 64 nodes, in increasing node
-// order.
+// Every run of consecutive inside nodes of a row (a line along the contiguous
+// axis), cut into segments of at most 64 nodes, in increasing node order.
 static void build_row_segments(HostLevel &L) {
     const int n = L.n;
     L.sp_list.clear();
-    for (int64_t r = 0; r < (int64_t)n * n; r++) {
+    for (int64_t r = 0; r < L.nn / n; r++) {
         const uint8_t *t = &L.type[(size_t)r * n];
         int k = 0;
         while (k < n) {
@@ -1319,6 +1318,7 @@ void build_hierarchy(int dim, int n, int n_coarse, const double *phi, double del
             for (int a = 0; a < tr; a++)
                 for (int b = 0; b < tc; b++)
                     if (active[(size_t)a * tc + b]) L.tiles.push_back((a << 16) | b);
+            build_row_segments(L);   // n < 2^15.5: node indices have 31 bits
         } else if (L.nn < ((int64_t)1 << 31)) {
             build_zmarch_items(L);
             build_span_items(L);
