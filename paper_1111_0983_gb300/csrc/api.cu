@@ -3,6 +3,7 @@
 // kernels.cu; geometry construction in setup.cpp.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstring>
 #include <exception>
@@ -370,6 +371,11 @@ T *relax(gcmg_ctx *c, LevelView<T> v, T *out, T *wb, int l, bool extra) {
                                  : 0.0;
         timer_mark(c, GCMG_KERNEL_SMOOTH, l, bytes);
         timer_mark(c, GCMG_KERNEL_BOUNDARY, l, bytes);
+        // FP32: the junction solve as one launch, from a copy of the values it
+        // reads (wb is free here).  FP64 keeps two: the defects that every CTA
+        // computes again cost GB300's FP64 pipe more than the launch (1025^2:
+        // 426 us a cycle with two, 460 with one)
+        T *z = sizeof(T) == 4 && c->p.junction_solve && g.js_n > 0 ? wb : nullptr;
         bool split = false;
         if constexpr (std::is_same<T, float>::value) {
             if (c->split2d_strips > 0 && g.nstrips >= c->split2d_strips) {
@@ -378,18 +384,22 @@ T *relax(gcmg_ctx *c, LevelView<T> v, T *out, T *wb, int l, bool extra) {
                     ck(cudaEventCreateWithFlags(&c->ev_fork, cudaEventDisableTiming), "cudaEventCreate");
                     ck(cudaEventCreateWithFlags(&c->ev_join, cudaEventDisableTiming), "cudaEventCreate");
                 }
-                launch_relax2d_split(v, out, g, b2view<T>(g.b2, v), c->p.lambda, c->stream, c->sstream, c->ev_fork,
+                launch_relax2d_split(v, out, g, b2view<T>(g.b2, v), c->p.lambda, z, c->stream, c->sstream, c->ev_fork,
                                      c->ev_join);
                 split = true;
             }
         }
-        if (!split) launch_relax2d<T>(v, out, g, b2view<T>(g.b2, v), c->p.lambda, c->stream);
+        if (!split) launch_relax2d<T>(v, out, g, b2view<T>(g.b2, v), c->p.lambda, z, c->stream);
         timer_mark(c, GCMG_KERNEL_BOUNDARY, l);
         timer_mark(c, GCMG_KERNEL_SMOOTH, l);
         v.u = out;
         if (c->p.junction_solve) {
             const DevData<T> &D = data<T>(c)[l];
-            launch_junction_solve<T>(v, g, D.js_inv, D.js_r, c->stream, nullptr);
+            if constexpr (std::is_same<T, float>::value) {
+                if (z) launch_js(v, g, D.js_inv, z, c->stream);
+            } else {
+                launch_junction_solve<T>(v, g, D.js_inv, D.js_r, c->stream, nullptr);
+            }
         } else if (c->p.junction_sweeps > 0 && g.jz.ncomp > 0) {
             if (g.jz.in_smem) {
                 launch_local<T>(lview<T>(g.jz, v), dim, 0, c->p.junction_sweeps, c->stream);
@@ -992,6 +1002,13 @@ void upload_js(gcmg_ctx *c, int l) {
     }
     free_tracked(c, g.js_aoff);
     g.js_aoff = nullptr;
+    launch_mark_types(g.type, g.js_read, g.js_nread, NODE_JS, false, c->stream);
+    if (g.js_nread > 0) ck(cudaStreamSynchronize(c->stream), "sync");   // the list goes
+    free_tracked(c, g.js_read);
+    free_tracked(c, g.js_chunk);
+    g.js_read = nullptr;
+    g.js_chunk = nullptr;
+    g.js_nread = g.js_nchunk = g.js_mmax = 0;
     auto drop = [&](auto &D) {
         free_tracked(c, D.js_inv);
         free_tracked(c, D.js_r);
@@ -1028,14 +1045,28 @@ void upload_js(gcmg_ctx *c, int l) {
     g.js_rlen = nr;
     g.js_aoff_h = aoff;
     g.js_roff_h = roff;
+    // on the device a component's inside nodes come first, then its ghosts (the
+    // host's node order keeps the band of its elimination narrow)
+    std::vector<int32_t> ord(g.js_n), node(g.js_n), ghost(g.js_n), inside(g.js_ncomp, 0);
     std::vector<double> inv((size_t)na, 0.0);
     for (int k = 0; k < g.js_ncomp; k++) {
-        const int m = L.js_off[k + 1] - L.js_off[k], mp = (m + 3) & ~3;
-        for (int i = 0; i < m; i++)
-            std::copy_n(L.js_inv.begin() + L.js_aoff[k] + (int64_t)i * m, m, inv.begin() + aoff[k] + (int64_t)i * mp);
+        const int o = L.js_off[k], m = L.js_off[k + 1] - o, mp = (m + 3) & ~3;
+        int at = o;
+        for (int kind = 0; kind < 2; kind++)
+            for (int i = o; i < o + m; i++)
+                if ((L.js_ghost[i] >= 0) == (kind == 1)) {
+                    ord[at++] = i;
+                    if (kind == 0) inside[k]++;
+                }
+        for (int i = 0; i < m; i++) {
+            node[o + i] = L.js_node[ord[o + i]];
+            ghost[o + i] = L.js_ghost[ord[o + i]];
+            const double *row = &L.js_inv[L.js_aoff[k] + (int64_t)(ord[o + i] - o) * m];
+            for (int j = 0; j < m; j++) inv[aoff[k] + (int64_t)i * mp + j] = row[ord[o + j] - o];
+        }
     }
-    g.js_node = upload<int32_t>(c, L.js_node.data(), L.js_node.size());
-    g.js_ghost = upload<int32_t>(c, L.js_ghost.data(), L.js_ghost.size());
+    g.js_node = upload<int32_t>(c, node.data(), node.size());
+    g.js_ghost = upload<int32_t>(c, ghost.data(), ghost.size());
     g.js_comp = upload<int32_t>(c, comp.data(), comp.size());
     g.js_off = upload<int32_t>(c, L.js_off.data(), L.js_off.size());
     g.js_roff = upload<int32_t>(c, roff.data(), roff.size());
@@ -1052,6 +1083,35 @@ void upload_js(gcmg_ctx *c, int l) {
         const std::vector<float> inv32(inv.begin(), inv.end()), zero(nr, 0.f);
         c->D32[l].js_inv = upload<float>(c, inv32.data(), inv32.size());
         c->D32[l].js_r = upload<float>(c, zero.data(), zero.size());
+    }
+    if (L.dim == 2) {
+        // k_js: rows of a component a CTA, a warp each, as many as spread the
+        // level's rows over one CTA an SM (8 to 12 warps)
+        int sms = 1;
+        ck(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device), "attr");
+        g.js_warps = std::min(12, std::max(8, (g.js_n + sms - 1) / sms));
+        std::vector<JsChunk> chunk;
+        for (int k = 0; k < g.js_ncomp; k++) {
+            const int o = L.js_off[k], m = L.js_off[k + 1] - o, mp = (m + 3) & ~3;
+            g.js_mmax = std::max(g.js_mmax, m);
+            for (int r = 0; r < m; r += g.js_warps)
+                chunk.push_back({aoff[k] + (int64_t)r * mp, o, m, inside[k], o + r, std::min(g.js_warps, m - r), 0});
+        }
+        g.js_nchunk = (int)chunk.size();
+        g.js_chunk = upload<JsChunk>(c, chunk.data(), chunk.size());
+        // the nodes the solved equations read
+        std::vector<int32_t> rd;
+        for (int k = 0; k < g.js_n; k++) {
+            const int32_t p = L.js_node[k], q = L.js_ghost[k];
+            if (q >= 0) rd.insert(rd.end(), &L.stn[(int64_t)q * KMAX], &L.stn[(int64_t)q * KMAX] + 9);
+            else rd.insert(rd.end(), {p, p - 1, p + 1, p - L.n, p + L.n});
+        }
+        std::sort(rd.begin(), rd.end());
+        rd.erase(std::unique(rd.begin(), rd.end()), rd.end());
+        g.js_nread = (int)rd.size();
+        g.js_read = upload<int32_t>(c, rd.data(), rd.size());
+        launch_mark_types(g.type, g.js_read, g.js_nread, NODE_JS, true, c->stream);
+        ck(cudaStreamSynchronize(c->stream), "sync");   // the host lists die at scope end
     }
     ck(cudaStreamSynchronize(c->stream), "sync");   // the staging vectors die at return
 }

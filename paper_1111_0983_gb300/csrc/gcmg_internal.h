@@ -38,8 +38,9 @@ constexpr int ZM_MROW = (ZM_TX + 2 + 31) / 32;
 constexpr int ZM_MPLANE = ((ZM_TY + 2) * ZM_MROW + 3) / 4 * 4;
 
 // NODE_WB marks, in the device copy of the type grid only, the nodes that the
-// 2D boundary blocks write back through the write-back grid
-enum : uint8_t { NODE_OUT = 0, NODE_IN = 1, NODE_GHOST = 2, NODE_KIND = 3, NODE_BAND = 4, NODE_WB = 8 };
+// 2D boundary blocks write back through the write-back grid; NODE_JS, there
+// too, the nodes that the equations of the exact junction solve read
+enum : uint8_t { NODE_OUT = 0, NODE_IN = 1, NODE_GHOST = 2, NODE_KIND = 3, NODE_BAND = 4, NODE_WB = 8, NODE_JS = 16 };
 enum : uint8_t { STENCIL_QUAD = 0, STENCIL_LIN = 1, STENCIL_CORNER = 2, STENCIL_AXIS = 3 };
 
 struct GeomError {
@@ -248,6 +249,14 @@ struct Block2Host {
     std::vector<uint32_t> e_red, e_black, p_red, p_black, g0, g1;   // 4 words a record
 };
 Block2Host build_blocks2(const HostLevel &L);
+// Work of one CTA of the junction solve's single launch (k_js): `rows` rows
+// from k0 of the component at o with m rows, its first mi at inside nodes; a:
+// the chunk's first entry in the inverses
+struct JsChunk {
+    int64_t a;
+    int32_t o, m, mi, k0, rows, pad;
+};
+
 // Integer geometry of a level on the device (shared by both precisions).
 struct DevGeom {
     int dim = 2, n = 0;
@@ -300,6 +309,12 @@ struct DevGeom {
     std::vector<int64_t> js_aoff_h;     // host copies of the padded offsets (ncomp + 1)
     std::vector<int32_t> js_roff_h;
     int64_t *js_aoff = nullptr;
+    // 2D: the CTAs of k_js (js_warps rows at most each), the longest component,
+    // and the nodes marked NODE_JS
+    JsChunk *js_chunk = nullptr;
+    int js_nchunk = 0, js_warps = 0, js_mmax = 0;
+    int32_t *js_read = nullptr;
+    int js_nread = 0;
 };
 
 // Floating-point data of a level in precision T.

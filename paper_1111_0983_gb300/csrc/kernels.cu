@@ -1342,68 +1342,68 @@ void launch_rb(const LevelView<T> &v, int dim, int color, cudaStream_t s) {
 template <typename T, int SR, int NT, int M>
 __global__ void __launch_bounds__(NT, M == 1 ? 2 : 1)
     k_relax2d(LevelView<T> v, T *__restrict__ out, const int32_t *__restrict__ strips, int ns, int nsc,
-              Block2View<T> J, int lambda) {
+              Block2View<T> J, int lambda, T *__restrict__ z) {
     if (sizeof(T) == 4) pdl_trigger();
     if ((int)blockIdx.x < nsc) {
         const int s = blockIdx.x * (NT / 32) + (threadIdx.x >> 5);
         const int32_t st = s < ns ? strips[s] : 0;   // static: read before the wait
         pdl_wait();
-        if (s < ns) rb_strip<T, SR, true>(v, out, st);   // uniform over the warp
+        if (s < ns) rb_strip<T, SR, true>(v, out, st, z);   // uniform over the warp
         return;
     }
-    block2<T, NT, M>(J, v.u, out, (int)blockIdx.x - nsc, lambda, true);
+    block2<T, NT, M>(J, v.u, out, z, (int)blockIdx.x - nsc, lambda, true);
 }
 
 // the blocks, after the CTAs of the first ns strips (0: the blocks alone)
 template <typename T, int SR, int NT, int M>
 void launch_relax2d_as(cudaStream_t s, const LevelView<T> &v, T *out, const DevGeom &g, int ns, const Block2View<T> &J,
-                       int lambda) {
+                       int lambda, T *z) {
     const int nsc = (ns + NT / 32 - 1) / (NT / 32);
     pdl_launch(k_relax2d<T, SR, NT, M>, dim3((unsigned)(nsc + J.p.ncomp)), dim3(NT), block2_smem<T>(J.p), s, v, out,
-               g.strips, ns, nsc, J, lambda);
+               g.strips, ns, nsc, J, lambda, z);
 }
 
 template <typename T>
 void launch_relax2d_strips(cudaStream_t s, const LevelView<T> &v, T *out, const DevGeom &g, int ns,
-                           const Block2View<T> &J, int lambda) {
-    if (J.p.nt == 512) launch_relax2d_as<T, 8, 512, 2>(s, v, out, g, ns, J, lambda);
-    else if (J.p.m == 2) launch_relax2d_as<T, 8, 256, 2>(s, v, out, g, ns, J, lambda);
-    else launch_relax2d_as<T, 8, 256, 1>(s, v, out, g, ns, J, lambda);
+                           const Block2View<T> &J, int lambda, T *z) {
+    if (J.p.nt == 512) launch_relax2d_as<T, 8, 512, 2>(s, v, out, g, ns, J, lambda, z);
+    else if (J.p.m == 2) launch_relax2d_as<T, 8, 256, 2>(s, v, out, g, ns, J, lambda, z);
+    else launch_relax2d_as<T, 8, 256, 1>(s, v, out, g, ns, J, lambda, z);
 }
 
 template <typename T>
-void launch_relax2d(const LevelView<T> &v, T *out, const DevGeom &g, const Block2View<T> &J, int lambda,
+void launch_relax2d(const LevelView<T> &v, T *out, const DevGeom &g, const Block2View<T> &J, int lambda, T *z,
                     cudaStream_t s) {
     g_launches++;
-    launch_relax2d_strips<T>(s, v, out, g, g.nstrips, J, lambda);
+    launch_relax2d_strips<T>(s, v, out, g, g.nstrips, J, lambda, z);
 }
 
 // both colours in one pass over the active 2D strips: 4 warps a CTA, one strip a warp
 // (INTERIOR_ONLY: the boundary blocks, launched beside, store the band and ghosts)
 template <typename T, int SR, bool INTERIOR_ONLY = false>
 __global__ void __launch_bounds__(128) k_rb_strip(LevelView<T> v, T *__restrict__ out,
-                                                  const int32_t *__restrict__ strips, int ns) {
+                                                  const int32_t *__restrict__ strips, int ns, T *__restrict__ z) {
     pdl_wait();
     const int s = blockIdx.x * 4 + (threadIdx.x >> 5);
-    if (s < ns) rb_strip<T, SR, INTERIOR_ONLY>(v, out, strips[s]);   // uniform over the warp
+    if (s < ns) rb_strip<T, SR, INTERIOR_ONLY>(v, out, strips[s], z);   // uniform over the warp
 }
 
 template <int SR>
-static void launch_strips_interior(const LevelView<float> &v, float *out, const DevGeom &g, cudaStream_t s) {
+static void launch_strips_interior(const LevelView<float> &v, float *out, const DevGeom &g, float *z, cudaStream_t s) {
     pdl_launch(k_rb_strip<float, SR, true>, dim3((unsigned)((g.nstrips + 3) / 4)), dim3(128), 0, s, v, out, g.strips,
-               g.nstrips);
+               g.nstrips, z);
 }
 
 void launch_relax2d_split(const LevelView<float> &v, float *out, const DevGeom &g, const Block2View<float> &J,
-                          int lambda, cudaStream_t s, cudaStream_t side, cudaEvent_t fork, cudaEvent_t join) {
+                          int lambda, float *z, cudaStream_t s, cudaStream_t side, cudaEvent_t fork, cudaEvent_t join) {
     // the boundary blocks (k_relax2d without strips) on the side stream, the
     // strips (interior nodes off the band) on the main one: both read v.u and
     // store disjoint nodes of out, as the merged launch does
     g_launches += 2;
     cudaEventRecord(fork, s);
     cudaStreamWaitEvent(side, fork, 0);
-    launch_relax2d_strips<float>(side, v, out, g, 0, J, lambda);
-    launch_strips_interior<8>(v, out, g, s);
+    launch_relax2d_strips<float>(side, v, out, g, 0, J, lambda, z);
+    launch_strips_interior<8>(v, out, g, z, s);
     cudaEventRecord(join, side);
     cudaStreamWaitEvent(s, join, 0);
 }
@@ -1413,9 +1413,9 @@ void launch_rb_strip(const LevelView<T> &v, T *out, const DevGeom &g, cudaStream
     if (g.nstrips <= 0) return;
     g_launches++;
     const dim3 grid((unsigned)((g.nstrips + 3) / 4));
-    if (g.strip_rows == 32) pdl_launch(k_rb_strip<T, 32>, grid, dim3(128), 0, s, v, out, g.strips, g.nstrips);
-    else if (g.strip_rows == 16) pdl_launch(k_rb_strip<T, 16>, grid, dim3(128), 0, s, v, out, g.strips, g.nstrips);
-    else pdl_launch(k_rb_strip<T, 8>, grid, dim3(128), 0, s, v, out, g.strips, g.nstrips);
+    if (g.strip_rows == 32) pdl_launch(k_rb_strip<T, 32>, grid, dim3(128), 0, s, v, out, g.strips, g.nstrips, (T *)nullptr);
+    else if (g.strip_rows == 16) pdl_launch(k_rb_strip<T, 16>, grid, dim3(128), 0, s, v, out, g.strips, g.nstrips, (T *)nullptr);
+    else pdl_launch(k_rb_strip<T, 8>, grid, dim3(128), 0, s, v, out, g.strips, g.nstrips, (T *)nullptr);
 }
 
 template <typename T>
@@ -1820,6 +1820,48 @@ __global__ void __launch_bounds__(kThreads) k_js_defect(LevelView<T> v, const in
     }
 }
 
+// The exact junction solve in one launch: a CTA computes every defect of its
+// component into shared memory (from z, the grid the relaxation has stored the
+// nodes they read into, since other CTAs are updating u) and applies its rows of
+// the inverse, a warp each.  650 defects a CTA again and again are cheap next to
+// a launch: the two of defects and rows took 3.7 us of a relaxation at 1025^2,
+// this one takes 2.7 (a mixed cycle 166 -> 152 us).  Rows and inverse entries are
+// fixed and loaded before the wait.
+template <typename T>
+__global__ void __launch_bounds__(384) k_js(LevelView<T> v, const T *__restrict__ z, const int32_t *__restrict__ node,
+                                            const int32_t *__restrict__ ghost, const JsChunk *__restrict__ chunk,
+                                            const T *__restrict__ inv) {
+    extern __shared__ __align__(16) unsigned char smem_js[];
+    using V = typename Vec16<T>::type;
+    constexpr int MAXV = 8;   // vectors of its row a lane loads before the wait
+    if (sizeof(T) == 4) pdl_trigger();
+    T *rs = reinterpret_cast<T *>(smem_js);
+    const JsChunk c = chunk[blockIdx.x];
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int nv = ((c.m + 3) & ~3) / Vec16<T>::n;
+    const bool on = w < c.rows;   // uniform over the warp
+    const V *a = reinterpret_cast<const V *>(inv + c.a) + (int64_t)w * nv;
+    V av[MAXV];
+    int nd = 0;
+    if (on) {
+#pragma unroll
+        for (int e = 0; e < MAXV; e++)
+            if (lane + 32 * e < nv) av[e] = a[lane + 32 * e];
+        nd = node[c.k0 + w];
+    }
+    dev::js_component_defects<T, 3>(v, z, node + c.o, ghost + c.o, c.m, c.mi, rs);
+    __syncthreads();
+    if (!on) return;
+    const V *rr = reinterpret_cast<const V *>(rs);
+    T s = 0;
+#pragma unroll
+    for (int e = 0; e < MAXV; e++)
+        if (lane + 32 * e < nv) s = Vec16<T>::dot(s, av[e], rr[lane + 32 * e]);
+    for (int j = lane + 32 * MAXV; j < nv; j += 32) s = Vec16<T>::dot(s, a[j], rr[j]);
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (lane == 0) v.u[nd] = z[nd] + s;
+}
+
 // R rows a warp, 8 warps a CTA: R = 4 amortises the per-CTA address chain
 // over 4 rows once the launch fills the GPU several times over; a small
 // launch (a single domain: about a thousand rows a level) keeps one row a
@@ -1838,6 +1880,27 @@ __global__ void __launch_bounds__(256)
     }
     pdl_wait();
     dev::js_apply_span<T, R>(u, node, comp, off, aoff, roff, inv, r, k0, min(k0 + R, n), threadIdx.x & 31);
+}
+
+void launch_js(const LevelView<float> &v, const DevGeom &g, const float *inv, const float *z, cudaStream_t s) {
+    if (g.js_nchunk <= 0) return;
+    g_launches++;
+    pdl_launch(k_js<float>, dim3((unsigned)g.js_nchunk), dim3(32 * g.js_warps),
+               sizeof(float) * (((size_t)g.js_mmax + 3) & ~3), s,
+               v, z, (const int32_t *)g.js_node, (const int32_t *)g.js_ghost, (const JsChunk *)g.js_chunk, inv);
+}
+
+__global__ void k_mark_types(uint8_t *__restrict__ type, const int32_t *__restrict__ list, int n, uint8_t bit, int set) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    const int p = list[i];   // each node once
+    type[p] = set ? type[p] | bit : type[p] & (uint8_t)~bit;
+}
+
+void launch_mark_types(uint8_t *type, const int32_t *list, int n, uint8_t bit, bool set, cudaStream_t s) {
+    if (n <= 0) return;
+    g_launches++;
+    k_mark_types<<<blocks_for(n), kThreads, 0, s>>>(type, list, n, bit, (int)set);
 }
 
 template <typename T>
@@ -1967,7 +2030,7 @@ void launch_add_correction(const DevGeom &g, double *u64, const float *e32, cuda
     template void launch_rb_stream3d<T>(const LevelView<T> &, T *, const DevGeom &, cudaStream_t);  \
     template bool launch_rb_rows<T>(const LevelView<T> &, const DevGeom &, cudaStream_t);           \
     template void launch_relax2d<T>(const LevelView<T> &, T *, const DevGeom &, const Block2View<T> &, int,  \
-                                    cudaStream_t);                                                       \
+                                    T *, cudaStream_t);                                                       \
     template bool launch_boundary3d<T>(const LevelView<T> &, BoundaryProgram3, int, cudaStream_t);  \
     template bool launch_boundary3d_cluster<T>(const LevelView<T> &, const BoundaryProgram3 &, cudaStream_t); \
     template size_t local_smem_bytes<T>(const LocalView<T> &, int);                                       \

@@ -19,14 +19,15 @@ void launch_kaczmarz(const LevelView<double> &v, const int32_t *rows, const std:
 template <typename T>
 void launch_rb(const LevelView<T> &v, int dim, int color, cudaStream_t s);
 // one 2D relaxation (interior sweep, ghost sweep, band sweeps) in one launch:
-// strips (of 8 rows) and boundary blocks both read v.u and write out
+// strips (of 8 rows) and boundary blocks both read v.u and write out; z: null,
+// or a grid that also gets the nodes marked NODE_JS (for launch_js)
 template <typename T>
-void launch_relax2d(const LevelView<T> &v, T *out, const DevGeom &g, const Block2View<T> &J, int lambda,
+void launch_relax2d(const LevelView<T> &v, T *out, const DevGeom &g, const Block2View<T> &J, int lambda, T *z,
                     cudaStream_t s);
 // the same as two launches side by side: the boundary blocks on `side`, the
 // strips' interior nodes on `s` (fork and join through the two events)
 void launch_relax2d_split(const LevelView<float> &v, float *out, const DevGeom &g, const Block2View<float> &J,
-                          int lambda, cudaStream_t s, cudaStream_t side, cudaEvent_t fork, cudaEvent_t join);
+                          int lambda, float *z, cudaStream_t s, cudaStream_t side, cudaEvent_t fork, cudaEvent_t join);
 // dynamic shared memory of the boundary blocks
 template <typename T>
 size_t block2_smem(const Block2Dev &p) { return sizeof(T) * ((size_t)p.nodes + 2 * (size_t)p.gh); }
@@ -80,6 +81,11 @@ void launch_coarse_solve(const LevelView<T> &v, const DevGeom &g, const T *Ainv,
 template <typename T>
 void launch_junction_solve(const LevelView<T> &v, const DevGeom &g, const T *inv, T *r, cudaStream_t s,
                            const LocalView<T> *pending = nullptr);
+// 2D exact junction solve in one launch (FP32): u += A_ZZ^-1 r per component,
+// the defects r from z, which holds u at the nodes they read
+void launch_js(const LevelView<float> &v, const DevGeom &g, const float *inv, const float *z, cudaStream_t s);
+// sets or clears a bit of the type grid at n distinct nodes
+void launch_mark_types(uint8_t *type, const int32_t *list, int n, uint8_t bit, bool set, cudaStream_t s);
 template <typename T>
 void launch_mask_unknowns(const uint8_t *type, T *u, int64_t nn, cudaStream_t s);
 // Boundary types of the ng ghosts of a level (step `step` = 2^l of the fine

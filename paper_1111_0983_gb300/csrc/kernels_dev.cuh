@@ -250,9 +250,11 @@ __device__ __forceinline__ double quarter(double s) {
 }
 
 // INTERIOR_ONLY: store only the inside nodes outside the boundary band (the
-// boundary blocks of the same launch store the band nodes and the ghosts)
+// boundary blocks of the same launch store the band nodes and the ghosts); z:
+// when not null, the nodes marked NODE_JS into that grid too
 template <typename T, int SR, bool INTERIOR_ONLY = false>
-__device__ __forceinline__ void rb_strip(const LevelView<T> &v, T *__restrict__ out, int strip) {
+__device__ __forceinline__ void rb_strip(const LevelView<T> &v, T *__restrict__ out, int strip,
+                                         T *__restrict__ z = nullptr) {
     constexpr int PD = STRIP_PD;
     constexpr unsigned FULL = 0xffffffffu;
     const int lane = threadIdx.x & 31;
@@ -319,8 +321,14 @@ __device__ __forceinline__ void rb_strip(const LevelView<T> &v, T *__restrict__ 
                 auto stored = [](uint8_t k) {
                     return INTERIOR_ONLY ? (k & (NODE_KIND | NODE_BAND)) == NODE_IN : (k & NODE_KIND) != NODE_OUT;
                 };
-                if (stored(kp0) && c0 < n) out[b + c0] = o0;
-                if (stored(kp1) && c1 < n) out[b + c1] = o1;
+                if (stored(kp0) && c0 < n) {
+                    out[b + c0] = o0;
+                    if (INTERIOR_ONLY && z && (kp0 & NODE_JS)) z[b + c0] = o0;
+                }
+                if (stored(kp1) && c1 < n) {
+                    out[b + c1] = o1;
+                    if (INTERIOR_ONLY && z && (kp1 & NODE_JS)) z[b + c1] = o1;
+                }
             }
         }
         ra0 = rb0;
@@ -497,7 +505,7 @@ __device__ __forceinline__ void local_body(const LocalView<T> &J, const T *src, 
 // inside node the block reads (the sums of the strips), the ghost sweep, then
 // reps x (red band, black band, Jacobi ghosts) on the band nodes and ghosts
 // within the reach of those phases (the block's halo); the block's own band
-// nodes and ghosts are stored into dst.  A phase is one record a thread (M at
+// nodes and ghosts are stored into dst (and z, if given).  A phase is one record a thread (M at
 // most), held in registers with its weights and h^2 f, so that it costs its
 // shared-memory reads, its sum and one barrier: the records are loaded at once
 // by the threads that use them (one round trip, before the wait for the
@@ -509,8 +517,8 @@ __device__ __forceinline__ void local_body(const LocalView<T> &J, const T *src, 
 // this form (430): a relaxation with its junction solve 8.6 -> 7.2 us; FP64 30
 // -> 20 us, where the interior sweep and the blocks had been two launches.
 template <typename T, int NT, int M>
-__device__ __forceinline__ void block2(const Block2View<T> &J, const T *__restrict__ src, T *__restrict__ dst, int c,
-                                       int reps, bool early) {
+__device__ __forceinline__ void block2(const Block2View<T> &J, const T *__restrict__ src, T *__restrict__ dst,
+                                       T *__restrict__ z, int c, int reps, bool early) {
     constexpr int RP = M + 1, RN = 4 * M, RW = 2 * M;
     extern __shared__ __align__(16) unsigned char smem_dyn[];
     T *val = reinterpret_cast<T *>(smem_dyn);   // nodes, then two values a ghost
@@ -637,7 +645,11 @@ __device__ __forceinline__ void block2(const Block2View<T> &J, const T *__restri
     }
 #pragma unroll
     for (int k = 0; k < RW; k++)
-        if (wb[k].x >= 0) dst[wb[k].x] = at((unsigned)wb[k].y);
+        if (wb[k].x >= 0) {
+            const T x = at((unsigned)wb[k].y);
+            dst[wb[k].x] = x;
+            if (z) z[wb[k].x] = x;
+        }
 }
 
 // write-back node i of the flat list: u = wb
@@ -1228,6 +1240,77 @@ __device__ __forceinline__ void js_apply_row_early(T *__restrict__ u, const int3
     for (int j = lane + 32 * MAXV; j < nv; j += 32) s = Vec16<T>::dot(s, a[j], rr[j]);
     for (int w = 16; w > 0; w >>= 1) s += __shfl_xor_sync(0xffffffffu, s, w);
     if (lane == 0) u[nd] = uo + s;
+}
+
+// The defects of the m equations of one component of a 2D junction solve (mi
+// inside nodes, then ghosts) into shared memory (rs, padded with zeros to a
+// multiple of 4), by a CTA: u is read from z, which nothing writes meanwhile.
+// The ghosts start at a warp of their own, so that no warp takes both branches;
+// up to KJ equations a thread have their fixed data (nodes, ghost stencils,
+// weights) loaded before the wait for the previous launch, then all their
+// values at once.  The sums of js_defect.
+template <typename T, int KJ>
+__device__ __forceinline__ void js_component_defects(const LevelView<T> &v, const T *__restrict__ z,
+                                                     const int32_t *__restrict__ node,
+                                                     const int32_t *__restrict__ ghost, int m, int mi, T *rs) {
+    const int tid = threadIdx.x, nt = blockDim.x;
+    const int shift = ((mi + 31) & ~31) - mi;   // thread index t: equation t (t < mi), then t - shift
+    int32_t q[KJ], x[KJ][9];
+    T w[KJ][9];
+#pragma unroll
+    for (int k = 0; k < KJ; k++) {
+        const int t = tid + k * nt;
+        q[k] = -1;
+        if (t < mi) x[k][0] = node[t];
+        else if (t >= mi + shift && t < m + shift) q[k] = ghost[t - shift];
+    }
+#pragma unroll
+    for (int k = 0; k < KJ; k++)
+        if (q[k] >= 0) {
+#pragma unroll
+            for (int i = 0; i < 9; i++) {
+                x[k][i] = v.gstn[(int64_t)i * v.ng + q[k]];
+                w[k][i] = v.gw[(int64_t)i * v.ng + q[k]];
+            }
+        }
+    const int s0 = (int)v.s0;
+    pdl_wait();
+    T y[KJ][9], b[KJ];
+#pragma unroll
+    for (int k = 0; k < KJ; k++) {
+        if (tid + k * nt < mi) {
+            const int p = x[k][0];
+            y[k][0] = z[p];
+            y[k][1] = z[p - 1];
+            y[k][2] = z[p + 1];
+            y[k][3] = z[p - s0];
+            y[k][4] = z[p + s0];
+            b[k] = v.f[p];
+        } else if (q[k] >= 0) {
+#pragma unroll
+            for (int i = 0; i < 9; i++) y[k][i] = z[x[k][i]];
+            b[k] = v.gg[q[k]];
+        }
+    }
+#pragma unroll
+    for (int k = 0; k < KJ; k++) {
+        if (tid + k * nt < mi) {
+            const T up = y[k][0];
+            const T lap = (y[k][1] - up) + (y[k][2] - up) + (y[k][3] - up) + (y[k][4] - up);
+            rs[tid + k * nt] = b[k] + lap * v.inv_h2;
+        } else if (q[k] >= 0) {
+            T s = 0;
+#pragma unroll
+            for (int i = 0; i < 9; i++) s += w[k][i] * y[k][i];
+            rs[tid + k * nt - shift] = b[k] - s;
+        }
+    }
+    LevelView<T> vz = v;
+    vz.u = const_cast<T *>(z);
+    for (int t = tid + KJ * nt; t < m + shift; t += nt)
+        if (t < mi) rs[t] = js_defect<T, 2>(vz, node[t], -1);
+        else if (t >= mi + shift) rs[t - shift] = js_defect<T, 2>(vz, node[t - shift], ghost[t - shift]);
+    if (tid < 4 && m + tid < ((m + 3) & ~3)) rs[m + tid] = 0;
 }
 
 // one row k (the form of the fused coarse cycle)
