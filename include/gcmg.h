@@ -444,7 +444,8 @@ gcmg_status gcmg_batch_set_graph(gcmg_batch *batch, int on);
  * one warp): 0 = 8 rows, 1 = 16 rows, 2 = 32 rows. */
 gcmg_status gcmg_batch_set_tiles(gcmg_batch *batch, int variant);
 
-/* Autotuner: times the batched interior sweeps of one cycle with every strip
+/* Autotuner: times the launches with the batched interior sweeps of one cycle
+ * (which also hold the boundary blocks where those fit) with every strip
  * height, selects the fastest (*best) and reports each time in ms[0..2]. */
 gcmg_status gcmg_batch_autotune(gcmg_batch *batch, int *best, double *ms);
 

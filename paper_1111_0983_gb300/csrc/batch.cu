@@ -36,16 +36,14 @@ struct BItem {
     int32_t start;   // tile / component / first node / first ghost / block
 };
 
-// the junction-solve product of up to kJsRows rows of one component of one
-// domain level, with every address resolved on the host
+// the junction solve of up to kJsRows rows of one component of one domain
+// level, with the component's and the rows' addresses resolved on the host
 struct JsItem {
-    const float *a;          // the first row of the chunk in the component's padded inverse
-    const float *r;          // the component's padded defect vector
-    const int32_t *node;     // the chunk's row nodes
-    float *u0, *u1;          // the level's two u grids
-    int rows, mp, dom, pad;  // rows of the chunk, padded row length, domain
+    const float *a;              // the first row of the chunk in the component's padded inverse
+    const int32_t *node, *ghost; // the component's nodes and ghost numbers, inside nodes first
+    int view, m, mi;             // the level's view; the component's rows, those at inside nodes
+    int k0, rows, pad;           // first row of the chunk within the component, rows
 };
-
 
 // one level of one domain, in FP32 (the cycle precision of the batch)
 struct BView32 {
@@ -56,6 +54,10 @@ struct BView32 {
     const int32_t *tiles;    // active sweep strips of the selected height
     int ntiles;
     LocalView<float> bz, jz; // boundary blocks, junction zone
+    Block2View<float> b2;    // boundary blocks as per-thread records
+    float *z;                // copy of u at the nodes the junction solve reads
+    const int32_t *js_read;  // those nodes
+    int js_nread;
     const int32_t *gt_ptr, *gt_col;
     const float *gt_val;
     const int32_t *unk_node, *unk_ghost;
@@ -63,12 +65,6 @@ struct BView32 {
     int nunk;
     int dom;
     const int *active;       // per-domain flag: still iterating
-    // exact junction solve of this level
-    const int32_t *js_node, *js_ghost, *js_comp, *js_off, *js_roff, *js_rpos;
-    const int64_t *js_aoff;
-    const float *js_inv;
-    float *js_r;
-    int js_n;
 };
 
 // level 0 of one domain in FP64 plus its FP32 correction arrays
@@ -98,10 +94,40 @@ const int kStripRows[kVariants] = {8, 16, 32};
 // (0: v.u, 1: u2); the sweep reads that grid and writes the other.
 __device__ __forceinline__ float *ugrid(const BView32 &w, int k) { return k ? w.u2 : w.v.u; }
 
-// both colours of the sweep: an item is 4 consecutive strips of one view, one a warp
+// A kernel's items, views and lists are fixed while a solve runs: read before
+// pdl_wait.  The per-domain flags (kb_check writes them) and the grids after it.
+
+// one relaxation up to the band sweeps: an item is NT / 32 consecutive strips of
+// one view (start >= 0), one a warp, or boundary block ~start; both read grid
+// src and store disjoint nodes of the other.  A block is a chain of latencies:
+// its launch is bound by how many run at once (three CTAs an SM instead of two,
+// two instead of one for M = 2: 48 stars 25.6 -> 23.3 ms a solve)
+template <int SR, int NT, int M>
+__global__ void __launch_bounds__(NT, NT == 512 ? 1 : M == 1 ? 3 : 2) kb_relax(const BView32 *__restrict__ V,
+                                                               const BItem *__restrict__ it, int src, int lambda) {
+    const BItem b = it[blockIdx.x];
+    const BView32 &w = V[b.view];
+    float *out = ugrid(w, src ^ 1);
+    const float *u = ugrid(w, src);
+    if (b.start < 0) {
+        block2<float, NT, M>(w.b2, u, out, w.z, ~b.start, lambda, w.active + w.dom);
+        return;
+    }
+    const int s = b.start + (threadIdx.x >> 5);
+    const int32_t st = s < w.ntiles ? w.tiles[s] : 0;
+    pdl_wait();
+    if (s >= w.ntiles || !w.active[w.dom]) return;   // uniform over the warp
+    LevelView<float> v = w.v;
+    v.u = const_cast<float *>(u);
+    rb_strip<float, SR, true>(v, out, st, w.z);
+}
+
+// both colours of the sweep alone (blocks too large for kb_relax): an item is 4
+// consecutive strips of one view, one a warp
 template <int SR>
 __global__ void __launch_bounds__(128, 8) kb_fused(const BView32 *__restrict__ V, const BItem *__restrict__ it, int src) {
     const BItem b = it[blockIdx.x];
+    pdl_wait();
     if (!V[b.view].active[V[b.view].dom]) return;
     const BView32 &w = V[b.view];
     const int s = b.start + (threadIdx.x >> 5);
@@ -114,6 +140,7 @@ __global__ void __launch_bounds__(128, 8) kb_fused(const BView32 *__restrict__ V
 __global__ void __launch_bounds__(256) kb_local_copyback(const BView32 *__restrict__ V, const BItem *__restrict__ it,
                                                          int cur, int npt) {
     const BItem b = it[blockIdx.x];
+    pdl_wait();
     if (!V[b.view].active[V[b.view].dom]) return;
     float *u = ugrid(V[b.view], cur);
     for_span(b, npt, [&](int64_t i) { local_copyback<float>(V[b.view].bz, u, (int)i); });
@@ -124,115 +151,144 @@ __global__ void __launch_bounds__(LOCAL_THREADS, 2) kb_local(const BView32 *__re
                                                              const BItem *__restrict__ it, int junction,
                                                              int lead_ghost, int reps, int cur) {
     const BItem b = it[blockIdx.x];
+    pdl_wait();
     if (!V[b.view].active[V[b.view].dom]) return;
     const LocalView<float> &J = junction ? V[b.view].jz : V[b.view].bz;
     float *u = ugrid(V[b.view], cur);
     local_body<float, 2, EPT>(J, u, J.wb ? J.wb : u, b.start, lead_ghost, reps);
 }
 
-// exact junction solve: defects of the solved equations (dense items), then
-// u += A_ZZ^-1 r (kJsWarpRows rows a warp, kJsRows rows an item)
-constexpr int kJsWarpRows = 4;
-constexpr int kJsRows = 8 * kJsWarpRows;
-
-// WB: the boundary blocks' write-back is performed here too (items cover
-// max(js_n, nwb) indexes); the defects read the write-back nodes from the
-// write-back grid
-template <bool WB>
-__global__ void kb_js_defect(const BView32 *__restrict__ V, const BItem *__restrict__ it, int cur, int npt) {
+// z = u at the nodes the junction solve reads (after a relaxation by kb_fused and kb_local)
+__global__ void kb_js_copy(const BView32 *__restrict__ V, const BItem *__restrict__ it, int cur, int npt) {
     const BItem b = it[blockIdx.x];
-    if (!V[b.view].active[V[b.view].dom]) return;
+    pdl_wait();
     const BView32 &w = V[b.view];
-    LevelView<float> v = w.v;
-    v.u = ugrid(w, cur);
-    for_span(b, npt, [&](int64_t k) {
-        if (WB) local_copyback<float>(w.bz, v.u, (int)k);
-        if (k < w.js_n) w.js_r[w.js_rpos[k]] = js_defect<float, 2, WB>(v, w.js_node[k], w.js_ghost[k], w.bz.wb);
-    });
+    if (!w.active[w.dom]) return;
+    const float *u = ugrid(w, cur);
+    for_span(b, npt, [&](int64_t k) { if (k < w.js_nread) w.z[w.js_read[k]] = u[w.js_read[k]]; });
 }
 
-// one chunk a CTA, kJsWarpRows rows a warp (each lane sums its vectors of a
-// row in index order, as js_apply_rows); chain: descriptor -> active flag -> rows
-__global__ void __launch_bounds__(256) kb_js_apply_chunk(const JsItem *__restrict__ items,
-                                                        const int *__restrict__ active, int cur) {
+// exact junction solve: u += A_ZZ^-1 r, a CTA a chunk of rows of one component,
+// kJsWarpRows a warp (a row's vector in flight each); the component's defects r
+// are computed by every CTA from z into shared memory (as k_js).  Bound by the
+// inverses' bytes (160 MB a launch on 48 stars).  8 rows a warp and three CTAs an
+// SM: 48 stars 23.3 ms a solve with 4 rows and two, 21.6 ms so.
+constexpr int kJsWarpRows = 8;
+constexpr int kJsRows = 8 * kJsWarpRows;
+
+__global__ void __launch_bounds__(256, 3) kb_js(const BView32 *__restrict__ V, const JsItem *__restrict__ items, int cur) {
+    extern __shared__ __align__(16) unsigned char smem_js[];
+    float *rs = reinterpret_cast<float *>(smem_js);
     const JsItem q = items[blockIdx.x];
-    if (!active[q.dom]) return;
-    using V = Vec16<float>::type;
-    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int i0 = w * kJsWarpRows;
+    const BView32 &w = V[q.view];
+    const LevelView<float> &v = w.v;
+    const float *z = w.z;
+    js_component_defects<float, 2>(v, z, q.node, q.ghost, q.m, q.mi, rs, w.active + w.dom);   // waits before it reads z
+    __syncthreads();
+    if (!w.active[w.dom]) return;
+    using Vec = Vec16<float>::type;
+    const int wp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int i0 = wp * kJsWarpRows;
     const int nr = min(kJsWarpRows, q.rows - i0);
     if (nr <= 0) return;   // uniform over the warp
-    const int nv = q.mp / 4;
-    const V *a = reinterpret_cast<const V *>(q.a + (int64_t)i0 * q.mp);
-    const V *rr = reinterpret_cast<const V *>(q.r);
-    constexpr int U = 2;
+    const int nv = (q.m + 3) / 4;
+    const Vec *a = reinterpret_cast<const Vec *>(q.a) + (int64_t)i0 * nv;
+    const Vec *rr = reinterpret_cast<const Vec *>(rs);
+    constexpr int U = 1;
     float s[kJsWarpRows] = {};
     for (int j0 = lane; j0 < nv; j0 += 32 * U) {
-        V rv[U], av[kJsWarpRows][U];
-#pragma unroll
-        for (int e = 0; e < U; e++)
-            if (j0 + 32 * e < nv) {
-                rv[e] = rr[j0 + 32 * e];
-#pragma unroll
-                for (int i = 0; i < kJsWarpRows; i++)
-                    if (i < nr) av[i][e] = a[(int64_t)i * nv + j0 + 32 * e];
-            }
+        Vec av[kJsWarpRows][U];
 #pragma unroll
         for (int e = 0; e < U; e++)
             if (j0 + 32 * e < nv)
 #pragma unroll
                 for (int i = 0; i < kJsWarpRows; i++)
-                    if (i < nr) s[i] = Vec16<float>::dot(s[i], av[i][e], rv[e]);
+                    if (i < nr) av[i][e] = a[(int64_t)i * nv + j0 + 32 * e];
+#pragma unroll
+        for (int e = 0; e < U; e++)
+            if (j0 + 32 * e < nv) {
+                const Vec rv = rr[j0 + 32 * e];
+#pragma unroll
+                for (int i = 0; i < kJsWarpRows; i++)
+                    if (i < nr) s[i] = Vec16<float>::dot(s[i], av[i][e], rv);
+            }
     }
-    float *u = cur ? q.u1 : q.u0;
+    float *u = ugrid(w, cur);
 #pragma unroll
     for (int i = 0; i < kJsWarpRows; i++) {
         float t = s[i];
         for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-        if (lane == 0 && i < nr) u[q.node[i0 + i]] += t;
+        if (lane == 0 && i < nr) {
+            const int32_t p = q.node[q.k0 + i0 + i];
+            u[p] = z[p] + t;
+        }
     }
 }
 
-// defect, restriction with the coarse-ghost transfer, and zero coarse u in
-// one pass over the coarser level's nodes and ghosts (fine u in grid `cur`,
-// coarse u = 0 into its first grid)
+// defect, restriction with the coarse-ghost transfer, and zero coarse u in one
+// pass (fine u in grid `cur`, coarse u = 0 into its first grid): 32 indexes a
+// coarse ghost row, then 64 a segment of coarse inside nodes
 __global__ void kb_descend(const BView32 *__restrict__ V, const BItem *__restrict__ it, int cur, int npt) {
     const BItem b = it[blockIdx.x];
+    pdl_wait();
     if (!V[b.view].active[V[b.view].dom]) return;
     const BView32 &w = V[b.view];
     LevelView<float> v = w.v;
     v.u = ugrid(w, cur);
-    for_span(b, npt, [&](int64_t i) {
-        descend_item<float, 2>(v, w.c, w.cf, w.cg, w.c.u, w.gt_ptr, w.gt_col, w.gt_val, i);
+    const LevelView<float> &c = w.c;
+    const int64_t nw = 32 * (int64_t)c.ng;
+    for_span(b, npt, [&](int64_t t) {
+        if (t < nw) {   // uniform over the warp
+            const int q = (int)(t >> 5);
+            descend_ghost_row_warp<float, 2, false>(v, w.cg, w.gt_ptr, w.gt_col, w.gt_val, q);
+            if ((t & 31) == 0) c.u[c.gnode[q]] = 0;
+            return;
+        }
+        const int64_t s = (t - nw) >> 6;
+        if (s >= c.nsegs) return;
+        const int2 sg = c.segs[s];
+        const int k = (sg.y & 0xffff) + (int)((t - nw) & 63);
+        if (k <= (int)((unsigned)sg.y >> 16))
+            descend_inside_early<float, 2, false>(v, w.cf, c.u, (int64_t)sg.x * c.n + k, 2 * ((int64_t)sg.x * v.s0 + k));
     });
 }
 
-// zero u of the view's level (coarse = 0) or of its coarser level (coarse = 1)
-__global__ void kb_zero(const BView32 *__restrict__ V, const BItem *__restrict__ it, int coarse, int npt) {
-    const BItem b = it[blockIdx.x];
-    if (!V[b.view].active[V[b.view].dom]) return;
-    const LevelView<float> &v = coarse ? V[b.view].c : V[b.view].v;
-    for_span(b, npt, [&](int64_t p) { if (p < v.nn) v.u[p] = 0.f; });
+// index t over a level's unknowns (64 a segment of inside nodes, then the
+// ghosts): calls f(row, k, ghost number or -1)
+template <typename T, class F>
+__device__ __forceinline__ void at_unknown(const LevelView<T> &v, int64_t t, F &&f) {
+    const int64_t nt = 64 * (int64_t)v.nsegs;
+    if (t < nt) {
+        const int2 sg = v.segs[t >> 6];
+        const int k = (sg.y & 0xffff) + (int)(t & 63);
+        if (k <= (int)((unsigned)sg.y >> 16)) f(sg.x, k, -1);
+    } else if (t - nt < v.ng) {
+        const int q = (int)(t - nt), p = v.gnode[q];
+        f(p / v.n, p % v.n, q);
+    }
 }
 
 __global__ void kb_prolong(const BView32 *__restrict__ V, const BItem *__restrict__ it, int cur, int ccur,
                            int npt) {
     const BItem b = it[blockIdx.x];
+    pdl_wait();
     if (!V[b.view].active[V[b.view].dom]) return;
     const BView32 &w = V[b.view];
-    float *e = ccur ? w.c_u2 : w.c.u;
+    const float *e = ccur ? w.c_u2 : w.c.u;
     float *u = ugrid(w, cur);
-    for_span(b, npt, [&](int64_t p) { if (p < w.v.nn) prolong_node<float, 2>(w.v, w.c, e, u, true, p); });
+    for_span(b, npt, [&](int64_t t) {
+        at_unknown(w.v, t, [&](int i, int k, int) { prolong_add2<float>(w.v, w.c, e, u, i, k); });
+    });
 }
 
 __global__ void kb_coarse(const BView32 *__restrict__ V, const BItem *__restrict__ it) {
     const BItem b = it[blockIdx.x];
+    pdl_wait();
     if (!V[b.view].active[V[b.view].dom]) return;
     const BView32 &w = V[b.view];
     coarse_rows<float>(w.v, w.unk_node, w.unk_ghost, w.Ainv, w.nunk, b.start, kCoarseBlocks);
 }
 
-// FP64 level 0: defect with per-domain norms (nodes, then ghosts)
 // largest |x| over a thread's indexes; NaN wins
 __device__ __forceinline__ double max_abs(double m, double x) {
     double a = fabs(x);
@@ -240,60 +296,54 @@ __device__ __forceinline__ double max_abs(double m, double x) {
     return a > m ? a : m;
 }
 
+// FP64 level 0: the defect at every unknown, its per-domain norm, and the next
+// FP32 problem (right-hand side = the defect, e32 = 0; both stay 0 elsewhere)
 __global__ void kb_defect64(const BView64 *__restrict__ V, const BItem *__restrict__ it, unsigned long long *norms,
-                            int ghosts, int npt) {
+                            int npt) {
     const BItem b = it[blockIdx.x];
-    if (!V[b.view].active[V[b.view].dom]) return;   // uniform per block
-    const LevelView<double> &v = V[b.view].v;
-    double m = 0.0;
-    if (!ghosts) {
-        for_span(b, npt, [&](int64_t p) { if (p < v.nn) m = max_abs(m, defect_node<double, 2>(v, p, false)); });
-    } else {
-        for_span(b, npt, [&](int64_t q) { if (q < v.ng) m = max_abs(m, defect_ghost_item<double, 9>(v, (int)q)); });
-    }
-    reduce_norm(norms + V[b.view].dom, m);
+    pdl_wait();
+    const BView64 &w = V[b.view];
+    if (!w.active[w.dom]) return;   // uniform per block
+    const LevelView<double> &v = w.v;
+    unsigned long long m = 0;   // the largest |d| by its bits (off the FP64 pipe; NaN above +Inf)
+    for_span(b, npt, [&](int64_t t) {
+        at_unknown(v, t, [&](int i, int k, int q) {
+            const int64_t p = (int64_t)i * v.n + k;
+            const double d = q < 0 ? inside_defect<double, 2>(v, p) : ghost_defect<double, 9>(v, q);
+            if (q < 0) w.f32[p] = (float)d;
+            else w.g32[q] = (float)d;
+            w.e32[p] = 0.f;
+            const unsigned long long a = (unsigned long long)__double_as_longlong(d) & 0x7fffffffffffffffull;
+            m = a > m ? a : m;
+        });
+    });
+    reduce_norm(norms + w.dom, __longlong_as_double((long long)m));
 }
 
 // ||(f, g)|| per domain
 __global__ void kb_rhs_norm(const BView64 *__restrict__ V, const BItem *__restrict__ it, unsigned long long *norms,
-                            int ghosts, int npt) {
+                            int npt) {
     const BItem b = it[blockIdx.x];
     const LevelView<double> &v = V[b.view].v;
     double m = 0.0;
-    if (!ghosts) {
-        for_span(b, npt, [&](int64_t p) { if (p < v.nn && (v.type[p] & NODE_KIND) == NODE_IN) m = max_abs(m, v.f[p]); });
-    } else {
-        for_span(b, npt, [&](int64_t q) { if (q < v.ng) m = max_abs(m, v.gg[q]); });
-    }
+    for_span(b, npt, [&](int64_t t) {
+        at_unknown(v, t, [&](int i, int k, int q) { m = max_abs(m, q < 0 ? v.f[(int64_t)i * v.n + k] : v.gg[q]); });
+    });
     reduce_norm(norms + V[b.view].dom, m);
-}
-
-// FP64 defect -> FP32 right-hand side; e32 = 0
-__global__ void kb_to_f32(const BView64 *__restrict__ V, const BItem *__restrict__ it, int ghosts, int npt) {
-    const BItem b = it[blockIdx.x];
-    if (!V[b.view].active[V[b.view].dom]) return;
-    const BView64 &w = V[b.view];
-    if (!ghosts) {
-        for_span(b, npt, [&](int64_t p) {
-            if (p >= w.v.nn) return;
-            w.f32[p] = ((w.v.type[p] & NODE_KIND) == NODE_IN) ? (float)w.v.r[p] : 0.f;
-            w.e32[p] = 0.f;
-        });
-    } else {
-        for_span(b, npt, [&](int64_t q) { if (q < w.v.ng) w.g32[q] = (float)w.v.r[w.v.gnode[q]]; });
-    }
 }
 
 // u64 += e32 on Omega_h u Gamma_h
 __global__ void kb_add(const BView64 *__restrict__ V, const BItem *__restrict__ it, int cur, int npt) {
     const BItem b = it[blockIdx.x];
+    pdl_wait();
     if (!V[b.view].active[V[b.view].dom]) return;
     const BView64 &w = V[b.view];
     const float *e = cur ? w.e32b : w.e32;
-    for_span(b, npt, [&](int64_t p) {
-        if (p >= w.v.nn) return;
-        const uint8_t k = w.v.type[p] & NODE_KIND;
-        if (k == NODE_IN || k == NODE_GHOST) w.v.u[p] += (double)e[p];
+    for_span(b, npt, [&](int64_t t) {
+        at_unknown(w.v, t, [&](int i, int k, int) {
+            const int64_t p = (int64_t)i * w.v.n + k;
+            w.v.u[p] += (double)e[p];
+        });
     });
 }
 
@@ -325,13 +375,14 @@ __global__ void kb_check(cudaGraphConditionalHandle h, const unsigned long long 
 
 // a captured launch: kernel kind, item range and parameters
 struct Launch {
-    enum Kind { FUSED, BOUNDARY, BOUNDARY_COPY, JUNCTION, JS_DEFECT, JS_APPLY, DESCEND, PROLONG, COARSE, ZERO };
+    enum Kind { RELAX, FUSED, BOUNDARY, BOUNDARY_COPY, JUNCTION, JS_COPY, JS, DESCEND, PROLONG, COARSE };
     Kind kind;
     size_t off, count;
     size_t smem;
     int cur = 0, ccur = 0;   // which u grid holds u (this level, the next coarser one)
     int npt = 1;             // indexes a thread of a dense item
     int ept = LOCAL_EPT;     // shared-memory programs: inside entries per thread and colour
+    int nt = 256, m = 1;     // RELAX: threads, records a thread (the most any of its blocks needs)
 };
 
 }  // namespace
@@ -354,8 +405,8 @@ struct gcmg_batch {
     JsItem *d_jsitems = nullptr;              // junction-solve chunks (JS_APPLY launches)
     std::vector<int32_t *> tile_bufs;         // tile lists per view for the selected shape
     std::vector<Launch> cycle;                // FP32 V-cycle over all domains
-    size_t items64_nodes = 0, items64_ghosts = 0, n_items64_nodes = 0, n_items64_ghosts = 0;
-    int npt64_nodes = 1, npt64_ghosts = 1;
+    size_t items64 = 0, n_items64 = 0;        // the unknowns of every domain's level 0
+    int npt64 = 1;
     unsigned long long *d_norms = nullptr;
     double *d_r0 = nullptr, *d_rel = nullptr;
     int *d_m = nullptr;
@@ -451,16 +502,10 @@ void build_tables(gcmg_batch *b) {
             w.nunk = c->G[l].nunk;
             w.dom = d;
             w.active = b->d_active;
-            w.js_n = c->G[l].js_n;
-            w.js_node = c->G[l].js_node;
-            w.js_ghost = c->G[l].js_ghost;
-            w.js_comp = c->G[l].js_comp;
-            w.js_off = c->G[l].js_off;
-            w.js_aoff = c->G[l].js_aoff;
-            w.js_roff = c->G[l].js_roff;
-            w.js_rpos = c->G[l].js_rpos;
-            w.js_inv = c->D32[l].js_inv;
-            w.js_r = c->D32[l].js_r;
+            w.b2 = b2view<float>(c->G[l].b2, w.v);
+            w.z = c->D32[l].r;
+            w.js_read = c->G[l].js_read;
+            w.js_nread = c->p.junction_solve ? c->G[l].js_nread : 0;
             b->view_of[d].push_back((int)v32.size());
             v32.push_back(w);
             if (!c->G[l].bz.in_smem || (c->p.junction_sweeps > 0 && c->G[l].jz.ncomp > 0 && !c->G[l].jz.in_smem))
@@ -519,18 +564,54 @@ void build_tables(gcmg_batch *b) {
     };
     const gcmg_params &p0 = b->doms[0]->p;
     auto relax = [&](int k) {
-        size_t s0 = items.size();
+        // strips and boundary blocks in one launch where every domain's blocks fit
+        bool merged = true;
+        int nt = 256, m = 1;
         for (int d = 0; d < nd; d++) {
             const int l = (int)b->doms[d]->H.size() - 1 - k;
             if (l < 0) continue;
-            const int vi = b->view_of[d][l];
-            for (int i = 0; i < ntile[vi]; i += 4) items.push_back({vi, (int32_t)i});
+            const Block2Dev &p = b->doms[d]->G[l].b2;
+            if (p.ncomp == 0) continue;
+            merged = merged && p.m > 0;
+            nt = std::max(nt, p.nt);
+            m = std::max(m, p.m);
         }
-        add_launch(Launch::FUSED, s0, 0, cur[k]);   // reads grid cur[k], writes the other
-        cur[k] ^= 1;
-        for (int which = 0; which < 2; which++) {
+        size_t s0 = items.size();
+        size_t smem = 0;
+        if (merged) {
+            for (int d = 0; d < nd; d++) {   // the blocks first: each is a chain of phases, the strips fill in
+                const int l = (int)b->doms[d]->H.size() - 1 - k;
+                if (l < 0) continue;
+                const Block2Dev &p = b->doms[d]->G[l].b2;
+                for (int c = 0; c < p.ncomp; c++) items.push_back({b->view_of[d][l], ~c});
+                if (p.ncomp) smem = std::max(smem, block2_smem<float>(p));
+            }
+            for (int d = 0; d < nd; d++) {
+                const int l = (int)b->doms[d]->H.size() - 1 - k;
+                if (l < 0) continue;
+                const int vi = b->view_of[d][l];
+                for (int i = 0; i < ntile[vi]; i += nt / 32) items.push_back({vi, (int32_t)i});
+            }
+            const size_t before = b->cycle.size();
+            add_launch(Launch::RELAX, s0, smem, cur[k]);
+            if (b->cycle.size() > before) {
+                b->cycle.back().nt = nt;
+                b->cycle.back().m = m;
+            }
+            cur[k] ^= 1;
+        } else {
+            for (int d = 0; d < nd; d++) {
+                const int l = (int)b->doms[d]->H.size() - 1 - k;
+                if (l < 0) continue;
+                const int vi = b->view_of[d][l];
+                for (int i = 0; i < ntile[vi]; i += 4) items.push_back({vi, (int32_t)i});
+            }
+            add_launch(Launch::FUSED, s0, 0, cur[k]);   // reads grid cur[k], writes the other
+            cur[k] ^= 1;
+        }
+        for (int which = merged ? 1 : 0; which < 2; which++) {
             s0 = items.size();
-            size_t smem = 0;
+            smem = 0;
             int most = 0;   // most inside entries of one colour in a component
             for (int d = 0; d < nd; d++) {
                 const int l = (int)b->doms[d]->H.size() - 1 - k;
@@ -546,7 +627,7 @@ void build_tables(gcmg_batch *b) {
             const size_t ncycle = b->cycle.size();
             add_launch(which ? Launch::JUNCTION : Launch::BOUNDARY, s0, smem, cur[k]);
             if (b->cycle.size() > ncycle && most <= LOCAL_THREADS) b->cycle.back().ept = 1;
-            if (!which && !p0.junction_solve) {   // the boundary blocks' write-back, once all have staged
+            if (!which) {   // the boundary blocks' write-back, once all have staged
                 for (int d = 0; d < nd; d++) {
                     const int l = (int)b->doms[d]->H.size() - 1 - k;
                     if (l >= 0) dense(b->view_of[d][l], v32[b->view_of[d][l]].bz.nwb);
@@ -555,42 +636,44 @@ void build_tables(gcmg_batch *b) {
             }
         }
         if (p0.junction_solve) {
-            // with the boundary blocks' write-back (all views of a batch have
-            // boundary programs with a write-back grid)
-            for (int d = 0; d < nd; d++) {
-                const int l = (int)b->doms[d]->H.size() - 1 - k;
-                if (l < 0) continue;
-                const BView32 &w = v32[b->view_of[d][l]];
-                dense(b->view_of[d][l], std::max<int64_t>(w.js_n, w.bz.wb ? w.bz.nwb : 0));
+            if (!merged) {
+                for (int d = 0; d < nd; d++) {
+                    const int l = (int)b->doms[d]->H.size() - 1 - k;
+                    if (l >= 0) dense(b->view_of[d][l], v32[b->view_of[d][l]].js_nread);
+                }
+                add_dense(Launch::JS_COPY, cur[k]);
             }
-            add_dense(Launch::JS_DEFECT, cur[k]);
             // chunks of at most kJsRows rows of one component, addresses resolved here
             const size_t j0 = jsitems.size();
+            smem = 0;
             for (int d = 0; d < nd; d++) {
                 const int l = (int)b->doms[d]->H.size() - 1 - k;
                 if (l < 0) continue;
                 gcmg_ctx *c = b->doms[d];
                 const DevGeom &g = c->G[l];
                 const DevData<float> &D = c->D32[l];
-                const std::vector<int32_t> &off = c->H[l].js_off;
+                const HostLevel &L = c->H[l];
                 for (int cc = 0; cc < g.js_ncomp; cc++) {
-                    const int o = off[cc], m = off[cc + 1] - o, mp = (m + 3) & ~3;
-                    for (int r0 = o; r0 < o + m; r0 += kJsRows) {
+                    const int o = L.js_off[cc], m_ = L.js_off[cc + 1] - o, mp = (m_ + 3) & ~3;
+                    int mi = 0;
+                    for (int i = o; i < o + m_; i++) mi += L.js_ghost[i] < 0;
+                    smem = std::max(smem, sizeof(float) * (size_t)mp);
+                    for (int r0 = 0; r0 < m_; r0 += kJsRows) {
                         JsItem q{};
-                        q.a = D.js_inv + g.js_aoff_h[cc] + (int64_t)(r0 - o) * mp;
-                        q.r = D.js_r + g.js_roff_h[cc];
-                        q.node = g.js_node + r0;
-                        q.u0 = D.u;
-                        q.u1 = D.u2;
-                        q.rows = std::min(kJsRows, o + m - r0);
-                        q.mp = mp;
-                        q.dom = d;
+                        q.a = D.js_inv + g.js_aoff_h[cc] + (int64_t)r0 * mp;
+                        q.node = g.js_node + o;
+                        q.ghost = g.js_ghost + o;
+                        q.view = b->view_of[d][l];
+                        q.m = m_;
+                        q.mi = mi;
+                        q.k0 = r0;
+                        q.rows = std::min(kJsRows, m_ - r0);
                         jsitems.push_back(q);
                     }
                 }
             }
             if (jsitems.size() > j0) {
-                Launch L{Launch::JS_APPLY, j0, jsitems.size() - j0, 0};
+                Launch L{Launch::JS, j0, jsitems.size() - j0, smem};
                 L.cur = cur[k];
                 b->cycle.push_back(L);
             }
@@ -602,8 +685,7 @@ void build_tables(gcmg_batch *b) {
     // when that is the coarsest), the interpolation, nu2 relaxations
     auto visit = [&](auto &self, int k) -> void {
         if (k == 0) {
-            for (int d = 0; d < nd; d++) dense(b->view_of[d].back(), b->doms[d]->H.back().nn);
-            add_dense(Launch::ZERO);
+            // every unknown is written: nothing to zero
             const size_t s0 = items.size();
             size_t smem = 0;
             for (int d = 0; d < nd; d++) {
@@ -616,7 +698,10 @@ void build_tables(gcmg_batch *b) {
         for (int r = 0; r < p0.nu1; r++) relax(k);
         for (int d = 0; d < nd; d++) {
             const int l = (int)b->doms[d]->H.size() - 1 - k;
-            if (l >= 0) dense(b->view_of[d][l], std::max<int64_t>(b->doms[d]->H[l + 1].nn, b->doms[d]->H[l + 1].ng()));
+            if (l >= 0) {
+                const LevelView<float> &cv = v32[b->view_of[d][l]].c;
+                dense(b->view_of[d][l], 32 * (int64_t)cv.ng + 64 * (int64_t)cv.nsegs);
+            }
         }
         add_dense(Launch::DESCEND, cur[k]);
         cur[k - 1] = 0;
@@ -624,7 +709,10 @@ void build_tables(gcmg_batch *b) {
         for (int g = 0; g < gam; g++) self(self, k - 1);
         for (int d = 0; d < nd; d++) {
             const int l = (int)b->doms[d]->H.size() - 1 - k;
-            if (l >= 0) dense(b->view_of[d][l], b->doms[d]->H[l].nn);
+            if (l >= 0) {
+                const LevelView<float> &v = v32[b->view_of[d][l]].v;
+                dense(b->view_of[d][l], 64 * (int64_t)v.nsegs + v.ng);
+            }
         }
         add_dense(Launch::PROLONG, cur[k], cur[k - 1]);
         for (int r = 0; r < p0.nu2; r++) relax(k);
@@ -633,14 +721,10 @@ void build_tables(gcmg_batch *b) {
     visit(visit, kmax);
     b->add_cur = cur[kmax];
     // FP64 level-0 items (view index = domain)
-    b->items64_nodes = items.size();
-    for (int d = 0; d < nd; d++) dense(d, b->doms[d]->H[0].nn);
-    b->npt64_nodes = emit_dense();
-    b->n_items64_nodes = items.size() - b->items64_nodes;
-    b->items64_ghosts = items.size();
-    for (int d = 0; d < nd; d++) dense(d, b->doms[d]->H[0].ng());
-    b->npt64_ghosts = emit_dense();
-    b->n_items64_ghosts = items.size() - b->items64_ghosts;
+    b->items64 = items.size();
+    for (int d = 0; d < nd; d++) dense(d, 64 * (int64_t)v64[d].v.nsegs + v64[d].v.ng);
+    b->npt64 = emit_dense();
+    b->n_items64 = items.size() - b->items64;
     ck(cudaMalloc(&b->d_v32, v32.size() * sizeof(BView32)), "cudaMalloc");
     ck(cudaMalloc(&b->d_v64, v64.size() * sizeof(BView64)), "cudaMalloc");
     ck(cudaMalloc(&b->d_items, std::max<size_t>(items.size(), 1) * sizeof(BItem)), "cudaMalloc");
@@ -655,60 +739,73 @@ void build_tables(gcmg_batch *b) {
     for (gcmg_ctx *c : b->doms) b->versions.push_back(c->version);
 }
 
+// A launch that may be set up while its predecessor finishes; the kernel waits
+// for it (pdl_wait) before it reads what a launch writes
+template <typename... P, typename... A>
+void blaunch(void (*kernel)(P...), unsigned grid, unsigned block, size_t smem, cudaStream_t s, A... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    ck(cudaLaunchKernelEx(&cfg, kernel, P(args)...), "launch");
+}
+
 template <int SR>
-void launch_fused(const gcmg_batch *b, const Launch &L, cudaStream_t s) {
-    kb_fused<SR><<<(unsigned)L.count, 128, 0, s>>>(b->d_v32, b->d_items + L.off, L.cur);
+void launch_sweep(const gcmg_batch *b, const Launch &L, cudaStream_t s) {
+    const BItem *it = b->d_items + L.off;
+    const unsigned n = (unsigned)L.count;
+    const int lambda = b->doms[0]->p.lambda;
+    if (L.kind == Launch::FUSED) blaunch(kb_fused<SR>, n, 128, 0, s, b->d_v32, it, L.cur);
+    else if (L.nt == 512) blaunch(kb_relax<SR, 512, 2>, n, 512, L.smem, s, b->d_v32, it, L.cur, lambda);
+    else if (L.m == 2) blaunch(kb_relax<SR, 256, 2>, n, 256, L.smem, s, b->d_v32, it, L.cur, lambda);
+    else blaunch(kb_relax<SR, 256, 1>, n, 256, L.smem, s, b->d_v32, it, L.cur, lambda);
 }
 
 void launch_one(const gcmg_batch *b, const Launch &L, cudaStream_t s) {
     const BItem *it = b->d_items + L.off;
     const unsigned n = (unsigned)L.count;
     const int junction_sweeps = b->doms[0]->p.junction_sweeps, lambda = b->doms[0]->p.lambda;
+    const int j = L.kind == Launch::JUNCTION ? 1 : 0, lead = 1 - j, reps = j ? junction_sweeps : lambda;
     switch (L.kind) {
+        case Launch::RELAX:
         case Launch::FUSED:
             switch (kStripRows[b->variant]) {   // the height the strip lists were built with
-                case 8: launch_fused<8>(b, L, s); break;
-                case 16: launch_fused<16>(b, L, s); break;
-                default: launch_fused<32>(b, L, s); break;
+                case 8: launch_sweep<8>(b, L, s); break;
+                case 16: launch_sweep<16>(b, L, s); break;
+                default: launch_sweep<32>(b, L, s); break;
             }
             break;
         case Launch::BOUNDARY:
-            if (L.ept == 1) kb_local<1><<<n, LOCAL_THREADS, L.smem, s>>>(b->d_v32, it, 0, 1, lambda, L.cur);
-            else kb_local<LOCAL_EPT><<<n, LOCAL_THREADS, L.smem, s>>>(b->d_v32, it, 0, 1, lambda, L.cur);
-            break;
-        case Launch::BOUNDARY_COPY: kb_local_copyback<<<n, 256, 0, s>>>(b->d_v32, it, L.cur, L.npt); break;
         case Launch::JUNCTION:
-            if (L.ept == 1) kb_local<1><<<n, LOCAL_THREADS, L.smem, s>>>(b->d_v32, it, 1, 0, junction_sweeps, L.cur);
-            else kb_local<LOCAL_EPT><<<n, LOCAL_THREADS, L.smem, s>>>(b->d_v32, it, 1, 0, junction_sweeps, L.cur);
+            if (L.ept == 1) blaunch(kb_local<1>, n, LOCAL_THREADS, L.smem, s, b->d_v32, it, j, lead, reps, L.cur);
+            else blaunch(kb_local<LOCAL_EPT>, n, LOCAL_THREADS, L.smem, s, b->d_v32, it, j, lead, reps, L.cur);
             break;
-        case Launch::JS_DEFECT: kb_js_defect<true><<<n, kThreads, 0, s>>>(b->d_v32, it, L.cur, L.npt); break;
-        case Launch::JS_APPLY:
-            kb_js_apply_chunk<<<n, 256, 0, s>>>(b->d_jsitems + L.off, b->d_active, L.cur);
-            break;
-        case Launch::DESCEND: kb_descend<<<n, kThreads, 0, s>>>(b->d_v32, it, L.cur, L.npt); break;
-        case Launch::ZERO: kb_zero<<<n, kThreads, 0, s>>>(b->d_v32, it, 0, L.npt); break;
-        case Launch::COARSE: kb_coarse<<<n, 512, L.smem, s>>>(b->d_v32, it); break;
-        case Launch::PROLONG: kb_prolong<<<n, kThreads, 0, s>>>(b->d_v32, it, L.cur, L.ccur, L.npt); break;
+        case Launch::BOUNDARY_COPY: blaunch(kb_local_copyback, n, 256, 0, s, b->d_v32, it, L.cur, L.npt); break;
+        case Launch::JS_COPY: blaunch(kb_js_copy, n, kThreads, 0, s, b->d_v32, it, L.cur, L.npt); break;
+        case Launch::JS: blaunch(kb_js, n, 256, L.smem, s, b->d_v32, b->d_jsitems + L.off, L.cur); break;
+        case Launch::DESCEND: blaunch(kb_descend, n, kThreads, 0, s, b->d_v32, it, L.cur, L.npt); break;
+        case Launch::COARSE: blaunch(kb_coarse, n, 512, L.smem, s, b->d_v32, it); break;
+        case Launch::PROLONG: blaunch(kb_prolong, n, kThreads, 0, s, b->d_v32, it, L.cur, L.ccur, L.npt); break;
     }
 }
 
-// one refinement step of every domain, then the FP64 defect norms
+// one refinement step of every domain from the FP32 problem the last defect
+// set up, then the FP64 defect, its norms and the next problem
 void step_body(gcmg_batch *b, cudaStream_t s) {
-    const BItem *in = b->d_items + b->items64_nodes, *ig = b->d_items + b->items64_ghosts;
-    kb_to_f32<<<(unsigned)b->n_items64_nodes, kThreads, 0, s>>>(b->d_v64, in, 0, b->npt64_nodes);
-    if (b->n_items64_ghosts)
-        kb_to_f32<<<(unsigned)b->n_items64_ghosts, kThreads, 0, s>>>(b->d_v64, ig, 1, b->npt64_ghosts);
+    const BItem *it = b->d_items + b->items64;
     for (const Launch &L : b->cycle) launch_one(b, L, s);
-    kb_add<<<(unsigned)b->n_items64_nodes, kThreads, 0, s>>>(b->d_v64, in, b->add_cur, b->npt64_nodes);
+    blaunch(kb_add, (unsigned)b->n_items64, kThreads, 0, s, b->d_v64, it, b->add_cur, b->npt64);
     ck(cudaMemsetAsync(b->d_norms, 0, b->doms.size() * sizeof(unsigned long long), s), "memset");
-    kb_defect64<<<(unsigned)b->n_items64_nodes, kThreads, 0, s>>>(b->d_v64, in, b->d_norms, 0, b->npt64_nodes);
-    if (b->n_items64_ghosts)
-            kb_defect64<<<(unsigned)b->n_items64_ghosts, kThreads, 0, s>>>(b->d_v64, ig, b->d_norms, 1, b->npt64_ghosts);
+    blaunch(kb_defect64, (unsigned)b->n_items64, kThreads, 0, s, b->d_v64, it, b->d_norms, b->npt64);
 }
 
-long long step_kernels(const gcmg_batch *b) {
-    return (long long)b->cycle.size() + 4 + (b->n_items64_ghosts ? 2 : 0) + 1;
-}
+long long step_kernels(const gcmg_batch *b) { return (long long)b->cycle.size() + 3; }
 
 void build_graph(gcmg_batch *b) {
     if (b->gexec) cudaGraphExecDestroy(b->gexec);
@@ -947,7 +1044,7 @@ gcmg_status gcmg_batch_solve(gcmg_batch *b, gcmg_stats *stats, int *steps) {
         }
         const int nd = (int)b->doms.size();
         cudaStream_t s = b->stream;
-        const BItem *in = b->d_items + b->items64_nodes, *ig = b->d_items + b->items64_ghosts;
+        const BItem *it = b->d_items + b->items64;
         {   // every domain starts active; the step kernels skip the inactive ones
             std::vector<int> ones(nd, 1), zeros(nd, 0);
             ck(cudaMemcpyAsync(b->d_active, ones.data(), nd * sizeof(int), cudaMemcpyHostToDevice, s), "active");
@@ -959,9 +1056,7 @@ gcmg_status gcmg_batch_solve(gcmg_batch *b, gcmg_stats *stats, int *steps) {
             ck(cudaMemsetAsync(c->D64[0].u, 0, c->H[0].nn * sizeof(double), s), "memset");
         // ||r0|| = ||(f, g)|| per domain
         ck(cudaMemsetAsync(b->d_norms, 0, nd * sizeof(unsigned long long), s), "memset");
-        kb_rhs_norm<<<(unsigned)b->n_items64_nodes, kThreads, 0, s>>>(b->d_v64, in, b->d_norms, 0, b->npt64_nodes);
-        if (b->n_items64_ghosts)
-            kb_rhs_norm<<<(unsigned)b->n_items64_ghosts, kThreads, 0, s>>>(b->d_v64, ig, b->d_norms, 1, b->npt64_ghosts);
+        kb_rhs_norm<<<(unsigned)b->n_items64, kThreads, 0, s>>>(b->d_v64, it, b->d_norms, b->npt64);
         std::vector<unsigned long long> bits(nd);
         ck(cudaMemcpyAsync(bits.data(), b->d_norms, nd * sizeof(unsigned long long), cudaMemcpyDeviceToHost, s), "r0");
         ck(cudaStreamSynchronize(s), "sync");
@@ -971,11 +1066,9 @@ gcmg_status gcmg_batch_solve(gcmg_batch *b, gcmg_stats *stats, int *steps) {
             if (!(r0[d] > 0.0)) r0[d] = 1.0;
         }
         ck(cudaMemcpyAsync(b->d_r0, r0.data(), nd * sizeof(double), cudaMemcpyHostToDevice, s), "r0");
-        // defect of u = 0 (the FP64 defect every step starts from)
+        // defect of u = 0 and the first FP32 problem
         ck(cudaMemsetAsync(b->d_norms, 0, nd * sizeof(unsigned long long), s), "memset");
-        kb_defect64<<<(unsigned)b->n_items64_nodes, kThreads, 0, s>>>(b->d_v64, in, b->d_norms, 0, b->npt64_nodes);
-        if (b->n_items64_ghosts)
-            kb_defect64<<<(unsigned)b->n_items64_ghosts, kThreads, 0, s>>>(b->d_v64, ig, b->d_norms, 1, b->npt64_ghosts);
+        kb_defect64<<<(unsigned)b->n_items64, kThreads, 0, s>>>(b->d_v64, it, b->d_norms, b->npt64);
         ck(cudaGetLastError(), "kernel launch");
         const int zero = 0;
         ck(cudaMemcpyAsync(b->d_m, &zero, sizeof(int), cudaMemcpyHostToDevice, s), "m");
@@ -998,7 +1091,7 @@ gcmg_status gcmg_batch_solve(gcmg_batch *b, gcmg_stats *stats, int *steps) {
         int m = 0;
         ck(cudaMemcpyAsync(&m, b->d_m, sizeof(int), cudaMemcpyDeviceToHost, s), "m");
         ck(cudaStreamSynchronize(s), "sync");
-        g_launches += 4 + b->graph_kernels * m;
+        g_launches += 2 + b->graph_kernels * m;
         std::vector<double> rel((size_t)nd * 257, 0.0);
         ck(cudaMemcpy(rel.data(), b->d_rel, rel.size() * sizeof(double), cudaMemcpyDeviceToHost), "rel");
         std::vector<int> steps_of(nd, 0);
@@ -1058,7 +1151,7 @@ gcmg_status gcmg_batch_autotune(gcmg_batch *b, int *best, double *ms) {
             for (int rep = 0; rep < 3; rep++) {   // warm-up, then timed twice
                 ck(cudaEventRecord(e0, b->stream), "event");
                 for (const Launch &L : b->cycle)
-                    if (L.kind == Launch::FUSED) launch_one(b, L, b->stream);
+                    if (L.kind == Launch::RELAX || L.kind == Launch::FUSED) launch_one(b, L, b->stream);
                 ck(cudaEventRecord(e1, b->stream), "event");
             }
             ck(cudaEventSynchronize(e1), "sync");

@@ -1351,7 +1351,7 @@ __global__ void __launch_bounds__(NT, M == 1 ? 2 : 1)
         if (s < ns) rb_strip<T, SR, true>(v, out, st, z);   // uniform over the warp
         return;
     }
-    block2<T, NT, M>(J, v.u, out, z, (int)blockIdx.x - nsc, lambda, true);
+    block2<T, NT, M>(J, v.u, out, z, (int)blockIdx.x - nsc, lambda);
 }
 
 // the blocks, after the CTAs of the first ns strips (0: the blocks alone)

@@ -509,7 +509,8 @@ __device__ __forceinline__ void local_body(const LocalView<T> &J, const T *src, 
 // most), held in registers with its weights and h^2 f, so that it costs its
 // shared-memory reads, its sum and one barrier: the records are loaded at once
 // by the threads that use them (one round trip, before the wait for the
-// previous launch where `early`), then the values through them (another).
+// previous launch), then the values through them (another).  go: where given, a
+// flag read after the wait; 0: nothing is done.
 // Updated ghosts have two values, the ghost sweep reads one and writes the
 // other, so it takes one barrier instead of two.
 // Measured, the flower at 1025^2, a block's lists staged in shared memory by 512
@@ -518,7 +519,7 @@ __device__ __forceinline__ void local_body(const LocalView<T> &J, const T *src, 
 // -> 20 us, where the interior sweep and the blocks had been two launches.
 template <typename T, int NT, int M>
 __device__ __forceinline__ void block2(const Block2View<T> &J, const T *__restrict__ src, T *__restrict__ dst,
-                                       T *__restrict__ z, int c, int reps, bool early) {
+                                       T *__restrict__ z, int c, int reps, const int *go = nullptr) {
     constexpr int RP = M + 1, RN = 4 * M, RW = 2 * M;
     extern __shared__ __align__(16) unsigned char smem_dyn[];
     T *val = reinterpret_cast<T *>(smem_dyn);   // nodes, then two values a ghost
@@ -554,7 +555,8 @@ __device__ __forceinline__ void block2(const Block2View<T> &J, const T *__restri
 #pragma unroll
             for (int i = 0; i < 9; i++) w[k][i] = J.gw[(int64_t)i * J.ng + gb[k].w];
         }
-    if (early) pdl_wait();
+    pdl_wait();
+    if (go && !*go) return;   // uniform over the CTA
     T v[RN], fr[M], fb[M], fpr[RP], fpb[RP], gg[M], g0[M];
 #pragma unroll
     for (int k = 0; k < RN; k++)
@@ -1101,6 +1103,35 @@ __device__ __forceinline__ void prolong_node(const LevelView<T> &F, const LevelV
     else out[p] = val;
 }
 
+// 2D: the interpolation added at unknown k of row i: the parents' types, then
+// their values, loaded together (two round trips).  The sums of prolong_node.
+template <typename T>
+__device__ __forceinline__ void prolong_add2(const LevelView<T> &F, const LevelView<T> &C, const T *__restrict__ e,
+                                             T *__restrict__ out, int i, int k) {
+    const int64_t p = (int64_t)i * F.n + k, X0 = (int64_t)(i / 2) * C.s0 + k / 2;
+    const unsigned odd = (i & 1) << 1 | (k & 1);   // the axes along which the node has two parents
+    const T old = out[p];
+    unsigned use = 0;
+#pragma unroll
+    for (int s = 0; s < 4; s++)
+        if ((s & ~odd) == 0) {
+            const uint8_t kc = C.type[X0 + (s >> 1) * C.s0 + (s & 1)] & NODE_KIND;
+            use |= (unsigned)(kc == NODE_IN || kc == NODE_GHOST) << s;
+        }
+    T ev[4];
+#pragma unroll
+    for (int s = 0; s < 4; s++) ev[s] = (use >> s & 1u) ? e[X0 + (s >> 1) * C.s0 + (s & 1)] : (T)0;
+    T num = 0, den = 0;
+    const T w = (T)1 / (T)(1 << __popc(odd));   // a power of two: exact
+#pragma unroll
+    for (int s = 0; s < 4; s++)
+        if (use >> s & 1u) {
+            num += w * ev[s];
+            den += w;
+        }
+    out[p] = old + (den > (T)0 ? num / den : (T)0);
+}
+
 // --------------------------------------------------------------- coarsest
 // ---------------------------------------------------- exact junction solve
 // Defect of the equation of row k of the junction solve: at an inside node
@@ -1252,7 +1283,8 @@ __device__ __forceinline__ void js_apply_row_early(T *__restrict__ u, const int3
 template <typename T, int KJ>
 __device__ __forceinline__ void js_component_defects(const LevelView<T> &v, const T *__restrict__ z,
                                                      const int32_t *__restrict__ node,
-                                                     const int32_t *__restrict__ ghost, int m, int mi, T *rs) {
+                                                     const int32_t *__restrict__ ghost, int m, int mi, T *rs,
+                                                     const int *go = nullptr) {
     const int tid = threadIdx.x, nt = blockDim.x;
     const int shift = ((mi + 31) & ~31) - mi;   // thread index t: equation t (t < mi), then t - shift
     int32_t q[KJ], x[KJ][9];
@@ -1275,6 +1307,7 @@ __device__ __forceinline__ void js_component_defects(const LevelView<T> &v, cons
         }
     const int s0 = (int)v.s0;
     pdl_wait();
+    if (go && !*go) return;   // uniform over the CTA
     T y[KJ][9], b[KJ];
 #pragma unroll
     for (int k = 0; k < KJ; k++) {

@@ -1,0 +1,42 @@
+"""Batched solves in every form of the relaxation launch -- one and two records
+a thread, 512 threads (many extra sweeps: halos that cover the domain) -- with
+the exact junction solve and with junction sweeps: every domain equals the
+single-domain solver's solution to 1e-10 (the bound of test_gpu_batch.py)."""
+import numpy as np
+import pytest
+
+from helpers import rel_maxdiff
+from paper_1111_0983_gb300 import inputs
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("kw", [dict(), dict(lam=30), dict(lam=7, delta_over_h=6.0),
+                                dict(junction_solve=0, junction_sweeps=3, junction_radius=2.0)])
+def test_batch_equals_single(kw):
+    from paper_1111_0983_gb300 import gcmg
+    probs = [inputs.star(i, params=dict(inputs.star_params(i), n=n)) for i, n in ((0, 257), (1, 129), (5, 257))]
+    sizes = [P.meta["n"] for P in probs]
+
+    def data(S, P, n):
+        for l in range(S.nlev):
+            S.set_bc_types(l, P.bc_types(S.ghosts(l)["B"]))
+        G = S.ghosts(0)
+        g = P.g_values(G["B"], G["nu"], P.bc_types(G["B"]))
+        S.set_rhs(torch.from_numpy(P.f_grid(n)).cuda(), torch.from_numpy(g).cuda())
+
+    B = gcmg.Batch([P.phi_grid(n) for P, n in zip(probs, sizes)], 33, rtol=1e-11, max_cycles=200, **kw)
+    for S, P, n in zip(B.domains, probs, sizes):
+        data(S, P, n)
+    for _ in range(2):   # the second solve finds the first one's grids
+        stats, _ = B.solve()
+    assert all(s["converged"] for s in stats)
+    for k, (P, n) in enumerate(zip(probs, sizes)):
+        S = gcmg.Solver(P.phi_grid(n), 33, precision=1, rtol=1e-11, max_cycles=200, **kw)
+        data(S, P, n)
+        u = torch.zeros((n, n), dtype=torch.float64, device="cuda")
+        assert S.solve(u)["converged"]
+        ub = torch.zeros_like(u)
+        B.solution(k, ub)
+        assert rel_maxdiff(ub.cpu().numpy(), u.cpu().numpy(), (S.node_types(0) & 3) > 0) <= 1e-10
