@@ -52,9 +52,9 @@ constexpr int64_t kClusterWork = 65536;
 // phases of a relaxation as one cluster over distributed shared memory, larger
 // ones the junction zone alone.  Beyond, the 16 SMs' work a phase (and their
 // shared memory: 29 values a ghost) costs more than a launch saves.  A cycle of
-// the torus, launch a phase -> cluster: 33^3 173 -> 142 us, 65^3 376 -> 275,
-// 97^3 (two levels) 469 -> 316, FP64 65^3 746 -> 513; the zone alone on 129^3
-// and 257^3: 46 -> 21 and 52 -> 25 us a relaxation
+// the torus, launch a phase -> cluster: 33^3 173 -> 119 us, 65^3 376 -> 238,
+// 97^3 (two levels) 469 -> 306, FP64 65^3 746 -> 490; the zone alone on 129^3
+// and 257^3: 46 -> 15 and 52 -> 19 us a relaxation
 constexpr int64_t kC3Ghosts32 = 12000, kC3Ghosts64 = 6000;
 
 // Rows of the Kaczmarz comparison smoother on level l (2D): the ghosts and the

@@ -136,59 +136,142 @@ Cluster3Program build_cluster3(const HostLevel &L, bool band) {
         return 27;
     };
     auto is_ghost = [&](int64_t p) { return (L.type[p] & NODE_KIND) == NODE_GHOST; };
-    // order within a rank: inside (red, black; band only, both, zone only), then ghosts (zone ones last)
-    auto klass = [](const Node &x) {
-        if (x.q >= 0) return x.inzone ? 9 : 8;
-        return (x.black ? 3 : 0) + (x.inband ? (x.inzone ? 1 : 0) : 2);
-    };
+    // order of a rank's own nodes: inside, then ghosts (zone ones last)
+    auto klass = [](const Node &x) { return x.q < 0 ? 0 : x.inzone ? 2 : 1; };
     for (int r = 0; r < C3_RANKS; r++)
         std::sort(N.begin() + start[r], N.begin() + start[r + 1], [&](const Node &x, const Node &y) {
             const int a = klass(x), b = klass(y);
             return a != b ? a < b : x.p < y.p;
         });
+    struct Entry {
+        int32_t i;       // index in N
+        uint8_t band, zone;
+    };
     struct Rank {
         std::vector<int32_t> in, gs;   // slots -> node
-        int own_in = 0, own_g = 0;
-        int bound[11] = {};
+        std::vector<Entry> ent;        // own and halo entries, in sweep order
+        int own_in = 0, own_g = 0, zone_g = 0;
+        int hi[4] = {}, hg[3] = {};
+        int bound[7] = {};             // entries before (colour, class) 3 * colour + class
     };
     std::vector<Rank> R(C3_RANKS);
     std::vector<NodeMap> slot;         // per rank: node -> slot (inside or ghost)
-    // (slot, rank) pairs of the copies of an updated node, by its index in N
+    // (rank, slot) pairs of the copies of an updated node, by its index in N
     std::vector<std::vector<uint32_t>> cps(N.size());
     Cluster3Layout &y = out.lay;
     for (size_t i = 0; i < N.size(); i++) at.set(N[i].p, (int32_t)i);
     for (int r = 0; r < C3_RANKS; r++) {
         Rank &K = R[r];
-        slot.emplace_back(4 * (start[r + 1] - start[r]) + 16);
+        const int32_t b0 = (int32_t)start[r], e0 = (int32_t)start[r + 1];
+        slot.emplace_back(4 * (size_t)(e0 - b0) + 16);
         NodeMap &S = slot.back();
-        for (size_t i = start[r]; i < start[r + 1]; i++) {
+        for (int32_t i = b0; i < e0; i++) {
             std::vector<int32_t> &l = N[i].q >= 0 ? K.gs : K.in;
             S.set(N[i].p, (int32_t)l.size());
             l.push_back(N[i].p);
-            for (int k = klass(N[i]) + 1; k < 11; k++) K.bound[k]++;
+            K.zone_g += N[i].q >= 0 && N[i].inzone;
         }
         K.own_in = (int)K.in.size();
         K.own_g = (int)K.gs.size();
-        int64_t rd[27];
-        for (size_t i = start[r]; i < start[r + 1]; i++) {
-            const int m = reads(N[i], rd);
-            for (int k = 0; k < m; k++) {
-                if (S.get(rd[k], -1) >= 0) continue;
-                std::vector<int32_t> &l = is_ghost(rd[k]) ? K.gs : K.in;
-                S.set(rd[k], (int32_t)l.size());
-                l.push_back((int32_t)rd[k]);
-                const int32_t o = at.get(rd[k], -1);   // updated by another rank: a copy there
-                if (o >= 0) cps[o].push_back((uint32_t)r << 16 | (uint32_t)(l.size() - 1));
+        // the entries: a sweep's own nodes, the blacks its own ghosts read, the
+        // reds those blacks and ghosts read
+        NodeMap ent_of(2 * (size_t)(e0 - b0) + 16);   // node -> entry
+        auto entry = [&](int32_t i, bool zone) {
+            const int32_t k = ent_of.get(N[i].p, -1);
+            if (k >= 0) {
+                (zone ? K.ent[k].zone : K.ent[k].band) = 1;
+                return;
             }
+            ent_of.set(N[i].p, (int32_t)K.ent.size());
+            K.ent.push_back({i, (uint8_t)!zone, (uint8_t)zone});
+        };
+        int64_t rd[27];
+        for (int zone = band ? 0 : 1; zone < 2; zone++) {
+            auto in_sweep = [&](const Node &x) { return zone ? x.inzone != 0 : x.inband != 0; };
+            // inside nodes of one colour that the updates of `list` read
+            auto cone = [&](const std::vector<int32_t> &list, int black) {
+                for (int32_t i : list) {
+                    const int m = reads(N[i], rd);
+                    for (int k = 0; k < m; k++) {
+                        const int32_t o = at.get(rd[k], -1);
+                        if (o >= 0 && N[o].q < 0 && N[o].black == black && in_sweep(N[o])) entry(o, zone != 0);
+                    }
+                }
+            };
+            std::vector<int32_t> g, bl;
+            for (int32_t i = b0; i < e0; i++) {
+                if (!in_sweep(N[i])) continue;
+                if (N[i].q >= 0) g.push_back(i);
+                else entry(i, zone != 0);
+            }
+            cone(g, 1);
+            for (const Entry &x : K.ent)
+                if (N[x.i].black && (zone ? x.zone : x.band)) bl.push_back(x.i);
+            cone(bl, 0);
+            cone(g, 0);
         }
+        auto cls = [&](const Entry &x) { return 3 * (int)N[x.i].black + (x.band ? (x.zone ? 1 : 0) : 2); };
+        std::sort(K.ent.begin(), K.ent.end(), [&](const Entry &x, const Entry &z) {
+            return cls(x) != cls(z) ? cls(x) < cls(z) : N[x.i].p < N[z.i].p;
+        });
+        for (const Entry &x : K.ent)
+            for (int k = cls(x) + 1; k < 7; k++) K.bound[k]++;
+        // every other node the updates touch: halo (updated by another rank) or read only
+        std::vector<int32_t> halo_in, halo_g, fixed_in, fixed_g;
+        auto touch = [&](int64_t p) {
+            if (S.get(p, -1) >= 0) return;
+            S.set(p, 0);   // seen; numbered below
+            const bool upd = at.get(p, -1) >= 0;
+            if (is_ghost(p)) (upd ? halo_g : fixed_g).push_back((int32_t)p);
+            else (upd ? halo_in : fixed_in).push_back((int32_t)p);
+        };
+        for (const Entry &x : K.ent) {
+            touch(N[x.i].p);
+            const int m = reads(N[x.i], rd);
+            for (int k = 0; k < m; k++) touch(rd[k]);
+        }
+        for (int32_t i = b0; i < e0; i++)
+            if (N[i].q >= 0) {
+                const int m = reads(N[i], rd);
+                for (int k = 0; k < m; k++) touch(rd[k]);
+            }
+        auto group = [&](int32_t p) {   // band only, both, zone only
+            const Node &x = N[at.get(p, -1)];
+            return x.inband ? (x.inzone ? 1 : 0) : 2;
+        };
+        auto by_group = [&](int32_t a, int32_t c) { return group(a) != group(c) ? group(a) < group(c) : a < c; };
+        std::sort(halo_in.begin(), halo_in.end(), by_group);
+        std::sort(halo_g.begin(), halo_g.end(), by_group);
+        K.hi[0] = K.hi[1] = K.hi[2] = K.hi[3] = K.own_in;
+        for (int32_t p : halo_in)
+            for (int k = group(p) + 1; k < 4; k++) K.hi[k]++;
+        K.hg[0] = K.hg[1] = K.own_g;
+        K.hg[2] = K.own_g + (int)halo_g.size();
+        for (int32_t p : halo_g) K.hg[1] += group(p) == 0;
+        for (const auto *l : {&halo_in, &fixed_in})
+            for (int32_t p : *l) {
+                S.set(p, (int32_t)K.in.size());
+                K.in.push_back(p);
+            }
+        for (const auto *l : {&halo_g, &fixed_g})
+            for (int32_t p : *l) {
+                S.set(p, (int32_t)K.gs.size());
+                K.gs.push_back(p);
+            }
         y.max_in = std::max(y.max_in, (int)K.in.size());
         y.max_gs = std::max(y.max_gs, (int)K.gs.size());
-        y.max_e = std::max(y.max_e, K.own_in);
+        y.max_e = std::max(y.max_e, (int)K.ent.size());
         y.max_g = std::max(y.max_g, K.own_g);
     }
     y.max_in = (y.max_in + 3) & ~3;
     y.max_gs = (y.max_gs + 3) & ~3;
     if (y.max_in + y.max_gs >= 0x8000) return out;
+    for (int r = 0; r < C3_RANKS; r++) {   // the halo slots are copies of other ranks' nodes
+        const Rank &K = R[r];
+        for (int i = K.own_in; i < K.hi[3]; i++) cps[at.get(K.in[i], -1)].push_back((uint32_t)r << 16 | (uint32_t)i);
+        for (int i = K.own_g; i < K.hg[2]; i++)
+            cps[at.get(K.gs[i], -1)].push_back((uint32_t)r << 16 | (uint32_t)(y.max_in + i));
+    }
     int max_c = 0;
     for (int r = 0; r < C3_RANKS; r++) {
         int nc = 0;
@@ -211,6 +294,7 @@ Cluster3Program build_cluster3(const HostLevel &L, bool band) {
         h[C3_NGS] = (int)K.gs.size();
         h[C3_OWN_IN] = K.own_in;
         h[C3_OWN_G] = K.own_g;
+        h[C3_NE] = (int)K.ent.size();
         h[C3_RB0] = K.bound[0];
         h[C3_RB1] = K.bound[2];
         h[C3_RZ0] = K.bound[1];
@@ -219,7 +303,9 @@ Cluster3Program build_cluster3(const HostLevel &L, bool band) {
         h[C3_BB1] = K.bound[5];
         h[C3_BZ0] = K.bound[4];
         h[C3_BZ1] = K.bound[6];
-        h[C3_GZ] = K.bound[9] - K.bound[8];
+        h[C3_GZ] = K.own_g - K.zone_g;
+        for (int k = 0; k < 4; k++) h[C3_HI0 + k] = K.hi[k];
+        for (int k = 0; k < 3; k++) h[C3_HG0 + k] = K.hg[k];
         int32_t *ln = reinterpret_cast<int32_t *>(rec + y.lnode);
         std::copy(K.in.begin(), K.in.end(), ln);
         std::copy(K.gs.begin(), K.gs.end(), ln + y.max_in);
@@ -227,33 +313,37 @@ Cluster3Program build_cluster3(const HostLevel &L, bool band) {
         int32_t *gq = reinterpret_cast<int32_t *>(rec + y.gq);
         uint16_t *gst = reinterpret_cast<uint16_t *>(rec + y.gst);
         uint32_t *cp = reinterpret_cast<uint32_t *>(rec + y.copies);
-        int nc = 0, ie = 0, ig = 0;
+        int nc = 0;
         int64_t rd[27];
-        for (size_t i = start[r]; i < start[r + 1]; i++) {
+        auto copies_of = [&](int32_t i) {   // only this rank's own nodes are sent
             uint16_t first = 0xffff;
-            if (!cps[i].empty()) {
+            if (i >= (int32_t)start[r] && i < (int32_t)start[r + 1] && !cps[i].empty()) {
                 first = (uint16_t)nc;
                 for (uint32_t c : cps[i]) cp[nc++] = c;
                 cp[nc - 1] |= 0x80000000u;
             }
-            const int m = reads(N[i], rd);
-            uint16_t src[27];
-            for (int k = 0; k < m; k++) {
-                const int s = slot[r].get(rd[k], -1);
-                src[k] = (uint16_t)(is_ghost(rd[k]) ? 0x8000 | (y.max_in + s) : s);
-            }
-            if (N[i].q < 0) {
-                uint16_t *e = ent + 8 * ie;
-                e[0] = (uint16_t)ie;   // an own inside entry's slot is its number
-                for (int k = 0; k < 6; k++) e[1 + k] = src[k];
-                e[7] = first;
-                ie++;
-            } else {
-                gq[ig] = N[i].q;
-                for (int k = 0; k < 28; k++)
-                    gst[((size_t)(k / 8) * y.max_g + ig) * 8 + k % 8] = k < 27 ? src[k] : first;
-                ig++;
-            }
+            return first;
+        };
+        auto source = [&](int64_t p) {
+            const int s = slot[r].get(p, -1);
+            return (uint16_t)(is_ghost(p) ? 0x8000 | (y.max_in + s) : s);
+        };
+        for (size_t k = 0; k < K.ent.size(); k++) {
+            const Node &x = N[K.ent[k].i];
+            uint16_t *e = ent + 8 * k;
+            e[0] = source(x.p);
+            reads(x, rd);
+            for (int a = 0; a < 6; a++) e[1 + a] = source(rd[a]);
+            e[7] = copies_of(K.ent[k].i);
+        }
+        int ig = 0;
+        for (int32_t i = (int32_t)start[r]; i < (int32_t)start[r + 1]; i++) {
+            if (N[i].q < 0) continue;
+            gq[ig] = N[i].q;
+            reads(N[i], rd);
+            for (int k = 0; k < 28; k++)
+                gst[((size_t)(k / 8) * y.max_g + ig) * 8 + k % 8] = k < 27 ? source(rd[k]) : copies_of(i);
+            ig++;
         }
     }
     return out;

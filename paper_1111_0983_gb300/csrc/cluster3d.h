@@ -12,32 +12,39 @@
 namespace gcmg {
 
 constexpr int C3_RANKS = 16;      // CTAs of the cluster
-constexpr int C3_THREADS = 512;
+constexpr int C3_THREADS = 512;   // of a CTA, at most
 
-// Header of a rank's record: counts and list bounds (ints).  Inside entries
-// are ordered by colour, within a colour band only | band and zone | zone
-// only, so that a band sweep and a zone sweep each take one range.
+// Header of a rank's record: counts and list bounds (ints).  A sweep (red,
+// black, ghosts) runs in a rank without waiting for the others: besides its own
+// nodes it updates the inside nodes of other ranks that its own updates of the
+// same sweep read (halo entries).  Entries are ordered by colour, within a colour
+// band sweep only | both | zone sweep only, so that a sweep takes one range.
 enum {
-    C3_NIN,                   // inside slots (own updated nodes first)
-    C3_NGS,                   // ghost slots (own updated ghosts first)
-    C3_OWN_IN, C3_OWN_G,      // updated nodes of this rank, written back
+    C3_NIN,                   // inside slots: own, halo, read only
+    C3_NGS,                   // ghost slots: own, halo, read only
+    C3_OWN_IN, C3_OWN_G,      // own nodes, written back
+    C3_NE,                    // inside entries
     C3_RB0, C3_RB1,           // red entries of a band sweep
     C3_RZ0, C3_RZ1,           // red entries of a zone sweep
     C3_BB0, C3_BB1, C3_BZ0, C3_BZ1,   // black
     C3_GZ,                    // first zone ghost among the own ghosts
-    C3_HDR = 16
+    // halo slots, refreshed after a sweep: inside band only from HI0 on, both
+    // from HI1, zone only from HI2, end HI3; ghosts off the zone from HG0, in the
+    // zone from HG1, end HG2
+    C3_HI0, C3_HI1, C3_HI2, C3_HI3, C3_HG0, C3_HG1, C3_HG2,
+    C3_HDR = 24
 };
 
 // The partition of the updated nodes over the cluster's ranks.  Every rank
 // has a record of `stride` bytes with the same section offsets:
 //   ints    header
 //   lnode   int32 per slot: global node (inside slots, then ghost slots)
-//   ent     8 x uint16 per inside entry: own slot, 6 sources in the order of
+//   ent     8 x uint16 per inside entry: its slot, 6 sources in the order of
 //           the sweeps' sum, first copy (0xffff: none)
 //   gq      int32 per own ghost: ghost number
 //   gst     4 x max_g x 8 uint16: the 27 stencil sources, first copy
-//   copies  uint32: rank << 16 | slot, bit 31 = last; where the entry's value
-//           is also kept (the ranks that read it)
+//   copies  uint32: rank << 16 | slot (ghosts: max_in + ghost slot), bit 31 =
+//           last; the halo slots of other ranks that hold the entry's value
 // A source is an inside slot, or 0x8000 | (max_in + ghost slot).
 struct Cluster3Layout {
     int stride = 0, lnode = 0, ent = 0, gq = 0, gst = 0, copies = 0;   // bytes

@@ -1,8 +1,9 @@
 // Test program (built and run by tests/test_cluster3.py, host only): the 3D
 // cluster programs of a torus, phase by phase as the kernel runs them, against
 // the same sweeps over the level's lists on the global grid.  Prints one line
-// "name failures count" per check: values (bitwise), reads of something
-// written in the same phase (a race between two barriers), bounds.
+// "name failures count" per check: values (bitwise), copies that nobody sent,
+// reads of something written in the same phase (a race between two block
+// barriers), bounds.
 #include <cmath>
 #include <cstdio>
 #include <cstdlib>
@@ -17,18 +18,17 @@ struct Rank {
     const int32_t *h, *lnode, *gq;
     const uint16_t *ent, *gst;
     const uint32_t *copies;
-    std::vector<double> val;
-    std::vector<uint8_t> wrote;   // in the current phase
+    std::vector<double> val, inbox[2];
 };
 
-static long race = 0, bounds = 0;
+static long race = 0, bounds = 0, stale = 0;
 
 struct Program {
     const HostLevel &L;
     const Cluster3Program &P;
     const std::vector<double> &f, &g;
     std::vector<Rank> R;
-    int par = 0;
+    int par = 0, in = 0;
     Program(const HostLevel &l, const Cluster3Program &p, const std::vector<double> &u, const std::vector<double> &f_,
             const std::vector<double> &g_)
         : L(l), P(p), f(f_), g(g_), R(C3_RANKS) {
@@ -43,100 +43,111 @@ struct Program {
             K.gst = (const uint16_t *)(rec + y.gst);
             K.copies = (const uint32_t *)(rec + y.copies);
             K.val.assign(y.max_in + 2 * y.max_gs, NAN);
-            K.wrote.assign(K.val.size(), 0);
-            if (K.h[C3_NIN] > y.max_in || K.h[C3_NGS] > y.max_gs || K.h[C3_OWN_IN] > y.max_e || K.h[C3_OWN_G] > y.max_g)
+            for (auto &b : K.inbox) b.assign(y.max_in + y.max_gs, NAN);
+            if (K.h[C3_NIN] > y.max_in || K.h[C3_NGS] > y.max_gs || K.h[C3_NE] > y.max_e || K.h[C3_OWN_G] > y.max_g ||
+                K.h[C3_HI3] > K.h[C3_NIN] || K.h[C3_HG2] > K.h[C3_NGS] || K.h[C3_OWN_IN] > K.h[C3_HI0])
                 bounds++;
             for (int i = 0; i < K.h[C3_NIN]; i++) K.val[i] = u[K.lnode[i]];
             for (int i = 0; i < K.h[C3_NGS]; i++)
                 K.val[y.max_in + i] = K.val[y.max_in + y.max_gs + i] = u[K.lnode[y.max_in + i]];
         }
     }
-    double rd(Rank &K, unsigned s) {
+    // one rank's phase between two block barriers: what it reads must not be what it writes
+    std::vector<size_t> reads;
+    std::vector<std::pair<size_t, double>> writes;
+    double get(Rank &K, unsigned s) {
         const size_t a = (s & 0x7fffu) + ((s >> 15) ? (size_t)par * P.lay.max_gs : 0);
         if (a >= K.val.size()) { bounds++; return NAN; }
-        if (K.wrote[a]) race++;
+        reads.push_back(a);
         return K.val[a];
     }
-    struct Write { int rank; size_t a; double x; };
-    std::vector<Write> writes;
-    void put(int r, size_t a, double x) {
-        if (r >= C3_RANKS || a >= R[r].val.size()) { bounds++; return; }
-        writes.push_back({r, a, x});
+    void put(Rank &K, size_t a, double x) {
+        if (a >= K.val.size()) { bounds++; return; }
+        writes.push_back({a, x});
     }
-    void send(Rank &K, unsigned first, size_t add, double x) {
+    void block_barrier(Rank &K) {
+        std::vector<uint8_t> wrote(K.val.size(), 0);
+        for (auto &w : writes) { if (wrote[w.first]++) race++; K.val[w.first] = w.second; }
+        for (size_t a : reads) if (wrote[a]) race++;
+        reads.clear();
+        writes.clear();
+    }
+    void send(Rank &K, unsigned first, double x) {
         if (first == 0xffff) return;
         for (unsigned c = first;; c++) {
             if ((uint8_t *)(K.copies + c + 1) > (uint8_t *)K.h + P.lay.stride) { bounds++; return; }
             const uint32_t w = K.copies[c];
-            put((int)((w >> 16) & 0x7fff), (w & 0xffff) + add, x);
+            const int r = (int)((w >> 16) & 0x7fff);
+            if (r >= C3_RANKS || (w & 0xffff) >= R[r].inbox[0].size()) { bounds++; return; }
+            R[r].inbox[in][w & 0xffff] = x;
             if (w >> 31) break;
         }
     }
-    // a barrier: the phase's writes become visible; whatever it read must not be among them
-    std::vector<std::pair<int, size_t>> reads;
-    void barrier() {
-        for (const Write &w : writes) {
-            R[w.rank].wrote[w.a]++;
-            R[w.rank].val[w.a] = w.x;
+    void inside(Rank &K, int lo, int hi) {
+        for (int e = K.h[lo]; e < K.h[hi]; e++) {
+            const uint16_t *q = K.ent + 8 * e;
+            double nb = get(K, q[1]) + get(K, q[2]) + get(K, q[3]) + get(K, q[4]);
+            nb += get(K, q[5]) + get(K, q[6]);
+            const double x = (L.h * L.h * f[K.lnode[q[0]]] + nb) * (1.0 / 6.0);
+            put(K, q[0], x);
+            send(K, q[7], x);
         }
-        for (const auto &q : reads)
-            if (R[q.first].wrote[q.second]) race++;
-        for (const Write &w : writes) R[w.rank].wrote[w.a] = 0;
-        writes.clear();
-        reads.clear();
+        block_barrier(K);
     }
-    double get(int r, unsigned s) {
-        reads.push_back({r, (s & 0x7fffu) + ((s >> 15) ? (size_t)par * P.lay.max_gs : 0)});
-        return rd(R[r], s);
-    }
-    void inside(int lo, int hi) {
-        for (int r = 0; r < C3_RANKS; r++) {
-            Rank &K = R[r];
-            for (int e = K.h[lo]; e < K.h[hi]; e++) {
-                const uint16_t *q = K.ent + 8 * e;
-                double nb = get(r, q[1]) + get(r, q[2]) + get(r, q[3]) + get(r, q[4]);
-                nb += get(r, q[5]) + get(r, q[6]);
-                const double x = (L.h * L.h * f[K.lnode[e]] + nb) * (1.0 / 6.0);
-                put(r, q[0], x);
-                send(K, q[7], 0, x);
-            }
-        }
-        barrier();
-    }
-    void ghosts(bool zone) {
+    void ghosts(Rank &K, bool zone) {
         const Cluster3Layout &y = P.lay;
         const size_t po = (size_t)(1 - par) * y.max_gs;
-        for (int r = 0; r < C3_RANKS; r++) {
-            Rank &K = R[r];
-            for (int e = zone ? K.h[C3_GZ] : 0; e < K.h[C3_OWN_G]; e++) {
-                auto src = [&](int k) { return K.gst[((size_t)(k / 8) * y.max_g + e) * 8 + k % 8]; };
-                const int64_t q = K.gq[e];
-                double s = 0;
-                for (int k = 0; k < 27; k++) s += L.wD[q * KMAX + k] * get(r, src(k));
-                const double x = get(r, 0x8000u | (unsigned)(y.max_in + e)) + 0.9 * (g[q] - s);
-                put(r, y.max_in + po + e, x);
-                send(K, src(27), y.max_in + po, x);
-            }
+        for (int e = zone ? K.h[C3_GZ] : 0; e < K.h[C3_OWN_G]; e++) {
+            auto src = [&](int k) { return K.gst[((size_t)(k / 8) * y.max_g + e) * 8 + k % 8]; };
+            const int64_t q = K.gq[e];
+            double s = 0;
+            for (int k = 0; k < 27; k++) s += L.wD[q * KMAX + k] * get(K, src(k));
+            const double x = get(K, 0x8000u | (unsigned)(y.max_in + e)) + 0.9 * (g[q] - s);
+            put(K, y.max_in + po + e, x);
+            send(K, src(27), x);
         }
-        barrier();
+        block_barrier(K);
+    }
+    void refresh(int i0, int i1, int g0, int g1) {   // header fields; -1: nothing
+        const Cluster3Layout &y = P.lay;
         par ^= 1;
+        for (Rank &K : R) {
+            for (int i = i0 < 0 ? 0 : K.h[i0]; i < (i0 < 0 ? 0 : K.h[i1]); i++) {
+                if (K.inbox[in][i] != K.inbox[in][i]) stale++;   // nobody sent it in this sweep
+                K.val[i] = K.inbox[in][i];
+            }
+            for (int i = K.h[g0]; i < K.h[g1]; i++) {
+                if (K.inbox[in][y.max_in + i] != K.inbox[in][y.max_in + i]) stale++;
+                K.val[y.max_in + par * y.max_gs + i] = K.inbox[in][y.max_in + i];
+            }
+            K.inbox[in].assign(y.max_in + y.max_gs, NAN);
+        }
+        in ^= 1;
     }
     void run(bool lead, int lambda, int mu) {
         const Cluster3Layout &y = P.lay;
-        if (lead) ghosts(false);
+        if (lead) {
+            for (Rank &K : R) ghosts(K, false);
+            refresh(-1, -1, C3_HG0, C3_HG2);
+        }
         for (int k = 0; k < lambda; k++) {
-            inside(C3_RB0, C3_RB1);
-            inside(C3_BB0, C3_BB1);
-            ghosts(false);
+            for (Rank &K : R) {
+                inside(K, C3_RB0, C3_RB1);
+                inside(K, C3_BB0, C3_BB1);
+                ghosts(K, false);
+            }
+            refresh(C3_HI0, C3_HI2, C3_HG0, C3_HG2);
         }
         for (int k = 0; k < mu; k++) {
-            if (k == 0 && P.band)
-                for (int r = 0; r < C3_RANKS; r++)
-                    for (int i = 0; i < R[r].h[C3_NGS]; i++)
-                        put(r, y.max_in + (par ^ 1) * y.max_gs + i, R[r].val[y.max_in + par * y.max_gs + i]);
-            inside(C3_RZ0, C3_RZ1);
-            inside(C3_BZ0, C3_BZ1);
-            ghosts(P.band);
+            for (Rank &K : R) {
+                if (k == 0 && P.band)
+                    for (int i = 0; i < K.h[C3_NGS]; i++)
+                        put(K, y.max_in + (par ^ 1) * y.max_gs + i, K.val[y.max_in + par * y.max_gs + i]);
+                inside(K, C3_RZ0, C3_RZ1);
+                inside(K, C3_BZ0, C3_BZ1);
+                ghosts(K, P.band);
+            }
+            refresh(C3_HI1, C3_HI3, C3_HG1, C3_HG2);
         }
     }
 };
@@ -224,6 +235,7 @@ int main(int argc, char **argv) {
             }
         }
     }
+    report("stale", stale, 1);
     report("race", race, 1);
     report("bounds", bounds, 1);
     return fails ? 1 : 0;

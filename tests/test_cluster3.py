@@ -1,9 +1,10 @@
 """The 3D cluster programs (csrc/cluster3d.cpp), without a GPU: the host code
 is compiled with g++ together with cluster3_check.cpp, which runs the phases
-of every level's program rank by rank -- own values, copies sent to the other
-ranks, two values a ghost -- and compares them bitwise with the same sweeps
-over the level's lists; a phase reads nothing that it writes (the barriers
-suffice), and every index stays in its section.  Levels from 9^3 (a few nodes
+of every level's program rank by rank -- a whole sweep each, own values sent into
+the other ranks' inboxes, two values a ghost -- and compares them bitwise with
+the same sweeps over the level's lists; a phase reads nothing that it writes,
+every copy is sent in the sweep that changes it, and every index stays in its
+section.  Levels from 9^3 (a few nodes
 a rank) up, with and without a junction zone, sizes off powers of two."""
 import os
 import shutil
@@ -32,5 +33,5 @@ def test_cluster_programs_equal_the_list_sweeps(checker, n, nc):
     rows = [ln.split() for ln in out.stdout.splitlines()]
     assert rows and out.returncode == 0, out.stdout + out.stderr
     assert all(int(r[1]) == 0 for r in rows), rows
-    assert {r[0] for r in rows} >= {"band_and_zone", "zone", "race", "bounds"}
+    assert {r[0] for r in rows} >= {"band_and_zone", "zone", "stale", "race", "bounds"}
     assert all(int(r[2]) > 0 for r in rows), rows
