@@ -49,13 +49,21 @@ int kslots(int dim) { return dim == 2 ? 9 : 27; }
 constexpr int64_t kClusterWork = 65536;
 
 // 3D levels with at most this many ghosts (FP32 / FP64 cycles) run all boundary
-// phases of a relaxation as one cluster over distributed shared memory, larger
-// ones the junction zone alone.  Beyond, the 16 SMs' work a phase (and their
-// shared memory: 29 values a ghost) costs more than a launch saves.  A cycle of
-// the torus, launch a phase -> cluster: 33^3 173 -> 119 us, 65^3 376 -> 238,
-// 97^3 (two levels) 469 -> 306, FP64 65^3 746 -> 490; the zone alone on 129^3
-// and 257^3: 46 -> 15 and 52 -> 19 us a relaxation
-constexpr int64_t kC3Ghosts32 = 12000, kC3Ghosts64 = 6000;
+// phases of a relaxation as one cluster over distributed shared memory; larger
+// ones the junction zone alone, and the band a launch a sweep.  A cycle of the
+// torus, launch a phase -> cluster: 33^3 173 -> 119 us, 65^3 376 -> 238, FP64
+// 65^3 746 -> 490; the zone alone on 129^3 and 257^3: 46 -> 15 and 52 -> 19 us a
+// relaxation.  Where the line lies, cluster against a launch a sweep: FP32
+// 65^3 (4,532 ghosts) 242 and 242, 81^3 (7,000) 260 and 249, 97^3 (9,972) 308
+// and 263; FP64 49^3 (2,568) 251 and 255, 65^3 497 and 466
+constexpr int64_t kC3Ghosts32 = 6000, kC3Ghosts64 = 4000;
+// Larger levels: ghosts a block of the band sweeps, and at least three blocks
+// an SM in FP32, two in FP64 (fewer leave the SM waiting in a block's barriers,
+// more repeat more of each other's nodes).  Measured, us a cycle against a
+// launch a phase: FP32 129^3 448 -> 393 (2 blocks an SM 400, 4: 391, 6: 425),
+// 257^3 861 -> 720 (747, 721, 786), 385^3 1353 -> 1268 (115 ghosts 1328, 345:
+// 1468); FP64 129^3 847 -> 800 (3: 800, 4: 860).
+constexpr int64_t kS3Ghosts = 230;
 
 // Rows of the Kaczmarz comparison smoother on level l (2D): the ghosts and the
 // inside nodes of the band, grouped by the colour (i mod 5) + 5 (j mod 5) of
@@ -462,9 +470,8 @@ T *relax(gcmg_ctx *c, LevelView<T> v, T *out, T *wb, int l, bool extra) {
         bool done = false, zdone = false;
         // mode 0: the cluster program of the level, if it has one
         const Cluster3Dev *C3 = nullptr;
-        if (dim == 3 && extra && c->p.smoother == 0 && !c->coop3d && !c->cluster3d && !c->junction_blocks &&
-            c->c3[l].records && (sizeof(T) == 4 ? c->c3[l].fits32 : c->c3[l].fits64))
-            C3 = &c->c3[l];
+        const bool mode0 = dim == 3 && extra && c->p.smoother == 0 && !c->coop3d && !c->cluster3d && !c->junction_blocks;
+        if (mode0 && c->c3[l].records && (sizeof(T) == 4 ? c->c3[l].fits32 : c->c3[l].fits64)) C3 = &c->c3[l];
         const int mu = !c->p.junction_solve && g.jz.ncomp > 0 ? c->p.junction_sweeps : 0;
         if (C3 && C3->band) {
             timer_mark(c, GCMG_KERNEL_BOUNDARY, l);
@@ -520,7 +527,11 @@ T *relax(gcmg_ctx *c, LevelView<T> v, T *out, T *wb, int l, bool extra) {
             const bool zmerge = !zcluster && !c->p.junction_solve && c->p.junction_sweeps > 0 && g.jz.ncomp > 0 &&
                                 !jz_smem && g.jz.zred_src;
             launch_ghost_new<T>(v, nullptr, g.ng, c->stream);
-            for (int k = 0; k < c->p.lambda; k++) {
+            // a launch a sweep where the level has blocks for it in this precision
+            const bool sweeps = mode0 && !zmerge && c->s3[l].records && c->p.lambda >= 2 &&
+                                (sizeof(T) == 4) == (c->p.precision == 1);
+            if (sweeps) launch_sweep3<T>(v, c->s3[l], c->p.lambda, c->stream);
+            for (int k = 0; k < (sweeps ? 0 : c->p.lambda); k++) {
                 launch_rb_list_store<T>(v, g.red, g.red_src, g.nred, nullptr, g.ng, c->stream);
                 launch_rb_list<T>(v, dim, g.black, g.nblack, c->stream);
                 launch_ghost_new<T>(v, nullptr, g.ng, c->stream);
@@ -536,7 +547,7 @@ T *relax(gcmg_ctx *c, LevelView<T> v, T *out, T *wb, int l, bool extra) {
                 launch_ghost_store<T>(v, g.jz.zghost, g.jz.nzghost, c->stream);
                 return v.u;
             }
-            launch_ghost_store<T>(v, nullptr, g.ng, c->stream);
+            if (!sweeps) launch_ghost_store<T>(v, nullptr, g.ng, c->stream);
             if (zcluster) {
                 launch_cluster3<T>(v, *C3, false, 0, mu, c->stream);
                 return v.u;
@@ -593,6 +604,27 @@ void check_program_fits(gcmg_ctx *c, LocalDev &z) {
     // the attribute is per kernel: allow the device maximum once for all levels
     local_prepare<double>(c->p.dim, (size_t)dev_max);
     local_prepare<float>(c->p.dim, (size_t)dev_max);
+}
+
+// builds level l's band-sweep blocks (3D) where the cluster does not take them
+void build_sweep3_dev(gcmg_ctx *c, int l) {
+    if (c->p.dim != 3) return;
+    if (c->s3.empty()) c->s3.resize(c->H.size());
+    const HostLevel &L = c->H[l];
+    const bool f32 = c->p.precision == 1;
+    if (L.ng() <= (f32 ? kC3Ghosts32 : kC3Ghosts64) || c->p.lambda < 2) return;
+    int sms = 1;
+    ck(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device), "attr");
+    const int blocks = (int)std::max<int64_t>((f32 ? 3 : 2) * sms, (L.ng() + kS3Ghosts - 1) / kS3Ghosts);
+    const Sweep3Program P = build_sweep3(L, blocks);
+    if (P.records.empty() || !(f32 ? sweep3_fits<float>(P.lay, c->device) : sweep3_fits<double>(P.lay, c->device))) return;
+    Sweep3Dev &d = c->s3[l];
+    d.lay = P.lay;
+    d.records = upload<uint8_t>(c, P.records.data(), P.records.size());
+    const size_t sz = f32 ? sizeof(float) : sizeof(double);
+    for (void *&x : d.x) x = dalloc<uint8_t>(c, sz * (size_t)P.lay.inside);
+    d.g = dalloc<uint8_t>(c, sz * (size_t)L.ng());
+    ck(cudaStreamSynchronize(c->stream), "sync");   // the host records die at return
 }
 
 // (re)builds level l's cluster program (3D) for its current junction zone: the
@@ -965,7 +997,10 @@ gcmg_status create_from_levels(const gcmg_params &q, std::vector<HostLevel> &&H,
             c->D32.resize(nl);
             for (int l = 0; l < nl; l++) alloc_data<float>(c, l, c->D32[l], true);
         }
-        for (int l = 0; l < nl; l++) update_cluster3(c, l);
+        for (int l = 0; l < nl; l++) {
+            update_cluster3(c, l);
+            build_sweep3_dev(c, l);
+        }
         c->d_norm = dalloc<unsigned long long>(c, 2);
         c->d_rel = dalloc<double>(c, 257);
         c->d_r0 = dalloc<double>(c, 2);   // r0, the last relative residual

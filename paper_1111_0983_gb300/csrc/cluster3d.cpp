@@ -3,7 +3,9 @@
 #include "cluster3d.h"
 
 #include <algorithm>
+#include <atomic>
 #include <cstring>
+#include <thread>
 
 namespace gcmg {
 
@@ -53,8 +55,9 @@ struct Node {
 };
 
 // splits nodes [b, e) into `parts` ranges of about equal weight by cutting the
-// longest axis of their box at the weighted median, again and again
-void bisect(std::vector<Node> &N, size_t b, size_t e, int parts, int first, std::vector<size_t> &start) {
+// longest axis of their box at the weighted share, again and again
+void bisect(std::vector<Node> &N, std::vector<Node> &tmp, size_t b, size_t e, int parts, int first,
+            std::vector<size_t> &start) {
     if (parts == 1) {
         start[first] = b;
         return;
@@ -70,15 +73,19 @@ void bisect(std::vector<Node> &N, size_t b, size_t e, int parts, int first, std:
         if (hi[a] - lo[a] > hi[ax] - lo[ax]) ax = a;
     // a ghost's update reads 27 values, an inside node's 7
     auto weight = [](const Node &x) { return x.q >= 0 ? 4 : 1; };
-    std::sort(N.begin() + b, N.begin() + e, [ax](const Node &x, const Node &y) {
-        return x.c[ax] != y.c[ax] ? x.c[ax] < y.c[ax] : x.p < y.p;
-    });
     int64_t total = 0, run = 0;
-    for (size_t i = b; i < e; i++) total += weight(N[i]);
+    std::vector<size_t> at(e > b ? hi[ax] - lo[ax] + 2 : 1, 0);   // counting sort along the axis
+    for (size_t i = b; i < e; i++) {
+        at[N[i].c[ax] - lo[ax] + 1]++;
+        total += weight(N[i]);
+    }
+    for (size_t k = 1; k < at.size(); k++) at[k] += at[k - 1];
+    for (size_t i = b; i < e; i++) tmp[b + at[N[i].c[ax] - lo[ax]]++] = N[i];
+    std::copy(tmp.begin() + b, tmp.begin() + e, N.begin() + b);
     size_t m = b;
-    while (m < e && 2 * run < total) run += weight(N[m++]);
-    bisect(N, b, m, parts / 2, first, start);
-    bisect(N, m, e, parts - parts / 2, first + parts / 2, start);
+    while (m < e && parts * run < total * (parts / 2)) run += weight(N[m++]);
+    bisect(N, tmp, b, m, parts / 2, first, start);
+    bisect(N, tmp, m, e, parts - parts / 2, first + parts / 2, start);
 }
 
 int align16(int x) { return (x + 15) & ~15; }
@@ -122,7 +129,8 @@ Cluster3Program build_cluster3(const HostLevel &L, bool band) {
     for (int32_t q : Z.zghost) add(L.ghost_node[q], q, false, true);
     if (N.empty()) return out;
     std::vector<size_t> start(C3_RANKS + 1, N.size());
-    bisect(N, 0, N.size(), C3_RANKS, 0, start);
+    std::vector<Node> tmp(N.size());
+    bisect(N, tmp, 0, N.size(), C3_RANKS, 0, start);
     auto reads = [&](const Node &x, int64_t *rd) {
         if (x.q < 0) {   // the order of the sweeps' sum: axis 2, axis 0, axis 1
             const int64_t s[3] = {L.stride[2], L.stride[0], L.stride[1]};
@@ -346,6 +354,191 @@ Cluster3Program build_cluster3(const HostLevel &L, bool band) {
             ig++;
         }
     }
+    return out;
+}
+
+Sweep3Program build_sweep3(const HostLevel &L, int blocks) {
+    Sweep3Program out;
+    if (L.dim != 3 || blocks < 1) return out;
+    std::vector<Node> N;
+    N.reserve(L.band_red.size() + L.band_black.size() + L.ghost_node.size());
+    auto add = [&](int64_t p, int32_t q) {
+        Node x;
+        x.p = (int32_t)p;
+        x.q = q;
+        x.c[0] = (int)(p / L.stride[0]);
+        x.c[1] = (int)(p % L.stride[0] / L.stride[1]);
+        x.c[2] = (int)(p % L.stride[1]);
+        x.black = (x.c[0] + x.c[1] + x.c[2]) & 1;
+        x.inband = 1;
+        x.inzone = 0;
+        N.push_back(x);
+    };
+    for (int32_t p : L.band_red) add(p, -1);
+    for (int32_t p : L.band_black) add(p, -1);
+    for (int64_t q = 0; q < L.ng(); q++) add(L.ghost_node[q], (int32_t)q);
+    if (N.empty()) return out;
+    std::vector<size_t> start(blocks + 1, N.size());
+    std::vector<Node> tmp(N.size());
+    bisect(N, tmp, 0, N.size(), blocks, 0, start);
+    NodeMap at(N.size());   // updated node -> index in N
+    std::vector<int32_t> base(blocks + 1, 0);
+    for (int r = 0; r < blocks; r++) {
+        std::sort(N.begin() + start[r], N.begin() + start[r + 1], [](const Node &x, const Node &y) {
+            const int a = x.q < 0 ? x.black : 2, b = y.q < 0 ? y.black : 2;
+            return a != b ? a < b : x.p < y.p;
+        });
+        int ni = 0;
+        for (size_t i = start[r]; i < start[r + 1]; i++) ni += N[i].q < 0;
+        base[r + 1] = base[r] + ni;
+    }
+    std::vector<int32_t> cid(N.size(), -1);   // place of an inside node in the compact array
+    for (int r = 0; r < blocks; r++)
+        for (size_t i = start[r]; i < start[r + 1]; i++) {
+            at.set(N[i].p, (int32_t)i);
+            if (N[i].q < 0) cid[i] = base[r] + (int32_t)(i - start[r]);   // inside nodes come first
+        }
+    struct Block {
+        std::vector<int32_t> in, gs, red, black;   // slots -> node; entries (index in N)
+        std::vector<uint16_t> ent, gst;
+        std::vector<int32_t> in_cid, gs_q;
+        int own_in = 0, own_g = 0;
+    };
+    std::vector<Block> B(blocks);
+    std::atomic<int> next{0};
+    auto work = [&]() {
+        int64_t rd[27];
+        for (int r = next++; r < blocks; r = next++) {
+            Block &K = B[r];
+            const int32_t b0 = (int32_t)start[r], e0 = (int32_t)start[r + 1];
+            NodeMap S(6 * (size_t)(e0 - b0) + 64), in_ent(4 * (size_t)(e0 - b0) + 64);
+            auto reads = [&](const Node &x) {
+                if (x.q < 0) {   // the order of the sweeps' sum: axis 2, axis 0, axis 1
+                    const int64_t s[3] = {L.stride[2], L.stride[0], L.stride[1]};
+                    for (int a = 0; a < 3; a++) {
+                        rd[2 * a] = x.p - s[a];
+                        rd[2 * a + 1] = x.p + s[a];
+                    }
+                    return 6;
+                }
+                for (int k = 0; k < 27; k++) rd[k] = L.stn[(int64_t)x.q * KMAX + k];
+                return 27;
+            };
+            auto touch = [&](int64_t p) {
+                if (S.get(p, -1) >= 0) return;
+                const int32_t o = at.get(p, -1);
+                if ((L.type[p] & NODE_KIND) == NODE_GHOST) {
+                    S.set(p, (int32_t)K.gs.size());
+                    K.gs.push_back((int32_t)p);
+                    K.gs_q.push_back(N[o].q);   // every ghost is updated
+                } else {
+                    S.set(p, (int32_t)K.in.size());
+                    K.in.push_back((int32_t)p);
+                    K.in_cid.push_back(o < 0 ? -1 : cid[o]);
+                }
+            };
+            for (int32_t i = b0; i < e0; i++) {
+                touch(N[i].p);
+                if (N[i].q < 0) {
+                    in_ent.set(N[i].p, 1);
+                    (N[i].black ? K.black : K.red).push_back(i);
+                    K.own_in++;
+                } else {
+                    K.own_g++;
+                }
+            }
+            // the blacks the own ghosts read, the reds those blacks and ghosts read
+            auto cone = [&](int32_t i, int black) {
+                const int m = reads(N[i]);
+                for (int k = 0; k < m; k++) {
+                    const int32_t o = at.get(rd[k], -1);
+                    if (o < 0 || N[o].q >= 0 || N[o].black != black || in_ent.get(N[o].p, 0)) continue;
+                    in_ent.set(N[o].p, 1);
+                    (black ? K.black : K.red).push_back(o);
+                }
+            };
+            for (int32_t i = b0; i < e0; i++)
+                if (N[i].q >= 0) cone(i, 1);
+            for (size_t k = 0; k < K.black.size(); k++) cone(K.black[k], 0);
+            for (int32_t i = b0; i < e0; i++)
+                if (N[i].q >= 0) cone(i, 0);
+            for (const auto *l : {&K.red, &K.black})
+                for (int32_t i : *l) {
+                    touch(N[i].p);
+                    const int m = reads(N[i]);
+                    for (int k = 0; k < m; k++) touch(rd[k]);
+                }
+            for (int32_t i = b0; i < e0; i++)
+                if (N[i].q >= 0) {
+                    const int m = reads(N[i]);
+                    for (int k = 0; k < m; k++) touch(rd[k]);
+                }
+        }
+    };
+    auto parallel = [](auto &&f) {
+        std::vector<std::thread> pool;
+        const unsigned nt = std::max(1u, std::min(16u, std::thread::hardware_concurrency()));
+        for (unsigned t = 1; t < nt; t++) pool.emplace_back(f);
+        f();
+        for (auto &t : pool) t.join();
+    };
+    parallel(work);
+    Sweep3Layout &y = out.lay;
+    y.blocks = blocks;
+    y.inside = base[blocks];
+    for (const Block &K : B) {
+        y.max_in = std::max(y.max_in, (int)K.in.size());
+        y.max_gs = std::max(y.max_gs, (int)K.gs.size());
+        y.max_e = std::max(y.max_e, (int)(K.red.size() + K.black.size()));
+        y.max_g = std::max(y.max_g, K.own_g);
+    }
+    y.max_in = (y.max_in + 3) & ~3;
+    if (y.max_in + y.max_gs >= 0x10000) return out;
+    y.node = S3_HDR * 4;
+    y.cid = y.node + 4 * y.max_in;
+    y.gslot = y.cid + 4 * y.max_in;
+    y.ent = align16(y.gslot + 4 * y.max_gs);
+    y.gst = y.ent + 16 * y.max_e;
+    y.stride = y.gst + 64 * y.max_g;
+    out.records.assign((size_t)blocks * y.stride, 0);
+    next = 0;
+    auto write = [&]() {
+        for (int r = next++; r < blocks; r = next++) {
+            const Block &K = B[r];
+            NodeMap S(2 * (K.in.size() + K.gs.size()) + 64);
+            for (size_t i = 0; i < K.in.size(); i++) S.set(K.in[i], (int32_t)i);
+            for (size_t i = 0; i < K.gs.size(); i++) S.set(K.gs[i], y.max_in + (int32_t)i);
+            uint8_t *rec = out.records.data() + (size_t)r * y.stride;
+            int32_t *h = reinterpret_cast<int32_t *>(rec);
+            h[S3_NIN] = (int)K.in.size();
+            h[S3_NGS] = (int)K.gs.size();
+            h[S3_OWN_IN] = K.own_in;
+            h[S3_OWN_G] = K.own_g;
+            h[S3_RED] = (int)K.red.size();
+            h[S3_NE] = (int)(K.red.size() + K.black.size());
+            h[S3_BASE] = base[r];
+            std::copy(K.in.begin(), K.in.end(), reinterpret_cast<int32_t *>(rec + y.node));
+            std::copy(K.in_cid.begin(), K.in_cid.end(), reinterpret_cast<int32_t *>(rec + y.cid));
+            std::copy(K.gs_q.begin(), K.gs_q.end(), reinterpret_cast<int32_t *>(rec + y.gslot));
+            uint16_t *e = reinterpret_cast<uint16_t *>(rec + y.ent), *g = reinterpret_cast<uint16_t *>(rec + y.gst);
+            const int64_t s[3] = {L.stride[2], L.stride[0], L.stride[1]};
+            for (const auto *l : {&K.red, &K.black})
+                for (int32_t i : *l) {
+                    const int64_t p = N[i].p;
+                    e[0] = (uint16_t)S.get(p, 0);
+                    for (int a = 0; a < 3; a++) {
+                        e[1 + 2 * a] = (uint16_t)S.get(p - s[a], 0);
+                        e[2 + 2 * a] = (uint16_t)S.get(p + s[a], 0);
+                    }
+                    e += 8;
+                }
+            for (int k = 0; k < K.own_g; k++)
+                for (int a = 0; a < 27; a++)
+                    g[((size_t)(a / 8) * y.max_g + k) * 8 + a % 8] =
+                        (uint16_t)S.get(L.stn[(int64_t)K.gs_q[k] * KMAX + a], 0);
+        }
+    };
+    parallel(write);
     return out;
 }
 

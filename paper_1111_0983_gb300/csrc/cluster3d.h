@@ -79,4 +79,45 @@ bool cluster3_fits(const Cluster3Layout &l, int device);
 template <typename T>
 void launch_cluster3(const LevelView<T> &v, const Cluster3Dev &P, bool lead, int lambda, int mu, cudaStream_t s);
 
+// ---- band sweeps of larger levels, one launch a sweep
+// The updated nodes are split into blocks; a block runs a whole band sweep
+// (red, black, ghosts) on its own nodes and the inside nodes of other blocks
+// that its updates read.  Between launches the own values of all blocks lie in
+// compact arrays (block after block), the ghosts' in arrays over the ghosts.
+// Every block has a record of `stride` bytes with the same section offsets:
+//   ints   header (S3_*)
+//   node   int32 per inside slot: grid node (own, halo, read only)
+//   cid    int32 per inside slot: place in the compact array, -1: read only
+//   gslot  int32 per ghost slot (own first): ghost number
+//   ent    8 x uint16 per entry, red then black: its slot, 6 sources in the
+//          order of the sweeps' sum
+//   gst    4 x max_g x 8 uint16: the 27 stencil sources of an own ghost
+// A source is an inside slot or max_in + ghost slot.
+enum { S3_NIN, S3_NGS, S3_OWN_IN, S3_OWN_G, S3_RED, S3_NE, S3_BASE, S3_HDR = 8 };
+struct Sweep3Layout {
+    int blocks = 0, stride = 0, node = 0, cid = 0, gslot = 0, ent = 0, gst = 0;
+    int max_in = 0, max_gs = 0, max_e = 0, max_g = 0;
+    int inside = 0;   // entries of the compact array
+};
+struct Sweep3Program {
+    Sweep3Layout lay;
+    std::vector<uint8_t> records;   // blocks * stride; empty: no program
+};
+Sweep3Program build_sweep3(const HostLevel &L, int blocks);
+
+struct Sweep3Dev {
+    Sweep3Layout lay;
+    uint8_t *records = nullptr;
+    void *x[2] = {nullptr, nullptr};   // compact values of the inside nodes (the cycle precision)
+    void *g = nullptr;                 // ghost values beside LevelView::gtmp
+};
+template <typename T>
+size_t sweep3_smem(const Sweep3Layout &l);
+template <typename T>
+bool sweep3_fits(const Sweep3Layout &l, int device);
+// lambda >= 2 band sweeps after the ghosts' new values have been put into
+// v.gtmp; leaves u with every new value
+template <typename T>
+void launch_sweep3(const LevelView<T> &v, const Sweep3Dev &P, int lambda, cudaStream_t s);
+
 }  // namespace gcmg

@@ -25,6 +25,7 @@ struct gcmg_ctx {
     std::vector<DevData<double>> D64;
     std::vector<DevData<float>> D32;
     std::vector<gcmg::Cluster3Dev> c3;      // 3D: the levels' boundary phases as one cluster launch
+    std::vector<gcmg::Sweep3Dev> s3;        // 3D: larger levels' band sweeps as a launch each (cycle precision)
     bool rhs_set = false;
     bool js64 = false;                      // FP64 junction-solve inverses kept (single relaxations)
     // the fused coarse cycle (coarse.cu): its first level (-1: per-level
