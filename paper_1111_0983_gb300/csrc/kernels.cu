@@ -619,24 +619,42 @@ __global__ void __launch_bounds__(256) k_rb_rows(LevelView<T> v, const int2 *__r
     }
 }
 
-// The defect f + Lap_h u (TGCS step 3) at every inside node of a level into r, over the row segments: a warp takes G segments at once, lane l the
-// nodes k0 + l and k0 + l + 32 of each, all loads issued before the first
-// store; with norm, its max-norm.  MIXED (the FP64 finest level of the mixed
-// form): also f32 = the defect rounded to FP32 and e32 = 0 at those nodes.
-// The expression of defect_node.
+// The defect (TGCS step 3) at every unknown of a level into r: f + Lap_h u at
+// the inside nodes over the row segments (a warp takes G segments at once, lane
+// l the nodes k0 + l and k0 + l + 32 of each, all loads issued before the first
+// store), g - L_G u at the ghosts by the first gb CTAs; with norm, its max-norm.
+// MIXED (the FP64 finest level of the mixed form): also the next FP32 problem,
+// f32 and g32 = the defects rounded to FP32 and e32 = 0.  The expressions of
+// defect_node and defect_ghost_item.  The ghosts had a launch of their own:
+// without it the star on 257^2 (mixed) 1035 -> 995 us a solve, the flower on
+// 1025^2 in FP64 6.03 -> 5.87 ms, the torus on 257^3 (mixed) 11.38 -> 11.00 ms.
 template <typename T, int D, int G, bool MIXED>
 __global__ void __launch_bounds__(256) k_defect_rows(LevelView<T> v, unsigned long long *norm, float *__restrict__ f32,
-                                                    float *__restrict__ e32) {
+                                                    float *__restrict__ g32, float *__restrict__ e32, int gb) {
     if (MIXED) pdl_trigger();
+    if ((int)blockIdx.x < gb) {
+        const int q = blockIdx.x * blockDim.x + threadIdx.x;
+        pdl_wait();
+        double val = 0.0;
+        if (q < v.ng) {
+            val = defect_ghost_item<T, D == 2 ? 9 : 27>(v, q);
+            if (MIXED) {
+                g32[q] = (float)val;
+                e32[v.gnode[q]] = 0.0f;
+            }
+        }
+        reduce_norm(norm, val);
+        return;
+    }
     const int lane = threadIdx.x & 31;
-    const int nw = (int)((gridDim.x * blockDim.x) >> 5);
+    const int nw = (int)(((gridDim.x - gb) * blockDim.x) >> 5);
     const int n = v.n, nseg = v.nsegs;
     const int2 *__restrict__ segs = v.segs;
     pdl_wait();
     // the max-norm on the bit patterns of |d| (integer compares; the order of
     // non-negative doubles, NaN above +Inf, which reduce_norm maps to +Inf)
     unsigned long long mb = 0;
-    for (int q = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5) * G; q < nseg; q += nw * G) {
+    for (int q = (int)(((blockIdx.x - gb) * blockDim.x + threadIdx.x) >> 5) * G; q < nseg; q += nw * G) {
         T d[2 * G];
         int64_t p[2 * G];
         bool on[2 * G];
@@ -1287,24 +1305,6 @@ __global__ void k_coarse_solve(LevelView<T> v, const int32_t *__restrict__ unk_n
 }
 
 // ------------------------------------------------------- mixed precision
-// Ghost rows of the FP64 defect of the finest level that sets up the next FP32
-// correction problem (the inside nodes: k_defect_rows): r, the defects rounded
-// to FP32 into g32, e32 = 0 at the ghosts
-template <int K>
-__global__ void k_defect_ghost_mixed(LevelView<double> v, unsigned long long *norm, float *__restrict__ g32,
-                                     float *__restrict__ e32) {
-    pdl_trigger();
-    pdl_wait();
-    const int q = blockIdx.x * blockDim.x + threadIdx.x;
-    double val = 0.0;
-    if (q < v.ng) {
-        val = defect_ghost_item<double, K>(v, q);
-        g32[q] = (float)val;
-        e32[v.gnode[q]] = 0.0f;
-    }
-    reduce_norm(norm, val);
-}
-
 // keep u = 0 off Omega_h u Gamma_h
 template <typename T>
 __global__ void k_mask_unknowns(const uint8_t *__restrict__ type, T *__restrict__ u, int64_t nn) {
@@ -1632,26 +1632,31 @@ void launch_ghost_relax_list(const LevelView<T> &v, int dim, const int32_t *list
 // at once pay the memory's latency once for G, but a warp's arithmetic (the
 // FP64 form's exact sum above all) is a chain
 template <typename T, int D, int G, bool MIXED>
-static void launch_defect_rows(const LevelView<T> &v, unsigned long long *norm, float *f32, float *e32, cudaStream_t s) {
+static void launch_defect_rows(const LevelView<T> &v, unsigned long long *norm, float *f32, float *g32, float *e32,
+                               cudaStream_t s) {
     static unsigned resident = 0, resident1 = 0;
+    g_launches++;
+    const unsigned gb = (unsigned)((v.ng + 255) / 256);
     if (v.nsegs >= 32 * G * num_sms())
         pdl_launch(k_defect_rows<T, D, G, MIXED>,
-                   dim3(segment_blocks(k_defect_rows<T, D, G, MIXED>, v.nsegs, G, resident)), dim3(256), 0, s, v, norm,
-                   f32, e32);
+                   dim3(gb + segment_blocks(k_defect_rows<T, D, G, MIXED>, v.nsegs, G, resident)), dim3(256), 0, s, v,
+                   norm, f32, g32, e32, (int)gb);
     else
         pdl_launch(k_defect_rows<T, D, 1, MIXED>,
-                   dim3(segment_blocks(k_defect_rows<T, D, 1, MIXED>, v.nsegs, 1, resident1)), dim3(256), 0, s, v, norm,
-                   f32, e32);
+                   dim3(gb + segment_blocks(k_defect_rows<T, D, 1, MIXED>, v.nsegs, 1, resident1)), dim3(256), 0, s, v,
+                   norm, f32, g32, e32, (int)gb);
 }
 
 template <typename T>
 void launch_defect(const LevelView<T> &v, int dim, bool zero_rest, unsigned long long *norm, cudaStream_t s) {
+    if (!zero_rest) {   // inside nodes over the row segments, and the ghosts
+        if (dim == 2) launch_defect_rows<T, 2, 4, false>(v, norm, nullptr, nullptr, nullptr, s);
+        else launch_defect_rows<T, 3, 4, false>(v, norm, nullptr, nullptr, nullptr, s);
+        return;
+    }
     g_launches += v.ng > 0 ? 2 : 1;
-    const unsigned nb = std::min(blocks_for(level_threads(v, !zero_rest)), kNormBlocks);
-    if (!zero_rest) {   // inside nodes over the row segments
-        if (dim == 2) launch_defect_rows<T, 2, 4, false>(v, norm, nullptr, nullptr, s);
-        else launch_defect_rows<T, 3, 4, false>(v, norm, nullptr, nullptr, s);
-    } else if (dim == 2) pdl_launch(k_defect_interior<T, 2>, dim3(nb), dim3(kThreads), 0, s, v, zero_rest, norm);
+    const unsigned nb = std::min(blocks_for(level_threads(v, false)), kNormBlocks);
+    if (dim == 2) pdl_launch(k_defect_interior<T, 2>, dim3(nb), dim3(kThreads), 0, s, v, zero_rest, norm);
     else pdl_launch(k_defect_interior<T, 3>, dim3(nb), dim3(kThreads), 0, s, v, zero_rest, norm);
     if (v.ng > 0) {
         if (dim == 2) pdl_launch(k_defect_ghost<T, 9>, dim3(blocks_for(v.ng)), dim3(kThreads), 0, s, v, norm);
@@ -1697,13 +1702,7 @@ void launch_descend(const LevelView<T> &F, const LevelView<T> &C, const DevGeom 
         // segments, then the ghosts), so that each fine defect is computed
         // once rather than once per coarse node whose 27-node neighbourhood
         // holds it (27/8 times on average); the same values as on the spot
-        g_launches++;
-        launch_defect_rows<T, 3, 4, false>(F, nullptr, nullptr, nullptr, s);
-        if (F.ng > 0) {
-            g_launches++;
-            pdl_launch(k_defect_ghost<T, 27>, dim3(blocks_for(F.ng)), dim3(kThreads), 0, s, F,
-                       (unsigned long long *)nullptr);
-        }
+        launch_defect_rows<T, 3, 4, false>(F, nullptr, nullptr, nullptr, nullptr, s);
         if (C.ng > 0) {
             g_launches++;
             pdl_launch(k_ghost_rows<T, true>, dim3(blocks_for(32 * (int64_t)C.ng)), dim3(kThreads), 0, s,
@@ -1975,15 +1974,9 @@ void launch_mask_unknowns(const uint8_t *type, T *u, int64_t nn, cudaStream_t s)
 
 void launch_defect_mixed(const LevelView<double> &v, int dim, unsigned long long *norm, float *f32, float *g32,
                          float *e32, cudaStream_t s) {
-    g_launches += v.ng > 0 ? 2 : 1;
-    // the inside nodes over the segments, e32 = 0 at the ghosts by the ghost
-    // launch; the other nodes of f32 and e32 are 0 from the start
-    if (dim == 2) launch_defect_rows<double, 2, 2, true>(v, norm, f32, e32, s);
-    else launch_defect_rows<double, 3, 2, true>(v, norm, f32, e32, s);
-    if (v.ng > 0) {
-        if (dim == 2) pdl_launch(k_defect_ghost_mixed<9>, dim3(blocks_for(v.ng)), dim3(kThreads), 0, s, v, norm, g32, e32);
-        else pdl_launch(k_defect_ghost_mixed<27>, dim3(blocks_for(v.ng)), dim3(kThreads), 0, s, v, norm, g32, e32);
-    }
+    // nodes off Omega_h u Gamma_h: f32 and e32 are 0 from the start
+    if (dim == 2) launch_defect_rows<double, 2, 2, true>(v, norm, f32, g32, e32, s);
+    else launch_defect_rows<double, 3, 2, true>(v, norm, f32, g32, e32, s);
 }
 
 void launch_add_correction(const DevGeom &g, double *u64, const float *e32, cudaStream_t s) {
