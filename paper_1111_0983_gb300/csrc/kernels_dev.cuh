@@ -773,14 +773,11 @@ __device__ __forceinline__ int64_t fine_image(int64_t X, int64_t cs0, int64_t cs
     return 2 * j0 * fs0 + 2 * j1 * fs1 + 2 * j2;
 }
 
-// wait: call pdl_wait once the node types are read, before any value (the
-// types are fixed while a solve runs; the values come from earlier launches)
 // skipped: when not null, a neighbourhood that is not all members is not
 // searched: *skipped is set and 0 returned (the caller handles those nodes
 // in another launch)
 template <typename T, int D, typename Get>
-__device__ T partial_transfer_of(const LevelView<T> &F, int64_t p, bool interior, Get value, bool wait = false,
-                                 bool *skipped = nullptr) {
+__device__ T partial_transfer_of(const LevelView<T> &F, int64_t p, bool interior, Get value, bool *skipped = nullptr) {
     const int cube = D == 2 ? 9 : 27;
     const unsigned full = (1u << cube) - 1u;
     unsigned member = 0;
@@ -803,7 +800,6 @@ __device__ T partial_transfer_of(const LevelView<T> &F, int64_t p, bool interior
         best = 1;  // full weighting fast path
     } else if (skipped) {
         *skipped = true;
-        if (wait) pdl_wait();
         return (T)0;
     } else {
         for (int b = 0; b < nbox; b++) {
@@ -814,32 +810,6 @@ __device__ T partial_transfer_of(const LevelView<T> &F, int64_t p, bool interior
             else if (sz == best) { count++; bestset |= 1ull << b; }
         }
     }
-    // the members' weights: the largest boxes in increasing order (as a scan of
-    // all boxes would)
-    auto weight = [&](int c) {
-        int rem = c;
-        int o[3] = {0, 0, 0};
-        for (int a = D - 1; a >= 0; a--) {
-            o[a] = rem % 3 - 1;
-            rem /= 3;
-        }
-        T w = 0;
-        for (unsigned long long bs = bestset; bs; bs &= bs - 1) {
-            const int b = __ffsll((long long)bs) - 1;
-            T wb = 1;
-            for (int a = 0; a < D; a++) wb *= w1d<T>((b >> (2 * a)) & 3, o[a]);
-            w += wb;
-        }
-        return w / (T)count;
-    };
-    // in 2D before the wait, being fixed as the types are: at 1025^2 a mixed
-    // cycle 155.2 -> 150.4 us, at 257^2 98.0 -> 92.8 (3D takes a launch of its own)
-    T early[D == 2 ? 9 : 1];
-    const bool pre = D == 2 && wait;
-    if (pre && count > 0)
-#pragma unroll
-        for (int c = 0; c < (D == 2 ? 9 : 1); c++) early[c] = ((member >> c) & 1u) ? weight(c) : (T)0;
-    if (wait) pdl_wait();
     if (member == full) {
         // full weighting: every value loaded before the first product (one
         // round trip, not 3^D), then the same sum in the same order as below
@@ -888,7 +858,21 @@ __device__ T partial_transfer_of(const LevelView<T> &F, int64_t p, bool interior
 #pragma unroll
     for (int c = 0; c < cube; c++) {
         if (!((member >> c) & 1u)) continue;
-        const T w = pre ? early[D == 2 ? c : 0] : weight(c);
+        int rem = c;
+        int o[3] = {0, 0, 0};
+        for (int a = D - 1; a >= 0; a--) {
+            o[a] = rem % 3 - 1;
+            rem /= 3;
+        }
+        // the largest boxes in increasing order (as a scan of all boxes would)
+        T w = 0;
+        for (unsigned long long bs = bestset; bs; bs &= bs - 1) {
+            const int b = __ffsll((long long)bs) - 1;
+            T wb = 1;
+            for (int a = 0; a < D; a++) wb *= w1d<T>((b >> (2 * a)) & 3, o[a]);
+            w += wb;
+        }
+        w /= (T)count;
         if (w != (T)0) acc += w * val[c];
     }
     return acc;
@@ -938,7 +922,7 @@ __device__ __forceinline__ void descend_node(const LevelView<T> &F, const LevelV
     bool skipped = false;
     const T v = partial_transfer_of<T, D>(F, fine_image<D>(i, C.s0, C.s1, F.s0, F.s1), true,
                                           [&](int64_t q) { return FROM_R ? F.r[q] : inside_defect<T, D>(F, q); },
-                                          false, full_only ? &skipped : nullptr);
+                                          full_only ? &skipped : nullptr);
     if (!skipped) fc[i] = v;
 }
 
@@ -948,16 +932,81 @@ __device__ __forceinline__ T transfer_term(const LevelView<T> &F, int col) {
     return FROM_R ? F.r[F.gnode[col]] : ghost_defect<T, D == 2 ? 9 : 27>(F, col);
 }
 
-// descend_node at coarse inside node i (fine image p) in a launch that starts
-// before its predecessor ends: the node types are read first, then pdl_wait
-// (again harmless when the warp has waited before), then the defects
+// The weights of partial_transfer_of over the inside set in 2D (the same
+// products and sums; 0 for non-members), bit c of the 3^2 neighbourhood in w[c]
+template <typename T>
+__device__ __forceinline__ void partial_weights2(const LevelView<T> &F, int64_t p, T (&w)[9]) {
+    unsigned member = 0;
+#pragma unroll
+    for (int c = 0; c < 9; c++)
+        if ((F.type[p + (c / 3 - 1) * F.s0 + (c % 3 - 1)] & NODE_KIND) == NODE_IN) member |= 1u << c;
+    if (member == 0x1ffu) {
+#pragma unroll
+        for (int c = 0; c < 9; c++) w[c] = w1d<T>(0, c / 3 - 1) * w1d<T>(0, c % 3 - 1);
+        return;
+    }
+    int best = 0, count = 0;
+    unsigned bestset = 0;   // the largest boxes inside the set
+    for (int b = 0; b < 16; b++) {
+        const unsigned m = box_mask<2>(b);
+        if (m & ~member) continue;
+        const int sz = __popc(m);
+        if (sz > best) { best = sz; count = 1; bestset = 1u << b; }
+        else if (sz == best) { count++; bestset |= 1u << b; }
+    }
+#pragma unroll
+    for (int c = 0; c < 9; c++) w[c] = 0;
+    for (unsigned bs = bestset; bs; bs &= bs - 1) {   // in increasing order
+        const int b = __ffs((int)bs) - 1;
+#pragma unroll
+        for (int c = 0; c < 9; c++) w[c] += w1d<T>(b & 3, c / 3 - 1) * w1d<T>((b >> 2) & 3, c % 3 - 1);
+    }
+    if (count > 1)
+#pragma unroll
+        for (int c = 0; c < 9; c++) w[c] /= (T)count;
+}
+
+// descend_node at coarse inside node i (fine image p) in 2D, in a launch that
+// starts before its predecessor ends: the node types and the weights from them
+// first, then pdl_wait (again harmless when the warp has waited before), then
+// the defects.  u and f are read at every node that a full neighbourhood needs
+// (all within 2 of the fine image of a node that is not on the box edge, so in
+// the grid), members or not: one round trip, where a load a member under its own
+// test had been up to nine.  A mixed cycle with the weights after the wait and loads
+// under tests, the weights before it, and so: 1025^2 155, 150, 138 us; 257^2 98,
+// 93, 83; 4097^2 342, 338, 316; FP64 (the defects from r) 1025^2 419 -> 400.
 template <typename T, int D, bool FROM_R>
 __device__ __forceinline__ void descend_inside_early(const LevelView<T> &F, T *__restrict__ fc, T *__restrict__ uc,
                                                      int64_t i, int64_t p) {
-    const T v = partial_transfer_of<T, D>(F, p, true,
-                                          [&](int64_t q) { return FROM_R ? F.r[q] : inside_defect<T, D>(F, q); }, true);
+    T w[9], val[9];
+    partial_weights2<T>(F, p, w);
+    pdl_wait();
+    if (FROM_R) {
+#pragma unroll
+        for (int c = 0; c < 9; c++) val[c] = F.r[p + (c / 3 - 1) * F.s0 + (c % 3 - 1)];
+    } else {
+        T u[5][5], f[9];
+#pragma unroll
+        for (int a = 0; a < 5; a++)
+#pragma unroll
+            for (int b = 0; b < 5; b++)
+                if ((a > 0 && a < 4) || (b > 0 && b < 4)) u[a][b] = F.u[p + (a - 2) * F.s0 + (b - 2)];
+#pragma unroll
+        for (int c = 0; c < 9; c++) f[c] = F.f[p + (c / 3 - 1) * F.s0 + (c % 3 - 1)];
+#pragma unroll
+        for (int c = 0; c < 9; c++) {   // inside_defect
+            const int a = c / 3 + 1, b = c % 3 + 1;
+            const T up = u[a][b];
+            const T lap = (u[a][b - 1] - up) + (u[a][b + 1] - up) + (u[a - 1][b] - up) + (u[a + 1][b] - up);
+            val[c] = f[c] + lap * F.inv_h2;
+        }
+    }
+    T acc = 0;
+#pragma unroll
+    for (int c = 0; c < 9; c++)
+        if (w[c] != (T)0) acc += w[c] * val[c];
     uc[i] = 0;
-    fc[i] = v;
+    fc[i] = acc;
 }
 
 // both parts at index i, the ghost row summed by one thread
