@@ -773,7 +773,7 @@ def run_gcmg(args):
              "share_of_solve": (k_ms / ms) if ms > 0 else None}
     if P.dim == 3 and kern == "rows":
         sweep["launch_note"] = ("a unit is one sweep: the red and the black launch, timed together; the kernels "
-                                "that take most of the solve's time are the boundary phases' short list launches "
+                                "that take most of the solve's time are the boundary phases' launches "
                                 "(latency bound), see the launch list under profiles/")
     roofline = sweep
     if b_launches:
