@@ -46,7 +46,8 @@ constexpr int kCin[kLayers] = {4, 32, 32, 32, 32, 32};
 constexpr int kCout[kLayers] = {32, 32, 32, 32, 32, 2};
 constexpr int kTile = 128;            // pixels per CTA (M)
 constexpr int kMaxDil = 96;
-constexpr int kRing = 4;              // row segments in shared memory
+constexpr int kRing = 4;              // row segments in shared memory (convolution: at least,
+constexpr int kMaxRing = 8;           // and at most, see ConvArgs::ring)
 constexpr int kAcc = 4;               // TMEM accumulators of the convolution
 constexpr int kDzStages = 4;          // staged gradient tiles of the weight gradients
 constexpr int kConvThreads = 192;     // producer, MMA issuer, four epilogue warps
@@ -182,6 +183,7 @@ struct ConvArgs {
     Geo geo;
     Chains ch;
     int dil;
+    int ring;             // segments in shared memory
     int *err;
 };
 
@@ -198,12 +200,12 @@ __device__ __forceinline__ void mbar_expect(uint32_t mbar, uint32_t bytes) {
 }
 
 // Positions number the segments a CTA loads, over all of its items; position p
-// lies in ring slot p % kRing.  Tile k of an item whose first segment has
+// lies in ring slot p % ring.  Tile k of an item whose first segment has
 // position p0 reads positions p0 + k, + 1, + 2 (tap rows -1, 0, +1).
 // Every wait is bounded; after one that ran out (ok = false) a role waits no
 // more, and the kernel reports it through a.err.
-// Four CTAs an SM at small dilations, two at 81 (TMEM columns, shared memory):
-// with one segment in flight a CTA, several CTAs hide the copies' latency.
+// Several CTAs an SM (TMEM columns, shared memory), each with ring - 3 segments
+// in flight: three of six slots at small dilations, two of five at 81.
 // Measured, 8 images of 513^2, 32 -> 32 channels, forward: 366 us a layer with
 // three segments a tile, one accumulator and the border's tiles computed too;
 // 81-96 us so (2.9-3.4 TB/s of activations read and written once).  Backward to
@@ -212,17 +214,17 @@ template <int GIN, int NOUT, int MODE>
 __global__ void __launch_bounds__(kConvThreads) k_conv(ConvArgs a) {
     extern __shared__ __align__(128) unsigned char smem[];
     const int seg = kTile + 2 * a.dil;                            // pixels of a segment
-    uint4 *sx = reinterpret_cast<uint4 *>(smem);                  // [kRing][GIN][seg]
-    uint4 *sw = sx + kRing * GIN * seg;                           // 9 * GIN * NOUT rows
+    uint4 *sx = reinterpret_cast<uint4 *>(smem);                  // [ring][GIN][seg]
+    uint4 *sw = sx + a.ring * GIN * seg;                           // 9 * GIN * NOUT rows
     uint64_t *bars = reinterpret_cast<uint64_t *>(sw + 9 * GIN * NOUT);
-    uint32_t *tslot = reinterpret_cast<uint32_t *>(bars + 2 * kRing + 2 * kAcc + 1);
-    const uint32_t full = smem_u32(bars), empty = full + 8 * kRing, afull = empty + 8 * kRing,
+    uint32_t *tslot = reinterpret_cast<uint32_t *>(bars + 2 * kMaxRing + 2 * kAcc + 1);
+    const uint32_t full = smem_u32(bars), empty = full + 8 * kMaxRing, afull = empty + 8 * kMaxRing,
                    afree = afull + 8 * kAcc, wbar = afree + 8 * kAcc;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
     if (warp == 1) tmem_alloc<kAcc * NOUT>(smem_u32(tslot));
     if (threadIdx.x == 0) {
-        for (int i = 0; i < kRing; i++) {
+        for (int i = 0; i < a.ring; i++) {
             mbar_init(full + 8 * i, 1);
             mbar_init(empty + 8 * i, 1);
         }
@@ -246,25 +248,29 @@ __global__ void __launch_bounds__(kConvThreads) k_conv(ConvArgs a) {
         if (lane == 0) {   // producer
             mbar_expect(wbar, 9 * GIN * NOUT * 16);
             bulk_g2s(smem_u32(sw), a.w, 9 * GIN * NOUT * 16, wbar);
-            int pos = 0;
+            int s = 0, round = 0, sent = 0;   // slot of the next position and how often the ring was filled
             for (int t = blockIdx.x; t < a.ch.items; t += gridDim.x) {
                 if (!a.ch.item(t, &b, &c, &row0, &cnt)) continue;
                 // pixel of the first segment: row row0 - dil, columns from dil before the tile
                 long q = ((long)b * a.geo.Hp + a.geo.P + row0 - a.dil) * a.geo.Wp + a.geo.P + c * kTile - a.dil;
-                for (int p = 0; p < cnt + 2; p++, pos++, q += (long)a.dil * a.geo.Wp) {
-                    const int s = pos % kRing;
-                    wait(empty + 8 * s, (uint32_t)(pos / kRing) + 1u);
+                for (int p = 0; p < cnt + 2; p++, q += (long)a.dil * a.geo.Wp) {
+                    wait(empty + 8 * s, (uint32_t)round + 1u);
                     if (!ok) break;
                     mbar_expect(full + 8 * s, (uint32_t)(GIN * seg * 16));
                     for (int g = 0; g < GIN; g++)
                         bulk_g2s(smem_u32(sx + (s * GIN + g) * seg), a.x + (long)g * a.geo.gs + q, (uint32_t)(seg * 16),
                                  full + 8 * s);
+                    sent = min(sent + 1, a.ring);
+                    if (++s == a.ring) s = 0, round++;
                 }
                 if (!ok) break;
             }
             // every copy has landed before the CTA ends (in a complete run the
             // MMAs have waited for them already)
-            for (int p = max(0, pos - kRing); p < pos; p++) mbar_wait(full + 8 * (p % kRing), (uint32_t)(p / kRing) & 1u);
+            for (; sent > 0; sent--) {
+                if (--s < 0) s = a.ring - 1, round--;
+                mbar_wait(full + 8 * s, (uint32_t)round & 1u);
+            }
             mbar_wait(wbar, 0);
         }
         __syncwarp();
@@ -272,13 +278,17 @@ __global__ void __launch_bounds__(kConvThreads) k_conv(ConvArgs a) {
         if (lane == 0) {   // MMA issuer
             constexpr uint32_t idesc = idesc_bf16(kTile, NOUT, 0, 0);
             const uint32_t xa = smem_u32(sx), wa = smem_u32(sw);
-            int pos = 0, tile = 0;
+            int tile = 0;
+            int s0 = 0, sn = 0, round = 0;   // slot of the tile's first position; of the next one to arrive
+            auto after = [&](int i, int d) { return i + d < a.ring ? i + d : i + d - a.ring; };
             wait(wbar, 0);
             for (int t = blockIdx.x; t < a.ch.items && ok; t += gridDim.x) {
                 if (!a.ch.item(t, &b, &c, &row0, &cnt)) continue;
                 for (int k = 0; k < cnt; k++, tile++) {
-                    for (int p = k ? pos + k + 2 : pos; p <= pos + k + 2; p++)
-                        wait(full + 8 * (p % kRing), (uint32_t)(p / kRing));
+                    for (int p = k ? 2 : 0; p < 3; p++) {
+                        wait(full + 8 * sn, (uint32_t)round);
+                        if (++sn == a.ring) sn = 0, round++;
+                    }
                     const int ac = tile % kAcc;
                     wait(afree + 8 * ac, (uint32_t)(tile / kAcc) + 1u);
                     if (!ok) break;
@@ -287,7 +297,7 @@ __global__ void __launch_bounds__(kConvThreads) k_conv(ConvArgs a) {
                     uint32_t acc = 0;
 #pragma unroll 1
                     for (int tr = 0; tr < 3; tr++) {
-                        const uint32_t xs = xa + (uint32_t)(((pos + k + tr) % kRing) * GIN * seg) * 16;
+                        const uint32_t xs = xa + (uint32_t)(after(s0, tr) * GIN * seg) * 16;
 #pragma unroll
                         for (int tc = 0; tc < 3; tc++)
 #pragma unroll
@@ -300,13 +310,14 @@ __global__ void __launch_bounds__(kConvThreads) k_conv(ConvArgs a) {
                             }
                     }
                     mma_commit(afull + 8 * ac);
-                    mma_commit(empty + 8 * ((pos + k) % kRing));
+                    mma_commit(empty + 8 * s0);
                     if (k + 1 == cnt) {   // the item's last two segments serve no other tile
-                        mma_commit(empty + 8 * ((pos + k + 1) % kRing));
-                        mma_commit(empty + 8 * ((pos + k + 2) % kRing));
+                        mma_commit(empty + 8 * after(s0, 1));
+                        mma_commit(empty + 8 * after(s0, 2));
+                        s0 = after(s0, 2);
                     }
+                    s0 = after(s0, 1);
                 }
-                pos += cnt + 2;
             }
         }
         __syncwarp();
@@ -405,8 +416,9 @@ __global__ void __launch_bounds__(kConvThreads) k_conv(ConvArgs a) {
 // operand, whatever N.  A slot holds tap row (slot - first position) mod 4 of
 // the tile, so the accumulators are kept per class = first position mod 4; the
 // class's fourth slot (being loaded, or of the next item) yields rows nobody
-// reads.  Pixels past the image's last column are staged as zeros.  Bound by
-// the latency of the one x segment in flight (the ring's fourth slot).
+// reads.  Pixels past the image's last column are staged as zeros.  Not bound by the
+// one x segment in flight (the ring's fourth slot): three chains a CTA, each with
+// a ring, and five gradient stages measured 225 us where this form takes 195.
 // Measured, 8 images of 513^2: 2469 us a layer with a tap and 16 pixels an MMA
 // and nothing staged ahead, 253 us with the ring and one MMA a tap column, 195
 // us with one MMA for the three.
@@ -770,6 +782,7 @@ struct gcmg_cnn {
     int sms = 148;
     size_t guard = 0;            // zero rows before and after each channel group
     size_t smem_sm = 0;          // shared memory of an SM
+    size_t smem_cta = 0;         // of a CTA at most
     std::string err;
     std::vector<void *> allocs;
 };
@@ -803,8 +816,8 @@ int groups_in(int l) { return l == 0 ? 2 : 4; }
 int nout_of(int l) { return l == kLayers - 1 ? 16 : 32; }
 
 // shared memory of the convolution: the ring, the weights, the barriers
-size_t conv_smem(int gin, int nout, int dil) {
-    return (size_t)(kRing * gin * (kTile + 2 * dil) + 9 * gin * nout) * 16 + 16 * 16;
+size_t conv_smem(int gin, int nout, int dil, int ring) {
+    return (size_t)(ring * gin * (kTile + 2 * dil) + 9 * gin * nout) * 16 + (2 * kMaxRing + 2 * kAcc + 2) * 8;
 }
 // of the weight gradients: 16 channel groups of x (the MMA's M rows), the
 // staged gradients, the reduction buffer, the barriers; the kernel holds 512
@@ -860,9 +873,20 @@ void prep_weights(gcmg_cnn *c) {
 
 template <int GIN, int NOUT, int MODE>
 void launch_conv(gcmg_cnn *c, ConvArgs a) {
-    const size_t smem = conv_smem(GIN, NOUT, a.dil);
     // resident CTAs an SM: shared memory (1 KB each is the system's), TMEM columns
-    const int per_sm = std::max(1, std::min({(int)(c->smem_sm / (smem + 1024)), 512 / (kAcc * NOUT), 4}));
+    auto resident = [&](int ring) {
+        const size_t smem = conv_smem(GIN, NOUT, a.dil, ring);
+        return smem > c->smem_cta ? 0 : std::min({(int)(c->smem_sm / (smem + 1024)), 512 / (kAcc * NOUT), 4});
+    };
+    // the ring with the most segments in flight an SM of those that leave three
+    // CTAs there (or what the smallest ring leaves, if fewer): a forward pass of 8
+    // images of 513^2 takes 550 us with rings of 4, 509 so, 567 with two CTAs
+    a.ring = kRing;
+    const int least = std::min(3, resident(kRing));
+    for (int r = kRing + 1; r <= kMaxRing; r++)
+        if (resident(r) >= least && resident(r) * (r - 3) > resident(a.ring) * (a.ring - 3)) a.ring = r;
+    const size_t smem = conv_smem(GIN, NOUT, a.dil, a.ring);
+    const int per_sm = std::max(1, resident(a.ring));
     a.ch = make_chains(c, a.dil, per_sm * c->sms);
     const unsigned grid = (unsigned)std::min(a.ch.items, per_sm * c->sms);
     k_conv<GIN, NOUT, MODE><<<grid, kConvThreads, smem, c->stream>>>(a);
@@ -1019,6 +1043,7 @@ gcmg_status gcmg_cnn_create(int batch, int H, int W, const int *dilations, void 
         ck(cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, c->device), "attr");
         ck(cudaDeviceGetAttribute(&per_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, c->device), "attr");
         c->smem_sm = (size_t)per_sm;
+        c->smem_cta = (size_t)most;
         const auto allow = [&](auto *kernel) {
             ck(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, most), "attr");
         };
