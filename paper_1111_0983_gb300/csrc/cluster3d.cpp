@@ -5,6 +5,8 @@
 #include <algorithm>
 #include <atomic>
 #include <cstring>
+#include <exception>
+#include <mutex>
 #include <thread>
 
 namespace gcmg {
@@ -88,6 +90,34 @@ void bisect(std::vector<Node> &N, std::vector<Node> &tmp, size_t b, size_t e, in
     bisect(N, tmp, m, e, parts - parts / 2, first + parts / 2, start);
 }
 
+// f(0) .. f(n - 1), independent of each other, over the host's threads; an
+// exception of one (or of the creation of a thread) reaches the caller after all
+// threads have ended
+template <typename F>
+void for_each_index(int n, F &&f) {
+    std::atomic<int> next{0};
+    std::mutex lock;
+    std::exception_ptr error;
+    auto work = [&]() {
+        try {
+            for (int i = next++; i < n; i = next++) f(i);
+        } catch (...) {
+            next = n;
+            std::lock_guard<std::mutex> g(lock);
+            if (!error) error = std::current_exception();
+        }
+    };
+    std::vector<std::thread> pool;
+    try {
+        const unsigned nt = std::max(1u, std::min(16u, std::thread::hardware_concurrency()));
+        for (unsigned t = 1; t < nt; t++) pool.emplace_back(work);
+    } catch (...) {   // fewer threads then
+    }
+    work();
+    for (auto &t : pool) t.join();
+    if (error) std::rethrow_exception(error);
+}
+
 int align16(int x) { return (x + 15) & ~15; }
 
 }  // namespace
@@ -168,11 +198,11 @@ Cluster3Program build_cluster3(const HostLevel &L, bool band) {
     std::vector<std::vector<uint32_t>> cps(N.size());
     Cluster3Layout &y = out.lay;
     for (size_t i = 0; i < N.size(); i++) at.set(N[i].p, (int32_t)i);
-    for (int r = 0; r < C3_RANKS; r++) {
+    for (int r = 0; r < C3_RANKS; r++) slot.emplace_back(4 * (start[r + 1] - start[r]) + 16);
+    for_each_index(C3_RANKS, [&](int r) {
         Rank &K = R[r];
         const int32_t b0 = (int32_t)start[r], e0 = (int32_t)start[r + 1];
-        slot.emplace_back(4 * (size_t)(e0 - b0) + 16);
-        NodeMap &S = slot.back();
+        NodeMap &S = slot[r];
         for (int32_t i = b0; i < e0; i++) {
             std::vector<int32_t> &l = N[i].q >= 0 ? K.gs : K.in;
             S.set(N[i].p, (int32_t)l.size());
@@ -266,6 +296,8 @@ Cluster3Program build_cluster3(const HostLevel &L, bool band) {
                 S.set(p, (int32_t)K.gs.size());
                 K.gs.push_back(p);
             }
+    });
+    for (const Rank &K : R) {
         y.max_in = std::max(y.max_in, (int)K.in.size());
         y.max_gs = std::max(y.max_gs, (int)K.gs.size());
         y.max_e = std::max(y.max_e, (int)K.ent.size());
@@ -294,7 +326,7 @@ Cluster3Program build_cluster3(const HostLevel &L, bool band) {
     y.copies = y.gst + 64 * y.max_g;
     y.stride = align16(y.copies + 4 * max_c);
     out.records.assign((size_t)C3_RANKS * y.stride, 0);
-    for (int r = 0; r < C3_RANKS; r++) {
+    for_each_index(C3_RANKS, [&](int r) {
         const Rank &K = R[r];
         uint8_t *rec = out.records.data() + (size_t)r * y.stride;
         int32_t *h = reinterpret_cast<int32_t *>(rec);
@@ -353,7 +385,7 @@ Cluster3Program build_cluster3(const HostLevel &L, bool band) {
                 gst[((size_t)(k / 8) * y.max_g + ig) * 8 + k % 8] = k < 27 ? source(rd[k]) : copies_of(i);
             ig++;
         }
-    }
+    });
     return out;
 }
 
@@ -405,84 +437,74 @@ Sweep3Program build_sweep3(const HostLevel &L, int blocks) {
         int own_in = 0, own_g = 0;
     };
     std::vector<Block> B(blocks);
-    std::atomic<int> next{0};
-    auto work = [&]() {
+    auto work = [&](int r) {
         int64_t rd[27];
-        for (int r = next++; r < blocks; r = next++) {
-            Block &K = B[r];
-            const int32_t b0 = (int32_t)start[r], e0 = (int32_t)start[r + 1];
-            NodeMap S(6 * (size_t)(e0 - b0) + 64), in_ent(4 * (size_t)(e0 - b0) + 64);
-            auto reads = [&](const Node &x) {
-                if (x.q < 0) {   // the order of the sweeps' sum: axis 2, axis 0, axis 1
-                    const int64_t s[3] = {L.stride[2], L.stride[0], L.stride[1]};
-                    for (int a = 0; a < 3; a++) {
-                        rd[2 * a] = x.p - s[a];
-                        rd[2 * a + 1] = x.p + s[a];
-                    }
-                    return 6;
+        Block &K = B[r];
+        const int32_t b0 = (int32_t)start[r], e0 = (int32_t)start[r + 1];
+        NodeMap S(6 * (size_t)(e0 - b0) + 64), in_ent(4 * (size_t)(e0 - b0) + 64);
+        auto reads = [&](const Node &x) {
+            if (x.q < 0) {   // the order of the sweeps' sum: axis 2, axis 0, axis 1
+                const int64_t s[3] = {L.stride[2], L.stride[0], L.stride[1]};
+                for (int a = 0; a < 3; a++) {
+                    rd[2 * a] = x.p - s[a];
+                    rd[2 * a + 1] = x.p + s[a];
                 }
-                for (int k = 0; k < 27; k++) rd[k] = L.stn[(int64_t)x.q * KMAX + k];
-                return 27;
-            };
-            auto touch = [&](int64_t p) {
-                if (S.get(p, -1) >= 0) return;
-                const int32_t o = at.get(p, -1);
-                if ((L.type[p] & NODE_KIND) == NODE_GHOST) {
-                    S.set(p, (int32_t)K.gs.size());
-                    K.gs.push_back((int32_t)p);
-                    K.gs_q.push_back(N[o].q);   // every ghost is updated
-                } else {
-                    S.set(p, (int32_t)K.in.size());
-                    K.in.push_back((int32_t)p);
-                    K.in_cid.push_back(o < 0 ? -1 : cid[o]);
-                }
-            };
-            for (int32_t i = b0; i < e0; i++) {
-                touch(N[i].p);
-                if (N[i].q < 0) {
-                    in_ent.set(N[i].p, 1);
-                    (N[i].black ? K.black : K.red).push_back(i);
-                    K.own_in++;
-                } else {
-                    K.own_g++;
-                }
+                return 6;
             }
-            // the blacks the own ghosts read, the reds those blacks and ghosts read
-            auto cone = [&](int32_t i, int black) {
-                const int m = reads(N[i]);
-                for (int k = 0; k < m; k++) {
-                    const int32_t o = at.get(rd[k], -1);
-                    if (o < 0 || N[o].q >= 0 || N[o].black != black || in_ent.get(N[o].p, 0)) continue;
-                    in_ent.set(N[o].p, 1);
-                    (black ? K.black : K.red).push_back(o);
-                }
-            };
-            for (int32_t i = b0; i < e0; i++)
-                if (N[i].q >= 0) cone(i, 1);
-            for (size_t k = 0; k < K.black.size(); k++) cone(K.black[k], 0);
-            for (int32_t i = b0; i < e0; i++)
-                if (N[i].q >= 0) cone(i, 0);
-            for (const auto *l : {&K.red, &K.black})
-                for (int32_t i : *l) {
-                    touch(N[i].p);
-                    const int m = reads(N[i]);
-                    for (int k = 0; k < m; k++) touch(rd[k]);
-                }
-            for (int32_t i = b0; i < e0; i++)
-                if (N[i].q >= 0) {
-                    const int m = reads(N[i]);
-                    for (int k = 0; k < m; k++) touch(rd[k]);
-                }
+            for (int k = 0; k < 27; k++) rd[k] = L.stn[(int64_t)x.q * KMAX + k];
+            return 27;
+        };
+        auto touch = [&](int64_t p) {
+            if (S.get(p, -1) >= 0) return;
+            const int32_t o = at.get(p, -1);
+            if ((L.type[p] & NODE_KIND) == NODE_GHOST) {
+                S.set(p, (int32_t)K.gs.size());
+                K.gs.push_back((int32_t)p);
+                K.gs_q.push_back(N[o].q);   // every ghost is updated
+            } else {
+                S.set(p, (int32_t)K.in.size());
+                K.in.push_back((int32_t)p);
+                K.in_cid.push_back(o < 0 ? -1 : cid[o]);
+            }
+        };
+        for (int32_t i = b0; i < e0; i++) {
+            touch(N[i].p);
+            if (N[i].q < 0) {
+                in_ent.set(N[i].p, 1);
+                (N[i].black ? K.black : K.red).push_back(i);
+                K.own_in++;
+            } else {
+                K.own_g++;
+            }
         }
+        // the blacks the own ghosts read, the reds those blacks and ghosts read
+        auto cone = [&](int32_t i, int black) {
+            const int m = reads(N[i]);
+            for (int k = 0; k < m; k++) {
+                const int32_t o = at.get(rd[k], -1);
+                if (o < 0 || N[o].q >= 0 || N[o].black != black || in_ent.get(N[o].p, 0)) continue;
+                in_ent.set(N[o].p, 1);
+                (black ? K.black : K.red).push_back(o);
+            }
+        };
+        for (int32_t i = b0; i < e0; i++)
+            if (N[i].q >= 0) cone(i, 1);
+        for (size_t k = 0; k < K.black.size(); k++) cone(K.black[k], 0);
+        for (int32_t i = b0; i < e0; i++)
+            if (N[i].q >= 0) cone(i, 0);
+        for (const auto *l : {&K.red, &K.black})
+            for (int32_t i : *l) {
+                touch(N[i].p);
+                const int m = reads(N[i]);
+                for (int k = 0; k < m; k++) touch(rd[k]);
+            }
+        for (int32_t i = b0; i < e0; i++)
+            if (N[i].q >= 0) {
+                const int m = reads(N[i]);
+                for (int k = 0; k < m; k++) touch(rd[k]);
+            }
     };
-    auto parallel = [](auto &&f) {
-        std::vector<std::thread> pool;
-        const unsigned nt = std::max(1u, std::min(16u, std::thread::hardware_concurrency()));
-        for (unsigned t = 1; t < nt; t++) pool.emplace_back(f);
-        f();
-        for (auto &t : pool) t.join();
-    };
-    parallel(work);
+    for_each_index(blocks, work);
     Sweep3Layout &y = out.lay;
     y.blocks = blocks;
     y.inside = base[blocks];
@@ -501,44 +523,41 @@ Sweep3Program build_sweep3(const HostLevel &L, int blocks) {
     y.gst = y.ent + 16 * y.max_e;
     y.stride = y.gst + 64 * y.max_g;
     out.records.assign((size_t)blocks * y.stride, 0);
-    next = 0;
-    auto write = [&]() {
-        for (int r = next++; r < blocks; r = next++) {
-            const Block &K = B[r];
-            NodeMap S(2 * (K.in.size() + K.gs.size()) + 64);
-            for (size_t i = 0; i < K.in.size(); i++) S.set(K.in[i], (int32_t)i);
-            for (size_t i = 0; i < K.gs.size(); i++) S.set(K.gs[i], y.max_in + (int32_t)i);
-            uint8_t *rec = out.records.data() + (size_t)r * y.stride;
-            int32_t *h = reinterpret_cast<int32_t *>(rec);
-            h[S3_NIN] = (int)K.in.size();
-            h[S3_NGS] = (int)K.gs.size();
-            h[S3_OWN_IN] = K.own_in;
-            h[S3_OWN_G] = K.own_g;
-            h[S3_RED] = (int)K.red.size();
-            h[S3_NE] = (int)(K.red.size() + K.black.size());
-            h[S3_BASE] = base[r];
-            std::copy(K.in.begin(), K.in.end(), reinterpret_cast<int32_t *>(rec + y.node));
-            std::copy(K.in_cid.begin(), K.in_cid.end(), reinterpret_cast<int32_t *>(rec + y.cid));
-            std::copy(K.gs_q.begin(), K.gs_q.end(), reinterpret_cast<int32_t *>(rec + y.gslot));
-            uint16_t *e = reinterpret_cast<uint16_t *>(rec + y.ent), *g = reinterpret_cast<uint16_t *>(rec + y.gst);
-            const int64_t s[3] = {L.stride[2], L.stride[0], L.stride[1]};
-            for (const auto *l : {&K.red, &K.black})
-                for (int32_t i : *l) {
-                    const int64_t p = N[i].p;
-                    e[0] = (uint16_t)S.get(p, 0);
-                    for (int a = 0; a < 3; a++) {
-                        e[1 + 2 * a] = (uint16_t)S.get(p - s[a], 0);
-                        e[2 + 2 * a] = (uint16_t)S.get(p + s[a], 0);
-                    }
-                    e += 8;
+    auto write = [&](int r) {
+        const Block &K = B[r];
+        NodeMap S(2 * (K.in.size() + K.gs.size()) + 64);
+        for (size_t i = 0; i < K.in.size(); i++) S.set(K.in[i], (int32_t)i);
+        for (size_t i = 0; i < K.gs.size(); i++) S.set(K.gs[i], y.max_in + (int32_t)i);
+        uint8_t *rec = out.records.data() + (size_t)r * y.stride;
+        int32_t *h = reinterpret_cast<int32_t *>(rec);
+        h[S3_NIN] = (int)K.in.size();
+        h[S3_NGS] = (int)K.gs.size();
+        h[S3_OWN_IN] = K.own_in;
+        h[S3_OWN_G] = K.own_g;
+        h[S3_RED] = (int)K.red.size();
+        h[S3_NE] = (int)(K.red.size() + K.black.size());
+        h[S3_BASE] = base[r];
+        std::copy(K.in.begin(), K.in.end(), reinterpret_cast<int32_t *>(rec + y.node));
+        std::copy(K.in_cid.begin(), K.in_cid.end(), reinterpret_cast<int32_t *>(rec + y.cid));
+        std::copy(K.gs_q.begin(), K.gs_q.end(), reinterpret_cast<int32_t *>(rec + y.gslot));
+        uint16_t *e = reinterpret_cast<uint16_t *>(rec + y.ent), *g = reinterpret_cast<uint16_t *>(rec + y.gst);
+        const int64_t s[3] = {L.stride[2], L.stride[0], L.stride[1]};
+        for (const auto *l : {&K.red, &K.black})
+            for (int32_t i : *l) {
+                const int64_t p = N[i].p;
+                e[0] = (uint16_t)S.get(p, 0);
+                for (int a = 0; a < 3; a++) {
+                    e[1 + 2 * a] = (uint16_t)S.get(p - s[a], 0);
+                    e[2 + 2 * a] = (uint16_t)S.get(p + s[a], 0);
                 }
-            for (int k = 0; k < K.own_g; k++)
-                for (int a = 0; a < 27; a++)
-                    g[((size_t)(a / 8) * y.max_g + k) * 8 + a % 8] =
-                        (uint16_t)S.get(L.stn[(int64_t)K.gs_q[k] * KMAX + a], 0);
-        }
+                e += 8;
+            }
+        for (int k = 0; k < K.own_g; k++)
+            for (int a = 0; a < 27; a++)
+                g[((size_t)(a / 8) * y.max_g + k) * 8 + a % 8] =
+                    (uint16_t)S.get(L.stn[(int64_t)K.gs_q[k] * KMAX + a], 0);
     };
-    parallel(write);
+    for_each_index(blocks, write);
     return out;
 }
 
