@@ -332,9 +332,10 @@ gcmg_status gcmg_kernel_timing_ex(gcmg_ctx *ctx, int64_t *launches, double *tota
  * of Sec. 3.2 and the junction sweeps) is launched; every mode gives the same
  * results bitwise.  mode 0 (default): on small levels all phases, on the
  * others the junction sweeps, as one thread-block cluster whose CTAs hold the
- * values in shared memory and send each other what they read; the remaining
- * phases one launch each, the store of each Jacobi ghost sweep merged into the
- * launch of the next red band or junction-zone sweep; 1: on levels whose ghost, band and junction lists
+ * values in shared memory and send each other what they read; the band sweeps of
+ * the others a launch each over blocks in shared memory; what neither takes one
+ * launch a phase, the store of each Jacobi ghost sweep merged into the launch of
+ * the next red band or junction-zone sweep; 1: on levels whose ghost, band and junction lists
  * hold at most 65,536 entries all phases as one thread-block cluster of 16
  * CTAs with hardware barriers between them and the values in global memory,
  * one launch a phase on the other levels; 2: all phases as one grid with
