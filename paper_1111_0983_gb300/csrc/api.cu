@@ -242,8 +242,23 @@ void free_tracked(gcmg_ctx *c, void *p) {
         }
 }
 
+void destroy_graph(gcmg_ctx *c) {
+    if (c->gexec) cudaGraphExecDestroy(c->gexec);
+    if (c->graph) cudaGraphDestroy(c->graph);
+    c->gexec = nullptr;
+    c->graph = nullptr;
+}
+
+// device arrays that launches take by pointer move: a captured graph of this
+// context holds the old ones, and so do the tables of a batch it belongs to
+void arrays_move(gcmg_ctx *c) {
+    destroy_graph(c);
+    c->version++;
+}
+
 // (re)uploads a local program of level l
 void upload_program(gcmg_ctx *c, const LocalProgram &J, LocalDev &z) {
+    arrays_move(c);
     int32_t **arrs[] = {&z.node_off, &z.wb_cnt, &z.lnode, &z.int_off, &z.red_cnt, &z.int_glob,
                         &z.int_me, &z.int_nb, &z.gh_off, &z.gh_me, &z.gh_q, &z.gh_stn,
                         &z.zred, &z.zblack, &z.zghost, &z.wb_list, &z.node_base, &z.zred_src};
@@ -832,13 +847,6 @@ void loop_body(gcmg_ctx *c) {
     fine_defect(c);
 }
 
-void destroy_graph(gcmg_ctx *c) {
-    if (c->gexec) cudaGraphExecDestroy(c->gexec);
-    if (c->graph) cudaGraphDestroy(c->graph);
-    c->gexec = nullptr;
-    c->graph = nullptr;
-}
-
 void build_graph(gcmg_ctx *c) {
     destroy_graph(c);
     if (!c->gstream) ck(cudaStreamCreateWithFlags(&c->gstream, cudaStreamNonBlocking), "cudaStreamCreate");
@@ -1029,6 +1037,7 @@ void upload_inverse(gcmg_ctx *c) {
 
 // (re)uploads the exact junction solve of level l
 void upload_js(gcmg_ctx *c, int l) {
+    arrays_move(c);
     const HostLevel &L = c->H[l];
     DevGeom &g = c->G[l];
     for (int32_t **a : {&g.js_node, &g.js_ghost, &g.js_comp, &g.js_off, &g.js_roff, &g.js_rpos}) {
@@ -1157,7 +1166,6 @@ void ensure_junction_solve(gcmg_ctx *c) {
     for (int l = 0; l < (int)c->H.size(); l++) {
         HostLevel &L = c->H[l];
         if (!L.js_dirty) continue;
-        destroy_graph(c);   // a captured graph holds the arrays reallocated below
         build_junction_solve(L, c->p.junction_radius);
         upload_js(c, l);
         L.js_dirty = false;
@@ -1322,8 +1330,7 @@ gcmg_status gcmg_set_bc_types(gcmg_ctx *c, int l, const uint8_t *types) {
     GCMG_GUARD(c, {
         ck(cudaSetDevice(c->device), "cudaSetDevice");
         HostLevel &L = c->H[l];
-        destroy_graph(c);   // the junction arrays are reallocated below
-        c->version++;
+        arrays_move(c);   // the junction arrays are reallocated below
         for (int64_t q = 0; q < L.ng(); q++) L.bc[q] = types[q] ? 1 : 0;
         if (l + 1 == (int)c->H.size()) L.ainv_dirty = true;   // rebuilt before the next solve
         if (c->p.junction_solve) {
@@ -1770,7 +1777,6 @@ gcmg_status gcmg_relax(gcmg_ctx *c, int l, double *u, const double *f, const dou
             c->js64 = true;
             for (int k = 0; k < (int)c->H.size(); k++) {
                 if (c->H[k].js_node.empty() || c->D64[k].js_inv) continue;
-                destroy_graph(c);   // a captured graph holds the arrays reallocated below
                 upload_js(c, k);
             }
         }

@@ -85,7 +85,7 @@ struct gcmg_ctx {
     std::vector<int64_t> bz_units;         // per level: distinct values a boundary-block launch moves
     std::vector<void *> allocs;
     std::string err;
-    int version = 0;                        // bumped when the boundary types change
+    int version = 0;                        // bumped when device arrays move (a batch's tables hold them)
 };
 
 
