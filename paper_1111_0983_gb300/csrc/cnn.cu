@@ -218,6 +218,7 @@ __global__ void __launch_bounds__(kConvThreads) k_conv(ConvArgs a) {
     uint4 *sw = sx + a.ring * GIN * seg;                           // 9 * GIN * NOUT rows
     uint64_t *bars = reinterpret_cast<uint64_t *>(sw + 9 * GIN * NOUT);
     uint32_t *tslot = reinterpret_cast<uint32_t *>(bars + 2 * kMaxRing + 2 * kAcc + 1);
+    float *part = reinterpret_cast<float *>(tslot + 2);            // MODE 2: a warp's sums, NOUT each
     const uint32_t full = smem_u32(bars), empty = full + 8 * kMaxRing, afull = empty + 8 * kMaxRing,
                    afree = afull + 8 * kAcc, wbar = afree + 8 * kAcc;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -389,13 +390,18 @@ __global__ void __launch_bounds__(kConvThreads) k_conv(ConvArgs a) {
                 }
             }
         }
+        // one sum a CTA: the atomics of all CTAs go to the same NOUT words, one after
+        // the other (16 images of 128 x 16, 456 CTAs: 63-72 us a layer with a sum a warp, 18 so)
         if (MODE == 2) {
 #pragma unroll
             for (int e = 0; e < NOUT; e++) {
                 float s = dbs[e];
                 for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-                if (lane == 0) atomicAdd(&a.db[e], s);
+                if (lane == 0) part[ew * NOUT + e] = s;
             }
+            asm volatile("bar.sync 1, 128;" ::: "memory");   // the epilogue warps
+            const int e = ew * 32 + lane;
+            if (e < NOUT) atomicAdd(&a.db[e], (part[e] + part[NOUT + e]) + (part[2 * NOUT + e] + part[3 * NOUT + e]));
         }
     }
     if (!ok) atomicExch(a.err, 1);
@@ -815,9 +821,9 @@ T *alloc(gcmg_cnn *c, size_t n) {
 int groups_in(int l) { return l == 0 ? 2 : 4; }
 int nout_of(int l) { return l == kLayers - 1 ? 16 : 32; }
 
-// shared memory of the convolution: the ring, the weights, the barriers
+// shared memory of the convolution: the ring, the weights, the barriers, the epilogue warps' sums
 size_t conv_smem(int gin, int nout, int dil, int ring) {
-    return (size_t)(ring * gin * (kTile + 2 * dil) + 9 * gin * nout) * 16 + (2 * kMaxRing + 2 * kAcc + 2) * 8;
+    return (size_t)(ring * gin * (kTile + 2 * dil) + 9 * gin * nout) * 16 + (2 * kMaxRing + 2 * kAcc + 2) * 8 + 16 * nout;
 }
 // of the weight gradients: 16 channel groups of x (the MMA's M rows), the
 // staged gradients, the reduction buffer, the barriers; the kernel holds 512
