@@ -15,8 +15,11 @@
 // 128 of the MMAs).  With dilation d the tiles of rows i, i + d, i + 2d, ... in
 // one column of tiles share their input rows: row i is tap row +1, 0 and -1 of
 // three successive tiles.  A CTA therefore walks down such a chain with a ring
-// of four row segments of 128 + 2d pixels in shared memory: each tile brings in
-// one new segment (18.6 KB at d = 81) instead of three.
+// of row segments of 128 + 2d pixels in shared memory (four to eight in the
+// convolution, as shared memory allows; four of 128 in the weight gradients):
+// each tile brings in one new segment (18.6 KB at d = 81) instead of three.
+// Images much narrower than 128 pixels take tiles over their flattened rows, each
+// with three segments of its own (cnn_tiles.h).
 //
 // Convolution (forward, and backward to the input): N = output channels, K =
 // input channels in slices of 16, summed over the 9 taps.  Warp roles: a
@@ -37,19 +40,24 @@
 #include <string>
 #include <vector>
 
+#include "cnn_tiles.h"
 #include "gcmg_cnn.h"
 
 namespace {
 
+using namespace gcmg_cnn_tiles;
+
 constexpr int kLayers = 6;
 constexpr int kCin[kLayers] = {4, 32, 32, 32, 32, 32};
 constexpr int kCout[kLayers] = {32, 32, 32, 32, 32, 2};
-constexpr int kTile = 128;            // pixels per CTA (M)
 constexpr int kMaxDil = 96;
 constexpr int kRing = 4;              // row segments in shared memory (convolution: at least,
 constexpr int kMaxRing = 8;           // and at most, see ConvArgs::ring)
 constexpr int kAcc = 4;               // TMEM accumulators of the convolution
 constexpr int kDzStages = 4;          // staged gradient tiles of the weight gradients
+// a CTA's share of the bias gradients (an atomic to each of the same 32 words, 26
+// ns) in tiles of the convolution (0.6 us)
+constexpr double kDbCta = 1.0 / 20;
 constexpr int kConvThreads = 192;     // producer, MMA issuer, four epilogue warps
 constexpr long kWaitLimit = 1L << 22; // bounded mbarrier polls
 
@@ -144,31 +152,7 @@ __device__ __forceinline__ uint32_t pack_bf16(float a, float b) {
 __device__ __forceinline__ float bf16_lo(uint32_t w) { return __uint_as_float(w << 16); }
 __device__ __forceinline__ float bf16_hi(uint32_t w) { return __uint_as_float(w & 0xFFFF0000u); }
 
-struct Geo {
-    int npix, Hp, Wp, H, W, P;
-    int gs;        // rows between channel groups (npix plus zero guard rows on both sides)
-};
-
 // ------------------------------------------------------------ convolution
-// Chains: item = ((image * cols + column) * res + residue) * parts + part; its
-// tiles are rows residue + (part * len + k) * dil, k < cnt.
-struct Chains {
-    int H, dil, cols, res, parts, len, items;
-    // false: the part lies past the chain's end
-    __device__ __forceinline__ bool item(int t, int *b, int *c, int *row0, int *cnt) const {
-        const int part = t % parts;
-        t /= parts;
-        const int r = t % res;
-        t /= res;
-        *c = t % cols;
-        *b = t / cols;
-        const int n = (H - r + dil - 1) / dil, j0 = part * len;
-        *row0 = r + j0 * dil;
-        *cnt = min(len, n - j0);
-        return *cnt > 0;
-    }
-};
-
 // MODE 0: y = bf16(relu(acc + bias)); 1: out[b][c][i][j] = acc + bias (c < 2);
 // 2: y = bf16(acc * (gate > 0)) (backward to the input of the layer below) and
 // db[c] += the sum of the stored values over the pixels
@@ -181,7 +165,7 @@ struct ConvArgs {
     const uint4 *gate;    // MODE 2: [NOUT / 8][npix]
     float *db;            // MODE 2: NOUT
     Geo geo;
-    Chains ch;
+    Tiles ch;
     int dil;
     int ring;             // segments in shared memory
     int *err;
@@ -243,7 +227,7 @@ __global__ void __launch_bounds__(kConvThreads) k_conv(ConvArgs a) {
     auto wait = [&](uint32_t bar, uint32_t parity) {
         if (ok) ok = mbar_wait(bar, parity & 1u);
     };
-    int b, c, row0, cnt;
+    TileItem it;
 
     if (warp == 0) {
         if (lane == 0) {   // producer
@@ -251,10 +235,10 @@ __global__ void __launch_bounds__(kConvThreads) k_conv(ConvArgs a) {
             bulk_g2s(smem_u32(sw), a.w, 9 * GIN * NOUT * 16, wbar);
             int s = 0, round = 0, sent = 0;   // slot of the next position and how often the ring was filled
             for (int t = blockIdx.x; t < a.ch.items; t += gridDim.x) {
-                if (!a.ch.item(t, &b, &c, &row0, &cnt)) continue;
-                // pixel of the first segment: row row0 - dil, columns from dil before the tile
-                long q = ((long)b * a.geo.Hp + a.geo.P + row0 - a.dil) * a.geo.Wp + a.geo.P + c * kTile - a.dil;
-                for (int p = 0; p < cnt + 2; p++, q += (long)a.dil * a.geo.Wp) {
+                if (!a.ch.item(a.geo, t, &it)) continue;
+                // pixel of the first segment: dil rows and dil columns before the tile
+                long q = it.q - (long)a.dil * a.geo.Wp - a.dil;
+                for (int p = 0; p < it.cnt + 2; p++, q += (long)a.dil * a.geo.Wp) {
                     wait(empty + 8 * s, (uint32_t)round + 1u);
                     if (!ok) break;
                     mbar_expect(full + 8 * s, (uint32_t)(GIN * seg * 16));
@@ -284,8 +268,8 @@ __global__ void __launch_bounds__(kConvThreads) k_conv(ConvArgs a) {
             auto after = [&](int i, int d) { return i + d < a.ring ? i + d : i + d - a.ring; };
             wait(wbar, 0);
             for (int t = blockIdx.x; t < a.ch.items && ok; t += gridDim.x) {
-                if (!a.ch.item(t, &b, &c, &row0, &cnt)) continue;
-                for (int k = 0; k < cnt; k++, tile++) {
+                if (!a.ch.item(a.geo, t, &it)) continue;
+                for (int k = 0; k < it.cnt; k++, tile++) {
                     for (int p = k ? 2 : 0; p < 3; p++) {
                         wait(full + 8 * sn, (uint32_t)round);
                         if (++sn == a.ring) sn = 0, round++;
@@ -312,7 +296,7 @@ __global__ void __launch_bounds__(kConvThreads) k_conv(ConvArgs a) {
                     }
                     mma_commit(afull + 8 * ac);
                     mma_commit(empty + 8 * s0);
-                    if (k + 1 == cnt) {   // the item's last two segments serve no other tile
+                    if (k + 1 == it.cnt) {   // the item's last two segments serve no other tile
                         mma_commit(empty + 8 * after(s0, 1));
                         mma_commit(empty + 8 * after(s0, 2));
                         s0 = after(s0, 2);
@@ -335,12 +319,11 @@ __global__ void __launch_bounds__(kConvThreads) k_conv(ConvArgs a) {
         }
         int tile = 0;
         for (int t = blockIdx.x; t < a.ch.items && ok; t += gridDim.x) {
-            if (!a.ch.item(t, &b, &c, &row0, &cnt)) continue;
-            const int j = c * kTile + ew * 32 + lane;
-            const bool in = j < a.geo.W;
-            for (int k = 0; k < cnt && ok; k++, tile++) {
-                const int i = row0 + k * a.dil;
-                const long q = ((long)b * a.geo.Hp + a.geo.P + i) * a.geo.Wp + a.geo.P + j;
+            if (!a.ch.item(a.geo, t, &it)) continue;
+            for (int k = 0; k < it.cnt && ok; k++, tile++) {
+                int i, j;
+                const bool in = a.ch.at(a.geo, it, k, ew * 32 + lane, &i, &j);
+                const long q = it.q + (long)k * a.dil * a.geo.Wp + ew * 32 + lane;
                 uint4 gt[MODE == 2 ? NOUT / 8 : 1];
                 if (MODE == 2 && in) {
 #pragma unroll
@@ -360,7 +343,7 @@ __global__ void __launch_bounds__(kConvThreads) k_conv(ConvArgs a) {
                 if (!in) continue;
                 if (MODE == 1) {
                     for (int ch = 0; ch < 2; ch++)
-                        a.out[(((size_t)b * 2 + ch) * a.geo.H + i) * a.geo.W + j] = v[ch] + a.bias[ch];
+                        a.out[(((size_t)it.b * 2 + ch) * a.geo.H + i) * a.geo.W + j] = v[ch] + a.bias[ch];
                 } else {
 #pragma unroll
                     for (int g = 0; g < NOUT / 8; g++) {
@@ -434,7 +417,7 @@ struct DwArgs {
     float *dw;            // [co][ci][9] of this layer (FP32, accumulated)
     int cout, cin;        // real channel counts
     Geo geo;
-    Chains ch;
+    Tiles ch;
     int dil;
     int *err;
 };
@@ -473,25 +456,24 @@ __global__ void __launch_bounds__(128, 1) k_conv_dw(DwArgs a) {
     auto wait = [&](uint32_t bar, uint32_t parity) {
         if (ok) ok = mbar_wait(bar, parity & 1u);
     };
-    int b, c, row0, cnt;
+    TileItem it;
     unsigned used = 0;   // classes with an accumulator (the same in every thread)
     {
         int pos = 0;
         for (int t = blockIdx.x; t < a.ch.items; t += gridDim.x) {
-            if (!a.ch.item(t, &b, &c, &row0, &cnt)) continue;
-            for (int k = 0; k < min(cnt, kRing); k++) used |= 1u << ((pos + k) % kRing);
-            pos += cnt + 2;
+            if (!a.ch.item(a.geo, t, &it)) continue;
+            for (int k = 0; k < min(it.cnt, kRing); k++) used |= 1u << ((pos + k) % kRing);
+            pos += it.cnt + 2;
         }
     }
 
     if (warp == 0) {   // producer (the whole warp: it zeroes the tail of a gradient tile)
         int pos = 0, tile = 0;
         for (int t = blockIdx.x; t < a.ch.items && ok; t += gridDim.x) {
-            if (!a.ch.item(t, &b, &c, &row0, &cnt)) continue;
-            const long q0 = ((long)b * a.geo.Hp + a.geo.P + row0) * a.geo.Wp + a.geo.P + c * kTile;
-            const int width = min(kTile, a.geo.W - c * kTile), padded = (width + 15) & ~15;
-            for (int p = 0; p < cnt + 2 && ok; p++, pos++) {
-                const long q = q0 + (long)(p - 1) * a.dil * a.geo.Wp;
+            if (!a.ch.item(a.geo, t, &it)) continue;
+            const int width = it.width, padded = (width + 15) & ~15;
+            for (int p = 0; p < it.cnt + 2 && ok; p++, pos++) {
+                const long q = it.q + (long)(p - 1) * a.dil * a.geo.Wp;
                 const int s = pos % kRing;
                 wait(empty + 8 * s, (uint32_t)(pos / kRing) + 1u);
                 ok = __all_sync(0xffffffffu, ok);
@@ -502,7 +484,7 @@ __global__ void __launch_bounds__(128, 1) k_conv_dw(DwArgs a) {
                         bulk_g2s(smem_u32(sx + (s * GB + g) * kTile), a.x + (long)g * a.geo.gs + q, kTile * 16,
                                  full + 8 * s);
                 }
-                if (p < 1 || p > cnt) continue;   // the gradient tile of this row
+                if (p < 1 || p > it.cnt) continue;   // the gradient tile of this row
                 const int z = tile % kDzStages;
                 wait(zempty + 8 * z, (uint32_t)(tile / kDzStages) + 1u);
                 ok = __all_sync(0xffffffffu, ok);
@@ -540,9 +522,9 @@ __global__ void __launch_bounds__(128, 1) k_conv_dw(DwArgs a) {
             int pos = 0, tile = 0;
             unsigned begun = 0;
             for (int t = blockIdx.x; t < a.ch.items && ok; t += gridDim.x) {
-                if (!a.ch.item(t, &b, &c, &row0, &cnt)) continue;
-                const int steps = (min(kTile, a.geo.W - c * kTile) + 15) / 16;
-                for (int k = 0; k < cnt; k++, tile++) {
+                if (!a.ch.item(a.geo, t, &it)) continue;
+                const int steps = (it.width + 15) / 16;
+                for (int k = 0; k < it.cnt; k++, tile++) {
                     for (int p = k ? pos + k + 2 : pos; p <= pos + k + 2; p++)
                         wait(full + 8 * (p % kRing), (uint32_t)(p / kRing));
                     const int z = tile % kDzStages, cls = (pos + k) % kRing;
@@ -558,12 +540,12 @@ __global__ void __launch_bounds__(128, 1) k_conv_dw(DwArgs a) {
                     begun |= 1u << cls;
                     mma_commit(zempty + 8 * z);
                     mma_commit(empty + 8 * cls);
-                    if (k + 1 == cnt) {
+                    if (k + 1 == it.cnt) {
                         mma_commit(empty + 8 * ((pos + k + 1) % kRing));
                         mma_commit(empty + 8 * ((pos + k + 2) % kRing));
                     }
                 }
-                pos += cnt + 2;
+                pos += it.cnt + 2;
             }
             mma_commit(done);
             if (!mbar_wait(done, 0)) ok = false;
@@ -833,26 +815,6 @@ size_t dw_smem(int ga) {
     return std::max(need, (size_t)120 * 1024);
 }
 
-// work items of a chain kernel: chains cut into parts of at most `len` tiles,
-// short enough that every resident CTA (`slots`) gets about three
-Chains make_chains(const gcmg_cnn *c, int dil, int slots) {
-    Chains h;
-    h.H = c->H;
-    h.dil = dil;
-    h.cols = (c->W + kTile - 1) / kTile;
-    h.res = std::min(dil, c->H);
-    const int nmax = (c->H + dil - 1) / dil;   // tiles of the longest chain
-    const int64_t chains = (int64_t)c->batch * h.cols * h.res;
-    // a part of n tiles loads n + 2 segments: parts below 8 tiles only where a
-    // chain is that short or the CTAs would idle
-    const int64_t want = std::max<int64_t>(1, (int64_t)3 * slots / chains);
-    int len = std::max<int>(4, (int)((nmax + want - 1) / want));
-    h.parts = (nmax + len - 1) / len;
-    h.len = (nmax + h.parts - 1) / h.parts;
-    h.items = (int)(chains * h.parts);
-    return h;
-}
-
 #define CNN_GUARD(c, ...)                                             \
     try {                                                             \
         __VA_ARGS__                                                   \
@@ -893,17 +855,15 @@ void launch_conv(gcmg_cnn *c, ConvArgs a) {
         if (resident(r) >= least && resident(r) * (r - 3) > resident(a.ring) * (a.ring - 3)) a.ring = r;
     const size_t smem = conv_smem(GIN, NOUT, a.dil, a.ring);
     const int per_sm = std::max(1, resident(a.ring));
-    a.ch = make_chains(c, a.dil, per_sm * c->sms);
-    const unsigned grid = (unsigned)std::min(a.ch.items, per_sm * c->sms);
-    k_conv<GIN, NOUT, MODE><<<grid, kConvThreads, smem, c->stream>>>(a);
+    a.ch = make_tiles(c->geo, c->batch, a.dil, c->sms, per_sm, MODE == 2 ? kDbCta : 0.0);
+    k_conv<GIN, NOUT, MODE><<<(unsigned)a.ch.grid, kConvThreads, smem, c->stream>>>(a);
     ck(cudaGetLastError(), "conv launch");
 }
 
 template <int GA, int GB>
 void launch_dw(gcmg_cnn *c, DwArgs d) {
-    d.ch = make_chains(c, d.dil, c->sms);
-    const unsigned grid = (unsigned)std::min(d.ch.items, c->sms);
-    k_conv_dw<GA, GB><<<grid, 128, dw_smem(GA), c->stream>>>(d);
+    d.ch = make_tiles(c->geo, c->batch, d.dil, c->sms, 1, 0.0);
+    k_conv_dw<GA, GB><<<(unsigned)d.ch.grid, 128, dw_smem(GA), c->stream>>>(d);
     ck(cudaGetLastError(), "dw launch");
 }
 
