@@ -405,6 +405,12 @@ gcmg_status gcmg_span3d_info(const gcmg_ctx *ctx, int l, int *items, int *column
 /* Number of CUDA kernels this library has launched in the process so far. */
 int64_t gcmg_launch_counter(void);
 
+/* Number of 3D launch programs (cluster programs and band-sweep blocks, launch
+ * mode 0 of gcmg_set_boundary3d) built on the host in the process so far: one a
+ * level at creation or before its first relaxation, again after its boundary
+ * types changed. */
+int64_t gcmg_program_build_counter(void);
+
 /* ---- batched solves of many domains (not in the paper).
  * Independent 2D domains of uneven grid sizes are solved together: each step
  * of the cycle is one kernel launch over all domains and the whole solve --

@@ -56,6 +56,62 @@ struct Node {
     uint8_t black, inband, inzone;
 };
 
+// f(0) .. f(n - 1), independent of each other, over at most `most` of the host's
+// threads (the work's share of one should outweigh its start); an exception of one (or of the creation of a thread) reaches the caller after all
+// threads have ended
+template <typename F>
+void for_each_index(int n, size_t most, F &&f) {
+    std::atomic<int> next{0};
+    std::mutex lock;
+    std::exception_ptr error;
+    auto work = [&]() {
+        try {
+            for (int i = next++; i < n; i = next++) f(i);
+        } catch (...) {
+            next = n;
+            std::lock_guard<std::mutex> g(lock);
+            if (!error) error = std::current_exception();
+        }
+    };
+    std::vector<std::thread> pool;
+    try {
+        const unsigned nt = std::min({(unsigned)std::min<size_t>(most, 16), (unsigned)n, std::thread::hardware_concurrency()});
+        for (unsigned t = 1; t < nt; t++) pool.emplace_back(work);
+    } catch (...) {   // fewer threads then
+    }
+    work();
+    for (auto &t : pool) t.join();
+    if (error) std::rethrow_exception(error);
+}
+
+// f and g, at the same time if `apart` (and a thread can be had); an exception of
+// either reaches the caller after both have ended
+template <typename F, typename G>
+void both(bool apart, F &&f, G &&g) {
+    std::exception_ptr error;
+    std::thread t;
+    if (apart) try {
+            t = std::thread([&]() {
+                try {
+                    f();
+                } catch (...) {
+                    error = std::current_exception();
+                }
+            });
+        } catch (...) {   // here then
+            apart = false;
+        }
+    try {
+        if (!apart) f();
+        g();
+    } catch (...) {
+        if (t.joinable()) t.join();
+        throw;
+    }
+    if (t.joinable()) t.join();
+    if (error) std::rethrow_exception(error);
+}
+
 // splits nodes [b, e) into `parts` ranges of about equal weight by cutting the
 // longest axis of their box at the weighted share, again and again
 void bisect(std::vector<Node> &N, std::vector<Node> &tmp, size_t b, size_t e, int parts, int first,
@@ -86,43 +142,18 @@ void bisect(std::vector<Node> &N, std::vector<Node> &tmp, size_t b, size_t e, in
     std::copy(tmp.begin() + b, tmp.begin() + e, N.begin() + b);
     size_t m = b;
     while (m < e && parts * run < total * (parts / 2)) run += weight(N[m++]);
-    bisect(N, tmp, b, m, parts / 2, first, start);
-    bisect(N, tmp, m, e, parts - parts / 2, first + parts / 2, start);
-}
-
-// f(0) .. f(n - 1), independent of each other, over the host's threads; an
-// exception of one (or of the creation of a thread) reaches the caller after all
-// threads have ended
-template <typename F>
-void for_each_index(int n, F &&f) {
-    std::atomic<int> next{0};
-    std::mutex lock;
-    std::exception_ptr error;
-    auto work = [&]() {
-        try {
-            for (int i = next++; i < n; i = next++) f(i);
-        } catch (...) {
-            next = n;
-            std::lock_guard<std::mutex> g(lock);
-            if (!error) error = std::current_exception();
-        }
-    };
-    std::vector<std::thread> pool;
-    try {
-        const unsigned nt = std::max(1u, std::min(16u, std::thread::hardware_concurrency()));
-        for (unsigned t = 1; t < nt; t++) pool.emplace_back(work);
-    } catch (...) {   // fewer threads then
-    }
-    work();
-    for (auto &t : pool) t.join();
-    if (error) std::rethrow_exception(error);
+    both(e - b > 4096, [&]() { bisect(N, tmp, b, m, parts / 2, first, start); },
+         [&]() { bisect(N, tmp, m, e, parts - parts / 2, first + parts / 2, start); });
 }
 
 int align16(int x) { return (x + 15) & ~15; }
 
 }  // namespace
 
+std::atomic<long long> g_program_builds{0};
+
 Cluster3Program build_cluster3(const HostLevel &L, bool band) {
+    g_program_builds++;
     Cluster3Program out;
     out.band = band;
     if (L.dim != 3) return out;
@@ -176,11 +207,12 @@ Cluster3Program build_cluster3(const HostLevel &L, bool band) {
     auto is_ghost = [&](int64_t p) { return (L.type[p] & NODE_KIND) == NODE_GHOST; };
     // order of a rank's own nodes: inside, then ghosts (zone ones last)
     auto klass = [](const Node &x) { return x.q < 0 ? 0 : x.inzone ? 2 : 1; };
-    for (int r = 0; r < C3_RANKS; r++)
+    for_each_index(C3_RANKS, N.size() / 4096, [&](int r) {
         std::sort(N.begin() + start[r], N.begin() + start[r + 1], [&](const Node &x, const Node &y) {
             const int a = klass(x), b = klass(y);
             return a != b ? a < b : x.p < y.p;
         });
+    });
     struct Entry {
         int32_t i;       // index in N
         uint8_t band, zone;
@@ -199,7 +231,7 @@ Cluster3Program build_cluster3(const HostLevel &L, bool band) {
     Cluster3Layout &y = out.lay;
     for (size_t i = 0; i < N.size(); i++) at.set(N[i].p, (int32_t)i);
     for (int r = 0; r < C3_RANKS; r++) slot.emplace_back(4 * (start[r + 1] - start[r]) + 16);
-    for_each_index(C3_RANKS, [&](int r) {
+    for_each_index(C3_RANKS, N.size() / 256, [&](int r) {
         Rank &K = R[r];
         const int32_t b0 = (int32_t)start[r], e0 = (int32_t)start[r + 1];
         NodeMap &S = slot[r];
@@ -326,7 +358,7 @@ Cluster3Program build_cluster3(const HostLevel &L, bool band) {
     y.copies = y.gst + 64 * y.max_g;
     y.stride = align16(y.copies + 4 * max_c);
     out.records.assign((size_t)C3_RANKS * y.stride, 0);
-    for_each_index(C3_RANKS, [&](int r) {
+    for_each_index(C3_RANKS, N.size() / 256, [&](int r) {
         const Rank &K = R[r];
         uint8_t *rec = out.records.data() + (size_t)r * y.stride;
         int32_t *h = reinterpret_cast<int32_t *>(rec);
@@ -390,6 +422,7 @@ Cluster3Program build_cluster3(const HostLevel &L, bool band) {
 }
 
 Sweep3Program build_sweep3(const HostLevel &L, int blocks) {
+    g_program_builds++;
     Sweep3Program out;
     if (L.dim != 3 || blocks < 1) return out;
     std::vector<Node> N;
@@ -415,15 +448,14 @@ Sweep3Program build_sweep3(const HostLevel &L, int blocks) {
     bisect(N, tmp, 0, N.size(), blocks, 0, start);
     NodeMap at(N.size());   // updated node -> index in N
     std::vector<int32_t> base(blocks + 1, 0);
-    for (int r = 0; r < blocks; r++) {
+    for_each_index(blocks, N.size() / 4096, [&](int r) {
         std::sort(N.begin() + start[r], N.begin() + start[r + 1], [](const Node &x, const Node &y) {
             const int a = x.q < 0 ? x.black : 2, b = y.q < 0 ? y.black : 2;
             return a != b ? a < b : x.p < y.p;
         });
-        int ni = 0;
-        for (size_t i = start[r]; i < start[r + 1]; i++) ni += N[i].q < 0;
-        base[r + 1] = base[r] + ni;
-    }
+        for (size_t i = start[r]; i < start[r + 1]; i++) base[r + 1] += N[i].q < 0;
+    });
+    for (int r = 0; r < blocks; r++) base[r + 1] += base[r];
     std::vector<int32_t> cid(N.size(), -1);   // place of an inside node in the compact array
     for (int r = 0; r < blocks; r++)
         for (size_t i = start[r]; i < start[r + 1]; i++) {
@@ -504,7 +536,7 @@ Sweep3Program build_sweep3(const HostLevel &L, int blocks) {
                 for (int k = 0; k < m; k++) touch(rd[k]);
             }
     };
-    for_each_index(blocks, work);
+    for_each_index(blocks, N.size() / 256, work);
     Sweep3Layout &y = out.lay;
     y.blocks = blocks;
     y.inside = base[blocks];
@@ -557,7 +589,13 @@ Sweep3Program build_sweep3(const HostLevel &L, int blocks) {
                 g[((size_t)(a / 8) * y.max_g + k) * 8 + a % 8] =
                     (uint16_t)S.get(L.stn[(int64_t)K.gs_q[k] * KMAX + a], 0);
     };
-    for_each_index(blocks, write);
+    for_each_index(blocks, N.size() / 1024, write);
+    return out;
+}
+
+std::vector<Cluster3Program> build_cluster3_levels(const std::vector<HostLevel> &H, const std::vector<Cluster3Want> &want) {
+    std::vector<Cluster3Program> out(want.size());
+    for_each_index((int)want.size(), want.size(), [&](int i) { out[i] = build_cluster3(H[want[i].level], want[i].band); });
     return out;
 }
 

@@ -5,6 +5,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
 #include <vector>
 
 #include "gcmg_internal.h"
@@ -62,12 +63,23 @@ struct Cluster3Program {
 // slots do not fit 15 bits.
 Cluster3Program build_cluster3(const HostLevel &L, bool band);
 
+// Programs of several levels, built side by side on the host's threads.
+struct Cluster3Want {
+    int level;
+    bool band;
+};
+std::vector<Cluster3Program> build_cluster3_levels(const std::vector<HostLevel> &H, const std::vector<Cluster3Want> &want);
+
+// programs of either kind built on the host so far, by all contexts
+extern std::atomic<long long> g_program_builds;
+
 // Device copy of a program.
 struct Cluster3Dev {
     Cluster3Layout lay;
     uint8_t *records = nullptr;
     bool band = false;
     bool fits32 = false, fits64 = false;   // per precision: shared memory, and the cluster can be resident
+    bool stale = true;                     // to be built before the next relaxation that takes it
 };
 
 template <typename T>

@@ -170,7 +170,8 @@ Block2View<T> b2view(const Block2Dev &b, const LevelView<T> &v) {
 
 // Host geometry of a context's levels (no CUDA calls; thread safe): the
 // hierarchy of build_hierarchy plus the 2D boundary-block programs.
-void prepare_levels(const gcmg_params &p, const double *phi_host, std::vector<HostLevel> &H);
+void prepare_levels(const gcmg_params &p, const double *phi_host, std::vector<HostLevel> &H,
+                    const std::function<void()> &geometry_done = nullptr);
 // Validates p; GCMG_OK if usable.
 gcmg_status check_params(const gcmg_params &p);
 // Rebuilds (if out of date) and uploads the coarsest inverse; upload only.
@@ -183,6 +184,8 @@ void upload_inverse(gcmg_ctx *c);
 void coarse_prepare(gcmg_ctx *c);
 void launch_coarse_cycle(gcmg_ctx *c);
 // Creates a context from prepared levels (uploads everything to the current device).
-gcmg_status create_from_levels(const gcmg_params &p, std::vector<HostLevel> &&H, cudaStream_t stream, gcmg_ctx **out);
+struct Sweep3Builds;   // 3D: band-sweep programs being built (api.cu)
+gcmg_status create_from_levels(const gcmg_params &p, std::vector<HostLevel> &&H, cudaStream_t stream, gcmg_ctx **out,
+                               Sweep3Builds *sweeps = nullptr);
 
 }  // namespace gcmg

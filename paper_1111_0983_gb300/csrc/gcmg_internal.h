@@ -5,6 +5,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <functional>
 #include <string>
 #include <vector>
 
@@ -180,9 +181,12 @@ bool build_span_items(HostLevel &L, int C = 0, int seg = 0);
 
 // Builds all levels (throws GeomError).  phi: fine grid, n^dim values; h0:
 // fine spacing (0: 2 / (n - 1)); origin: coordinates of node 0 (null: -1 on
-// every axis).
+// every axis).  geometry_done is called once every level has its nodes, ghost
+// equations and lists, before the transfers between levels are built (which change
+// none of these).
 void build_hierarchy(int dim, int n, int n_coarse, const double *phi, double delta_over_h,
-                     std::vector<HostLevel> &levels, double h0 = 0.0, const double *origin = nullptr);
+                     std::vector<HostLevel> &levels, double h0 = 0.0, const double *origin = nullptr,
+                     const std::function<void()> &geometry_done = nullptr);
 // Partial-transfer weights (Sec. 2.5) at the fine image p of a coarse node over
 // the inside set (interior) or its complement; wt[3^dim], axis 0 slowest.
 bool partial_transfer_weights(const HostLevel &F, int64_t p, bool interior, double *wt);

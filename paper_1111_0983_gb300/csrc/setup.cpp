@@ -1244,7 +1244,8 @@ static void partial_weights_t(const HostLevel &F, int64_t p, T *w) {
 }
 
 void build_hierarchy(int dim, int n, int n_coarse, const double *phi, double delta_over_h,
-                     std::vector<HostLevel> &levels, double h0, const double *origin) {
+                     std::vector<HostLevel> &levels, double h0, const double *origin,
+                     const std::function<void()> &geometry_done) {
     if (!(h0 > 0.0)) h0 = 2.0 / (n - 1);
     levels.clear();
     int nl = 1;
@@ -1341,6 +1342,7 @@ void build_hierarchy(int dim, int n, int n_coarse, const double *phi, double del
         }
         levels.push_back(std::move(L));
     }
+    if (geometry_done) geometry_done();
     for (int l = 0; l + 1 < nl; l++) {
         build_extension(levels[l], levels[l + 1]);
         build_ghost_transfer(levels[l], levels[l + 1]);

@@ -103,6 +103,7 @@ def lib():
             "gcmg_fmg": (st, [vp, i32, vp]),
             "gcmg_reinit": (st, [i32, i32, vp, i32, vp, vp]),
             "gcmg_launch_counter": (i64, []),
+            "gcmg_program_build_counter": (i64, []),
             "gcmg_junction_zone": (st, [vp, i32, vp]),
             "gcmg_junction_solve_set": (st, [vp, i32, vp]),
             "gcmg_defect_noalloc": (st, [i32, i32, dbl, vp, vp, vp, i64, vp, vp, vp, vp, vp, C.POINTER(dbl), vp]),
@@ -381,6 +382,10 @@ class Solver:
 
 def launch_counter():
     return lib().gcmg_launch_counter()
+
+
+def program_build_counter():
+    return lib().gcmg_program_build_counter()
 
 
 def reinit(phi0, steps, stream=None):
