@@ -41,3 +41,34 @@ def test_sweep_launches_equal_one_grid(precision, n, nc, kw):
         assert torch.equal(u, runs[0][0])
         assert torch.equal(r, runs[0][2])
         np.testing.assert_array_equal(rel, runs[0][1])
+
+
+@pytest.mark.parametrize("precision,n,nc", [(0, 65, 17), (1, 65, 17), (0, 129, 17), (1, 129, 17)])
+def test_flat_domain_with_many_junctions(precision, n, nc):
+    """The same on a flat ellipsoid with a hole whose boundary changes type along
+    twelve curves (six sectors, another pattern below): the cluster programs on the
+    coarser levels, the band sweeps and the zone alone on the finer ones."""
+    from paper_1111_0983_gb300 import gcmg
+    x = np.linspace(-1.0, 1.0, n)
+    X, Y, Z = np.meshgrid(x, x, x, indexing="ij")
+    body = np.sqrt((X / 0.85) ** 2 + (Y / 0.7) ** 2 + (Z / 0.42) ** 2) - 1.0
+    phi = np.maximum(0.42 * body, 0.2 - np.sqrt((X - 0.1) ** 2 + (Y - 0.05) ** 2))
+    S = gcmg.Solver(phi, nc, precision=precision, rtol=1e-30, max_cycles=3)
+    for l in range(S.nlev):
+        B = S.ghosts(l)["B"]
+        S.set_bc_types(l, (np.sin(3 * np.arctan2(B[:, 1], B[:, 0]) + (B[:, 2] > 0)) > 0).astype(np.uint8))
+    rng = np.random.default_rng(n)
+    start = torch.from_numpy(rng.standard_normal((n,) * 3)).cuda()
+    start *= torch.from_numpy(S.node_types(0) & 3 > 0).cuda()
+    f = torch.from_numpy(rng.standard_normal((n,) * 3)).cuda()
+    g = torch.from_numpy(rng.standard_normal(S.num_ghosts(0))).cuda()
+    S.set_rhs(f, g)
+    runs = []
+    for mode in (0, 2):
+        S.set_boundary3d(mode)
+        u, r = torch.zeros_like(start), start.clone()
+        rel = S.solve(u)["rel"]
+        S.relax(0, r, f, g)
+        runs.append((u, rel, r))
+    assert torch.equal(runs[0][0], runs[1][0]) and torch.equal(runs[0][2], runs[1][2])
+    np.testing.assert_array_equal(runs[0][1], runs[1][1])
