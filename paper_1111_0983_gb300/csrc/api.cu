@@ -183,8 +183,7 @@ void upload_geometry(gcmg_ctx *c, int l) {
         // FP32 sweeps use strips of 8 rows (measured faster than the tiles on
         // every level: 4097^2 fine level 2.9 TB/s against 1.42, 1025^2 7.3 us
         // against 9.4); FP64 sweeps, bound by the FP64 pipe, keep the tiles
-        const std::vector<int32_t> st = strips_for(L, 8);
-        g.strip_rows = 8;
+        const std::vector<int32_t> st = strips_for(L, STRIP_ROWS);
         g.nstrips = (int)st.size();
         g.strips = upload<int32_t>(c, st.data(), st.size());
     }
@@ -391,7 +390,7 @@ T *relax(gcmg_ctx *c, LevelView<T> v, T *out, T *wb, int l, bool extra) {
     // 2D: the interior sweep, the ghost sweep and the band sweeps in one launch
     // (strips and boundary blocks both read v.u, write out); the blocks store
     // straight into out, so no write-back is pending
-    if (dim == 2 && extra && c->p.smoother == 0 && g.nstrips > 0 && g.strip_rows == 8 && g.b2.m > 0) {
+    if (dim == 2 && extra && c->p.smoother == 0 && g.nstrips > 0 && g.b2.m > 0) {
         // algorithmic bytes: the interior sweep's (u, f read and u written
         // once per inside node) and the boundary blocks' distinct values
         const double bytes = c->timing_kind >= 0

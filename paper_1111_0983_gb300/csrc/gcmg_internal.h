@@ -15,6 +15,7 @@ namespace gcmg {
 
 constexpr int KMAX = 27;   // ghost stencil slots (3^3)
 constexpr int STRIP_W = 60; // 2D sweep strips: owned columns (a warp holds 64)
+constexpr int STRIP_ROWS = 8; // and rows (a batch takes others too)
 constexpr int TILE_R = 16; // 2D interior tiles: rows (axis 0)
 constexpr int TILE_C = 64; //                    columns (axis 1, contiguous)
 constexpr int EMAX = 6;    // extension sources (2 d)
@@ -275,8 +276,8 @@ struct DevGeom {
     int32_t *red_src = nullptr;  // 3D: HostLevel::band_red_src
     int ntiles = 0;
     int32_t *tiles = nullptr;    // active 2D interior tiles
-    int nstrips = 0, strip_rows = 0;
-    int32_t *strips = nullptr;   // active 2D sweep strips (strip_rows x STRIP_W owned nodes)
+    int nstrips = 0;
+    int32_t *strips = nullptr;   // active 2D sweep strips (STRIP_ROWS x STRIP_W owned nodes)
     int nzm = 0;                 // 3D fused-sweep work items (HostLevel::zm pairs)
     int32_t *zm = nullptr;
     int32_t *zm_moff = nullptr;  // and their inside-node masks

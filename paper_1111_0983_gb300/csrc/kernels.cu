@@ -1243,10 +1243,9 @@ __global__ void k_descend_partial(LevelView<T> F, LevelView<T> C, T *__restrict_
 // 3D descent, coarse ghost rows (extension + partial transfer at coarse ghost
 // q as one sparse row over the fine ghost defects): a warp per row, the lanes
 // over every 32nd term, then a butterfly sum.  The fine ghost defects come
-// from rg[column] (FP32: computed once by k_ghost_defects) or, with GATHER,
-// from rg[gnode[column]] (FP64: the defect grid).
-template <typename T, bool GATHER>
-__global__ void k_ghost_rows(const T *__restrict__ rg, const int32_t *__restrict__ gnode, T *__restrict__ gc,
+// from the defect grid.
+template <typename T>
+__global__ void k_ghost_rows(const T *__restrict__ r, const int32_t *__restrict__ gnode, T *__restrict__ gc,
                              const int32_t *__restrict__ ptr, const int32_t *__restrict__ col,
                              const T *__restrict__ val, int nrows) {
     if (sizeof(T) == 4) pdl_trigger();
@@ -1255,19 +1254,9 @@ __global__ void k_ghost_rows(const T *__restrict__ rg, const int32_t *__restrict
     if (q >= nrows) return;   // uniform over the warp
     T s = 0;
     const int end = ptr[q + 1];
-    for (int j = ptr[q] + lane; j < end; j += 32) s = fma(val[j], rg[GATHER ? gnode[col[j]] : col[j]], s);
+    for (int j = ptr[q] + lane; j < end; j += 32) s = fma(val[j], r[gnode[col[j]]], s);
     for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
     if (lane == 0) gc[q] = s;
-}
-
-// g - L_G u at every ghost of a level into v.gtmp (free between
-// relaxations), for the 3D FP32 descent
-template <typename T, int K>
-__global__ void k_ghost_defects(LevelView<T> v) {
-    pdl_trigger();
-    pdl_wait();
-    const int q = blockIdx.x * blockDim.x + threadIdx.x;
-    if (q < v.ng) v.gtmp[q] = ghost_defect<T, K>(v, q);
 }
 
 template <typename T, int D>
@@ -1339,7 +1328,7 @@ void launch_rb(const LevelView<T> &v, int dim, int color, cudaStream_t s) {
 // (one a warp), the others a boundary block each.  Both read the grid before
 // the relaxation and store disjoint nodes of `out`, so nothing is written twice
 // and no CTA reads what another writes.
-template <typename T, int SR, int NT, int M>
+template <typename T, int NT, int M>
 __global__ void __launch_bounds__(NT, M == 1 ? 2 : 1)
     k_relax2d(LevelView<T> v, T *__restrict__ out, const int32_t *__restrict__ strips, int ns, int nsc,
               Block2View<T> J, int lambda, T *__restrict__ z) {
@@ -1348,27 +1337,27 @@ __global__ void __launch_bounds__(NT, M == 1 ? 2 : 1)
         const int s = blockIdx.x * (NT / 32) + (threadIdx.x >> 5);
         const int32_t st = s < ns ? strips[s] : 0;   // static: read before the wait
         pdl_wait();
-        if (s < ns) rb_strip<T, SR, true>(v, out, st, z);   // uniform over the warp
+        if (s < ns) rb_strip<T, STRIP_ROWS, true>(v, out, st, z);   // uniform over the warp
         return;
     }
     block2<T, NT, M>(J, v.u, out, z, (int)blockIdx.x - nsc, lambda);
 }
 
 // the blocks, after the CTAs of the first ns strips (0: the blocks alone)
-template <typename T, int SR, int NT, int M>
+template <typename T, int NT, int M>
 void launch_relax2d_as(cudaStream_t s, const LevelView<T> &v, T *out, const DevGeom &g, int ns, const Block2View<T> &J,
                        int lambda, T *z) {
     const int nsc = (ns + NT / 32 - 1) / (NT / 32);
-    pdl_launch(k_relax2d<T, SR, NT, M>, dim3((unsigned)(nsc + J.p.ncomp)), dim3(NT), block2_smem<T>(J.p), s, v, out,
+    pdl_launch(k_relax2d<T, NT, M>, dim3((unsigned)(nsc + J.p.ncomp)), dim3(NT), block2_smem<T>(J.p), s, v, out,
                g.strips, ns, nsc, J, lambda, z);
 }
 
 template <typename T>
 void launch_relax2d_strips(cudaStream_t s, const LevelView<T> &v, T *out, const DevGeom &g, int ns,
                            const Block2View<T> &J, int lambda, T *z) {
-    if (J.p.nt == 512) launch_relax2d_as<T, 8, 512, 2>(s, v, out, g, ns, J, lambda, z);
-    else if (J.p.m == 2) launch_relax2d_as<T, 8, 256, 2>(s, v, out, g, ns, J, lambda, z);
-    else launch_relax2d_as<T, 8, 256, 1>(s, v, out, g, ns, J, lambda, z);
+    if (J.p.nt == 512) launch_relax2d_as<T, 512, 2>(s, v, out, g, ns, J, lambda, z);
+    else if (J.p.m == 2) launch_relax2d_as<T, 256, 2>(s, v, out, g, ns, J, lambda, z);
+    else launch_relax2d_as<T, 256, 1>(s, v, out, g, ns, J, lambda, z);
 }
 
 template <typename T>
@@ -1388,9 +1377,8 @@ __global__ void __launch_bounds__(128) k_rb_strip(LevelView<T> v, T *__restrict_
     if (s < ns) rb_strip<T, SR, INTERIOR_ONLY>(v, out, strips[s], z);   // uniform over the warp
 }
 
-template <int SR>
 static void launch_strips_interior(const LevelView<float> &v, float *out, const DevGeom &g, float *z, cudaStream_t s) {
-    pdl_launch(k_rb_strip<float, SR, true>, dim3((unsigned)((g.nstrips + 3) / 4)), dim3(128), 0, s, v, out, g.strips,
+    pdl_launch(k_rb_strip<float, STRIP_ROWS, true>, dim3((unsigned)((g.nstrips + 3) / 4)), dim3(128), 0, s, v, out, g.strips,
                g.nstrips, z);
 }
 
@@ -1403,7 +1391,7 @@ void launch_relax2d_split(const LevelView<float> &v, float *out, const DevGeom &
     cudaEventRecord(fork, s);
     cudaStreamWaitEvent(side, fork, 0);
     launch_relax2d_strips<float>(side, v, out, g, 0, J, lambda, z);
-    launch_strips_interior<8>(v, out, g, z, s);
+    launch_strips_interior(v, out, g, z, s);
     cudaEventRecord(join, side);
     cudaStreamWaitEvent(s, join, 0);
 }
@@ -1413,9 +1401,7 @@ void launch_rb_strip(const LevelView<T> &v, T *out, const DevGeom &g, cudaStream
     if (g.nstrips <= 0) return;
     g_launches++;
     const dim3 grid((unsigned)((g.nstrips + 3) / 4));
-    if (g.strip_rows == 32) pdl_launch(k_rb_strip<T, 32>, grid, dim3(128), 0, s, v, out, g.strips, g.nstrips, (T *)nullptr);
-    else if (g.strip_rows == 16) pdl_launch(k_rb_strip<T, 16>, grid, dim3(128), 0, s, v, out, g.strips, g.nstrips, (T *)nullptr);
-    else pdl_launch(k_rb_strip<T, 8>, grid, dim3(128), 0, s, v, out, g.strips, g.nstrips, (T *)nullptr);
+    pdl_launch(k_rb_strip<T, STRIP_ROWS>, grid, dim3(128), 0, s, v, out, g.strips, g.nstrips, (T *)nullptr);
 }
 
 template <typename T>
@@ -1697,16 +1683,16 @@ void launch_descend(const LevelView<T> &F, const LevelView<T> &C, const DevGeom 
                     T *uc, cudaStream_t s, const T *pt_w) {
     // 3D: a thread a node of the coarse chunks; 2D: a warp per coarse ghost row, two per coarse segment
     const int64_t n = gf.dim == 3 ? level_threads(C, true) : 64 * (int64_t)C.nsegs + 32 * (int64_t)C.ng;
-    if (gf.dim == 3 && F.nsegs > 0) {
-        // 3D with row segments: one defect pass first (inside nodes over the
-        // segments, then the ghosts), so that each fine defect is computed
-        // once rather than once per coarse node whose 27-node neighbourhood
-        // holds it (27/8 times on average); the same values as on the spot
+    if (gf.dim == 3) {
+        // one defect pass first (inside nodes over the segments, and the
+        // ghosts), so that each fine defect is computed once rather than once
+        // per coarse node whose 27-node neighbourhood holds it (27/8 times on
+        // average); the same values as on the spot
         launch_defect_rows<T, 3, 4, false>(F, nullptr, nullptr, nullptr, nullptr, s);
         if (C.ng > 0) {
             g_launches++;
-            pdl_launch(k_ghost_rows<T, true>, dim3(blocks_for(32 * (int64_t)C.ng)), dim3(kThreads), 0, s,
-                       (const T *)F.r, F.gnode, gc, gf.gt_ptr, gf.gt_col, gt_val, C.ng);
+            pdl_launch(k_ghost_rows<T>, dim3(blocks_for(32 * (int64_t)C.ng)), dim3(kThreads), 0, s, (const T *)F.r,
+                       F.gnode, gc, gf.gt_ptr, gf.gt_col, gt_val, C.ng);
         }
         // the coarse nodes of full weighting first, then those whose fine
         // neighbourhood is partly outside
@@ -1720,26 +1706,11 @@ void launch_descend(const LevelView<T> &F, const LevelView<T> &C, const DevGeom 
         }
         return;
     }
-    constexpr bool from_r = sizeof(T) == 8;   // FP64: one defect pass first (see descend_item)
+    constexpr bool from_r = sizeof(T) == 8;   // FP64: one defect pass first (see descend_node)
     if (from_r) launch_defect<T>(F, gf.dim, false, nullptr, s);
-    if (gf.dim == 3 && C.ng > 0) {
-        // 3D: the fine ghost defects once (FP32: into F.gtmp; FP64: the
-        // defect pass above), then the coarse ghost rows a warp each
-        if (!from_r && F.ng > 0) {
-            g_launches++;
-            pdl_launch(k_ghost_defects<T, 27>, dim3(blocks_for(F.ng)), dim3(kThreads), 0, s, F);
-        }
-        g_launches++;
-        pdl_launch(k_ghost_rows<T, from_r>, dim3(blocks_for(32 * (int64_t)C.ng)), dim3(kThreads), 0, s,
-                   (const T *)(from_r ? F.r : F.gtmp), F.gnode, gc, gf.gt_ptr, gf.gt_col, gt_val, C.ng);
-    }
     g_launches++;
-    if (gf.dim == 2)
-        pdl_launch(k_descend<T, 2, from_r>, dim3(blocks_for(n)), dim3(kThreads), 0, s, F, C, fc, gc, uc, gf.gt_ptr, gf.gt_col, gt_val,
-                   false);
-    else
-        pdl_launch(k_descend<T, 3, from_r>, dim3(blocks_for(n)), dim3(kThreads), 0, s, F, C, fc, gc, uc, gf.gt_ptr, gf.gt_col, gt_val,
-                   false);
+    pdl_launch(k_descend<T, 2, from_r>, dim3(blocks_for(n)), dim3(kThreads), 0, s, F, C, fc, gc, uc, gf.gt_ptr, gf.gt_col, gt_val,
+               false);
 }
 
 template <typename T>

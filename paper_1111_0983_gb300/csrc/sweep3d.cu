@@ -23,11 +23,6 @@ using namespace dev;
 
 constexpr int S3_THREADS = 256;
 
-__device__ __forceinline__ void cp_async16(void *smem, const void *gmem) {
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(smem)), "l"(gmem)
-                 : "memory");
-}
-
 // xin: compact values of the updated inside nodes (null: from u), gin: the
 // ghosts' values; xout, gout: where the own new values go (null: into u, which
 // the launch then reads at nodes that no block updates only)
