@@ -180,9 +180,10 @@ void upload_geometry(gcmg_ctx *c, int l) {
     g.ntiles = (int)L.tiles.size();
     g.tiles = upload<int32_t>(c, L.tiles.data(), L.tiles.size());
     if (L.dim == 2) {
-        // FP32 sweeps use strips of 8 rows (measured faster than the tiles on
-        // every level: 4097^2 fine level 2.9 TB/s against 1.42, 1025^2 7.3 us
-        // against 9.4); FP64 sweeps, bound by the FP64 pipe, keep the tiles
+        // strips of 8 rows: in the merged relaxation of both precisions, and the
+        // FP32 sweeps by themselves (measured faster than the tiles on every
+        // level: 4097^2 fine level 2.9 TB/s against 1.42, 1025^2 7.3 us against
+        // 9.4); an FP64 sweep by itself, bound by the FP64 pipe, keeps the tiles
         const std::vector<int32_t> st = strips_for(L, STRIP_ROWS);
         g.nstrips = (int)st.size();
         g.strips = upload<int32_t>(c, st.data(), st.size());

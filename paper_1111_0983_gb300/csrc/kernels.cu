@@ -1316,14 +1316,6 @@ void launch_rb(const LevelView<T> &v, int dim, int color, cudaStream_t s) {
     else pdl_launch(k_rb_interior<T, 3>, dim3(blocks_for((int64_t)v.n * v.n * hc)), dim3(kThreads), 0, s, v, color);
 }
 
-// One FP32 2D relaxation in one launch: the first nsc CTAs sweep the strips
-// (one a warp) and store the inside nodes outside the band; the others run
-// the boundary blocks from the same grid v.u -- each block first takes the
-// interior sweep over what it reads, then the ghost sweep and the band
-// sweeps -- and store their band nodes and ghosts.  Every CTA reads only
-// v.u and the stored node sets are disjoint, so nothing is written twice and
-// no CTA reads a value another one writes.
-// EPT: inside entries per thread and colour the boundary blocks need
 // One 2D relaxation up to the band sweeps: the first nsc CTAs take the strips
 // (one a warp), the others a boundary block each.  Both read the grid before
 // the relaxation and store disjoint nodes of `out`, so nothing is written twice

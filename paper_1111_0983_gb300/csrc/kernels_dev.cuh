@@ -15,12 +15,6 @@ namespace dev {
 constexpr int LOCAL_THREADS = 512;
 constexpr int LOCAL_EPT = 4;     // inside entries per thread and colour in local programs (at most)
 
-// max-norm reduction on the bit pattern of a non-negative double (monotone
-// for non-negative IEEE values); NaN is folded into +Inf so that it is seen.
-// waits for the preceding kernel of the stream (programmatic dependent launch;
-// a no-op when the kernel was launched without it).  No kernel triggers its
-// dependents early: measured, a 1025^2 solve went from 4.84 to 5.13 ms when
-// every kernel did, the waiting CTAs taking SM slots from the running grid.
 // asynchronous global -> shared copy of one word (4 or 8 bytes): no register
 // holds it and the issuing thread does not wait for it
 template <typename W>
@@ -40,12 +34,17 @@ __device__ __forceinline__ void cp_async16(void *smem, const void *gmem) {
 // waits until this thread's asynchronous copies have landed (and are visible to it)
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
+// waits for the preceding kernel of the stream (programmatic dependent launch;
+// a no-op when the kernel was launched without it)
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 // lets the launch that depends on this grid start its CTAs now: they run
 // whatever precedes their pdl_wait (reads of data no launch writes) while
-// this grid works
+// this grid works.  The FP32 kernels of the cycle do; the FP64 ones do not, whose
+// waiting CTAs would take SM slots from the running grid
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
+// max-norm reduction on the bit pattern of a non-negative double (monotone
+// for non-negative IEEE values); NaN is folded into +Inf so that it is seen.
 __device__ __forceinline__ void atomic_max_abs(unsigned long long *bits, double v) {
     v = fabs(v);
     if (v != v) v = __longlong_as_double(0x7ff0000000000000ll);
@@ -669,8 +668,6 @@ __device__ __forceinline__ void local_copyback(const LocalView<T> &J, T *u, int 
 }
 
 // ------------------------------------------------------------------ defect
-// r = f + Lap_h u at inside node p (TGCS step 3), as a sum of differences so
-// that the O(u / h^2) terms do not cancel; with zero_rest, 0 at outside nodes.
 // The numerator sum_k u_k - 2d u_p of the 5/7-point Laplacian at inside node
 // p (neighbours in the order x-1, x+1, then the two slower axes).  FP32: the
 // sum of differences.  FP64: the exact integer sum of exact_lap.h rounded
@@ -696,6 +693,8 @@ __device__ __forceinline__ T lap_numerator(const LevelView<T> &v, int64_t p, T u
     return lap;
 }
 
+// r = f + Lap_h u at inside node p (TGCS step 3), as a sum of differences so
+// that the O(u / h^2) terms do not cancel; with zero_rest, 0 at outside nodes.
 // Returns the defect (0 off Omega_h) for the norm.
 template <typename T, int D>
 __device__ __forceinline__ double defect_node(const LevelView<T> &v, int64_t p, bool zero_rest) {
