@@ -406,9 +406,9 @@ gcmg_status gcmg_span3d_info(const gcmg_ctx *ctx, int l, int *items, int *column
 int64_t gcmg_launch_counter(void);
 
 /* Number of 3D launch programs (cluster programs and band-sweep blocks, launch
- * mode 0 of gcmg_set_boundary3d) built on the host in the process so far: one a
- * level at creation or before its first relaxation, again after its boundary
- * types changed. */
+ * mode 0 of gcmg_set_boundary3d) built on the host in the process so far: blocks
+ * at creation, a cluster program whenever its level's boundary types are set (or
+ * before the first relaxation, if they never are). */
 int64_t gcmg_program_build_counter(void);
 
 /* ---- batched solves of many domains (not in the paper).

@@ -1407,7 +1407,8 @@ gcmg_status gcmg_set_bc_types(gcmg_ctx *c, int l, const uint8_t *types) {
             upload_program(c, L.junction, c->G[l].jz);
             check_program_fits(c, c->G[l].jz);
         }
-        if (!c->c3.empty() && !c->p.junction_solve) c->c3[l].stale = true;   // its zone changed; rebuilt before it runs
+        if (!c->c3.empty() && !c->p.junction_solve) c->c3[l].stale = true;   // its zone changed
+        if (l + 1 < (int)c->H.size()) ensure_cluster3(c, l, l + 1);
         upload_ghost_data<double>(c, l, c->D64[l], false);
         if (!c->D32.empty()) upload_ghost_data<float>(c, l, c->D32[l], false);
         return GCMG_OK;

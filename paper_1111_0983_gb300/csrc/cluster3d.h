@@ -79,7 +79,7 @@ struct Cluster3Dev {
     uint8_t *records = nullptr;
     bool band = false;
     bool fits32 = false, fits64 = false;   // per precision: shared memory, and the cluster can be resident
-    bool stale = true;                     // to be built before the next relaxation that takes it
+    bool stale = true;                     // out of date with the boundary types
 };
 
 template <typename T>
