@@ -192,8 +192,10 @@ __device__ __forceinline__ void mbar_expect(uint32_t mbar, uint32_t bytes) {
 // in flight: three of six slots at small dilations, two of five at 81.
 // Measured, 8 images of 513^2, 32 -> 32 channels, forward: 366 us a layer with
 // three segments a tile, one accumulator and the border's tiles computed too;
-// 81-96 us so (2.9-3.4 TB/s of activations read and written once).  Backward to
-// the input 721 -> 124-149 us (reads the gate too).
+// 76-94 us so (2.9-3.6 TB/s of activations read and written once).  Backward to
+// the input 721 -> 101-123 us (reads the gate too).  Counters of a forward layer
+// (4 images): shared memory 64 % (the operands, read again for each tap), tensor
+// pipe 21 %, DRAM 31 %, L2 20 %.
 template <int GIN, int NOUT, int MODE>
 __global__ void __launch_bounds__(kConvThreads) k_conv(ConvArgs a) {
     extern __shared__ __align__(128) unsigned char smem[];
@@ -405,12 +407,14 @@ __global__ void __launch_bounds__(kConvThreads) k_conv(ConvArgs a) {
 // operand, whatever N.  A slot holds tap row (slot - first position) mod 4 of
 // the tile, so the accumulators are kept per class = first position mod 4; the
 // class's fourth slot (being loaded, or of the next item) yields rows nobody
-// reads.  Pixels past the image's last column are staged as zeros.  Not bound by the
-// one x segment in flight (the ring's fourth slot): three chains a CTA, each with
-// a ring, and five gradient stages measured 225 us where this form takes 195.
+// reads.  Pixels past the image's last column are staged as zeros.
 // Measured, 8 images of 513^2: 2469 us a layer with a tap and 16 pixels an MMA
-// and nothing staged ahead, 253 us with the ring and one MMA a tap column, 195
-// us with one MMA for the three.
+// and nothing staged ahead, 253 us with the ring and one MMA a tap column, 192
+// us with one MMA for the three.  Counters (4 images): no unit is busy -- tensor
+// pipe 10 %, its operand reads 11 %, shared memory 14 %, L2 13 %, DRAM 20 % -- and
+// the SMs' shares are uneven (608 MMAs on one, 446 on average): waits within the one
+// chain a CTA walks.  Three chains a CTA, each with a ring, and five gradient
+// stages measured 225 us all the same; why is open.
 struct DwArgs {
     const uint4 *dz;      // [GA][npix]
     const uint4 *x;       // [GB][npix]
