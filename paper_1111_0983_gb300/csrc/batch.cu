@@ -12,17 +12,15 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
-#include <atomic>
 #include <cmath>
 #include <cstring>
-#include <mutex>
 #include <new>
 #include <string>
-#include <thread>
 #include <vector>
 
 #include "ctx.h"
 #include "gcmg_internal.h"
+#include "host_threads.h"
 #include "kernels.h"
 #include "kernels_dev.cuh"
 
@@ -436,6 +434,8 @@ gcmg_status bfail(gcmg_batch *b, gcmg_status s, const std::string &m) {
         return bfail(b, GCMG_E_GEOM, g.msg);                                                     \
     } catch (const std::bad_alloc &) {                                                           \
         return bfail(b, GCMG_E_OOM, "allocation failed");                                        \
+    } catch (const std::exception &e) {                                                          \
+        return bfail(b, GCMG_E_ARG, e.what());                                                   \
     }
 
 void free_tables(gcmg_batch *b) {
@@ -883,22 +883,13 @@ gcmg_status gcmg_batch_create(int count, const gcmg_params *params, const double
         ck(cudaStreamSynchronize(b->stream), "sync");
         std::vector<std::vector<HostLevel>> H(count);
         std::vector<std::string> errs(count);
-        std::atomic<int> next{0};
-        const unsigned nt = std::max(1u, std::min(16u, std::thread::hardware_concurrency()));
-        std::vector<std::thread> pool;
-        for (unsigned t = 0; t < nt; t++)
-            pool.emplace_back([&]() {
-                for (int i = next++; i < count; i = next++) {
-                    try {
-                        prepare_levels(params[i], phi[i].data(), H[i]);
-                    } catch (const GeomError &g) {
-                        errs[i] = g.msg;
-                    } catch (const std::bad_alloc &) {
-                        errs[i] = "allocation failed";
-                    }
-                }
-            });
-        for (auto &t : pool) t.join();
+        for_each_index(count, 16, [&](int i) {
+            try {
+                prepare_levels(params[i], phi[i].data(), H[i]);
+            } catch (const GeomError &g) {
+                errs[i] = g.msg;
+            }
+        });
         for (int i = 0; i < count; i++)
             if (!errs[i].empty()) return bfail(b, GCMG_E_GEOM, "domain " + std::to_string(i) + ": " + errs[i]);
         for (int i = 0; i < count; i++) {
@@ -986,20 +977,13 @@ gcmg_status gcmg_batch_solve(gcmg_batch *b, gcmg_stats *stats, int *steps) {
             for (int d = 0; d < (int)b->doms.size(); d++)
                 if (b->doms[d]->H.back().ainv_dirty) dirty.push_back(d);
             std::vector<std::string> errs(dirty.size());
-            std::atomic<int> next{0};
-            const unsigned nt = std::max(1u, std::min(16u, std::thread::hardware_concurrency()));
-            std::vector<std::thread> pool;
-            for (unsigned t = 0; t < nt; t++)
-                pool.emplace_back([&]() {
-                    for (int i = next++; i < (int)dirty.size(); i = next++) {
-                        try {
-                            build_coarse_inverse(b->doms[dirty[i]]->H.back());
-                        } catch (const GeomError &g) {
-                            errs[i] = g.msg;
-                        }
-                    }
-                });
-            for (auto &t : pool) t.join();
+            for_each_index((int)dirty.size(), 16, [&](int i) {
+                try {
+                    build_coarse_inverse(b->doms[dirty[i]]->H.back());
+                } catch (const GeomError &g) {
+                    errs[i] = g.msg;
+                }
+            });
             for (size_t i = 0; i < dirty.size(); i++) {
                 if (!errs[i].empty()) return bfail(b, GCMG_E_GEOM, "domain " + std::to_string(dirty[i]) + ": " + errs[i]);
                 upload_inverse(b->doms[dirty[i]]);
@@ -1015,21 +999,14 @@ gcmg_status gcmg_batch_solve(gcmg_batch *b, gcmg_stats *stats, int *steps) {
                     if (c->H[l].js_dirty) dirty.push_back({d, l});
             }
             std::vector<std::string> errs(dirty.size());
-            std::atomic<int> next{0};
-            const unsigned nt = std::max(1u, std::min(16u, std::thread::hardware_concurrency()));
-            std::vector<std::thread> pool;
-            for (unsigned t = 0; t < nt; t++)
-                pool.emplace_back([&]() {
-                    for (int i = next++; i < (int)dirty.size(); i = next++) {
-                        gcmg_ctx *c = b->doms[dirty[i].first];
-                        try {
-                            build_junction_solve(c->H[dirty[i].second], c->p.junction_radius);
-                        } catch (const GeomError &g) {
-                            errs[i] = g.msg;
-                        }
-                    }
-                });
-            for (auto &t : pool) t.join();
+            for_each_index((int)dirty.size(), 16, [&](int i) {
+                gcmg_ctx *c = b->doms[dirty[i].first];
+                try {
+                    build_junction_solve(c->H[dirty[i].second], c->p.junction_radius);
+                } catch (const GeomError &g) {
+                    errs[i] = g.msg;
+                }
+            });
             for (size_t i = 0; i < dirty.size(); i++) {
                 const int d = dirty[i].first, l = dirty[i].second;
                 if (!errs[i].empty()) return bfail(b, GCMG_E_GEOM, "domain " + std::to_string(d) + ": " + errs[i]);

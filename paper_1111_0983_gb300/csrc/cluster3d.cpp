@@ -3,11 +3,11 @@
 #include "cluster3d.h"
 
 #include <algorithm>
-#include <atomic>
 #include <cstring>
 #include <exception>
-#include <mutex>
 #include <thread>
+
+#include "host_threads.h"
 
 namespace gcmg {
 
@@ -55,34 +55,6 @@ struct Node {
     int c[3];
     uint8_t black, inband, inzone;
 };
-
-// f(0) .. f(n - 1), independent of each other, over at most `most` of the host's
-// threads (the work's share of one should outweigh its start); an exception of one (or of the creation of a thread) reaches the caller after all
-// threads have ended
-template <typename F>
-void for_each_index(int n, size_t most, F &&f) {
-    std::atomic<int> next{0};
-    std::mutex lock;
-    std::exception_ptr error;
-    auto work = [&]() {
-        try {
-            for (int i = next++; i < n; i = next++) f(i);
-        } catch (...) {
-            next = n;
-            std::lock_guard<std::mutex> g(lock);
-            if (!error) error = std::current_exception();
-        }
-    };
-    std::vector<std::thread> pool;
-    try {
-        const unsigned nt = std::min({(unsigned)std::min<size_t>(most, 16), (unsigned)n, std::thread::hardware_concurrency()});
-        for (unsigned t = 1; t < nt; t++) pool.emplace_back(work);
-    } catch (...) {   // fewer threads then
-    }
-    work();
-    for (auto &t : pool) t.join();
-    if (error) std::rethrow_exception(error);
-}
 
 // f and g, at the same time if `apart` (and a thread can be had); an exception of
 // either reaches the caller after both have ended
