@@ -653,6 +653,7 @@ void build_tables(gcmg_batch *b) {
                 const DevGeom &g = c->G[l];
                 const DevData<float> &D = c->D32[l];
                 const HostLevel &L = c->H[l];
+                if (L.js_dirty) continue;   // rebuilt here, not yet there (a refused solve); a solve comes back with it
                 for (int cc = 0; cc < g.js_ncomp; cc++) {
                     const int o = L.js_off[cc], m_ = L.js_off[cc + 1] - o, mp = (m_ + 3) & ~3;
                     int mi = 0;

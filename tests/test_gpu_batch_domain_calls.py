@@ -44,3 +44,44 @@ def test_batch_after_calls_on_a_domain(kw):
             assert torch.equal(a, b)
         for a, b in zip(rels, rels2):
             np.testing.assert_array_equal(a, b)
+
+
+def test_batch_after_a_refused_solve():
+    """A solve that is refused for one domain's junction zone (beyond 4,096 nodes a
+    component) leaves the other's rebuilt on the host and not yet on the device; the
+    autotuner then takes neither, and the next solve is that of a new batch."""
+    from paper_1111_0983_gb300 import gcmg
+    sizes = (257, 65)
+    probs = [inputs.star(i, params=dict(inputs.star_params(i), n=n)) for i, n in zip((0, 1), sizes)]
+
+    def batch():
+        B = gcmg.Batch([P.phi_grid(n) for P, n in zip(probs, sizes)], 33, rtol=1e-10, junction_radius=64.0)
+        for S, P, n in zip(B.domains, probs, sizes):
+            G = S.ghosts(0)
+            g = P.g_values(G["B"], G["nu"], np.zeros(len(G["B"]), np.uint8))
+            S.set_rhs(torch.from_numpy(P.f_grid(n)).cuda(), torch.from_numpy(g).cuda())
+        return B
+
+    def mixed(S, on):   # types change across x = 0.05, or all Dirichlet
+        for l in range(S.nlev):
+            S.set_bc_types(l, ((S.ghosts(l)["B"][:, 0] > 0.05) & on).astype(np.uint8))
+
+    def solve(B):
+        B.solve()
+        us = [torch.zeros((n, n), dtype=torch.float64, device="cuda") for n in sizes]
+        for k, u in enumerate(us):
+            B.solution(k, u)
+        return us
+
+    B = batch()
+    mixed(B.domains[1], True)
+    solve(B)
+    mixed(B.domains[0], True)
+    mixed(B.domains[1], False)
+    with pytest.raises(gcmg.GcmgError, match="4096"):
+        B.solve()
+    B.autotune()
+    B.set_tiles(0)
+    mixed(B.domains[0], False)
+    for a, b in zip(solve(B), solve(batch())):
+        assert torch.equal(a, b)
