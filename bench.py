@@ -754,13 +754,13 @@ def run_gcmg(args):
     peak = peaks.get("hbm_gbs")
     # the interior sweep: both colours in one launch (2D strips / tiles, 3D
     # z-march) reading u and f and writing u once per inside node, plus in
-    # the merged FP32 2D relaxation the boundary blocks' values (the library
-    # gives those bytes)
+    # the merged 2D relaxation the boundary blocks' values (the library gives
+    # those bytes)
     elt = 4 if precision else 8
     alg_bytes = k_bytes / k_launches if k_launches and k_bytes > 0 else 3 * elt * n_in
     avg_ms = k_ms / max(k_launches, 1)
     achieved = alg_bytes / (avg_ms / 1e3) / 1e9 if k_launches else None
-    merged = P.dim == 2 and precision == 1 and b_launches > 0
+    merged = P.dim == 2 and b_launches > 0
     kern = ("relax2d" if merged else "fused2d") if P.dim == 2 else sweep3d_kernel(precision)[0]
     kname = f"rb_{kern}_{'f64' if precision == 0 else 'f32'}_{args.config}"
     kdesc = {"relax2d": "k_relax2d (fine level: interior sweep + ghost and band sweeps in one launch)",
@@ -779,7 +779,7 @@ def run_gcmg(args):
     if b_launches:
         bname = f"{'relax2d' if merged else 'local_bz'}_{'f64' if precision == 0 else 'f32'}_{args.config}"
         b_ach = (b_bytes / b_launches) / (b_ms / b_launches / 1e3) / 1e9 if b_ms > 0 else None
-        bdesc = ("k_relax2d (one FP32 relaxation: interior strips and boundary blocks in one launch, every level)"
+        bdesc = ("k_relax2d (one relaxation: interior strips and boundary blocks in one launch, every level)"
                  if merged else "k_local (2D boundary blocks: ghost sweep + lambda band sweeps in shared memory, "
                  "every level)")
         roofline = {"bound": "hbm", "kernel": bdesc, "achieved": b_ach, "peak": peak,
