@@ -528,7 +528,7 @@ def secondary(name, rtol, precision, args, stream, flush):
                 gbs = alg / (kms / kl / 1e3) / 1e9
                 peak = measured_peaks()[0].get("hbm_gbs")
                 kernel = (sweep3d_kernel(prec)[1] if P.dim == 3 else
-                          "k_rb_fused2d" if prec == 0 or kbytes <= 0 else
+                          "k_rb_fused2d" if kbytes <= 0 else
                           "k_relax2d (interior sweep + ghost and band sweeps)")
                 rec["fine_sweep"] = {"kernel": kernel, "alg_bytes_per_launch": alg,
                                      "avg_launch_ms": kms / kl, "achieved_GBs": gbs,
